@@ -132,15 +132,14 @@ typedef struct {
  * otherwise. Not for rg_render_batch's fused path (its plans take the lanes). */
 #define RG_FLAG_TILE_COUNTING_SORT (1u << 13)
 /* RoofGS: the fused front end with the ordered allocation (one contiguous run of entries
- * per block, 16-bit tile ids) and the two 8-bit radix passes over the tile id, instead of the
- * default row-bucketed front end. The row-bucketed front end (frames with an image, the
- * depth pre-sort and at most 256 x 256 tiles) runs a count kernel (the fused front end's
- * work without the emission), a per-tile-row scan of its block counts and a scatter kernel
- * that writes each Gaussian's tile-row runs straight into their tile row's part of the
- * entry array under the column-major key tx << 8 | ty; one 8-bit pass over the column then
- * groups the entries by tile. Both give the same entries per tile in the same order, hence
- * the same images; rg_inspect returns the entries in tile-id order either way. Other frames
- * always take the fused front end. */
+ * per block, 16-bit tile ids) and the radix passes over the tile bits, instead of the default:
+ * frames with the depth pre-sort and at most 512 x 512 tiles keep one run of tile columns per
+ * Gaussian and tile row, group the runs by tile row, and write every entry once, at its place
+ * in tile-id order (no entry keys, no radix pass). Both give the same entries per tile in the
+ * same order, hence the same images, and rg_inspect reports the same arrays. Other frames
+ * always take the fused front end. rg_stats.sort_passes reports one pass for a frame of runs
+ * with at most 256 x 256 tiles (the grouping by tile column), else the radix passes that it
+ * replaces. */
 #define RG_FLAG_ORDERED_FRONT_END (1u << 14)
 /* test hook for the failure path: the first radix pass of the entry sort never processes its
  * first tile, so the next tile's bounded look-back wait runs out (about a second); the frame
@@ -208,14 +207,12 @@ rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries);
  * precision and the quadratic form completed in dx, so the image stays within
  * 2e-4 per channel of an FP64 evaluation except where a pair's alpha or T lies
  * within rounding of the 1/255 or 1e-4 thresholds.
- * Pipeline (RoofGS): Gaussians ordered by quantized depth -> front end (by
- * default row-bucketed: the entries leave it grouped by tile row, in depth order)
- * -> stable radix sort of the remaining tile bits (one pass over the tile column;
- * two tile-bit passes after the fused front end of RG_FLAG_ORDERED_FRONT_END;
- * either way the order of the full 32-bit key; RG_FLAG_SORT_FULL_KEY sorts all
- * 32 bits in 4 passes instead) -> fast-exp rasterizer with 2 (dual-pixel), 1 or
- * 4 pixels per thread, each tile block finding its own range of the sorted
- * entries (Sec. IV).
+ * Pipeline (RoofGS): Gaussians ordered by quantized depth -> front end (one run of
+ * tile columns per Gaussian and tile row) -> grouping of the runs by tile, in depth
+ * order (the fused front end of RG_FLAG_ORDERED_FRONT_END and a stable radix sort of
+ * the tile bits instead; either way the order of the full 32-bit key;
+ * RG_FLAG_SORT_FULL_KEY sorts all 32 bits in 4 passes) -> fast-exp rasterizer with 2
+ * (dual-pixel), 1 or 4 pixels per thread (Sec. IV).
  * The number of entries stays on the device: with stats == NULL the call does
  * not synchronise; if the entries exceed the workspace the image is
  * incomplete and the overflow is recorded (see rg_scene_check). With stats
@@ -247,12 +244,11 @@ rg_status rg_stage_times(rg_scene* scene, float* ms7, int32_t* frames);
 
 /* rg_inspect selectors: copy internal buffers of the last frame to host memory */
 #define RG_INSPECT_KEYS 1        /* sorted keys: uint32 (RoofGS) or uint64 (exact), n_entries of them;
-                                    RoofGS frames with at most 16 tile bits sort 16-bit tile keys and
-                                    the 32-bit keys (tile << b_d | q_d) are rebuilt on the host from
-                                    the values and the per-Gaussian depth codes; the entries of a
-                                    row-bucketed frame (column-major tile keys) are first regrouped in
-                                    tile-id order from the tile ranges, so every frame reports the
-                                    order of the 32-bit key */
+                                    RoofGS frames of tile-row runs (the default) keep no keys, and those
+                                    that sort at most 16 tile bits keep 16-bit tile ids: the 32-bit keys
+                                    (tile << b_d | q_d) are rebuilt on the host from the tile ranges or
+                                    ids, the values and the per-Gaussian depth codes, so every frame
+                                    reports the order of the 32-bit key */
 #define RG_INSPECT_VALUES 2      /* sorted values: uint32 Gaussian indices (in the same order) */
 #define RG_INSPECT_RANGES 3      /* uint32 [tiles][2] = [start, end) per tile (of the same order) */
 #define RG_INSPECT_SH_CODES 4    /* int8 [n][16][3] compact SH codes */

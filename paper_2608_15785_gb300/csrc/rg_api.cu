@@ -114,43 +114,64 @@ rg_status make_layout(const rg_camera* c, FrameLayout& f, int tw, int th)
 // one device word set from the stream (test hook of RG_FLAG_TEST_STALL_SORT)
 __global__ void k_set_word(unsigned* p, unsigned v) { *p = v; }
 
-// the row-bucketed front end's buffer for n slots: rows per slot (4 B, padded to 16 B), the
-// row tests (3 x 16 B per slot), the per-block counts of up to 256 tile rows, the row totals
-size_t row_buffer_bytes(int64_t n)
+// entries (8 B each) the key buffers are sized for: the capacity, and the runs of an ordinary frame
+// when a small capacity was asked for (so that an overflowed frame still has all its runs)
+int64_t key_items(int64_t n_gauss, int64_t cap) { return std::max(cap, std::min<int64_t>(4 * n_gauss, MAX_CAP)); }
+
+// frames whose entries are written from tile-row runs (runs.cu)
+bool runs_possible(const Layout& L, int64_t n)
 {
-    const size_t nb = (size_t)((n + frontend_block_threads() - 1) / frontend_block_threads());
-    return ((size_t)n * 4 + 15) / 16 * 16 + (size_t)n * 48 + (size_t)256 * nb * 4 + 256 * 8;
+    return n > 0 && L.tiles_x <= RUN_MAX_GRID && L.tiles_y <= RUN_MAX_GRID;
 }
 
-// points the row-bucketed front end's arrays of a into w.rowbuf (n = a.n slots)
-void row_buffer_views(Workspace& w, FrontendArgs& a)
+// Arguments of runs.cu for a frame on workspace w: the runs live in the key buffers (list in
+// keys[0], the blocks' runs in keys[1]), the rest in runbuf. Returns the bytes of runbuf the frame
+// needs; the pointers are valid if runbuf has them.
+size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
 {
-    const size_t n = (size_t)a.n;
-    unsigned char* p = w.rowbuf.as<unsigned char>();
-    a.row_n = reinterpret_cast<unsigned*>(p);
-    p += (n * 4 + 15) / 16 * 16;
-    a.row_rt = reinterpret_cast<float4*>(p);
-    p += n * 48;
-    const size_t nb = (n + frontend_block_threads() - 1) / frontend_block_threads();
-    a.row_cnt = reinterpret_cast<unsigned*>(p);
-    p += (size_t)256 * nb * 4;
-    a.row_tot = reinterpret_cast<unsigned long long*>(p);
+    memset(&a, 0, sizeof(a));
+    a.rows = L.tiles_y;
+    a.cols = L.tiles_x;
+    a.blocks = (unsigned)((n + RUN_SLOTS - 1) / RUN_SLOTS);
+    a.run_cap = (unsigned)key_items(n, w.cap);
+    a.chunk_cap = run_chunk_cap(a.run_cap, a.rows, a.blocks);
+    a.cap = w.cap;
+    a.list = w.keys[0].as<uint2>();
+    a.runs = w.keys[1].as<unsigned>();
+    a.vals = w.vals[0].as<unsigned>();
+    a.ranges = w.ranges.as<uint2>();
+    a.ctr = w.ctrl.as<Counters>();
+    unsigned char* const p = w.runbuf.as<unsigned char>();
+    size_t at = 0;
+    auto part = [&](size_t bytes) {
+        unsigned char* q = p + at;
+        at += (bytes + 255) / 256 * 256;
+        return q;
+    };
+    const size_t per_row = (size_t)a.rows * a.blocks * 4;
+    a.cnt = reinterpret_cast<unsigned*>(part(per_row));
+    a.seg = reinterpret_cast<unsigned*>(part(per_row));
+    a.pre = reinterpret_cast<unsigned*>(part(per_row));
+    if (a.blocks <= RUN_SMALL_BLOCKS)
+        a.tot = reinterpret_cast<unsigned long long*>(w.ctrl.as<unsigned char>() + RUN_TOT_AT);
+    a.chunk = reinterpret_cast<RunChunk*>(part((size_t)a.chunk_cap * sizeof(RunChunk)));
+    a.row = reinterpret_cast<RunRow*>(part((size_t)a.rows * sizeof(RunRow)));
+    a.col = reinterpret_cast<unsigned*>(part((size_t)a.chunk_cap * run_pitch(a.cols) * 4));
+    return at;
 }
 
-rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, int tiles, int64_t cap)
+rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameLayout& F, int64_t cap)
 {
     const int64_t n = n_gauss > 0 ? n_gauss : 1;
     if (cap > MAX_CAP) return fail(RG_ERR_CAPACITY, "entry capacity above 2^30 - 1");
-    if (cap > w.cap || !w.keys[0].p) {
-        for (int k = 0; k < 2; k++) {
-            RG_TRY(ensure(w.keys[k], (size_t)cap * 8, "keys"));
-            RG_TRY(ensure(w.vals[k], (size_t)cap * 4, "values"));
-        }
+    for (int k = 0; k < 2; k++) RG_TRY(ensure(w.keys[k], (size_t)key_items(n, std::max(cap, w.cap)) * 8, "keys"));
+    if (cap > w.cap || !w.vals[0].p) {
+        for (int k = 0; k < 2; k++) RG_TRY(ensure(w.vals[k], (size_t)cap * 4, "values"));
         const int64_t max_tiles = (cap + sort_tile_items() - 1) / sort_tile_items();
         for (int k = 0; k < 2; k++) RG_TRY(ensure(w.sort_status[k], (size_t)max_tiles * 256 * 4, "sort status"));
         w.cap = cap;
     }
-    RG_TRY(ensure(w.ranges, (size_t)tiles * sizeof(uint2), "ranges"));
+    RG_TRY(ensure(w.ranges, (size_t)F.tiles * sizeof(uint2), "ranges"));
     RG_TRY(ensure(w.ctrl, CTRL_ALLOC, "counters"));
     const int64_t fe_blocks = (n + frontend_block_threads() - 1) / frontend_block_threads();
     RG_TRY(ensure(w.lb_status, (size_t)(std::max<int64_t>(fe_blocks, (n + 2047) / 2048) + 1) * 8, "look-back status"));
@@ -168,7 +189,10 @@ rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, int tiles, i
         // memory for any tile count) and tile totals: sized for any frame, so a workspace shared by
         // views of several resolutions never runs short
         RG_TRY(ensure(w.tsort, tilesort_matrix_bytes_max() + (size_t)tilesort_max_tiles() * 4, "tile counting sort"));
-        RG_TRY(ensure(w.rowbuf, row_buffer_bytes(n), "row buckets"));
+        if (runs_possible(F.lay, n)) {
+            RunArgs ra;
+            RG_TRY(ensure(w.runbuf, run_views(w, n, F.lay, ra), "tile-row runs"));
+        }
         for (int k = 0; k < 2; k++) {
             RG_TRY(ensure(w.gkeys[k], (size_t)n * 4, "depth keys"));
             RG_TRY(ensure(w.gvals[k], (size_t)n * 4, "depth order"));
@@ -326,11 +350,11 @@ rg_status roofgs_build(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_t
     }
     f.tile_shift = a.keys16 ? 0 : F.lay.b_d;
     w.last_key16 = a.keys16 != nullptr;
-    w.last_cols = false;
+    w.last_runs = false;
     w.last_tilesort = f.tile_sort;
     w.last_bd = F.lay.b_d;
     w.last_mode = RG_MODE_ROOFGS;
-    w.last_passes = sa.passes;
+    w.last_passes = w.last_stat_passes = sa.passes;
     w.last_tiles = F.tiles;
     return RG_OK;
 }
@@ -357,13 +381,12 @@ void roofgs_raster_args(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_
     r.cam = F.cam;
     r.out = out;
     r.rec = w.rec.as<float4>();
-    if (w.last_tilesort) { // the counting sort wrote the ranges: no search
+    if (w.last_tilesort || w.last_runs) { // the ranges were written with the entries: no search
     } else if (w.last_key16) {
         r.skeys16 = w.keys[fin].as<unsigned short>();
     } else {
         r.skeys = w.keys[fin].as<unsigned>();
     }
-    r.key_cols = w.last_key16 && w.last_cols;
     r.tile_shift = w.last_key16 ? 0 : F.lay.b_d;
     r.ranges_out = w.ranges.as<uint2>();
     r.ctr = w.ctrl.as<Counters>();
@@ -393,7 +416,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     const bool search_ranges = mode == RG_MODE_ROOFGS && out != nullptr && !tile_sort;
     w.last_key16 = false;
     w.last_tilesort = false;
-    w.last_cols = false;
+    w.last_runs = false;
     RG_CK(cudaMemsetAsync(w.ctrl.p, 0, CTRL_ALLOC, st));
     if (flags & RG_FLAG_TEST_STALL_SORT) { // tile 0 of the first entry-sort pass is never claimed
         k_set_word<<<1, 1, 0, st>>>(&ctr->sort_tile_ctr[0], 1u);
@@ -414,6 +437,8 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     sa.ctr = ctr;
     sa.sticky = sticky;
     int tile_shift;
+    bool runs = false;
+    RunArgs ra;
     TileSortArgs tsa;
     memset(&tsa, 0, sizeof(tsa));
     if (mode == RG_MODE_EXACT) {
@@ -466,18 +491,20 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     } else {
         RoofgsFrame f;
         RG_TRY(roofgs_build(s, w, F, flags, f));
-        // the row-bucketed front end: column-major 16-bit keys grouped by tile row, one 8-bit
-        // pass over the column left to the sort (the rasterizer finds the ranges)
-        const bool rows = !(flags & RG_FLAG_ORDERED_FRONT_END) && search_ranges && f.depth_order && f.fa.keys16 &&
-                          !f.tile_sort && F.lay.tiles_x <= 256 && F.lay.tiles_y <= 256 && n > 0;
-        if (rows) {
-            f.fa.rows = F.lay.tiles_y;
-            row_buffer_views(w, f.fa);
-            f.fa.hist_passes = 1; // the column digits
-            f.sa.passes = 1;
-            f.sa.bit0 = 8;
-            f.sa.rank_modes = sort_rank_modes(SORT_RANK_PEERS);
-            w.last_cols = true;
+        // entries written from tile-row runs, no sort of the entries. The stall hook needs an entry
+        // sort to stall, so its frames take the radix passes
+        runs = !(flags & (RG_FLAG_ORDERED_FRONT_END | RG_FLAG_TEST_STALL_SORT)) && out != nullptr && f.depth_order &&
+               !f.tile_sort && runs_possible(F.lay, n);
+        if (runs) {
+            if (run_views(w, n, F.lay, ra) > w.runbuf.bytes || (size_t)ra.run_cap * sizeof(uint2) > w.keys[0].bytes)
+                return fail(RG_ERR_CAPACITY, "workspace not sized for the frame");
+            ra.sticky = sticky;
+            w.last_key16 = false;
+            w.last_runs = true;
+            w.last_passes = 0;
+            // one pass over the tile column, or the tile-bit passes of larger grids, is what the
+            // grouping replaces
+            if (F.lay.tiles_x <= 256 && F.lay.tiles_y <= 256 && f.fa.keys16) w.last_stat_passes = 1;
         } else {
             RG_CK(cudaMemsetAsync(w.lb_status.p, 0,
                                   (size_t)((n + frontend_block_threads() - 1) / frontend_block_threads() + 1) * 8, st));
@@ -489,7 +516,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         if (ev) RG_CK(cudaEventRecord(E[1], st));
         {
             NvtxScope r_("rg front end");
-            if (rows) launch_frontend_rows(f.fa, st);
+            if (runs) launch_frontend_runs(f.fa, ra, st);
             else launch_frontend_fused(f.fa, st);
         }
         sa = f.sa;
@@ -497,8 +524,11 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         tsa = f.ts;
     }
     if (ev) RG_CK(cudaEventRecord(E[2], st));
-    if (ev && (sa.passes <= 0 || tile_sort)) RG_CK(cudaEventRecord(E[3], st));
-    if (tile_sort) {
+    if (ev && !runs && (sa.passes <= 0 || tile_sort)) RG_CK(cudaEventRecord(E[3], st));
+    if (runs) {
+        NvtxScope r_("rg sort");
+        launch_runs(ra, st, ev ? E[3] : nullptr);
+    } else if (tile_sort) {
         NvtxScope r_("rg sort");
         launch_tile_counting_sort(tsa, st);
     } else {
@@ -506,21 +536,22 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         launch_sort(sa, st, ev ? E[3] : nullptr);
     }
     if (ev) RG_CK(cudaEventRecord(E[4], st));
-    const int fin = sa.passes & 1;
+    if (!runs) w.last_passes = sa.passes;
+    const int fin = w.last_passes & 1;
     if (!search_ranges && !tile_sort) {
-        RangeArgs ra;
-        ra.keys = w.keys[fin].p;
-        ra.key_bytes = sa.key_bytes;
-        ra.tile_shift = tile_shift;
-        ra.ntiles = F.tiles;
-        ra.ranges = w.ranges.as<uint2>();
-        ra.ctr = ctr;
+        RangeArgs g;
+        g.keys = w.keys[fin].p;
+        g.key_bytes = sa.key_bytes;
+        g.tile_shift = tile_shift;
+        g.ntiles = F.tiles;
+        g.ranges = w.ranges.as<uint2>();
+        g.ctr = ctr;
         NvtxScope r_("rg ranges");
-        launch_ranges(ra, st);
+        launch_ranges(g, st);
     }
     if (ev) RG_CK(cudaEventRecord(E[5], st));
     w.last_mode = mode;
-    w.last_passes = sa.passes;
+    if (!runs) w.last_stat_passes = sa.passes;
     w.last_tiles = F.tiles;
     w.last_tilesort = tile_sort;
     if (!out) { // front end, sort and ranges only (the backward replays the blend itself)
@@ -552,9 +583,6 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     }
     if (ev) RG_CK(cudaEventRecord(E[6], st));
     RG_CK(cudaGetLastError());
-    w.last_mode = mode;
-    w.last_passes = sa.passes;
-    w.last_tiles = F.tiles;
     return RG_OK;
 }
 
@@ -699,7 +727,7 @@ rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries)
     RG_CK(cudaDeviceSynchronize());
     const int64_t cap = n_entries;
     for (int k = 0; k < 2; k++) {
-        RG_TRY(ensure(scene->ws.keys[k], (size_t)cap * 8, "keys"));
+        RG_TRY(ensure(scene->ws.keys[k], (size_t)key_items(scene->n, cap) * 8, "keys"));
         RG_TRY(ensure(scene->ws.vals[k], (size_t)cap * 4, "values"));
     }
     const int64_t max_tiles = (cap + sort_tile_items() - 1) / sort_tile_items();
@@ -871,7 +899,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, const rg_render_opts* opt
     cudaStream_t st = (cudaStream_t)stream;
     int64_t cap = s->ws.cap > 0 ? s->ws.cap : std::max<int64_t>(1 << 20, 4 * s->n);
     if (cap > MAX_CAP) cap = MAX_CAP;
-    RG_TRY(ensure_workspace(s->ws, s->n, mode, F.tiles, cap));
+    RG_TRY(ensure_workspace(s->ws, s->n, mode, F, cap));
     RG_TRY(render_once(s, s->ws, F, mode, opts->flags, out_chw, st, stats != nullptr));
     if (!stats) return RG_OK;
     Counters c;
@@ -885,6 +913,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, const rg_render_opts* opt
         if ((unsigned long long)want < c.n_entries_total)
             return fail(RG_ERR_CAPACITY, "frame needs more than 2^30 - 1 entries");
         RG_TRY(rg_scene_reserve(s, want));
+        RG_TRY(ensure_workspace(s->ws, s->n, mode, F, s->ws.cap));
         RG_TRY(render_once(s, s->ws, F, mode, opts->flags, out_chw, st, true));
         RG_CK(cudaMemcpyAsync(&c, s->ws.ctrl.p, sizeof(c), cudaMemcpyDeviceToHost, st));
         RG_CK(cudaStreamSynchronize(st));
@@ -906,7 +935,7 @@ rg_status rg_render(rg_scene* s, const rg_camera* cam, const rg_render_opts* opt
     stats->n_entries = (int64_t)c.n_entries_total;
     stats->capacity = s->ws.cap;
     stats->regrown = regrown;
-    stats->sort_passes = s->ws.last_passes;
+    stats->sort_passes = s->ws.last_stat_passes;
     stats->b_t = F.lay.b_t;
     stats->b_d = mode == RG_MODE_ROOFGS ? F.lay.b_d : 32;
     stats->tiles_x = F.lay.tiles_x;
@@ -967,47 +996,34 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
         Counters c;
         RG_CK(cudaMemcpy(&c, s->ws.ctrl.p, sizeof(c), cudaMemcpyDeviceToHost));
         const int fin = s->ws.last_passes & 1;
-        // column-major keys: the entries are regrouped tile by tile in tile-id order (each tile's
-        // range, in its order), which is the order of the entries sorted by tile id
-        std::vector<uint32_t> cval;
-        std::vector<uint2> cr;
-        if (s->ws.last_key16 && s->ws.last_cols) {
-            const size_t ne = c.n_entries;
-            std::vector<uint32_t> v(ne);
-            cr.resize((size_t)s->ws.last_tiles);
-            RG_CK(cudaMemcpy(cr.data(), s->ws.ranges.p, cr.size() * 8, cudaMemcpyDeviceToHost));
-            if (ne) RG_CK(cudaMemcpy(v.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
-            cval.reserve(ne);
-            uint32_t at = 0;
-            for (size_t t = 0; t < cr.size(); t++) {
-                const uint32_t b = cr[t].x, e = std::min<uint32_t>(cr[t].y, (uint32_t)ne);
-                const uint32_t len = e > b ? e - b : 0u;
-                for (uint32_t j = b; j < b + len; j++) cval.push_back(v[j]);
-                cr[t] = len ? make_uint2(at, at + len) : make_uint2(0u, 0u);
-                at += len;
-            }
+        const size_t ne = c.n_entries, ng = (size_t)n;
+        // a frame of runs: the values are slots of the depth order, which maps them to Gaussians
+        std::vector<uint32_t> val;
+        if (s->ws.last_runs && what != RG_INSPECT_RANGES) {
+            std::vector<uint32_t> order(ng);
+            val.resize(ne);
+            if (ne) RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
+            if (ng) RG_CK(cudaMemcpy(order.data(), s->ws.gvals[s->ws.last_gfin].p, ng * 4, cudaMemcpyDeviceToHost));
+            for (uint32_t& v : val) v = v < ng ? order[v] : 0u;
         }
-        if (what == RG_INSPECT_KEYS && s->ws.last_key16) {
-            // the entries carried 16-bit tile ids: each 32-bit key (tile << b_d | q_d) is rebuilt
-            // from the tile and the depth code of its Gaussian (the per-Gaussian depth sort's result);
-            // after the per-tile counting sort the tile of each slot follows from the ranges
-            const size_t ne = c.n_entries, ng = (size_t)n;
-            std::vector<uint16_t> t16(ne);
-            std::vector<uint32_t> val(ne), gq(ng), gi(ng), q(ng, 0u);
-            if (ne) {
-                if (s->ws.last_cols) {
-                    for (size_t t = 0; t < cr.size(); t++)
-                        for (uint32_t j = cr[t].x; j < cr[t].y; j++) t16[j] = (uint16_t)t;
-                    for (size_t j = 0; j < ne; j++) val[j] = j < cval.size() ? cval[j] : 0u;
-                } else if (s->ws.last_tilesort) {
-                    std::vector<uint2> rr((size_t)s->ws.last_tiles);
-                    RG_CK(cudaMemcpy(rr.data(), s->ws.ranges.p, rr.size() * 8, cudaMemcpyDeviceToHost));
-                    for (size_t t = 0; t < rr.size(); t++)
-                        for (uint32_t j = rr[t].x; j < rr[t].y && j < ne; j++) t16[j] = (uint16_t)t;
-                } else {
-                    RG_CK(cudaMemcpy(t16.data(), s->ws.keys[fin].p, ne * 2, cudaMemcpyDeviceToHost));
-                }
-                if (!s->ws.last_cols) RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
+        if (what == RG_INSPECT_KEYS && (s->ws.last_key16 || s->ws.last_runs)) {
+            // the entries carried 16-bit tile ids, or no key at all: each 32-bit key (tile << b_d | q_d)
+            // is rebuilt from the tile and the depth code of its Gaussian (the per-Gaussian depth
+            // sort's result); without stored keys the tile of each entry follows from the ranges
+            std::vector<uint32_t> tile(ne), gq(ng), gi(ng), q(ng, 0u);
+            if (ne && (s->ws.last_runs || s->ws.last_tilesort)) {
+                std::vector<uint2> rr((size_t)s->ws.last_tiles);
+                RG_CK(cudaMemcpy(rr.data(), s->ws.ranges.p, rr.size() * 8, cudaMemcpyDeviceToHost));
+                for (size_t t = 0; t < rr.size(); t++)
+                    for (uint32_t j = rr[t].x; j < rr[t].y && j < ne; j++) tile[j] = (uint32_t)t;
+            } else if (ne) {
+                std::vector<uint16_t> t16(ne);
+                RG_CK(cudaMemcpy(t16.data(), s->ws.keys[fin].p, ne * 2, cudaMemcpyDeviceToHost));
+                for (size_t j = 0; j < ne; j++) tile[j] = t16[j];
+            }
+            if (ne && !s->ws.last_runs) {
+                val.resize(ne);
+                RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
             }
             if (ng) {
                 RG_CK(cudaMemcpy(gq.data(), s->ws.gkeys[s->ws.last_gfin].p, ng * 4, cudaMemcpyDeviceToHost));
@@ -1019,7 +1035,7 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
             tmp.resize(ne * 4);
             for (size_t j = 0; j < ne; j++) {
                 const uint32_t qd = val[j] < ng ? q[val[j]] : 0u;
-                const uint32_t key = bd >= 32 ? qd : (((uint32_t)t16[j] << bd) | qd);
+                const uint32_t key = bd >= 32 ? qd : ((tile[j] << bd) | qd);
                 memcpy(&tmp[j * 4], &key, 4);
             }
             src = tmp.data();
@@ -1028,22 +1044,15 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
         } else if (what == RG_INSPECT_KEYS) {
             src = s->ws.keys[fin].p;
             bytes = (int64_t)c.n_entries * (s->ws.last_mode == RG_MODE_EXACT ? 8 : 4);
-        } else if (what == RG_INSPECT_VALUES && s->ws.last_key16 && s->ws.last_cols) {
-            cval.resize(c.n_entries, 0u);
-            tmp.resize(cval.size() * 4);
-            if (!cval.empty()) memcpy(tmp.data(), cval.data(), tmp.size());
+        } else if (what == RG_INSPECT_VALUES && s->ws.last_runs) {
+            tmp.resize(ne * 4);
+            if (ne) memcpy(tmp.data(), val.data(), tmp.size());
             src = tmp.data();
             device_src = false;
             bytes = (int64_t)tmp.size();
         } else if (what == RG_INSPECT_VALUES) {
             src = s->ws.vals[fin].p;
             bytes = (int64_t)c.n_entries * 4;
-        } else if (s->ws.last_key16 && s->ws.last_cols) {
-            tmp.resize(cr.size() * 8);
-            if (!cr.empty()) memcpy(tmp.data(), cr.data(), tmp.size());
-            src = tmp.data();
-            device_src = false;
-            bytes = (int64_t)tmp.size();
         } else {
             src = s->ws.ranges.p;
             bytes = (int64_t)s->ws.last_tiles * 8;
@@ -1124,7 +1133,7 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
     cudaStream_t st = (cudaStream_t)stream;
     int64_t cap = s->ws.cap > 0 ? s->ws.cap : std::max<int64_t>(1 << 20, 4 * s->n);
     if (cap > MAX_CAP) cap = MAX_CAP;
-    RG_TRY(ensure_workspace(s->ws, s->n, RG_MODE_EXACT, F.tiles, cap));
+    RG_TRY(ensure_workspace(s->ws, s->n, RG_MODE_EXACT, F, cap));
     // forward front end, sort and ranges of this camera (checked: the gradient needs every entry)
     for (int attempt = 0; attempt < 2; attempt++) {
         RG_TRY(render_once(s, s->ws, F, RG_MODE_EXACT, 0u, nullptr, st));
@@ -1137,6 +1146,7 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
         int64_t want = (int64_t)(c.n_entries_total + c.n_entries_total / 4 + 1024);
         if (want > MAX_CAP) return fail(RG_ERR_CAPACITY, "frame needs more than 2^30 - 1 entries");
         RG_TRY(rg_scene_reserve(s, want));
+        RG_TRY(ensure_workspace(s->ws, s->n, RG_MODE_EXACT, F, s->ws.cap));
     }
     RG_TRY(ensure(s->ws.gbuf, (size_t)(s->n > 0 ? s->n : 1) * 9 * 4, "gradient buffer"));
     RG_CK(cudaMemsetAsync(s->ws.gbuf.p, 0, (size_t)(s->n > 0 ? s->n : 1) * 9 * 4, st));

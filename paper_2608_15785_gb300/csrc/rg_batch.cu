@@ -91,16 +91,12 @@ bool fused_possible(const BatchPlan& P)
 rg_status plan_size(BatchPlan& P, const std::vector<FrameLayout>& F, float* const* outs, cudaStream_t st)
 {
     int64_t cap = 0;
-    int max_tiles = 1;
-    int64_t max_n = 1;
     std::vector<int64_t> view_entries(F.size(), 0);
     for (size_t v = 0; v < F.size(); v++) {
         rg_scene* s = P.scenes[v];
-        max_tiles = std::max(max_tiles, F[v].tiles);
-        max_n = std::max<int64_t>(max_n, s->n);
         int64_t c = P.ws[0].cap > 0 ? P.ws[0].cap : std::max<int64_t>(1 << 20, 4 * s->n);
         if (c > MAX_CAP) c = MAX_CAP;
-        RG_TRY(ensure_workspace(P.ws[0], s->n, P.mode, F[v].tiles, c));
+        RG_TRY(ensure_workspace(P.ws[0], s->n, P.mode, F[v], c));
         for (int attempt = 0; attempt < 2; attempt++) {
             RG_TRY(render_once(s, P.ws[0], F[v], P.mode, P.flags, outs[v], st));
             Counters c2;
@@ -112,25 +108,36 @@ rg_status plan_size(BatchPlan& P, const std::vector<FrameLayout>& F, float* cons
             if (c2.n_entries_total <= (unsigned long long)P.ws[0].cap) break;
             int64_t want = (int64_t)(c2.n_entries_total + c2.n_entries_total / 4 + 1024);
             if (want > MAX_CAP) return fail(RG_ERR_CAPACITY, "a view needs more than 2^30 - 1 entries");
-            RG_TRY(ensure_workspace(P.ws[0], s->n, P.mode, F[v].tiles, want));
+            RG_TRY(ensure_workspace(P.ws[0], s->n, P.mode, F[v], want));
         }
     }
     cap = std::min<int64_t>(MAX_CAP, cap + cap / 4 + 1024);
     for (int l = 0; l < BATCH_MAX_LANES; l++) {
         for (size_t v = 0; v < F.size(); v++)
-            RG_TRY(ensure_workspace(P.ws[l], P.scenes[v]->n, P.mode, max_tiles, std::max(cap, P.ws[l].cap)));
+            RG_TRY(ensure_workspace(P.ws[l], P.scenes[v]->n, P.mode, F[v], std::max(cap, P.ws[l].cap)));
     }
     if (fused_possible(P)) { // the fused path keeps every view's frame at once: one workspace per view
         if (!P.vws) P.vws.reset(new Workspace[F.size()]);
         for (size_t v = 0; v < F.size(); v++) {
             const int64_t c = std::min<int64_t>(MAX_CAP, view_entries[v] + view_entries[v] / 4 + 1024);
-            RG_TRY(ensure_workspace(P.vws[v], P.scenes[v]->n, P.mode, F[v].tiles, std::max(c, P.vws[v].cap)));
+            RG_TRY(ensure_workspace(P.vws[v], P.scenes[v]->n, P.mode, F[v], std::max(c, P.vws[v].cap)));
         }
         RG_TRY(ensure(P.claim, 256, "batch work counters"));
     }
     // the scenes' sticky flags of the sizing frames are not errors
     for (rg_scene* s : P.scenes) RG_CK(cudaMemsetAsync(s->sticky.p, 0, sizeof(Sticky), st));
     RG_CK(cudaStreamSynchronize(st));
+    return RG_OK;
+}
+
+// Grows the workspaces for the tile grids of F at the capacities they have.
+rg_status plan_fit(BatchPlan& P, const std::vector<FrameLayout>& F)
+{
+    for (size_t v = 0; v < F.size(); v++) {
+        for (int l = 0; l < BATCH_MAX_LANES; l++)
+            RG_TRY(ensure_workspace(P.ws[l], P.scenes[v]->n, P.mode, F[v], P.ws[l].cap));
+        if (P.vws) RG_TRY(ensure_workspace(P.vws[v], P.scenes[v]->n, P.mode, F[v], P.vws[v].cap));
+    }
     return RG_OK;
 }
 
@@ -405,6 +412,11 @@ rg_status rg_render_batch(rg_scene* const* scenes, const int32_t* scene_idx, con
             std::vector<FrameLayout> Fs;
             RG_TRY(layouts_for(cams, n, shape.first, shape.second, Fs));
             RG_TRY(plan_size(*np, Fs, outs, st));
+        }
+        for (auto shape : plan_shapes(*np)) { // a later shape may have raised the capacity
+            std::vector<FrameLayout> Fs;
+            RG_TRY(layouts_for(cams, n, shape.first, shape.second, Fs));
+            RG_TRY(plan_fit(*np, Fs));
         }
         RG_TRY(plan_tune(*np, cams, outs, st));
         if (g_plans.size() >= 8) g_plans.erase(g_plans.begin());

@@ -50,7 +50,8 @@ constexpr size_t CTRL_BYTES = sizeof(Counters) + 8 * 256 * sizeof(unsigned);
 // frame counters, the per-Gaussian depth sort's, then the producers' digit-count copies
 // ([copy][2][256] from the fused front end, [copy][8][256] from the exact duplicate)
 constexpr size_t FE_HIST_BYTES = (size_t)FE_HIST_COPIES * 8 * 256 * sizeof(unsigned);
-constexpr size_t CTRL_ALLOC = 2 * CTRL_BYTES + FE_HIST_BYTES;
+constexpr size_t RUN_TOT_AT = (2 * CTRL_BYTES + FE_HIST_BYTES + 15) / 16 * 16; // then RunArgs::tot
+constexpr size_t CTRL_ALLOC = RUN_TOT_AT + (size_t)RUN_MAX_GRID * 8;
 
 // Frame workspace: everything one frame in flight needs besides the scene.
 // rg_render uses the scene's own workspace; a batch lane or a server slot owns one.
@@ -66,14 +67,16 @@ struct Workspace {
     DevBuf gkeys[2], gvals[2], gstatus[2];                // RoofGS per-Gaussian depth sort
     DevBuf gbuf;                                          // backward: image-space gradients [n][9]
     DevBuf tsort;                                         // RoofGS per-tile counting sort: matrix + tile totals
-    DevBuf rowbuf; // RoofGS row-bucketed front end: rows and row tests per slot, counts per tile row
+    DevBuf runbuf; // tile-row runs: per-block counts and places, chunks, column counts (run_views)
     // last frame
     int last_mode = -1;
-    int last_passes = 0;
+    int last_passes = 0;     // radix passes over the entries (the result is in keys/vals[last_passes & 1])
+    int last_stat_passes = 0; // rg_stats.sort_passes
     int last_tiles = 0;
     bool last_key16 = false; // entries carried 16-bit tile ids (the 32-bit keys are rebuilt on inspection)
     bool last_tilesort = false; // the entries were grouped by the per-tile counting sort (keys rebuilt from ranges)
-    bool last_cols = false;  // the 16-bit keys were column-major (tx << 8 | ty): entries regrouped from the ranges
+    bool last_runs = false;  // the entries were written from tile-row runs: values are slots of the depth order
+                             // in tile-id order, in vals[0]
     int last_bd = 0;         // b_d of the last RoofGS frame
     int last_gfin = 0;       // buffer of the per-Gaussian depth sort's result
     // stage events
@@ -86,7 +89,7 @@ struct Workspace {
     {
         DevBuf* bufs[] = {&keys[0], &keys[1], &vals[0], &vals[1], &ranges, &ctrl, &lb_status, &sort_status[0],
                           &sort_status[1], &mean2, &depth, &quad, &rgb, &rect, &touched, &offsets, &rec, &gkeys[0],
-                          &gkeys[1], &gvals[0], &gvals[1], &gstatus[0], &gstatus[1], &gbuf, &tsort, &rowbuf};
+                          &gkeys[1], &gvals[0], &gvals[1], &gstatus[0], &gstatus[1], &gbuf, &tsort, &runbuf};
         for (DevBuf* b : bufs) b->release();
         if (ev_init)
             for (int f = 0; f < EV_RING; f++)
@@ -128,8 +131,8 @@ bool tile_shape_ok(int tw, int th);
 rg_status tile_shape(const rg_render_opts* o, int& tw, int& th);
 // checks the camera and derives the frame layout (Sec. IV-A.2 key split) for a tile shape
 rg_status make_layout(const rg_camera* c, FrameLayout& f, int tw = TILE, int th = TILE);
-// grows a workspace for a frame of n_gauss Gaussians, `tiles` tiles and `cap` entries
-rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, int tiles, int64_t cap);
+// grows a workspace for a frame of n_gauss Gaussians, F's tile grid and `cap` entries
+rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameLayout& F, int64_t cap);
 // creates the stage events of a workspace on first use
 void init_events(Workspace& w);
 // enqueues one frame on `st` (arguments and workspace already checked); out == nullptr stops

@@ -74,7 +74,10 @@ struct Counters {
     unsigned fe_block_ctr;   // virtual block ids of the fused front end / exact scan
     unsigned sort_tile_ctr[8];
     unsigned n_front;
+    unsigned n_row_runs;         // tile-row runs given a place in the rows' lists (runs.cu)
+    unsigned n_chunks;           // chunks of runs
     unsigned pad;
+    unsigned long long n_runs;   // tile-row runs the front end's blocks asked room for
     unsigned long long n_pairs;  // rasterizer work counters (counting launches only)
     unsigned long long n_blends;
 };
@@ -505,19 +508,70 @@ struct FrontendArgs {
     Sticky* sticky;
     unsigned* hist;             // [FE_HIST_COPIES][2][256] digit counts of the tile field, or null
     int hist_passes;            // 0, 1 or 2: 8-bit digits of the tile id counted (b_t <= 16)
-    // Row-bucketed front end (launch_frontend_rows): rows > 0 tile rows (at most 256, as are
-    // the tile columns); the entries carry the column-major 16-bit key tx << 8 | ty and come
-    // out grouped by tile row, which leaves one 8-bit sort pass (the column) to the sort
-    int rows;
-    unsigned* row_n;             // [N] tile rows of the Gaussian of each slot (0: none)
-    float4* row_rt;              // [3][N] its row test (RowTestS as three float4 planes)
-    unsigned* row_cnt;           // [rows][blocks] entries of each tile row per block, then their
-                                 // exclusive prefix over the blocks (saturated at 2^31 - 1)
-    unsigned long long* row_tot; // [rows] entries of each tile row
 };
 void launch_frontend_fused(const FrontendArgs& a, cudaStream_t s);
-// count kernel -> per-row scan of the block counts -> scatter kernel (a.rows > 0)
-void launch_frontend_rows(const FrontendArgs& a, cudaStream_t s);
+
+// ---------------------------------------------------------------------------
+// Tile-row runs (runs.cu): a Gaussian's entries in one tile row are consecutive tile columns.
+// ---------------------------------------------------------------------------
+constexpr int RUN_SLOTS = 256;     // slots (Gaussians in depth order) of a front-end block
+constexpr int RUN_MAX_GRID = 512;  // tile rows and tile columns at most (the front end's per-row
+                                   // shared memory, the collect kernel's column counts)
+// a block's count of one tile row: entries, and runs above them (at most 256 x 512 and 256)
+constexpr unsigned RUN_CNT_SHIFT = 20, RUN_CNT_ENTRIES = (1u << RUN_CNT_SHIFT) - 1u;
+// a tile row's count over all blocks of a small frame: entries (2^40), and runs above them
+constexpr int RUN_TOT_SHIFT = 40;
+constexpr unsigned long long RUN_TOT_ENTRIES = (1ull << RUN_TOT_SHIFT) - 1ull;
+constexpr unsigned RUN_SMALL_BLOCKS = 128; // front-end blocks of a small frame at most
+// a run in its block's list: slot in the block, first and last tile column
+__host__ __device__ __forceinline__ unsigned run_pack(unsigned slot, unsigned ta, unsigned tb)
+{
+    return slot | (ta << 8) | (tb << 20);
+}
+__host__ __device__ __forceinline__ unsigned run_slot(unsigned v) { return v & 255u; }
+__host__ __device__ __forceinline__ unsigned run_first(unsigned v) { return (v >> 8) & 0xfffu; }
+__host__ __device__ __forceinline__ unsigned run_last(unsigned v) { return v >> 20; }
+// words per chunk of the column counts
+__host__ __device__ __forceinline__ int run_pitch(int cols) { return (cols + 31) / 32 * 32; }
+
+struct RunChunk {
+    unsigned block;           // its first block
+    unsigned run;             // runs of the row before it
+    unsigned long long entry; // entries of the row before it
+};
+struct RunRow {
+    unsigned chunk, nchunks; // its chunks
+    unsigned base, runs;     // its part of the list
+    unsigned long long entries;
+};
+struct RunArgs {
+    int rows, cols;    // tile grid (each at most RUN_MAX_GRID)
+    unsigned blocks;   // front-end blocks: ceil(n / RUN_SLOTS)
+    unsigned run_cap;  // runs the buffers hold
+    unsigned chunk_cap;
+    int box_total;     // 1: the front end counted the frame's entries (n_entries_total; exact mode, whose
+                       // lists leave out entries below 1/255 on the whole tile); 0: the runs' entries
+    long long cap;     // entries the workspace holds
+    unsigned* cnt;     // [rows][blocks] entries | runs << RUN_CNT_SHIFT
+    unsigned* pre;     // [rows][blocks] runs of the row in the blocks before
+    unsigned long long* tot; // [rows] entries | runs << RUN_TOT_SHIFT, zeroed for every frame; null in a frame that
+                             // is not small (more than RUN_SMALL_BLOCKS blocks)
+    unsigned* seg;     // [rows][blocks] first run of the block's runs of the row
+    unsigned* runs;    // [run_cap] runs, by block, by tile row, by slot
+    uint2* list;       // [run_cap] (slot, first column | last column << 16), by tile row, by slot
+    RunChunk* chunk;   // [chunk_cap]
+    RunRow* row;       // [rows]
+    unsigned* col;     // [chunk_cap][run_pitch(cols)] entries per column, then their first slot in vals
+    unsigned* vals;    // [cap] slots, by tile id, by slot
+    uint2* ranges;     // [rows * cols] [start, end) of every tile, [0, 0) if empty
+    Counters* ctr;
+    Sticky* sticky;
+};
+unsigned run_chunk_cap(unsigned run_cap, int rows, unsigned blocks);
+// groups the runs the front end left in a.runs by tile: fills vals and ranges
+void launch_runs(const RunArgs& a, cudaStream_t s, cudaEvent_t ev_after_collect);
+// the front end of a frame of runs: projection, culling, colour, record per slot, runs per block
+void launch_frontend_runs(const FrontendArgs& a, const RunArgs& r, cudaStream_t s);
 
 // Views of a batch rendered by one launch of a stage (the batch's fused path).
 constexpr int MAX_BATCH_VIEWS = 32;
@@ -625,7 +679,6 @@ struct RasterArgs {
     // ranges_out; `ranges` is then unused
     const unsigned* skeys;
     const unsigned short* skeys16; // instead of skeys: 16-bit tile ids (tile_shift 0)
-    int key_cols;                  // skeys16 hold the column-major key tx << 8 | ty
     int tile_shift;
     uint2* ranges_out;
     const Counters* ctr;  // frame counters (n_entries) for the search

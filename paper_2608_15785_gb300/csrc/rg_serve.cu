@@ -73,7 +73,7 @@ namespace {
 rg_status slot_launch(rg_server* sv, ServeSlot& sl)
 {
     rg_scene* s = sv->scenes[sl.req.scene];
-    RG_TRY(ensure_workspace(sl.ws, s->n, sv->mode, sl.F.tiles, sl.ws.cap > 0 ? sl.ws.cap : (int64_t)1 << 20));
+    RG_TRY(ensure_workspace(sl.ws, s->n, sv->mode, sl.F, sl.ws.cap > 0 ? sl.ws.cap : (int64_t)1 << 20));
     RG_TRY(render_once(s, sl.ws, sl.F, sv->mode, sv->flags & ~RG_FLAG_STAGE_EVENTS, sl.out, sl.stream));
     RG_CK(cudaMemcpyAsync(sl.pinned_ctr, sl.ws.ctrl.p, sizeof(Counters), cudaMemcpyDeviceToHost, sl.stream));
     RG_CK(cudaEventRecord(sl.done, sl.stream));
@@ -108,7 +108,7 @@ void server_loop(rg_server* sv)
                 sl.attempts++;
                 rg_scene* s = sv->scenes[sl.req.scene];
                 rg_status e = want > MAX_CAP ? RG_ERR_CAPACITY
-                                             : ensure_workspace(sl.ws, s->n, sv->mode, sl.F.tiles, want);
+                                             : ensure_workspace(sl.ws, s->n, sv->mode, sl.F, want);
                 if (e == RG_OK) e = slot_launch(sv, sl);
                 if (e == RG_OK) continue;
                 sl.result = e;
@@ -213,7 +213,7 @@ rg_status rg_server_create(rg_scene* const* scenes, int32_t n_scenes, const rg_s
         probe->req.cam.height = sv->max_h;
         probe->req.scene = big;
         RG_TRY(make_layout(&probe->req.cam, probe->F));
-        RG_TRY(ensure_workspace(probe->ws, scenes[big]->n, sv->mode, probe->F.tiles, (int64_t)1 << 20));
+        RG_TRY(ensure_workspace(probe->ws, scenes[big]->n, sv->mode, probe->F, (int64_t)1 << 20));
         for (int attempt = 0; attempt < 2; attempt++) {
             RG_TRY(render_once(scenes[big], probe->ws, probe->F, sv->mode, sv->flags, probe->out, probe->stream));
             Counters c;
@@ -221,16 +221,20 @@ rg_status rg_server_create(rg_scene* const* scenes, int32_t n_scenes, const rg_s
             RG_CK(cudaStreamSynchronize(probe->stream));
             entries = (int64_t)c.n_entries_total;
             if (c.n_entries_total <= (unsigned long long)probe->ws.cap) break;
-            RG_TRY(ensure_workspace(probe->ws, scenes[big]->n, sv->mode, probe->F.tiles,
+            RG_TRY(ensure_workspace(probe->ws, scenes[big]->n, sv->mode, probe->F,
                                     std::min<int64_t>(MAX_CAP, entries + entries / 4 + 1024)));
         }
         RG_CK(cudaMemsetAsync(scenes[big]->sticky.p, 0, sizeof(Sticky), probe->stream));
     }
     const int64_t cap = std::min<int64_t>(MAX_CAP, std::max<int64_t>(1 << 20, entries + entries / 2 + 1024));
     const int64_t ngauss = scenes[big]->n;
-    const int64_t tiles = (int64_t)((sv->max_w + TILE - 1) / TILE) * ((sv->max_h + TILE - 1) / TILE);
+    FrameLayout largest; // the tile grid of the largest request
+    largest.lay.tiles_x = (sv->max_w + TILE - 1) / TILE;
+    largest.lay.tiles_y = (sv->max_h + TILE - 1) / TILE;
+    const int64_t tiles = (int64_t)largest.lay.tiles_x * largest.lay.tiles_y;
+    largest.tiles = (int)tiles;
     // bytes of one slot: 2 x (keys 8 B + values 4 B) per entry, sort status, per-Gaussian arrays (RoofGS:
-    // records, depth order, row tests and row counts), ranges, image
+    // records, depth order), ranges, image
     sv->slot_bytes = cap * 24 + (cap / 4096 + 1) * 2048 + ngauss * (sv->mode == RG_MODE_EXACT ? 72 : 112) +
                      tiles * 8 + (int64_t)out_bytes;
     int nslots = cfg->max_slots > 0 ? cfg->max_slots : 8;
@@ -248,7 +252,7 @@ rg_status rg_server_create(rg_scene* const* scenes, int32_t n_scenes, const rg_s
                 return fail(RG_ERR_OOM, "pinned counters");
         }
         for (int j = 0; j < n_scenes; j++)
-            RG_TRY(ensure_workspace(sl->ws, scenes[j]->n, sv->mode, (int)tiles, std::max(cap, sl->ws.cap)));
+            RG_TRY(ensure_workspace(sl->ws, scenes[j]->n, sv->mode, largest, std::max(cap, sl->ws.cap)));
         sv->slots.push_back(std::move(sl));
     }
     RG_CK(cudaDeviceSynchronize());

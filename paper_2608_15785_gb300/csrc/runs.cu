@@ -1,0 +1,625 @@
+// runs.cu -- grouping of the frame's entries by tile from tile-row runs.
+//
+// A Gaussian's entries in one tile row are a run of consecutive tile columns, so the depth-ordered
+// Gaussians are a list of runs about a fifth as long as the list of entries, and the entries never
+// need to be written before they are in their final place. The front end (emit_runs, frontend.cu)
+// leaves each block's runs grouped by tile row, in slot (depth) order within a row, and each (tile
+// row, block) count; here
+//  * k_run_rows: per tile row, cuts the row's blocks into chunks of at most CHUNK_RUNS runs;
+//  * k_run_collect: per chunk, gathers the blocks' runs into one list per tile row and counts the
+//    chunk's entries per tile column (a difference array: two shared atomics per run);
+//  * k_run_offsets: per tile row, turns the chunks' column counts into the first slot of every
+//    (chunk, column) and writes every tile's [start, end): the entries lie in tile-id order;
+//  * k_run_expand: per chunk, writes the values (slots) of every column. For every 32 runs and
+//    column one word says which of the 32 cover the column: a run toggles its bit at its first
+//    column and after its last (two shared atomics), a prefix XOR over the columns fills it in. A
+//    warp then takes a column: each lane holds 64 runs' bits, a scan of the bit counts places its
+//    values, and the column's values go to consecutive addresses in run (depth) order.
+// The order within a tile is that of the stable sort of the 32-bit (or 64-bit) keys, and no key is
+// stored, counted or moved.
+//
+// What bounds it: each run is moved twice (4 B block-local, 8 B by row) and each value written once,
+// so HBM is far from busy; k_run_expand, the longest, is bound by issue slots and the latency of its
+// shared-memory reads (ncu: 1.8 instructions per cycle with three blocks of 256 threads per SM and a
+// column at a time, 405 us at 4K with 3 M Gaussians; five blocks and two columns at a time 281 us).
+// Kernel times (ncu) of the front end and the grouping, against the scatter by tile row with one radix
+// pass it replaced: 4K, 3 M Gaussians 792 -> 591 us (front end 201, rows 14, collect 85, offsets 11,
+// expand 281); 8K, 1 M, against the fused front end with three radix passes 1295 -> 541 us; 1080p,
+// 500 k 93 -> 89 us; 256 x 256, 10 k 35 -> 26 us.
+#include "rg_internal.cuh"
+
+namespace rg {
+
+constexpr int RUN_THREADS = 256;
+constexpr int RUN_WARPS = RUN_THREADS / 32;
+constexpr int CHUNK_RUNS = 2048;                // runs of a chunk at most: 64 per lane of a warp
+constexpr int CHUNK_STEP = CHUNK_RUNS - RUN_SLOTS; // a chunk ends with the block that reaches this many
+constexpr int CHUNK_BLOCKS = 1024;              // blocks of a chunk at most (sparse tile rows)
+constexpr int COLS = 120;                       // tile columns expanded at a time (five blocks per SM)
+constexpr int PITCH = CHUNK_RUNS / 32 + 2;      // words per column: 64 masks, padded (8-byte loads, no bank conflicts)
+
+// chunks a tile row of a small frame has at most: its row r has chunks r * small_chunks(blocks) and up
+__host__ __device__ __forceinline__ unsigned small_chunks(unsigned blocks)
+{
+    return blocks * (unsigned)RUN_SLOTS / CHUNK_STEP + 1;
+}
+
+unsigned run_chunk_cap(unsigned run_cap, int rows, unsigned blocks)
+{
+    if (blocks <= RUN_SMALL_BLOCKS) return (unsigned)rows * small_chunks(blocks);
+    return run_cap / CHUNK_STEP + (unsigned)rows * (blocks / CHUNK_BLOCKS + 2);
+}
+
+template <typename T>
+__device__ __forceinline__ T run_warp_scan(T x)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+// inclusive scan over the block (every thread calls it); s_w: one word per warp; total = the sum
+template <int WARPS, typename T>
+__device__ __forceinline__ T run_block_scan(T v, T* s_w, T& total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const T x = run_warp_scan(v);
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    T before = 0, all = 0;
+#pragma unroll
+    for (int q = 0; q < WARPS; q++) {
+        const T t = s_w[q];
+        if (q < warp) before += t;
+        all += t;
+    }
+    total = all;
+    __syncthreads(); // s_w may be written again after the call
+    return x + before;
+}
+
+// The chunk of a block with `run` runs of its row before it: a new chunk starts where the runs before
+// a block reach the next multiple of CHUNK_STEP (the blocks of a chunk then hold at most CHUNK_STEP -
+// 1 + RUN_SLOTS runs) and at every CHUNK_BLOCKS-th block. Where both happen at once an empty chunk
+// lies between.
+__device__ __forceinline__ unsigned chunk_of(unsigned run, unsigned block)
+{
+    return run / CHUNK_STEP + block / CHUNK_BLOCKS;
+}
+
+// One block of 1024 threads per tile row: a scan of the blocks' counts, and the row's chunks.
+__global__ void __launch_bounds__(1024) k_run_rows(RunArgs a)
+{
+    constexpr int WARPS = 32;
+    __shared__ unsigned s_r[WARPS];
+    __shared__ unsigned long long s_e[WARPS];
+    __shared__ unsigned s_chunk;
+    grid_dependency_wait();
+    const unsigned row = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const unsigned* const cnt = a.cnt + (size_t)row * a.blocks;
+    const unsigned per = (a.blocks + 32u * WARPS - 1u) / (32u * WARPS), b0 = tid * per;
+    const unsigned b1 = b0 + per < a.blocks ? b0 + per : a.blocks;
+    unsigned p = 0, last = 0; // runs of this thread's blocks, of its last block
+    unsigned long long e = 0;
+#pragma unroll 4
+    for (unsigned b = b0; b < b1; b++) {
+        const unsigned c = cnt[b];
+        last = c >> RUN_CNT_SHIFT;
+        p += last;
+        e += c & RUN_CNT_ENTRIES;
+    }
+    const unsigned rx = run_warp_scan(p);
+    const unsigned long long ex = run_warp_scan(e);
+    if (lane == 31) {
+        s_r[warp] = rx;
+        s_e[warp] = ex;
+    }
+    __syncthreads();
+    unsigned rbefore = 0, rtot = 0;
+    unsigned long long ebefore = 0, etot = 0;
+#pragma unroll
+    for (int q = 0; q < WARPS; q++) {
+        if (q < (int)warp) {
+            rbefore += s_r[q];
+            ebefore += s_e[q];
+        }
+        rtot += s_r[q];
+        etot += s_e[q];
+    }
+    const unsigned rend = rbefore + rx; // runs up to the end of this thread's blocks
+    if (b0 < b1 && b1 == a.blocks) {    // the thread of the row's last block
+        const unsigned n = rtot ? chunk_of(rend - last, a.blocks - 1) + 1 : 0u;
+        // where the row's runs and chunks lie does not matter, only that no two rows share a place
+        const unsigned base = atomicAdd(&a.ctr->n_row_runs, rtot), chunk = atomicAdd(&a.ctr->n_chunks, n);
+        if (!a.box_total && etot) atomicAdd(&a.ctr->n_entries_total, etot);
+        a.row[row] = RunRow{chunk, n, base, rtot, etot};
+        s_chunk = chunk;
+    }
+    __syncthreads();
+    if (!rtot || b0 >= b1) return;
+    p = rend - p;
+    e = ebefore + ex - e;
+    int prev = -1; // chunk of the block before
+    if (b0) prev = (int)chunk_of(p - (cnt[b0 - 1] >> RUN_CNT_SHIFT), b0 - 1);
+    for (unsigned b = b0; b < b1; b++) {
+        const unsigned c = cnt[b];
+        a.pre[(size_t)row * a.blocks + b] = p;
+        for (const int k = (int)chunk_of(p, b); prev < k;) {
+            prev++;
+            a.chunk[s_chunk + (unsigned)prev] = RunChunk{b, p, e};
+        }
+        p += c >> RUN_CNT_SHIFT;
+        e += c & RUN_CNT_ENTRIES;
+    }
+}
+
+// runs of chunk c of a row: [first block, end block), [first run, end run) of the row's list
+__device__ __forceinline__ void chunk_bounds(const RunArgs& a, const RunRow& r, unsigned c, RunChunk& k, unsigned& bend,
+                                             unsigned& rend)
+{
+    k = a.chunk[r.chunk + c];
+    if (c + 1 < r.nchunks) {
+        const RunChunk n = a.chunk[r.chunk + c + 1];
+        bend = n.block;
+        rend = n.run;
+    } else {
+        bend = a.blocks;
+        rend = r.runs;
+    }
+}
+
+struct alignas(16) CollectSmem {
+    unsigned short own[CHUNK_RUNS];      // block (from the chunk's first) whose runs start at a run, 1-based; 0: none
+    int d[RUN_MAX_GRID + 1];             // the columns' difference array
+    unsigned from[CHUNK_BLOCKS];         // where run j of the chunk lies, if in the block: from + j
+    int w[RUN_WARPS];
+};
+
+// The runs of chunk `chunk` of a tile row: front-end blocks [block, bend), runs [run, run + n) of the
+// row. A thread takes eight consecutive runs; all its loads are in flight together. Which block a run
+// lies in follows from a maximum scan over the blocks' first runs. clip: the frame has more entries
+// than the workspace holds and keeps those whose place in (tile row, slot, column) order lies below
+// the capacity; `entry` entries of the frame lie before block `from` then.
+__device__ __forceinline__ void collect_chunk(const RunArgs& a, const RunRow& r, unsigned row, unsigned chunk,
+                                              unsigned block, unsigned bend, unsigned run, unsigned n, bool clip,
+                                              unsigned from, unsigned long long entry, CollectSmem& S)
+{
+    constexpr int PER = CHUNK_RUNS / RUN_THREADS;
+    const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const size_t at = (size_t)row * a.blocks;
+    for (int j = (int)tid; j <= a.cols; j += RUN_THREADS) S.d[j] = 0;
+    static_assert(CHUNK_RUNS * 2 == RUN_THREADS * 16, "16 bytes of own per thread");
+    reinterpret_cast<uint4*>(S.own)[tid] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+#pragma unroll 4
+    for (unsigned b = block + tid; b < bend; b += RUN_THREADS) {
+        const unsigned first = a.pre[at + b] - run;
+        if (a.cnt[at + b] >> RUN_CNT_SHIFT) {
+            S.own[first] = (unsigned short)(b - block + 1);
+            S.from[b - block] = a.seg[at + b] - first;
+        }
+    }
+    __syncthreads();
+    unsigned own[PER]; // block of each run, 1-based (a running maximum)
+    {
+        const uint4 q = reinterpret_cast<const uint4*>(S.own)[tid];
+        const unsigned w[4] = {q.x, q.y, q.z, q.w};
+        unsigned m = 0;
+#pragma unroll
+        for (int u = 0; u < PER; u++) {
+            const unsigned o = u & 1 ? w[u >> 1] >> 16 : w[u >> 1] & 0xffffu;
+            m = o > m ? o : m;
+            own[u] = m;
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, m, o);
+            if ((int)lane >= o) m = y > m ? y : m;
+        }
+        if (lane == 31) S.w[warp] = (int)m;
+        unsigned before = __shfl_up_sync(0xffffffffu, m, 1);
+        if (lane == 0) before = 0;
+        __syncthreads();
+        for (unsigned k = 0; k < warp; k++) before = (unsigned)S.w[k] > before ? (unsigned)S.w[k] : before;
+#pragma unroll
+        for (int u = 0; u < PER; u++) own[u] = before > own[u] ? before : own[u];
+    }
+    const unsigned j0 = PER * tid;
+    unsigned v[PER];
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+        const unsigned j = j0 + (unsigned)u;
+        v[u] = j < n ? a.runs[S.from[own[u] - 1] + j] : 0u;
+    }
+    uint2* const list = a.list + r.base + run;
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+        const unsigned j = j0 + (unsigned)u;
+        if (j >= n) break;
+        unsigned ta = run_first(v[u]), tb = run_last(v[u]);
+        const unsigned b = block + own[u] - 1;
+        if (clip) {
+            unsigned long long p = entry;
+            for (unsigned q = from; q < b; q++) p += a.cnt[at + q] & RUN_CNT_ENTRIES;
+            const unsigned f = a.seg[at + b], me = S.from[own[u] - 1] + j;
+            for (unsigned q = f; q < me; q++) p += run_last(a.runs[q]) - run_first(a.runs[q]) + 1u;
+            if (p >= (unsigned long long)a.cap) { // an empty run
+                ta = 1;
+                tb = 0;
+            } else if (p + (tb - ta + 1u) > (unsigned long long)a.cap) {
+                tb = ta + (unsigned)((unsigned long long)a.cap - p) - 1u;
+            }
+        }
+        list[j] = make_uint2(b * RUN_SLOTS + run_slot(v[u]), ta | (tb << 16));
+        if (ta <= tb) {
+            atomicAdd(&S.d[ta], 1);
+            atomicSub(&S.d[tb + 1], 1);
+        }
+    }
+    __syncthreads();
+    const int pitch = run_pitch(a.cols);
+    int carry = 0;
+    for (int g = 0; g < a.cols; g += RUN_THREADS) {
+        const int col = g + (int)tid;
+        int all;
+        const int x = run_block_scan<RUN_WARPS>(col < a.cols ? S.d[col] : 0, S.w, all);
+        if (col < a.cols) a.col[(size_t)chunk * pitch + col] = (unsigned)(carry + x);
+        carry += all;
+    }
+}
+
+// Grid (blocks per row, rows): block x of a row takes its chunks x, x + gridDim.x, ...
+__global__ void __launch_bounds__(RUN_THREADS) k_run_collect(RunArgs a)
+{
+    __shared__ CollectSmem S;
+    grid_dependency_wait();
+    const unsigned row = blockIdx.y;
+    const RunRow r = a.row[row];
+    if (blockIdx.x >= r.nchunks) return;
+    const bool clip = !a.box_total && a.ctr->n_entries_total > (unsigned long long)a.cap;
+    unsigned long long start = 0;
+    if (clip)
+        for (unsigned q = 0; q < row; q++) start += a.row[q].entries;
+    for (unsigned c = blockIdx.x; c < r.nchunks; c += gridDim.x) {
+        RunChunk k;
+        unsigned bend, rend;
+        chunk_bounds(a, r, c, k, bend, rend);
+        if (rend > k.run)
+            collect_chunk(a, r, row, r.chunk + c, k.block, bend, k.run, rend - k.run, clip, k.block, start + k.entry, S);
+        else // no run: no entries in any column
+            for (int j = (int)threadIdx.x; j < a.cols; j += RUN_THREADS)
+                a.col[(size_t)(r.chunk + c) * run_pitch(a.cols) + j] = 0u;
+    }
+}
+
+// Small frames (at most RUN_SMALL_BLOCKS front-end blocks), which the number of dependent launches
+// bounds: block x of a row takes chunk x, which it finds itself from the blocks' counts, and the
+// front end summed the rows' totals; k_run_rows and k_run_offsets are not launched.
+__global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
+{
+    __shared__ CollectSmem S;
+    __shared__ unsigned s_w[RUN_WARPS], s_first, s_end, s_run, s_rend, s_chunks;
+    __shared__ unsigned long long s_before, s_all;
+    static_assert(RUN_SMALL_BLOCKS <= RUN_THREADS, "one thread per front-end block");
+    grid_dependency_wait();
+    const unsigned row = blockIdx.y, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    if (warp == RUN_WARPS - 1) { // totals of the earlier rows, and of the frame
+        unsigned long long before = 0, all = 0;
+        for (unsigned q = lane; (int)q < a.rows; q += 32) {
+            const unsigned long long t = a.tot[q];
+            before += q < row ? t : 0ull;
+            all += t;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        if (lane == 0) {
+            s_before = before;
+            s_all = all & RUN_TOT_ENTRIES;
+        }
+    }
+    if (tid == 0) {
+        s_first = s_run = 0xffffffffu;
+        s_end = s_rend = 0u;
+    }
+    const unsigned rn = tid < a.blocks ? a.cnt[(size_t)row * a.blocks + tid] >> RUN_CNT_SHIFT : 0u;
+    unsigned rtot;
+    const unsigned p = run_block_scan<RUN_WARPS>(rn, s_w, rtot) - rn; // its barriers order the shared words above
+    if (tid < a.blocks && chunk_of(p, 0) == blockIdx.x) {
+        a.pre[(size_t)row * a.blocks + tid] = p;
+        atomicMin(&s_first, tid);
+        atomicMax(&s_end, tid + 1);
+        atomicMin(&s_run, p);
+        atomicMax(&s_rend, p + rn);
+    }
+    if (tid == a.blocks - 1) s_chunks = rtot ? chunk_of(p, 0) + 1 : 0u;
+    __syncthreads();
+    RunRow r{row * small_chunks(a.blocks), s_chunks, (unsigned)(s_before >> RUN_TOT_SHIFT), rtot,
+             a.tot[row] & RUN_TOT_ENTRIES};
+    if (tid == 0 && blockIdx.x == 0) {
+        a.row[row] = r;
+        if (row == 0 && !a.box_total) a.ctr->n_entries_total = s_all;
+    }
+    if (blockIdx.x >= r.nchunks) return;
+    if (tid == s_first) a.chunk[r.chunk + blockIdx.x] = RunChunk{tid, p, 0ull};
+    collect_chunk(a, r, row, r.chunk + blockIdx.x, s_first, s_end, s_run, s_rend - s_run,
+                  !a.box_total && s_all > (unsigned long long)a.cap, 0, s_before & RUN_TOT_ENTRIES, S);
+}
+
+// One block per tile row: OFF_SEGS segments of the row's chunks x OFF_COLS columns at a time.
+constexpr int OFF_SEGS = 4, OFF_COLS = 256;
+
+__global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
+{
+    __shared__ unsigned s_sum[OFF_SEGS][OFF_COLS];
+    __shared__ unsigned s_first[OFF_COLS];
+    __shared__ unsigned s_w[OFF_COLS / 32];
+    __shared__ unsigned s_start;
+    grid_dependency_wait();
+    const unsigned row = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const unsigned long long cap = (unsigned long long)a.cap;
+    const RunRow r = a.row[row];
+    const int pitch = run_pitch(a.cols);
+    const unsigned sg = tid / OFF_COLS, c = tid % OFF_COLS;
+    const unsigned per = (r.nchunks + OFF_SEGS - 1) / OFF_SEGS;
+    const unsigned k0 = sg * per, k1 = k0 + per < r.nchunks ? k0 + per : r.nchunks;
+    if (warp == OFF_SEGS * OFF_COLS / 32 - 1) { // entries of the earlier tile rows; of the frame (row 0)
+        unsigned long long before = 0, all = 0;
+        for (unsigned k = lane; (int)k < a.rows; k += 32) {
+            const unsigned long long e = a.row[k].entries;
+            before += k < row ? e : 0ull;
+            all += e;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        if (lane == 0) s_start = (unsigned)(before < cap ? before : cap);
+        if (lane == 0 && row == 0) {
+            const unsigned long long total = a.box_total ? a.ctr->n_entries_total : all;
+            a.ctr->n_entries = (unsigned)(total < cap ? total : cap);
+            if (total > cap) {
+                atomicOr(&a.ctr->overflow, 1u);
+                atomicOr(&a.sticky->overflow, 1u);
+            }
+        }
+    }
+    unsigned run = 0; // entries of the row's earlier columns
+    for (int g = 0; g < a.cols; g += OFF_COLS) {
+        const int col = g + (int)c;
+        unsigned* const p = a.col + (size_t)r.chunk * pitch + col;
+        unsigned sum = 0;
+        if (col < a.cols)
+#pragma unroll 8
+            for (unsigned k = k0; k < k1; k++) sum += p[(size_t)k * pitch];
+        s_sum[sg][c] = sum;
+        __syncthreads();
+        unsigned total = 0, incl = 0;
+        if (sg == 0) {
+#pragma unroll
+            for (int q = 0; q < OFF_SEGS; q++) total += s_sum[q][c];
+            incl = run_warp_scan(total);
+            if (lane == 31) s_w[warp] = incl;
+        }
+        __syncthreads();
+        unsigned row_all = 0;
+#pragma unroll
+        for (int q = 0; q < OFF_COLS / 32; q++) {
+            if (sg == 0 && q < (int)warp) incl += s_w[q];
+            row_all += s_w[q];
+        }
+        if (sg == 0) {
+            const unsigned first = s_start + run + incl - total;
+            s_first[c] = first;
+            if (col < a.cols) {
+                // entries past the capacity are not written
+                const unsigned b = first < a.cap ? first : (unsigned)a.cap;
+                const unsigned e = first + total < a.cap ? first + total : (unsigned)a.cap;
+                a.ranges[(size_t)row * a.cols + col] = e > b ? make_uint2(b, e) : make_uint2(0u, 0u);
+            }
+        }
+        __syncthreads();
+        if (col < a.cols) {
+            unsigned at = s_first[c];
+            for (unsigned q = 0; q < sg; q++) at += s_sum[q][c];
+#pragma unroll 8
+            for (unsigned k = k0; k < k1; k++) {
+                const unsigned n = p[(size_t)k * pitch];
+                p[(size_t)k * pitch] = at;
+                at += n;
+            }
+        }
+        run += row_all;
+        __syncthreads();
+    }
+}
+
+constexpr int SUBS = CHUNK_RUNS / 32, SEGS = RUN_THREADS / SUBS, SEG_COLS = COLS / SEGS;
+static_assert(SUBS == 64 && SEGS * SUBS == RUN_THREADS && SEG_COLS % 2 == 0, "a lane holds two words of 32 runs");
+
+struct ExpandSmem {
+    unsigned mask[COLS][PITCH];
+    unsigned seg[SEGS][SUBS]; // XOR of a segment of columns, then of the segments before it
+    unsigned id[CHUNK_RUNS];
+    unsigned first[RUN_MAX_GRID]; // first slot in vals of the chunk's entries of each column
+    unsigned w[RUN_WARPS];
+    unsigned start;
+};
+static_assert(sizeof(ExpandSmem) <= 48 * 1024, "no opt-in to more shared memory");
+
+// k_run_offsets for the chunk of one block of a small frame: the first slot of each of its columns
+// (S.first), from the column counts of all chunks of the row; block 0 of a row writes the ranges.
+__device__ __forceinline__ void small_offsets(const RunArgs& a, const RunRow& r, unsigned row, ExpandSmem& S)
+{
+    const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const unsigned long long cap = (unsigned long long)a.cap;
+    if (warp == RUN_WARPS - 1) {
+        unsigned long long before = 0;
+        for (unsigned q = lane; q < row; q += 32) before += a.tot[q] & RUN_TOT_ENTRIES;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        if (lane == 0) S.start = (unsigned)(before < cap ? before : cap);
+    }
+    if (blockIdx.x == 0 && row == 0 && tid == 0) {
+        const unsigned long long total = a.ctr->n_entries_total;
+        a.ctr->n_entries = (unsigned)(total < cap ? total : cap);
+        if (total > cap) {
+            atomicOr(&a.ctr->overflow, 1u);
+            atomicOr(&a.sticky->overflow, 1u);
+        }
+    }
+    const int pitch = run_pitch(a.cols);
+    unsigned run = 0; // entries of the row's earlier columns
+    for (int g = 0; g < a.cols; g += RUN_THREADS) {
+        const int col = g + (int)tid;
+        unsigned total = 0, before = 0; // of the column, of the earlier chunks
+        if (col < a.cols)
+            for (unsigned k = 0; k < r.nchunks; k++) {
+                const unsigned n = a.col[(size_t)(r.chunk + k) * pitch + col];
+                before += k < blockIdx.x ? n : 0u;
+                total += n;
+            }
+        unsigned all;
+        const unsigned incl = run_block_scan<RUN_WARPS>(total, S.w, all);
+        const unsigned first = S.start + run + incl - total;
+        if (col < a.cols) {
+            S.first[col] = first + before;
+            if (blockIdx.x == 0) {
+                const unsigned b = first < a.cap ? first : (unsigned)a.cap;
+                const unsigned e = first + total < a.cap ? first + total : (unsigned)a.cap;
+                a.ranges[(size_t)row * a.cols + col] = e > b ? make_uint2(b, e) : make_uint2(0u, 0u);
+            }
+        }
+        run += all;
+    }
+}
+
+// Grid as the collect kernel's.
+template <bool SMALL>
+__global__ void __launch_bounds__(RUN_THREADS, 5) k_run_expand(RunArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ExpandSmem& S = *reinterpret_cast<ExpandSmem*>(smem_raw);
+    grid_dependency_wait();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned row = blockIdx.y;
+    const RunRow r = a.row[row];
+    if (SMALL && (blockIdx.x == 0 || blockIdx.x < r.nchunks)) small_offsets(a, r, row, S);
+    if (blockIdx.x >= r.nchunks) return;
+    const int pitch = run_pitch(a.cols);
+    const unsigned cap = (unsigned)a.cap;
+    // groups of an even number of columns
+    const int groups = (a.cols + COLS - 1) / COLS, group = ((a.cols + groups - 1) / groups + 1) & ~1;
+    for (unsigned c = blockIdx.x; c < r.nchunks; c += gridDim.x) {
+        RunChunk k;
+        unsigned bend, rend;
+        chunk_bounds(a, r, c, k, bend, rend);
+        const unsigned n = rend - k.run; // at most CHUNK_RUNS
+        if (n == 0) continue;
+        const uint2* const list = a.list + r.base + k.run;
+        unsigned ends[CHUNK_RUNS / RUN_THREADS]; // the thread's runs: first and last column
+#pragma unroll
+        for (int u = 0; u < CHUNK_RUNS / RUN_THREADS; u++) {
+            const unsigned j = (unsigned)(u * RUN_THREADS + tid);
+            const uint2 q = j < n ? __ldg(&list[j]) : make_uint2(0u, 1u);
+            if (j < n) S.id[j] = q.x;
+            ends[u] = q.y;
+        }
+        if (!SMALL)
+            for (int j = tid; j < a.cols; j += RUN_THREADS) S.first[j] = __ldg(&a.col[(size_t)(r.chunk + c) * pitch + j]);
+        for (int g = 0; g < a.cols; g += group) {
+            const int cols = a.cols - g < group ? a.cols - g : group;
+            for (int j = tid; j < cols * PITCH / 2; j += RUN_THREADS)
+                reinterpret_cast<uint2*>(&S.mask[0][0])[j] = make_uint2(0u, 0u);
+            __syncthreads();
+            // run 32 s + l of the chunk: bit 31 - l of word s (the first run is the highest bit)
+#pragma unroll
+            for (int u = 0; u < CHUNK_RUNS / RUN_THREADS; u++) {
+                const int ta = (int)(ends[u] & 0xffffu) - g, tb = (int)(ends[u] >> 16) - g;
+                if (ta <= tb && tb >= 0 && ta < cols) { // an empty run has ta = 1, tb = 0
+                    const int sub = u * (RUN_THREADS / 32) + warp;
+                    atomicXor(&S.mask[ta > 0 ? ta : 0][sub], 0x80000000u >> lane);
+                    if (tb + 1 < cols) atomicXor(&S.mask[tb + 1][sub], 0x80000000u >> lane);
+                }
+            }
+            __syncthreads();
+            { // prefix XOR over the columns, in SEGS segments
+                const int sub = tid % SUBS, sg = tid / SUBS;
+                const int c0 = sg * SEG_COLS, c1 = c0 + SEG_COLS < cols ? c0 + SEG_COLS : cols;
+                unsigned x = 0;
+#pragma unroll 8
+                for (int q = c0; q < c1; q++) {
+                    x ^= S.mask[q][sub];
+                    S.mask[q][sub] = x;
+                }
+                S.seg[sg][sub] = x;
+                __syncthreads();
+                unsigned before = 0;
+                for (int q = 0; q < sg; q++) before ^= S.seg[q][sub];
+                __syncthreads();
+                S.seg[sg][sub] = before;
+            }
+            __syncthreads();
+            // a warp takes two columns at a time (one scan of 16-bit counts, two chains of stores)
+            for (int q = 2 * warp; q < cols; q += 2 * RUN_WARPS) {
+                const bool two = q + 1 < cols;
+                const uint2 b = *reinterpret_cast<const uint2*>(&S.seg[q / SEG_COLS][2 * lane]);
+                const uint2 m0 = *reinterpret_cast<const uint2*>(&S.mask[q][2 * lane]);
+                const uint2 m1 = two ? *reinterpret_cast<const uint2*>(&S.mask[q + 1][2 * lane]) : b;
+                unsigned lo0 = m0.x ^ b.x, hi0 = m0.y ^ b.y, lo1 = m1.x ^ b.x, hi1 = m1.y ^ b.y;
+                const unsigned cnt = (unsigned)(__popc(lo0) + __popc(hi0)) + ((unsigned)(__popc(lo1) + __popc(hi1)) << 16);
+                const unsigned excl = run_warp_scan(cnt) - cnt;
+                unsigned d0 = S.first[g + q] + (excl & 0xffffu), d1 = S.first[two ? g + q + 1 : g + q] + (excl >> 16);
+                const unsigned* const id = &S.id[64 * lane];
+                auto put = [&](unsigned& m, unsigned& d, int half) {
+                    if (m) {
+                        const int j = __clz((int)m);
+                        if (d < cap) a.vals[d] = id[half + j];
+                        d++;
+                        m ^= 0x80000000u >> j;
+                    }
+                };
+                while (lo0 | lo1) {
+                    put(lo0, d0, 0);
+                    put(lo1, d1, 0);
+                }
+                while (hi0 | hi1) {
+                    put(hi0, d0, 32);
+                    put(hi1, d1, 32);
+                }
+            }
+            __syncthreads(); // the masks are cleared for the next columns or chunk
+        }
+    }
+}
+
+void launch_runs(const RunArgs& a, cudaStream_t s, cudaEvent_t ev_after_collect)
+{
+    if (a.blocks == 0) return;
+    const dim3 block(RUN_THREADS);
+    if (a.tot) {
+        const dim3 grid(small_chunks(a.blocks), (unsigned)a.rows);
+        launch_dependent(k_run_collect_small, grid, block, 0, s, a);
+        if (ev_after_collect) cudaEventRecord(ev_after_collect, s);
+        launch_dependent(k_run_expand<true>, grid, block, sizeof(ExpandSmem), s, a);
+        return;
+    }
+    // at most the chunks a row can have, and about 8 waves of blocks over all rows
+    const unsigned most = a.blocks * (unsigned)RUN_SLOTS / CHUNK_STEP + a.blocks / CHUNK_BLOCKS + 1;
+    const unsigned want = (unsigned)(8 * 5 * device_sm_count() / a.rows + 1);
+    const dim3 grid(most < want ? most : want, (unsigned)a.rows);
+    launch_dependent(k_run_rows, dim3((unsigned)a.rows), dim3(1024), 0, s, a);
+    launch_dependent(k_run_collect, grid, block, 0, s, a);
+    if (ev_after_collect) cudaEventRecord(ev_after_collect, s);
+    launch_dependent(k_run_offsets, dim3((unsigned)a.rows), dim3(OFF_SEGS * OFF_COLS), 0, s, a);
+    launch_dependent(k_run_expand<false>, grid, block, sizeof(ExpandSmem), s, a);
+}
+
+} // namespace rg

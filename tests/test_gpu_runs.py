@@ -1,0 +1,92 @@
+"""Entries written from tile-row runs (the default RoofGS frame) at the sizes where their grouping
+changes shape: entries, ranges, counters and images bit-identical to the fused front end's with its
+radix passes, whose own parity with the oracle is tested elsewhere. Whole numbers: exact equality."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2608_15785_gb300 import binding, synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_15785_gb300.build import build
+    build()
+
+
+def _entries(gs):
+    return [gs.inspect(k) for k in (binding.RG_INSPECT_KEYS, binding.RG_INSPECT_VALUES, binding.RG_INSPECT_RANGES)]
+
+
+def _scene(n, scale=1.0, seed=3):
+    sc = synth.tiny_scene(n, seed=seed)
+    sc.scales = (sc.scales * np.float32(scale)).astype(np.float32)
+    return sc
+
+
+# n around the last small frame (128 blocks of 256 Gaussians); few tile rows with many runs each (several
+# chunks per row); sparse rows over more than 1,024 front-end blocks; 512 tile columns and rows (the
+# largest grid of runs, column groups) and 513 (the fused front end); one tile
+CASES = [(255, (64, 48), (16, 16), 1.0), (32_768, (256, 256), (16, 16), 1.0), (32_769, (256, 256), (16, 16), 1.0),
+         (60_000, (90, 40), (16, 16), 1.0), (400_000, (48, 48), (8, 32), 0.5), (300_000, (640, 1600), (32, 8), 0.05),
+         (4_000, (8192, 40), (16, 16), 3.0), (4_000, (40, 8192), (16, 16), 3.0), (40_000, (8192, 40), (16, 16), 2.0),
+         (4_000, (8208, 40), (16, 16), 3.0), (4_000, (40, 8208), (16, 16), 3.0), (5_000, (5, 7), (16, 16), 4.0)]
+
+
+@pytest.mark.parametrize("n,wh,tile,scale", CASES)
+def test_runs_equal_the_ordered_front_end(n, wh, tile, scale):
+    cam = synth.tiny_camera(*wh, bg=(0.2, 0.1, 0.3))
+    if wh[1] > 4 * wh[0]:
+        cam.fx = cam.fy = float(np.float32(wh[1] * 0.8))  # the cube over the whole height
+    gs = binding.Scene(_scene(n, scale))
+    a, sa = gs.render(cam, flags=binding.RG_FLAG_QUAD_PIXEL, stats=True, tile=tile)
+    ea = _entries(gs)
+    # (the first image is the counting launch's)
+    a = gs.render(cam, flags=binding.RG_FLAG_QUAD_PIXEL, tile=tile)
+    b, sb = gs.render(cam, flags=binding.RG_FLAG_QUAD_PIXEL | binding.RG_FLAG_ORDERED_FRONT_END, stats=True, tile=tile)
+    eb = _entries(gs)
+    assert sa["n_entries"] > 0
+    for f in ("n_entries", "n_visible", "n_front", "n_pairs", "n_blends"):
+        assert sa[f] == sb[f], f
+    for x, y in zip(ea, eb):
+        assert np.array_equal(x, y)
+    assert torch.equal(a, b)
+    gs.check()
+
+
+@pytest.mark.parametrize("n", [20_000, 40_000])
+def test_runs_beyond_the_capacity(n):
+    """A small and a larger frame with too few entries of room: the kept entries are those whose place
+    in (tile row, depth code, index, tile column) order lies below the capacity; the re-rendered frame
+    is complete."""
+    sc = _scene(n, 0.7)
+    cam = synth.tiny_camera(200, 150)
+    gs = binding.Scene(sc)
+    gs.reserve(9_000)
+    gs.render(cam)
+    torch.cuda.synchronize()
+    gk = gs.inspect(binding.RG_INSPECT_KEYS).view(np.uint32).astype(np.uint64)
+    gv = gs.inspect(binding.RG_INSPECT_VALUES)
+    k, v, _, _ = oracle.keys(sc, cam, oracle.ROOFGS, comp=oracle.compact(sc))
+    lay = oracle.layout(cam)
+    b_d = np.uint64(lay["b_d"])
+    tile = k >> b_d
+    tx, ty = tile % np.uint64(lay["tiles_x"]), tile // np.uint64(lay["tiles_x"])
+    assert gk.size == 9_000 < k.size
+    kept = np.lexsort((tx, v, k & ((np.uint64(1) << b_d) - np.uint64(1)), ty))[:9_000]
+    expect = kept[np.lexsort((v[kept], k[kept]))]
+    assert np.array_equal(gk, k[expect]) and np.array_equal(gv, v[expect])
+    with pytest.raises(binding.RgError) as e:
+        gs.check()
+    assert e.value.status == 4
+    img, st = gs.render(cam, stats=True)
+    assert st["regrown"] == 1 and st["n_entries"] == k.size
+    full = binding.Scene(sc)
+    assert torch.equal(img, full.render(cam, stats=True)[0])
