@@ -3,10 +3,9 @@
  *
  * Forward render of 3D Gaussian Splatting in two modes:
  *   RG_MODE_EXACT   the plain 3DGS path: FP32 attributes (236 bytes per
- *                   Gaussian, paper Sec. III-A, Eq. (3)), separate
- *                   preprocess / scan / duplicate kernels, 64-bit
- *                   tile|float-depth keys (Sec. IV-A.2), IEEE expf in the
- *                   rasterizer (Eqs. (7), (10)-(12));
+ *                   Gaussian, paper Sec. III-A, Eq. (3)), entries in the order
+ *                   of 64-bit tile|float-depth keys (Sec. IV-A.2), IEEE expf in
+ *                   the rasterizer (Eqs. (7), (10)-(12));
  *   RG_MODE_ROOFGS  the paper's method: compact attributes (FP32 mean, FP16
  *                   rotation and scale, INT8 spherical harmonics with one
  *                   scale per degree and channel, Sec. IV-A.1, Eq. (8)), one
@@ -201,8 +200,12 @@ rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries);
  * Render one view into out_chw, a caller-owned buffer of 3*H*W FP32 values laid
  * out [channel][row][column]: device memory, or pinned host memory that the
  * device addresses (the image is then written straight to the host).
- * Pipeline (exact): preprocess -> scan -> duplicate -> 64-bit radix sort ->
- * tile ranges -> rasterizer (Sec. II-A pipeline, Sec. III). The exponent of
+ * Pipeline (exact): Gaussians ordered by float depth -> preprocess -> entries grouped
+ * by tile in that order (the order of the 64-bit keys tile | float depth; tile grids
+ * above 512 x 512 tiles duplicate and sort such keys instead) -> rasterizer (Sec. II-A
+ * pipeline, Sec. III). Tiles of a Gaussian's 3-sigma rectangle where it stays below
+ * alpha = 1/255 are entries (rg_stats, capacity, rg_inspect) but take no part, except
+ * in a call given stats, whose pair counters are plain 3DGS's. The exponent of
  * Eq. (10) is evaluated from the projected mean carried at twice single
  * precision and the quadratic form completed in dx, so the image stays within
  * 2e-4 per channel of an FP64 evaluation except where a pair's alpha or T lies
@@ -235,9 +238,9 @@ rg_status rg_scene_check(rg_scene* scene, void* stream);
 /*
  * Per-stage device times (ms) of the frames rendered with RG_FLAG_STAGE_EVENTS
  * since the last call (at most the last 512 frames), summed: ms7[0] = depth order of
- * the Gaussians (RoofGS; 0 otherwise), ms7[1] = front end (RoofGS fused kernel; exact
- * preprocess + scan + duplicate), ms7[2] = sort histogram, ms7[3] = sort passes,
- * ms7[4] = tile ranges, ms7[5] = rasterizer, ms7[6] = whole frame. *frames receives
+ * the Gaussians, ms7[1] = front end, ms7[2] = collection of the tile-row runs (sort
+ * histogram in frames that sort entries), ms7[3] = entries written from them (sort
+ * passes), ms7[4] = tile ranges, ms7[5] = rasterizer, ms7[6] = whole frame. *frames receives
  * the number of frames summed. Synchronises the recorded events.
  */
 rg_status rg_stage_times(rg_scene* scene, float* ms7, int32_t* frames);

@@ -72,9 +72,10 @@ __global__ void __launch_bounds__(B_THREADS) k_raster_backward(BackwardArgs a)
         if (j < range.y) {
             unsigned id = a.vals[j];
             if (id >= (unsigned long long)a.n) id = 0;
-            const float4 m = a.mean2[id];
+            const float4* const rec = a.erec + 3 * (size_t)id;
+            const float4 m = __ldg(rec);
             s_xy[threadIdx.x] = make_float4(m.x - (float)x0, m.y, m.z - (float)y0, m.w);
-            s_co[threadIdx.x] = a.quad[id];
+            s_co[threadIdx.x] = __ldg(rec + 1);
         }
         __syncthreads();
         const int cnt = min((unsigned)B_THREADS, range.y - start);
@@ -114,10 +115,11 @@ __global__ void __launch_bounds__(B_THREADS) k_raster_backward(BackwardArgs a)
             unsigned id = a.vals[j];
             if (id >= (unsigned long long)a.n) id = 0;
             s_id[threadIdx.x] = id;
-            const float4 m = a.mean2[id];
+            const float4* const rec = a.erec + 3 * (size_t)id;
+            const float4 m = __ldg(rec);
             s_xy[threadIdx.x] = make_float4(m.x - (float)x0, m.y, m.z - (float)y0, m.w);
-            s_co[threadIdx.x] = a.quad[id];
-            s_rgb[threadIdx.x] = make_float4(a.rgb[3 * id], a.rgb[3 * id + 1], a.rgb[3 * id + 2], 0.f);
+            s_co[threadIdx.x] = __ldg(rec + 1);
+            s_rgb[threadIdx.x] = __ldg(rec + 2);
         }
         __syncthreads();
         const int cnt = min((long long)B_THREADS, (long long)range.y - start);
@@ -212,8 +214,9 @@ __device__ __forceinline__ void sh_basis_grad(float x, float y, float z, float g
 __global__ void __launch_bounds__(128) k_preprocess_backward(BackwardArgs a)
 {
     grid_dependency_wait();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    const long long slot = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (slot >= a.n) return;
+    const long long i = a.order ? (long long)a.order[slot] : slot;
     float* dm = a.dmeans + 3 * i;
     float* ds = a.dscales + 3 * i;
     float* dq = a.dquats + 4 * i;
@@ -222,8 +225,8 @@ __global__ void __launch_bounds__(128) k_preprocess_backward(BackwardArgs a)
     for (int k = 0; k < 4; k++) dq[k] = 0.f;
     for (int k = 0; k < 48; k++) dsh[k] = 0.f;
     a.dopac[i] = 0.f;
-    if (a.touched[i] == 0) return; // emitted no entry: no pixel depends on it
-    const float* g = a.gbuf + 9 * i;
+    if (a.touched[slot] == 0) return; // emitted no entry: no pixel depends on it
+    const float* g = a.gbuf + 9 * slot;
     const float g_u = g[0], g_v = g[1], g_A = g[2], g_B = g[3], g_C = g[4];
     a.dopac[i] = g[5];
     const CamDev& c = a.cam;

@@ -20,8 +20,10 @@
 //    runs.cu writes the entries from those runs, in their final place.
 //  * k_depth_keys: quantized depth and index of every Gaussian, the input of
 //    the per-Gaussian depth sort, and the digit counts of that sort.
-//  * k_exact_*: the plain 3DGS front end (preprocess -> scan -> duplicate,
-//    Sec. II-A), 64-bit keys of 32-bit tile id | 32-bit float depth.
+//  * k_exact_depth_keys, k_exact_runs: the plain 3DGS front end over tile-row runs, in
+//    the order of the float depth; k_exact_preprocess -> k_exact_scan ->
+//    k_exact_duplicate: the same entries one by one with 64-bit keys of 32-bit tile id |
+//    32-bit float depth (Sec. II-A), for tile grids too large for runs.
 //  * scene conversion: finite-value check, per-(degree, channel) max |SH|,
 //    and the compact attribute encoder.
 #include <atomic>
@@ -591,16 +593,23 @@ __global__ void __launch_bounds__(FE_THREADS, RG_FER_MIN_BLOCKS) k_frontend_runs
     }
 }
 
+// the shared memory of the largest tile grids needs the opt-in (once per device and kernel; setting it
+// twice does no harm)
+template <typename K>
+static void run_smem_opt_in(K kernel, std::atomic<bool> (&opted)[64])
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && opted[dev].load()) return;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RUN_MAX_GRID * (int)sizeof(RunRowSmem));
+    if (dev >= 0 && dev < 64) opted[dev].store(true);
+}
+
 void launch_frontend_runs(const FrontendArgs& a, const RunArgs& r, cudaStream_t s)
 {
     if (r.blocks == 0) return;
-    // the shared memory of the largest tile grids needs the opt-in (once per device)
     static std::atomic<bool> opted[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !opted[dev].exchange(true))
-        cudaFuncSetAttribute(k_frontend_runs, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             RUN_MAX_GRID * (int)sizeof(RunRowSmem));
+    run_smem_opt_in(k_frontend_runs, opted);
     launch_dependent(k_frontend_runs, dim3(r.blocks), dim3(FE_THREADS), (size_t)r.rows * sizeof(RunRowSmem), s, a, r);
 }
 
@@ -609,6 +618,37 @@ void launch_frontend_runs(const FrontendArgs& a, const RunArgs& r, cudaStream_t 
 // ---------------------------------------------------------------------------
 constexpr int EX_THREADS = 256;
 
+// The raster record of Gaussian i, binned as b: the exponent of Eq. (10) with the quadratic form
+// completed in dx, -1/2 ((Sigma'_yy / det) (dx - c dy)^2 + dy^2 / Sigma'_yy), c = Sigma'_xy / Sigma'_yy
+// (no cancellation for thin Gaussians), the mean as double-floats (b's FP32 u, v only bin the
+// Gaussian), and the degree-3 SH colour from FP32 coefficients.
+__device__ __forceinline__ void exact_record(const ExactArgs& a, long long i, const Binned& b, float mx, float my,
+                                             float mz, float4& mean, float4& quad, float4& rgb)
+{
+    quad = make_float4(-0.5f * __fdiv_rn(b.sc, b.det), __fdiv_rn(b.sb, b.sc), __fdiv_rn(-0.5f, b.sc), a.opac[i]);
+    mean = project_mean_df(a.cam, mx, my, mz);
+    float dx, dy, dz;
+    view_dir(a.cam, mx, my, mz, dx, dy, dz);
+    float Y[16];
+    sh_basis(dx, dy, dz, Y);
+    const int nk = (a.sh_degree + 1) * (a.sh_degree + 1);
+    const float4* shp = reinterpret_cast<const float4*>(a.sh + 48 * i);
+    float c[3] = {0.5f, 0.5f, 0.5f};
+#pragma unroll
+    for (int v4 = 0; v4 < 12; v4++) {
+        const float4 f = shp[v4];
+        const float e[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int j = 4 * v4 + u;
+            const int k = j / 3, ch = j % 3;
+            if (k < nk) c[ch] = fmaf(Y[k], e[u], c[ch]);
+        }
+    }
+    rgb = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), 0.0f);
+}
+
+// Front end in index order: the frames whose tile grid is too large for runs.
 __global__ void __launch_bounds__(EX_THREADS) k_exact_preprocess(ExactArgs a)
 {
     grid_dependency_wait();
@@ -628,37 +668,173 @@ __global__ void __launch_bounds__(EX_THREADS) k_exact_preprocess(ExactArgs a)
     const unsigned vm = __ballot_sync(__activemask(), vis);
     if (vis && __popc(vm & ((1u << (threadIdx.x & 31)) - 1u)) == 0) atomicAdd(&a.ctr->n_visible, (unsigned)__popc(vm));
     if (!vis) return;
-    // the rasterizer's exponent (Eq. (10)) with the quadratic form completed in dx:
-    // -1/2 ((Sigma'_yy / det) (dx - c dy)^2 + dy^2 / Sigma'_yy), c = Sigma'_xy / Sigma'_yy
-    // (no cancellation for thin Gaussians); the mean as double-floats (the FP32 u, v
-    // above only bin the Gaussian)
-    a.quad[i] = make_float4(-0.5f * __fdiv_rn(b.sc, b.det), __fdiv_rn(b.sb, b.sc), __fdiv_rn(-0.5f, b.sc), a.opac[i]);
-    a.mean2[i] = project_mean_df(a.cam, mx, my, mz);
     a.depth[i] = pz;
     a.rect[i] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
     a.touched[i] = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
-    // degree-3 SH colour from FP32 coefficients
-    float dx, dy, dz;
-    view_dir(a.cam, mx, my, mz, dx, dy, dz);
-    float Y[16];
-    sh_basis(dx, dy, dz, Y);
-    const int nk = (a.sh_degree + 1) * (a.sh_degree + 1);
-    const float4* shp = reinterpret_cast<const float4*>(a.sh + 48 * i);
-    float c[3] = {0.5f, 0.5f, 0.5f};
+    exact_record(a, i, b, mx, my, mz, a.rec[3 * i], a.rec[3 * i + 1], a.rec[3 * i + 2]);
+}
+
+__global__ void __launch_bounds__(256) k_exact_depth_keys(ExactArgs a, unsigned* keys, unsigned* vals, Counters* ctr,
+                                                          unsigned* hist, unsigned* status0, long long status_words)
+{
+    __shared__ unsigned s_h[4][256];
+    grid_dependency_wait();
+    for (int j = threadIdx.x; j < 4 * 256; j += 256) (&s_h[0][0])[j] = 0u;
+    for (long long j = (long long)blockIdx.x * 256 + threadIdx.x; j < status_words; j += (long long)gridDim.x * 256)
+        status0[j] = 0u;
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->n_entries = (unsigned)a.n;
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (long long)gridDim.x * 256) {
+        const float pz = view_z(a.cam, a.means[3 * i], a.means[3 * i + 1], a.means[3 * i + 2]);
+        // positive floats order as their bits
+        const unsigned k = pz > a.cam.zn && pz <= a.cam.zf ? __float_as_uint(pz) : 0xffffffffu;
+        keys[i] = k;
+        vals[i] = (unsigned)i;
 #pragma unroll
-    for (int v4 = 0; v4 < 12; v4++) {
-        const float4 f = shp[v4];
-        const float e[4] = {f.x, f.y, f.z, f.w};
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const int j = 4 * v4 + u;
-            const int k = j / 3, ch = j % 3;
-            if (k < nk) c[ch] = fmaf(Y[k], e[u], c[ch]);
-        }
+        for (int p = 0; p < 4; p++) atomicAdd(&s_h[p][(k >> (8 * p)) & 255u], 1u);
     }
-    a.rgb[3 * i] = clamp01(c[0]);
-    a.rgb[3 * i + 1] = clamp01(c[1]);
-    a.rgb[3 * i + 2] = clamp01(c[2]);
+    __syncthreads();
+    for (int j = threadIdx.x; j < 4 * 256; j += 256) {
+        const unsigned c = (&s_h[0][0])[j];
+        if (c) atomicAdd(&hist[j], c);
+    }
+}
+
+// Which tiles of a Gaussian's rectangle hold a pixel of alpha >= 1/255, from the rasterizer's own
+// record: -p = kx^-1 t^2 + sz dy^2 (t = dx - c dy) has to be at most `level` = ln(255 o). The level is
+// raised and the extents are widened by more than the FP32 rounding of this test and of
+// exact_power(), so no pair that the rasterizer would blend is lost:
+//  * exact_power() forms t from dx and c dy, each at most rx = sqrt(2 level Sigma'_xx) on the
+//    contour, with a rounding of 2^-23 of each; p then moves by at most 2 sqrt(level / kx) times that, and
+//    1 / kx = Sigma'_yy / (2 det) <= 1 / 0.6 by the dilation: 2.2e-6 rx. The level is raised by 0.01 + 1e-5 rx;
+//  * the extents below carry a few roundings of |u| + rx (2^-23 each); they are widened by 1/16 + 1e-5 (|u| + rx).
+// The pixels of a tile outside the rectangle's 3-sigma box count too, as the rasterizer evaluates them.
+struct ExactRow {
+    float u, v, level, kx, sz, c, ys, padx, pady;
+    int tx0, tx1, ty0;
+};
+
+__device__ __forceinline__ ExactRow exact_row(const Binned& b, const float4& mean, const float4& quad, bool& any)
+{
+    ExactRow r;
+    const float ext = sqrtf(12.0f * fmaxf(b.sa, b.sc)); // at least sqrt(2 level Sigma'_xx), level <= ln 255
+    r.level = LN255F + logf(quad.w) + 0.01f + 1e-5f * ext;
+    any = r.level > 0.0f;
+    r.u = mean.x;
+    r.v = mean.z;
+    r.kx = -1.0f / quad.x;
+    r.sz = -quad.z;
+    r.c = quad.y;
+    r.ys = r.c * sqrtf(r.level / (r.sz * (r.kx * r.sz + r.c * r.c))); // dy of the right-most point
+    r.padx = 0.0625f + 1e-5f * (fabsf(r.u) + ext);
+    r.pady = 0.0625f + 1e-5f * (fabsf(r.v) + ext);
+    r.tx0 = b.tx0;
+    r.tx1 = b.tx1;
+    r.ty0 = b.ty0;
+    return r;
+}
+
+// the tiles [txa, txb] of tile row ty; false if none. Comparisons are written so that a NaN keeps tiles.
+__device__ __forceinline__ bool exact_row_range(const ExactRow& g, int ty, const CamDev& cam, int& txa, int& txb)
+{
+    const float d0 = (float)(ty * cam.th) - g.v - g.pady, d1 = (float)(ty * cam.th + cam.th - 1) - g.v + g.pady;
+    const float near = fmaxf(fmaxf(d0, -d1), 0.0f); // the band's least |dy|
+    if (g.sz * near * near > g.level) return false;
+    const float yr = fminf(fmaxf(g.ys, d0), d1), yl = fminf(fmaxf(-g.ys, d0), d1);
+    const float xr = g.u + g.c * yr + sqrtf(fmaxf(g.level - g.sz * yr * yr, 0.0f) * g.kx) + g.padx;
+    const float xl = g.u + g.c * yl - sqrtf(fmaxf(g.level - g.sz * yl * yl, 0.0f) * g.kx) - g.padx;
+    const float a0 = fmaxf(ceilf(xl), 0.0f), a1 = fminf(floorf(xr), (float)(cam.W - 1)); // NaN: the whole row
+    if (a0 > a1) return false;
+    txa = max((int)a0 >> cam.tw_log2, g.tx0);
+    txb = min((int)a1 >> cam.tw_log2, g.tx1);
+    return txa <= txb;
+}
+
+// The front end of an exact frame of runs: one slot (Gaussian in depth order) per thread. Its record
+// goes to its slot; the frame's entries are counted by the rectangles (plain 3DGS's entries), while the
+// runs leave out the tiles where the Gaussian stays below 1/255 (about two thirds of the entries at
+// 4K), which the rasterizer would skip pixel by pixel. Bound by its depth-ordered gathers (236 B per
+// Gaussian; 405 us at 4K with 3 M, where the index-ordered preprocessing took 265). It pays for them many
+// times: with the entries in depth order no 64-bit key is written or sorted, and the whole exact frame
+// goes from 13.3 to 2.1 ms (4K, 3 M), 1.40 to 0.50 ms (1080p, 500 k).
+__global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunArgs r, int keep_all)
+{
+    __shared__ ExactRow s_row[FE_THREADS];
+    __shared__ unsigned long long s_sum[FE_WARPS];
+    static_assert(sizeof(s_row) >= FE_WARPS * RUN_CACHE * 4, "the runs are staged over the rows");
+    grid_dependency_wait();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long slot = (long long)blockIdx.x * FE_THREADS + tid;
+    bool front = false, vis = false;
+    int rows_l = 0;
+    unsigned tiles = 0;
+    if (slot < a.n) {
+        const long long i = (long long)a.order[slot];
+        const float mx = a.means[3 * i], my = a.means[3 * i + 1], mz = a.means[3 * i + 2];
+        const float pz = view_z(a.cam, mx, my, mz);
+        front = pz > a.cam.zn && pz <= a.cam.zf;
+        if (front) {
+            const float4 q = *reinterpret_cast<const float4*>(&a.quats[4 * i]);
+            Binned b;
+            vis = project_bin(a.cam, mx, my, mz, pz, q.x, q.y, q.z, q.w, a.scales[3 * i], a.scales[3 * i + 1],
+                              a.scales[3 * i + 2], false, 0.0f, b);
+            if (vis) {
+                float4 mean, quad, rgb;
+                exact_record(a, i, b, mx, my, mz, mean, quad, rgb);
+                a.rec[3 * slot] = mean;
+                a.rec[3 * slot + 1] = quad;
+                a.rec[3 * slot + 2] = rgb;
+                a.rect[slot] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
+                tiles = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
+                bool any;
+                s_row[tid] = exact_row(b, mean, quad, any);
+                if (any || keep_all) rows_l = b.ty1 - b.ty0 + 1;
+            }
+        }
+        a.touched[slot] = tiles;
+    }
+    emit_runs(r, blockIdx.x, rows_l, reinterpret_cast<unsigned*>(s_row), [&](int t, int k, int& ty, int& txa, int& txb) {
+        const ExactRow& G = s_row[t];
+        ty = G.ty0 + k;
+        if (keep_all) {
+            txa = G.tx0;
+            txb = G.tx1;
+            return true;
+        }
+        return exact_row_range(G, ty, a.cam, txa, txb);
+    });
+    unsigned long long sum = tiles;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) s_sum[warp] = sum;
+    const int nfront = __syncthreads_count(front);
+    const int nvis = __syncthreads_count(vis);
+    if (tid == 0) {
+        if (nvis) atomicAdd(&a.ctr->n_visible, (unsigned)nvis);
+        if (nfront) atomicAdd(&a.ctr->n_front, (unsigned)nfront);
+        sum = 0;
+        for (int q = 0; q < FE_WARPS; q++) sum += s_sum[q];
+        if (sum) atomicAdd(&a.ctr->n_entries_total, sum);
+    }
+}
+
+void launch_exact_depth_keys(const ExactArgs& a, unsigned* keys, unsigned* vals, Counters* ctr, unsigned* hist,
+                             unsigned* status0, cudaStream_t s)
+{
+    const int grid_cap = 8 * device_sm_count();
+    const long long need = (a.n + 255) / 256;
+    const unsigned blocks = (unsigned)(need < 1 ? 1 : (need < grid_cap ? need : grid_cap));
+    launch_dependent(k_exact_depth_keys, dim3(blocks), dim3(256), 0, s, a, keys, vals, ctr, hist, status0,
+                     sort_status_words(4, a.n));
+}
+
+void launch_exact_runs(const ExactArgs& a, const RunArgs& r, bool keep_all, cudaStream_t s)
+{
+    if (r.blocks == 0) return;
+    static std::atomic<bool> opted[64];
+    run_smem_opt_in(k_exact_runs, opted);
+    launch_dependent(k_exact_runs, dim3(r.blocks), dim3(FE_THREADS), (size_t)r.rows * sizeof(RunRowSmem), s, a, r,
+                     keep_all ? 1 : 0);
 }
 
 constexpr int SCAN_ITEMS = 8;

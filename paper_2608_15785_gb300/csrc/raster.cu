@@ -447,10 +447,11 @@ __global__ void __launch_bounds__(E_THREADS) k_raster_exact(RasterArgs a)
         if (j < range.y) {
             unsigned id = a.vals[j];
             if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
-            const float4 m = a.mean2[id];
+            const float4* const rec = a.erec + 3 * (size_t)id;
+            const float4 m = __ldg(rec);
             s_m[threadIdx.x] = make_float4(m.x - (float)x0, m.y, m.z - (float)y0, m.w);
-            s_q[threadIdx.x] = a.quad[id];
-            s_rgb[threadIdx.x] = make_float4(a.rgb[3 * id], a.rgb[3 * id + 1], a.rgb[3 * id + 2], 0.f);
+            s_q[threadIdx.x] = __ldg(rec + 1);
+            s_rgb[threadIdx.x] = __ldg(rec + 2);
         }
         __syncthreads();
         const int cnt = min((unsigned)E_THREADS, range.y - start);

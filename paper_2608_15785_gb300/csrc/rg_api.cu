@@ -160,6 +160,25 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     return at;
 }
 
+DepthSortViews depth_sort_views(const Workspace& w, int64_t n)
+{
+    DepthSortViews v;
+    unsigned char* const p = w.gsort.as<unsigned char>();
+    size_t at = 0;
+    auto part = [&](size_t words) {
+        unsigned* q = reinterpret_cast<unsigned*>(p + at);
+        at += (words * 4 + 255) / 256 * 256;
+        return q;
+    };
+    for (int k = 0; k < 2; k++) {
+        v.keys[k] = part((size_t)n);
+        v.vals[k] = part((size_t)n);
+        v.status[k] = part((size_t)((n + sort_tile_items() - 1) / sort_tile_items()) * 256);
+    }
+    v.bytes = at;
+    return v;
+}
+
 rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameLayout& F, int64_t cap)
 {
     const int64_t n = n_gauss > 0 ? n_gauss : 1;
@@ -176,29 +195,20 @@ rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameL
     const int64_t fe_blocks = (n + frontend_block_threads() - 1) / frontend_block_threads();
     RG_TRY(ensure(w.lb_status, (size_t)(std::max<int64_t>(fe_blocks, (n + 2047) / 2048) + 1) * 8, "look-back status"));
     if (mode == RG_MODE_EXACT) {
-        RG_TRY(ensure(w.mean2, (size_t)n * 16, "projected means"));
-        RG_TRY(ensure(w.depth, (size_t)n * 4, "depth"));
-        RG_TRY(ensure(w.quad, (size_t)n * 16, "exponent coefficients"));
-        RG_TRY(ensure(w.rgb, (size_t)n * 12, "rgb"));
+        RG_TRY(ensure(w.erec, (size_t)n * 48, "records"));
         RG_TRY(ensure(w.rect, (size_t)n * 16, "rect"));
         RG_TRY(ensure(w.touched, (size_t)n * 4, "touched"));
-        RG_TRY(ensure(w.offsets, (size_t)n * 4, "offsets"));
     } else {
         RG_TRY(ensure(w.rec, (size_t)n * 32, "records"));
         // the per-tile counting sort's count matrix (chunks x tiles, at most SMs x one block's shared
         // memory for any tile count) and tile totals: sized for any frame, so a workspace shared by
         // views of several resolutions never runs short
         RG_TRY(ensure(w.tsort, tilesort_matrix_bytes_max() + (size_t)tilesort_max_tiles() * 4, "tile counting sort"));
-        if (runs_possible(F.lay, n)) {
-            RunArgs ra;
-            RG_TRY(ensure(w.runbuf, run_views(w, n, F.lay, ra), "tile-row runs"));
-        }
-        for (int k = 0; k < 2; k++) {
-            RG_TRY(ensure(w.gkeys[k], (size_t)n * 4, "depth keys"));
-            RG_TRY(ensure(w.gvals[k], (size_t)n * 4, "depth order"));
-            RG_TRY(ensure(w.gstatus[k], (size_t)((n + sort_tile_items() - 1) / sort_tile_items()) * 256 * 4,
-                          "depth sort status"));
-        }
+    }
+    RG_TRY(ensure(w.gsort, depth_sort_views(w, n).bytes, "depth sort"));
+    if (runs_possible(F.lay, n)) {
+        RunArgs ra;
+        RG_TRY(ensure(w.runbuf, run_views(w, n, F.lay, ra), "tile-row runs"));
     }
     return RG_OK;
 }
@@ -232,6 +242,34 @@ struct NvtxScope {
 #define RG_EXACT_RANK_MODES sort_rank_modes(SORT_RANK_MATCH, SORT_RANK_MATCH, SORT_RANK_MATCH, SORT_RANK_MATCH) | \
                                 (sort_rank_modes(SORT_RANK_PEERS, SORT_RANK_PEERS) << 8)
 #endif
+
+// The per-Gaussian depth sort: `passes` 8-bit digits (at most 4) of the depth keys.
+static void depth_sort_args(Workspace& w, int64_t n, int passes, Sticky* sticky, SortArgs& ga)
+{
+    memset(&ga, 0, sizeof(ga));
+    const DepthSortViews g = depth_sort_views(w, n);
+    for (int k = 0; k < 2; k++) {
+        ga.keys[k] = g.keys[k];
+        ga.vals[k] = g.vals[k];
+        ga.status[k] = g.status[k];
+    }
+    ga.cap = n;
+    ga.key_bytes = 4;
+    ga.passes = passes;
+    ga.bit0 = 0;
+    // Gaussians in index order carry scattered depth digits: every pass ranks with the
+    // per-digit peer masks (measured 0.126 -> 0.124 ms at 4K, 0.086 -> 0.081 ms at 1080p
+    // against ballots on the first pass and match_any on the others)
+    ga.rank_modes = RG_DEPTH_RANK_MODES;
+    ga.hist = reinterpret_cast<unsigned*>(w.ctrl.as<unsigned char>() + CTRL_BYTES + sizeof(Counters));
+    ga.max_tiles = (n + sort_tile_items() - 1) / sort_tile_items();
+    ga.ctr = reinterpret_cast<Counters*>(w.ctrl.as<unsigned char>() + CTRL_BYTES);
+    ga.sticky = sticky;
+    // the depth keys' digits are counted as they are written, and the depth-key kernel clears the
+    // first pass's look-back status: no histogram kernel
+    ga.hist_pre = ga.hist;
+    ga.hist_done = 1;
+}
 
 // Arguments of a RoofGS frame's front end and sorts on workspace w (nothing launched;
 // records what rg_inspect needs about the frame in w).
@@ -281,28 +319,8 @@ rg_status roofgs_build(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_t
         // b_t tile bits alone yields the order of the full 32-bit key
         f.depth_order = true;
         SortArgs& ga = f.ga;
-        for (int k = 0; k < 2; k++) {
-            ga.keys[k] = w.gkeys[k].p;
-            ga.vals[k] = w.gvals[k].as<unsigned>();
-            ga.status[k] = w.gstatus[k].as<unsigned>();
-        }
-        ga.cap = n;
-        ga.key_bytes = 4;
-        ga.passes = (F.lay.b_d + 7) / 8;
-        ga.bit0 = 0;
-        // Gaussians in index order carry scattered depth digits: every pass ranks with the
-        // per-digit peer masks (measured 0.126 -> 0.124 ms at 4K, 0.086 -> 0.081 ms at 1080p
-        // against ballots on the first pass and match_any on the others)
-        ga.rank_modes = RG_DEPTH_RANK_MODES;
-        ga.hist = reinterpret_cast<unsigned*>(w.ctrl.as<unsigned char>() + CTRL_BYTES + sizeof(Counters));
-        ga.max_tiles = (n + sort_tile_items() - 1) / sort_tile_items();
-        ga.ctr = reinterpret_cast<Counters*>(w.ctrl.as<unsigned char>() + CTRL_BYTES);
-        ga.sticky = sticky;
-        // the depth keys' digits are counted as they are written (ga.passes <= 4), and the
-        // depth-key kernel clears the first pass's look-back status: no histogram kernel
-        ga.hist_pre = ga.hist;
-        ga.hist_done = 1;
-        a.order = w.gvals[ga.passes & 1].as<unsigned>();
+        depth_sort_args(w, n, (F.lay.b_d + 7) / 8, sticky, ga);
+        a.order = ga.vals[ga.passes & 1];
         sa.passes = (F.lay.b_t + 7) / 8;
         sa.bit0 = F.lay.b_d;
         // depth-ordered entries of one Gaussian row carry consecutive tiles, so the warp
@@ -361,9 +379,9 @@ rg_status roofgs_build(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_t
 
 // The per-Gaussian depth order of a RoofGS frame: quantized depth keys (with the sort's
 // digit counts), then their stable sort.
-void roofgs_depth_order(const RoofgsFrame& f, Workspace& w, cudaStream_t st)
+void roofgs_depth_order(const RoofgsFrame& f, cudaStream_t st)
 {
-    launch_depth_keys(f.fa, w.gkeys[0].as<unsigned>(), w.gvals[0].as<unsigned>(), f.ga.ctr, f.ga.hist, f.ga.passes,
+    launch_depth_keys(f.fa, (unsigned*)f.ga.keys[0], f.ga.vals[0], f.ga.ctr, f.ga.hist, f.ga.passes,
                       f.ga.status[0], st);
     launch_sort(f.ga, st, nullptr);
 }
@@ -422,7 +440,10 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         k_set_word<<<1, 1, 0, st>>>(&ctr->sort_tile_ctr[0], 1u);
         RG_CK(cudaGetLastError());
     }
-    if (!search_ranges) RG_CK(cudaMemsetAsync(w.ranges.p, 0, (size_t)F.tiles * sizeof(uint2), st));
+    // (the stall hook needs an entry sort to stall: its frames take the radix passes)
+    const bool exact_runs =
+        mode == RG_MODE_EXACT && !(flags & RG_FLAG_TEST_STALL_SORT) && runs_possible(F.lay, s->n);
+    if (!search_ranges && !exact_runs) RG_CK(cudaMemsetAsync(w.ranges.p, 0, (size_t)F.tiles * sizeof(uint2), st));
     const long long n = s->n;
     SortArgs sa;
     memset(&sa, 0, sizeof(sa));
@@ -453,36 +474,58 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         a.n = n;
         a.cam = F.cam;
         a.lay = F.lay;
-        a.mean2 = w.mean2.as<float4>();
-        a.depth = w.depth.as<float>();
-        a.quad = w.quad.as<float4>();
-        a.rgb = w.rgb.as<float>();
+        a.rec = w.erec.as<float4>();
         a.rect = w.rect.as<int4>();
         a.touched = w.touched.as<unsigned>();
-        a.offsets = w.offsets.as<unsigned>();
+        const DepthSortViews g = depth_sort_views(w, n); // unused by a frame without a depth order
+        a.depth = reinterpret_cast<float*>(g.keys[0]);
+        a.offsets = g.keys[1];
         a.keys = w.keys[0].as<unsigned long long>();
         a.vals = w.vals[0].as<unsigned>();
         a.cap = w.cap;
         a.status = w.lb_status.as<unsigned long long>();
         a.ctr = ctr;
         a.sticky = sticky;
-        RG_CK(cudaMemsetAsync(w.lb_status.p, 0, (size_t)((n + 2047) / 2048 + 1) * 8, st));
         sa.key_bytes = 8;
         sa.passes = (32 + F.lay.b_t + 7) / 8; // only the bits that can be non-zero
+        w.last_stat_passes = sa.passes;
+        // entries written from tile-row runs of the Gaussians in depth order: no sort of the entries
+        runs = exact_runs;
+        if (runs) {
+            if (run_views(w, n, F.lay, ra) > w.runbuf.bytes || (size_t)ra.run_cap * sizeof(uint2) > w.keys[0].bytes)
+                return fail(RG_ERR_CAPACITY, "workspace not sized for the frame");
+            ra.sticky = sticky;
+            ra.box_total = 1;
+            SortArgs ga;
+            depth_sort_args(w, n, 4, sticky, ga);
+            a.order = ga.vals[0]; // four passes
+            w.last_gfin = 0;
+            w.last_runs = true;
+            w.last_passes = 0;
+            {
+                NvtxScope r_("rg depth order");
+                launch_exact_depth_keys(a, (unsigned*)ga.keys[0], ga.vals[0], ga.ctr, ga.hist, ga.status[0], st);
+                launch_sort(ga, st, nullptr);
+            }
+            if (ev) RG_CK(cudaEventRecord(E[1], st));
+            NvtxScope r_("rg front end");
+            launch_exact_runs(a, ra, count, st);
+        }
         // passes 0-3 (depth bits: the entries of one Gaussian share them) rank with match_any,
         // the tile-bit passes 4-5 (consecutive tiles) with the peer masks: 4K sort 10.66 ->
         // 10.09 ms (every pass with the peer masks: 11.43 ms)
         sa.rank_modes = RG_EXACT_RANK_MODES;
         tile_shift = 32;
-        if (sa.passes <= 6) { // up to 2 tile-bit passes: the duplicate kernel counts every digit
+        if (!runs && sa.passes <= 6) { // up to 2 tile-bit passes: the duplicate kernel counts every digit
             a.hist = reinterpret_cast<unsigned*>(w.ctrl.as<unsigned char>() + 2 * CTRL_BYTES);
             a.tile_passes = sa.passes - 4;
             sa.hist_copies = a.hist;
             sa.hist_copy_stride = 8;
             sa.hist_pre = hist + 2 * 256; // rows 2-7 of the frame's [8][256] histograms
         }
-        if (ev) RG_CK(cudaEventRecord(E[1], st));
-        {
+        if (!runs) {
+            RG_CK(cudaMemsetAsync(w.lb_status.p, 0, (size_t)((n + 2047) / 2048 + 1) * 8, st));
+            if (ev) RG_CK(cudaEventRecord(E[1], st));
             NvtxScope r_("rg front end");
             launch_exact_preprocess(a, st);
             launch_exact_scan(a, st);
@@ -511,7 +554,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         }
         if (f.depth_order) {
             NvtxScope r_("rg depth order");
-            roofgs_depth_order(f, w, st);
+            roofgs_depth_order(f, st);
         }
         if (ev) RG_CK(cudaEventRecord(E[1], st));
         {
@@ -538,7 +581,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     if (ev) RG_CK(cudaEventRecord(E[4], st));
     if (!runs) w.last_passes = sa.passes;
     const int fin = w.last_passes & 1;
-    if (!search_ranges && !tile_sort) {
+    if (!search_ranges && !tile_sort && !runs) {
         RangeArgs g;
         g.keys = w.keys[fin].p;
         g.key_bytes = sa.key_bytes;
@@ -553,6 +596,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     w.last_mode = mode;
     if (!runs) w.last_stat_passes = sa.passes;
     w.last_tiles = F.tiles;
+    w.last_tiles_x = F.lay.tiles_x;
     w.last_tilesort = tile_sort;
     if (!out) { // front end, sort and ranges only (the backward replays the blend itself)
         if (ev) RG_CK(cudaEventRecord(E[6], st));
@@ -570,9 +614,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     r.out = out;
     r.count = count ? ctr : nullptr;
     if (mode == RG_MODE_EXACT) {
-        r.mean2 = w.mean2.as<float4>();
-        r.quad = w.quad.as<float4>();
-        r.rgb = w.rgb.as<float>();
+        r.erec = w.erec.as<float4>();
         NvtxScope r_("rg raster");
         launch_raster_exact(r, st);
     } else {
@@ -979,6 +1021,55 @@ rg_status rg_stage_times(rg_scene* s, float* ms7, int32_t* frames)
     return RG_OK;
 }
 
+// The entries of an exact frame of runs as plain 3DGS has them: every tile of every rectangle (the device
+// lists leave out tiles below 1/255), in the order of the 64-bit key tile << 32 | float depth, ties by
+// index; those that the capacity keeps are the first ones Gaussian by Gaussian, tiles ascending.
+static rg_status exact_runs_entries(rg_scene* s, const Counters& c, int32_t what, std::vector<unsigned char>& out)
+{
+    const Workspace& w = s->ws;
+    const size_t n = (size_t)s->n, tiles = (size_t)w.last_tiles, tx = (size_t)w.last_tiles_x, ne = c.n_entries;
+    std::vector<uint32_t> order(n), depth(n), touched(n), kept(n, 0u);
+    std::vector<int4> rect(n);
+    const DepthSortViews g = depth_sort_views(w, s->n);
+    RG_CK(cudaMemcpy(order.data(), g.vals[w.last_gfin], n * 4, cudaMemcpyDeviceToHost));
+    RG_CK(cudaMemcpy(depth.data(), g.keys[w.last_gfin], n * 4, cudaMemcpyDeviceToHost));
+    RG_CK(cudaMemcpy(touched.data(), w.touched.p, n * 4, cudaMemcpyDeviceToHost));
+    RG_CK(cudaMemcpy(rect.data(), w.rect.p, n * 16, cudaMemcpyDeviceToHost));
+    for (size_t k = 0; k < n; k++)
+        if (order[k] < n) kept[order[k]] = touched[k];
+    for (size_t i = 0, left = ne; i < n; i++) {
+        kept[i] = (uint32_t)std::min<size_t>(kept[i], left);
+        left -= kept[i];
+    }
+    auto each = [&](auto&& f) { // f(slot, Gaussian, tile) in depth order, tiles ascending
+        for (size_t k = 0; k < n; k++) {
+            if (order[k] >= n) continue;
+            uint32_t left = kept[order[k]];
+            const int4 r = rect[k];
+            for (int y = r.y; left && y <= r.w; y++)
+                for (int x = r.x; left && x <= r.z; x++, left--) f(k, order[k], (size_t)y * tx + (size_t)x);
+        }
+    };
+    std::vector<uint32_t> first(tiles + 1, 0u);
+    each([&](size_t, uint32_t, size_t t) { first[t + 1]++; });
+    for (size_t t = 0; t < tiles; t++) first[t + 1] += first[t];
+    if (what == RG_INSPECT_RANGES) {
+        std::vector<uint2> rr(tiles);
+        for (size_t t = 0; t < tiles; t++)
+            rr[t] = first[t + 1] > first[t] ? make_uint2(first[t], first[t + 1]) : make_uint2(0u, 0u);
+        out.resize(tiles * 8);
+        memcpy(out.data(), rr.data(), out.size());
+        return RG_OK;
+    }
+    const size_t item = what == RG_INSPECT_KEYS ? 8 : 4;
+    out.resize(ne * item);
+    each([&](size_t k, uint32_t i, size_t t) {
+        const uint64_t key = ((uint64_t)t << 32) | depth[k];
+        memcpy(&out[(size_t)first[t]++ * item], what == RG_INSPECT_KEYS ? (const void*)&key : (const void*)&i, item);
+    });
+    return RG_OK;
+}
+
 rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_bytes, int64_t* out_bytes)
 {
     if (!s) return fail(RG_ERR_INVALID_ARG, "scene is NULL");
@@ -997,13 +1088,21 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
         RG_CK(cudaMemcpy(&c, s->ws.ctrl.p, sizeof(c), cudaMemcpyDeviceToHost));
         const int fin = s->ws.last_passes & 1;
         const size_t ne = c.n_entries, ng = (size_t)n;
+        const DepthSortViews g = depth_sort_views(s->ws, n);
+        if (s->ws.last_runs && s->ws.last_mode == RG_MODE_EXACT) {
+            RG_TRY(exact_runs_entries(s, c, what, tmp));
+            src = tmp.data();
+            device_src = false;
+            bytes = (int64_t)tmp.size();
+            break;
+        }
         // a frame of runs: the values are slots of the depth order, which maps them to Gaussians
         std::vector<uint32_t> val;
         if (s->ws.last_runs && what != RG_INSPECT_RANGES) {
             std::vector<uint32_t> order(ng);
             val.resize(ne);
             if (ne) RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
-            if (ng) RG_CK(cudaMemcpy(order.data(), s->ws.gvals[s->ws.last_gfin].p, ng * 4, cudaMemcpyDeviceToHost));
+            if (ng) RG_CK(cudaMemcpy(order.data(), g.vals[s->ws.last_gfin], ng * 4, cudaMemcpyDeviceToHost));
             for (uint32_t& v : val) v = v < ng ? order[v] : 0u;
         }
         if (what == RG_INSPECT_KEYS && (s->ws.last_key16 || s->ws.last_runs)) {
@@ -1026,8 +1125,8 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
                 RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
             }
             if (ng) {
-                RG_CK(cudaMemcpy(gq.data(), s->ws.gkeys[s->ws.last_gfin].p, ng * 4, cudaMemcpyDeviceToHost));
-                RG_CK(cudaMemcpy(gi.data(), s->ws.gvals[s->ws.last_gfin].p, ng * 4, cudaMemcpyDeviceToHost));
+                RG_CK(cudaMemcpy(gq.data(), g.keys[s->ws.last_gfin], ng * 4, cudaMemcpyDeviceToHost));
+                RG_CK(cudaMemcpy(gi.data(), g.vals[s->ws.last_gfin], ng * 4, cudaMemcpyDeviceToHost));
             }
             for (size_t k = 0; k < ng; k++)
                 if (gi[k] < ng) q[gi[k]] = gq[k];
@@ -1159,9 +1258,8 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
     b.tiles_x = F.lay.tiles_x;
     b.tiles_y = F.lay.tiles_y;
     b.cam = F.cam;
-    b.mean2 = s->ws.mean2.as<float4>();
-    b.quad = s->ws.quad.as<float4>();
-    b.rgb = s->ws.rgb.as<float>();
+    b.erec = s->ws.erec.as<float4>();
+    b.order = s->ws.last_runs ? depth_sort_views(s->ws, s->n).vals[s->ws.last_gfin] : nullptr;
     b.touched = s->ws.touched.as<unsigned>();
     b.means = s->means.as<float>();
     b.scales = s->scales.as<float>();

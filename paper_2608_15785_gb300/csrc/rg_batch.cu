@@ -162,7 +162,7 @@ rg_status enqueue_fused(BatchPlan& P, const std::vector<FrameLayout>& F, float* 
         RG_TRY(roofgs_build(s, w, F[v], fl, f));
         RG_CK(cudaMemsetAsync(w.ctrl.p, 0, CTRL_ALLOC, ls));
         RG_CK(cudaMemsetAsync(w.lb_status.p, 0, (size_t)((s->n + bt - 1) / bt + 1) * 8, ls));
-        if (f.depth_order) roofgs_depth_order(f, w, ls);
+        if (f.depth_order) roofgs_depth_order(f, ls);
         fv->views[v] = f.fa;
         fv->block_prefix[v] = blocks;
         blocks += (unsigned)((s->n + bt - 1) / bt);

@@ -62,9 +62,9 @@ struct Workspace {
     DevBuf ctrl; // Counters followed by hist[8][256] (twice: frame, depth sort)
     DevBuf lb_status;
     DevBuf sort_status[2];
-    DevBuf mean2, depth, quad, rgb, rect, touched, offsets; // exact per-Gaussian
+    DevBuf erec, rect, touched;                           // exact per-Gaussian
     DevBuf rec;                                           // RoofGS raster records
-    DevBuf gkeys[2], gvals[2], gstatus[2];                // RoofGS per-Gaussian depth sort
+    DevBuf gsort;                                         // per-Gaussian depth sort (depth_sort_views)
     DevBuf gbuf;                                          // backward: image-space gradients [n][9]
     DevBuf tsort;                                         // RoofGS per-tile counting sort: matrix + tile totals
     DevBuf runbuf; // tile-row runs: per-block counts and places, chunks, column counts (run_views)
@@ -73,6 +73,7 @@ struct Workspace {
     int last_passes = 0;     // radix passes over the entries (the result is in keys/vals[last_passes & 1])
     int last_stat_passes = 0; // rg_stats.sort_passes
     int last_tiles = 0;
+    int last_tiles_x = 0;
     bool last_key16 = false; // entries carried 16-bit tile ids (the 32-bit keys are rebuilt on inspection)
     bool last_tilesort = false; // the entries were grouped by the per-tile counting sort (keys rebuilt from ranges)
     bool last_runs = false;  // the entries were written from tile-row runs: values are slots of the depth order
@@ -88,8 +89,7 @@ struct Workspace {
     void release()
     {
         DevBuf* bufs[] = {&keys[0], &keys[1], &vals[0], &vals[1], &ranges, &ctrl, &lb_status, &sort_status[0],
-                          &sort_status[1], &mean2, &depth, &quad, &rgb, &rect, &touched, &offsets, &rec, &gkeys[0],
-                          &gkeys[1], &gvals[0], &gvals[1], &gstatus[0], &gstatus[1], &gbuf, &tsort, &runbuf};
+                          &sort_status[1], &erec, &rect, &touched, &rec, &gsort, &gbuf, &tsort, &runbuf};
         for (DevBuf* b : bufs) b->release();
         if (ev_init)
             for (int f = 0; f < EV_RING; f++)
@@ -125,6 +125,15 @@ struct FrameLayout {
     int tiles;
 };
 
+// the per-Gaussian depth sort's arrays for n Gaussians: keys and values (4 B each) and look-back status,
+// twice; bytes: what gsort needs
+struct DepthSortViews {
+    unsigned* keys[2];
+    unsigned* vals[2];
+    unsigned* status[2];
+    size_t bytes;
+};
+DepthSortViews depth_sort_views(const Workspace& w, int64_t n);
 // tile shapes with kernels: 16 x 16, 32 x 8, 8 x 32
 bool tile_shape_ok(int tw, int th);
 // tile shape of a render option block (0 = the default 16 x 16); RG_ERR_UNSUPPORTED otherwise
@@ -152,7 +161,7 @@ struct RoofgsFrame {
 };
 // RG_ERR_UNSUPPORTED if the flags ask for what the frame cannot do
 rg_status roofgs_build(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_t flags, RoofgsFrame& f);
-void roofgs_depth_order(const RoofgsFrame& f, Workspace& w, cudaStream_t st);
+void roofgs_depth_order(const RoofgsFrame& f, cudaStream_t st);
 void roofgs_raster_args(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_t flags, float* out, RasterArgs& r);
 // frees a scene and its workspace
 void destroy_scene(rg_scene* s);

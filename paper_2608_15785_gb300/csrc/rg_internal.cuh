@@ -608,12 +608,14 @@ struct ExactArgs {
     long long n;
     CamDev cam;
     Layout lay;
-    float4* mean2;         // [N] projected mean as double-floats (u.hi, u.lo, v.hi, v.lo)
-    float* depth;
-    float4* quad;          // [N] (-Sigma'_yy / (2 det), Sigma'_xy / Sigma'_yy, -1 / (2 Sigma'_yy), opacity)
-    float* rgb;            // [N][3]
+    const unsigned* order; // [N] Gaussian of each slot (depth order) in a frame of tile-row runs, else null
+    // per slot (index without an order):
+    float4* rec;           // [N][3] projected mean as double-floats (u.hi, u.lo, v.hi, v.lo);
+                           // (-Sigma'_yy / (2 det), Sigma'_xy / Sigma'_yy, -1 / (2 Sigma'_yy), opacity); rgb
     int4* rect;            // [N] tx0, ty0, tx1, ty1
-    unsigned* touched;     // [N]
+    unsigned* touched;     // [N] tiles of the rectangle, 0 if culled
+    // without an order:
+    float* depth;
     unsigned* offsets;     // [N] exclusive scan of touched
     unsigned long long* keys; // [cap]
     unsigned* vals;
@@ -625,6 +627,13 @@ struct ExactArgs {
                            // 4-5: tile bits), counted by the duplicate kernel, or null
     int tile_passes;       // 1 or 2 tile-bit passes (b_t <= 16) when hist is set
 };
+// depth keys (float bits; culled Gaussians last) and indices of the per-Gaussian depth sort, their digit
+// counts (four passes), n in ctr, status0 cleared: as launch_depth_keys
+void launch_exact_depth_keys(const ExactArgs& a, unsigned* keys, unsigned* vals, Counters* ctr, unsigned* hist,
+                             unsigned* status0, cudaStream_t s);
+// the front end of an exact frame of runs (a.order set). keep_all: every tile of a rectangle (what the
+// counting rasterizer's work counters are about), else only those that a pixel of alpha >= 1/255 can lie in
+void launch_exact_runs(const ExactArgs& a, const RunArgs& r, bool keep_all, cudaStream_t s);
 void launch_exact_preprocess(const ExactArgs& a, cudaStream_t s);
 void launch_exact_scan(const ExactArgs& a, cudaStream_t s);
 void launch_exact_duplicate(const ExactArgs& a, cudaStream_t s);
@@ -691,10 +700,7 @@ struct RasterArgs {
     const float4* rec;
     int fast_exp;
     int ppt;              // pixels per thread: 1, 2 (Eq. (20)) or 4
-    // exact
-    const float4* mean2;
-    const float4* quad;
-    const float* rgb;
+    const float4* erec;   // exact (ExactArgs::rec)
     Counters* count;      // non-null: count evaluated / blended pairs (separate kernel variant)
 };
 void launch_raster_roofgs(const RasterArgs& a, cudaStream_t s);
@@ -739,17 +745,16 @@ struct BackwardArgs {
     long long n;
     int tiles_x, tiles_y;
     CamDev cam;
-    const float4* mean2;
-    const float4* quad;
-    const float* rgb;
+    const float4* erec;      // ExactArgs::rec
     const unsigned* touched;
+    const unsigned* order;   // Gaussian of each slot, or null (index order)
     // scene attributes (FP32)
     const float* means;
     const float* scales;
     const float* quats;
     const float* sh;
     int sh_degree;
-    // dL/dimage [3][H][W] and per-Gaussian image-space gradients [n][9]:
+    // dL/dimage [3][H][W] and per-slot image-space gradients [n][9]:
     // d(u, v), d(conic A, B, C), d(opacity), d(rgb)
     const float* dL_dimg;
     float* gbuf;

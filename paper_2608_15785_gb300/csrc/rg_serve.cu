@@ -235,7 +235,7 @@ rg_status rg_server_create(rg_scene* const* scenes, int32_t n_scenes, const rg_s
     largest.tiles = (int)tiles;
     // bytes of one slot: 2 x (keys 8 B + values 4 B) per entry, sort status, per-Gaussian arrays (RoofGS:
     // records, depth order), ranges, image
-    sv->slot_bytes = cap * 24 + (cap / 4096 + 1) * 2048 + ngauss * (sv->mode == RG_MODE_EXACT ? 72 : 112) +
+    sv->slot_bytes = cap * 24 + (cap / 4096 + 1) * 2048 + ngauss * (sv->mode == RG_MODE_EXACT ? 92 : 112) +
                      tiles * 8 + (int64_t)out_bytes;
     int nslots = cfg->max_slots > 0 ? cfg->max_slots : 8;
     nslots = (int)std::max<int64_t>(1, std::min<int64_t>(nslots, sv->budget / std::max<int64_t>(sv->slot_bytes, 1)));

@@ -25,7 +25,8 @@
 // Per pass every entry is read once and written once. The number of entries is
 // read on the device: no host round trip. k_ranges finds the per-tile
 // [start, end) of a sorted array (exact mode; RoofGS frames find their ranges
-// inside the rasterizer).
+// inside the rasterizer). Frames of at most 512 x 512 tiles sort only the Gaussians by
+// depth here: their entries are written from tile-row runs (runs.cu).
 #include <algorithm>
 #include <mutex>
 

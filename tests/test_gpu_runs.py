@@ -90,3 +90,38 @@ def test_runs_beyond_the_capacity(n):
     assert st["regrown"] == 1 and st["n_entries"] == k.size
     full = binding.Scene(sc)
     assert torch.equal(img, full.render(cam, stats=True)[0])
+
+
+# scales from specks to Gaussians wider than the image, seen from inside the cloud; thin ones; opacities
+# around 1/255; every tile shape, and small and larger frames
+EXACT_CASES = [(3_000, 0.05, False, (131, 77), (16, 16)), (40_000, 1.0, True, (640, 360), (16, 16)),
+               (2_000, 30.0, False, (333, 250), (32, 8)), (2_000, 30.0, True, (250, 333), (8, 32)),
+               (500, 300.0, True, (500, 400), (16, 16)), (40_000, 6.0, True, (320, 200), (32, 8)),
+               (2_000, 20.0, True, (8192, 48), (16, 16))]
+
+
+@pytest.mark.parametrize("n,scale,thin,wh,tile", EXACT_CASES)
+def test_exact_runs_leave_out_only_pairs_below_the_threshold(n, scale, thin, wh, tile):
+    """The timed exact frame leaves out the tiles that a Gaussian reaches below 1/255 everywhere: its
+    image equals bit by bit the counting frame's, which keeps every tile of the rectangles, and both
+    report the oracle's entries."""
+    sc = _scene(n, scale, seed=9)
+    rng = np.random.default_rng(1)
+    if thin:
+        sc.scales[:, 0] *= np.float32(0.01)
+    edge = rng.random(n) < 0.4
+    sc.opacities[edge] = rng.uniform(0.0, 0.012, int(edge.sum())).astype(np.float32)
+    sc.opacities[:2] = (0.0, 1.0)
+    cam = synth.look_at_camera((0.1, -0.2, -0.6), *wh, znear=0.02, zfar=5.0, bg=(0.3, 0.2, 0.1))
+    gs = binding.Scene(sc, storage=binding.RG_STORE_FP32)
+    full, st = gs.render(cam, mode="exact", stats=True, tile=tile)
+    k, v, _, _ = oracle.keys(sc, cam, oracle.EXACT, tile=tile)
+    ranges = gs.inspect(binding.RG_INSPECT_RANGES)
+    assert st["n_entries"] == k.size and 0 < st["n_blends"] < st["n_pairs"]
+    for frame in range(2):  # the counting frame, then the timed one
+        assert np.array_equal(gs.inspect(binding.RG_INSPECT_KEYS).view(np.uint64), k)
+        assert np.array_equal(gs.inspect(binding.RG_INSPECT_VALUES), v)
+        assert np.array_equal(gs.inspect(binding.RG_INSPECT_RANGES), ranges)
+        img = gs.render(cam, mode="exact", tile=tile)
+    assert torch.equal(img, full)
+    gs.check()
