@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
     int rows_l = 0;
     unsigned tiles = 0;
     if (slot < a.n) {
-        const long long i = (long long)a.order[slot];
+        const long long i = (long long)a.order[slot]; // below n
         const float mx = a.means[3 * i], my = a.means[3 * i + 1], mz = a.means[3 * i + 2];
         const float pz = view_z(a.cam, mx, my, mz);
         front = pz > a.cam.zn && pz <= a.cam.zf;
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
                 if (any || keep_all) rows_l = b.ty1 - b.ty0 + 1;
             }
         }
-        a.touched[slot] = tiles;
+        a.touched[i] = tiles;
     }
     emit_runs(r, blockIdx.x, rows_l, reinterpret_cast<unsigned*>(s_row), [&](int t, int k, int& ty, int& txa, int& txb) {
         const ExactRow& G = s_row[t];

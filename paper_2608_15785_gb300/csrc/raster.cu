@@ -485,10 +485,6 @@ __global__ void __launch_bounds__(E_THREADS) k_raster_exact_count(RasterArgs a)
     }
 }
 
-// The exponent below which a pair of opacity o is surely skipped: o exp(p) < 1/255 for every p below
-// it, whatever expf and the product round to (both within 1e-6; the margin is 1e-4). +inf for o = 0.
-__device__ __forceinline__ float exact_skip_below(float o) { return -(LN255F + logf(o)) - 1e-4f; }
-
 // One block of 256 / PPT threads per tile, PPT (2 or 4) vertically adjacent pixels per thread, blended in
 // pairs with packed FP32x2 arithmetic. Most pairs of a tile's list lie below 1/255 in most pixels: the
 // exponent alone decides those (exact_skip_below, staged with the record), and only a thread with a

@@ -1036,7 +1036,7 @@ static rg_status exact_runs_entries(rg_scene* s, const Counters& c, int32_t what
     RG_CK(cudaMemcpy(touched.data(), w.touched.p, n * 4, cudaMemcpyDeviceToHost));
     RG_CK(cudaMemcpy(rect.data(), w.rect.p, n * 16, cudaMemcpyDeviceToHost));
     for (size_t k = 0; k < n; k++)
-        if (order[k] < n) kept[order[k]] = touched[k];
+        kept[k] = touched[k];
     for (size_t i = 0, left = ne; i < n; i++) {
         kept[i] = (uint32_t)std::min<size_t>(kept[i], left);
         left -= kept[i];
@@ -1247,8 +1247,8 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
         RG_TRY(rg_scene_reserve(s, want));
         RG_TRY(ensure_workspace(s->ws, s->n, RG_MODE_EXACT, F, s->ws.cap));
     }
-    RG_TRY(ensure(s->ws.gbuf, (size_t)(s->n > 0 ? s->n : 1) * 9 * 4, "gradient buffer"));
-    RG_CK(cudaMemsetAsync(s->ws.gbuf.p, 0, (size_t)(s->n > 0 ? s->n : 1) * 9 * 4, st));
+    RG_TRY(ensure(s->ws.gbuf, (size_t)(s->n > 0 ? s->n : 1) * GBUF * 4, "gradient buffer"));
+    RG_CK(cudaMemsetAsync(s->ws.gbuf.p, 0, (size_t)(s->n > 0 ? s->n : 1) * GBUF * 4, st));
     BackwardArgs b;
     memset(&b, 0, sizeof(b));
     const int fin = s->ws.last_passes & 1;

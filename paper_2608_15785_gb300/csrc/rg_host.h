@@ -65,7 +65,7 @@ struct Workspace {
     DevBuf erec, rect, touched;                           // exact per-Gaussian
     DevBuf rec;                                           // RoofGS raster records
     DevBuf gsort;                                         // per-Gaussian depth sort (depth_sort_views)
-    DevBuf gbuf;                                          // backward: image-space gradients [n][9]
+    DevBuf gbuf;                                          // backward: per-Gaussian sums over pixels
     DevBuf tsort;                                         // RoofGS per-tile counting sort: matrix + tile totals
     DevBuf runbuf; // tile-row runs: per-block counts and places, chunks, column counts (run_views)
     // last frame

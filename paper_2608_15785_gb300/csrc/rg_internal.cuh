@@ -479,6 +479,10 @@ __device__ __forceinline__ float exact_power(const float4& m, const float4& quad
     return __fmaf_rn(__fmul_rn(quad.x, t), t, __fmul_rn(__fmul_rn(quad.z, dy), dy));
 }
 
+// The exponent below which a pair of opacity o is surely skipped: o exp(p) < 1/255 for every p below
+// it, whatever expf and the product round to (both within 1e-6; the margin is 1e-4). +inf for o = 0.
+__device__ __forceinline__ float exact_skip_below(float o) { return -(LN255F + logf(o)) - 1e-4f; }
+
 // ---------------------------------------------------------------------------
 // Host-side launchers (defined in the .cu files).
 // ---------------------------------------------------------------------------
@@ -613,6 +617,7 @@ struct ExactArgs {
     float4* rec;           // [N][3] projected mean as double-floats (u.hi, u.lo, v.hi, v.lo);
                            // (-Sigma'_yy / (2 det), Sigma'_xy / Sigma'_yy, -1 / (2 Sigma'_yy), opacity); rgb
     int4* rect;            // [N] tx0, ty0, tx1, ty1
+    // per Gaussian:
     unsigned* touched;     // [N] tiles of the rectangle, 0 if culled
     // without an order:
     float* depth;
@@ -738,6 +743,8 @@ size_t tilesort_matrix_bytes(int T);
 size_t tilesort_matrix_bytes_max();
 void launch_tile_counting_sort(const TileSortArgs& a, cudaStream_t s);
 
+constexpr int GBUF = 12; // words of gbuf per Gaussian (nine used)
+
 struct BackwardArgs {
     // forward state of the frame (exact mode)
     const uint2* ranges;
@@ -754,8 +761,8 @@ struct BackwardArgs {
     const float* quats;
     const float* sh;
     int sh_degree;
-    // dL/dimage [3][H][W] and per-slot image-space gradients [n][9]:
-    // d(u, v), d(conic A, B, C), d(opacity), d(rgb)
+    // dL/dimage [3][H][W] and the per-Gaussian sums over pixels [n][GBUF]: dL/dp times t, dy, t^2, t dy,
+    // dy^2 (backward.cu), d(opacity), d(rgb)
     const float* dL_dimg;
     float* gbuf;
     // outputs
