@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
     __shared__ float4 s_rgb[NT];
     __shared__ int s_last;
     grid_dependency_wait();
-    const int tile = blockIdx.x, th = threadIdx.x, lane = th & 31;
+    const int tile = (int)ordered_tile(a.tile_order, blockIdx.x), th = threadIdx.x, lane = th & 31;
     const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
     const int x0 = tx * a.cam.tw, y0 = ty * a.cam.th;
     const int lxi = th & (a.cam.tw - 1), lyi = (th >> a.cam.tw_log2) * PPT;

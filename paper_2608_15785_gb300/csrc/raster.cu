@@ -348,7 +348,7 @@ template <bool FAST, int PPT, bool COUNT>
 __global__ void __launch_bounds__(256 / PPT) k_raster_roofgs(RasterArgs a)
 {
     grid_dependency_wait();
-    raster_tile<FAST, PPT, COUNT>(a, blockIdx.x);
+    raster_tile<FAST, PPT, COUNT>(a, (int)ordered_tile(a.order, blockIdx.x));
 }
 
 // Every view of a batch in one persistent launch: each block takes (view, tile) items
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
     __shared__ float4 s_rg[NT]; // r, r, g, g
     __shared__ float2 s_bb[NT]; // b, b
     grid_dependency_wait();
-    const int tile = blockIdx.x, t = threadIdx.x;
+    const int tile = (int)ordered_tile(a.order, blockIdx.x), t = threadIdx.x;
     const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
     const int x0 = tx * a.cam.tw, y0 = ty * a.cam.th;
     const int lxi = t & (a.cam.tw - 1), lyi = (t >> a.cam.tw_log2) * PPT;

@@ -124,6 +124,21 @@ bool runs_possible(const Layout& L, int64_t n)
     return n > 0 && L.tiles_x <= RUN_MAX_GRID && L.tiles_y <= RUN_MAX_GRID;
 }
 
+// the order in which the rasterizers take the tiles, in frames whose tiles do not all fit on the GPU at
+// once (16 blocks of 64 threads per SM). Without it the heavy tiles of the image's centre were met last by
+// some SMs, and the others idled meanwhile for a sixth of the rasterizer's time at 1080p. Per pass, row-major /
+// longest first: RoofGS 1080p 312 / 292 us, 8K 2191 / 1879 us, exact 1080p 451 / 419 us, backward 1080p 1095 / 982 us
+static TileOrder tile_order(const Workspace& w, int tiles)
+{
+    TileOrder o = {nullptr, nullptr, 0};
+    if (tiles > 16 * device_sm_count()) {
+        o.list = reinterpret_cast<unsigned*>(w.ranges.as<uint2>() + tiles);
+        o.count = w.ctrl.as<Counters>()->tiles;
+        o.tiles = (unsigned)tiles;
+    }
+    return o;
+}
+
 // Arguments of runs.cu for a frame on workspace w: the runs live in the key buffers (list in
 // keys[0], the blocks' runs in keys[1]), the rest in runbuf. Returns the bytes of runbuf the frame
 // needs; the pointers are valid if runbuf has them.
@@ -141,6 +156,7 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     a.vals = w.vals[0].as<unsigned>();
     a.ranges = w.ranges.as<uint2>();
     a.ctr = w.ctrl.as<Counters>();
+    a.order = tile_order(w, a.rows * a.cols);
     unsigned char* const p = w.runbuf.as<unsigned char>();
     size_t at = 0;
     auto part = [&](size_t bytes) {
@@ -190,7 +206,7 @@ rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameL
         for (int k = 0; k < 2; k++) RG_TRY(ensure(w.sort_status[k], (size_t)max_tiles * 256 * 4, "sort status"));
         w.cap = cap;
     }
-    RG_TRY(ensure(w.ranges, (size_t)F.tiles * sizeof(uint2), "ranges"));
+    RG_TRY(ensure(w.ranges, (size_t)F.tiles * (sizeof(uint2) + 8 * 4), "ranges and tile order"));
     RG_TRY(ensure(w.ctrl, CTRL_ALLOC, "counters"));
     const int64_t fe_blocks = (n + frontend_block_threads() - 1) / frontend_block_threads();
     RG_TRY(ensure(w.lb_status, (size_t)(std::max<int64_t>(fe_blocks, (n + 2047) / 2048) + 1) * 8, "look-back status"));
@@ -615,11 +631,13 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     r.count = count ? ctr : nullptr;
     if (mode == RG_MODE_EXACT) {
         r.erec = w.erec.as<float4>();
+        if (runs) r.order = ra.order;
         NvtxScope r_("rg raster");
         launch_raster_exact(r, st);
     } else {
         roofgs_raster_args(s, w, F, flags, out, r);
         r.count = count ? ctr : nullptr;
+        if (runs) r.order = ra.order;
         NvtxScope r_("rg raster");
         launch_raster_roofgs(r, st);
     }
@@ -1258,6 +1276,7 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
     b.tiles_x = F.lay.tiles_x;
     b.tiles_y = F.lay.tiles_y;
     b.cam = F.cam;
+    if (s->ws.last_runs) b.tile_order = tile_order(s->ws, F.tiles);
     b.erec = s->ws.erec.as<float4>();
     b.order = s->ws.last_runs ? depth_sort_views(s->ws, s->n).vals[s->ws.last_gfin] : nullptr;
     b.touched = s->ws.touched.as<unsigned>();

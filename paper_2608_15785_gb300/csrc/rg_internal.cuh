@@ -77,6 +77,7 @@ struct Counters {
     unsigned n_row_runs;         // tile-row runs given a place in the rows' lists (runs.cu)
     unsigned n_chunks;           // chunks of runs
     unsigned pad;
+    alignas(16) unsigned tiles[8]; // tiles of each size class (TileOrder)
     unsigned long long n_runs;   // tile-row runs the front end's blocks asked room for
     unsigned long long n_pairs;  // rasterizer work counters (counting launches only)
     unsigned long long n_blends;
@@ -538,6 +539,47 @@ __host__ __device__ __forceinline__ unsigned run_last(unsigned v) { return v >> 
 // words per chunk of the column counts
 __host__ __device__ __forceinline__ int run_pitch(int cols) { return (cols + 31) / 32 * 32; }
 
+// The tiles of a frame by size class (octaves of their entries from 32 up), the longest first: a
+// rasterizer's blocks take them in this order, so that its last wave has only short tiles.
+struct TileOrder {
+    unsigned* list;        // [8][tiles] the tiles of each class, in any order; null: no order kept
+    const unsigned* count; // [8] (Counters::tiles)
+    unsigned tiles;
+};
+__device__ __forceinline__ unsigned tile_class(unsigned entries)
+{
+    const int b = 32 - __clz((int)entries) - 5;
+    return b < 0 ? 0u : (b > 7 ? 7u : (unsigned)b);
+}
+// the tile of block b of a rasterizer
+__device__ __forceinline__ unsigned ordered_tile(const TileOrder& o, unsigned b)
+{
+    if (!o.list) return b;
+    const uint4 lo = *reinterpret_cast<const uint4*>(o.count), hi = *reinterpret_cast<const uint4*>(o.count + 4);
+    const unsigned n[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    unsigned at = b, cls = 7;
+#pragma unroll
+    for (int c = 7; c > 0; c--) {
+        if (cls == (unsigned)c && at >= n[c]) {
+            at -= n[c];
+            cls = (unsigned)c - 1u;
+        }
+    }
+    return o.list[(size_t)cls * o.tiles + at];
+}
+// adds tile (if valid) of `entries` entries to the order; called by whole warps
+__device__ __forceinline__ void add_tile(const TileOrder& o, unsigned* count, bool valid, unsigned tile, unsigned entries)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned c = valid ? tile_class(entries) : 8u;
+    const unsigned peers = __match_any_sync(0xffffffffu, c);
+    const int leader = __ffs(peers) - 1;
+    unsigned at = 0;
+    if (valid && lane == leader) at = atomicAdd(&count[c], (unsigned)__popc(peers));
+    at = __shfl_sync(0xffffffffu, at, leader) + (unsigned)__popc(peers & ((1u << lane) - 1u));
+    if (valid) o.list[(size_t)c * o.tiles + at] = tile;
+}
+
 struct RunChunk {
     unsigned block;           // its first block
     unsigned run;             // runs of the row before it
@@ -568,6 +610,7 @@ struct RunArgs {
     unsigned* col;     // [chunk_cap][run_pitch(cols)] entries per column, then their first slot in vals
     unsigned* vals;    // [cap] slots, by tile id, by slot
     uint2* ranges;     // [rows * cols] [start, end) of every tile, [0, 0) if empty
+    TileOrder order;   // filled too if order.list is set
     Counters* ctr;
     Sticky* sticky;
 };
@@ -688,6 +731,7 @@ void launch_ranges(const RangeArgs& a, cudaStream_t s);
 
 struct RasterArgs {
     const uint2* ranges;
+    TileOrder order;
     // RoofGS: when set, every tile block finds its own [start, end) in the sorted keys
     // (tile id = key >> tile_shift, n_entries from the counters) and writes it to
     // ranges_out; `ranges` is then unused
@@ -748,6 +792,7 @@ constexpr int GBUF = 12; // words of gbuf per Gaussian (nine used)
 struct BackwardArgs {
     // forward state of the frame (exact mode)
     const uint2* ranges;
+    TileOrder tile_order;
     const unsigned* vals;
     long long n;
     int tiles_x, tiles_y;

@@ -424,6 +424,7 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
                 const unsigned e = first + total < a.cap ? first + total : (unsigned)a.cap;
                 a.ranges[(size_t)row * a.cols + col] = e > b ? make_uint2(b, e) : make_uint2(0u, 0u);
             }
+            if (a.order.list) add_tile(a.order, a.ctr->tiles, col < a.cols, row * (unsigned)a.cols + (unsigned)col, total);
         }
         __syncthreads();
         if (col < a.cols) {
@@ -497,6 +498,8 @@ __device__ __forceinline__ void small_offsets(const RunArgs& a, const RunRow& r,
                 a.ranges[(size_t)row * a.cols + col] = e > b ? make_uint2(b, e) : make_uint2(0u, 0u);
             }
         }
+        if (blockIdx.x == 0 && a.order.list)
+            add_tile(a.order, a.ctr->tiles, col < a.cols, row * (unsigned)a.cols + (unsigned)col, total);
         run += all;
     }
 }
