@@ -1034,21 +1034,34 @@ void launch_exact_duplicate(const ExactArgs& a, cudaStream_t s)
 // ---------------------------------------------------------------------------
 // Scene conversion (one-off at scene creation)
 // ---------------------------------------------------------------------------
-__global__ void k_check_finite(const float* p, long long count, unsigned* flag)
+__global__ void k_check_attributes(const float* means, const float* scales, const float* quats, const float* opac,
+                                   const float* sh, long long n, unsigned* flag)
 {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    bool bad = false;
-    for (; i < count; i += stride) bad |= !isfinite(p[i]);
-    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
+    bool bad = false, range = false;
+    auto finite = [&](const float* p, long long count) {
+        for (long long i = i0; i < count; i += stride) bad |= !isfinite(p[i]);
+    };
+    finite(means, 3 * n);
+    finite(scales, 3 * n);
+    finite(quats, 4 * n);
+    finite(sh, 48 * n);
+    for (long long i = i0; i < n; i += stride) {
+        bad |= !isfinite(opac[i]);
+        range |= !(opac[i] >= 0.0f && opac[i] <= 1.0f);
+    }
+    const unsigned f = __reduce_or_sync(0xffffffffu, (bad ? 1u : 0u) | (range ? 2u : 0u));
+    if (f && (threadIdx.x & 31) == 0) atomicOr(flag, f);
 }
 
-void launch_check_finite(const float* p, long long count, unsigned* flag, cudaStream_t s)
+void launch_check_attributes(const float* means, const float* scales, const float* quats, const float* opac,
+                             const float* sh, long long n, unsigned* flag, cudaStream_t s)
 {
-    if (count <= 0) return;
-    long long blocks = (count + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    k_check_finite<<<(unsigned)blocks, 256, 0, s>>>(p, count, flag);
+    if (n <= 0) return;
+    long long blocks = (48 * n + 255) / 256;
+    if (blocks > 16ll * device_sm_count()) blocks = 16ll * device_sm_count();
+    k_check_attributes<<<(unsigned)blocks, 256, 0, s>>>(means, scales, quats, opac, sh, n, flag);
 }
 
 // max |SH| per (degree, channel): float bits of non-negative values order like integers

@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -27,20 +28,104 @@ rg_status rg::fail(rg_status s, const std::string& msg)
 
 void rg::set_last_error(const char* msg) { g_err = msg; }
 
+namespace {
+
+struct KeptBlock {
+    void* p;
+    size_t bytes;
+    int dev;
+    uint64_t at; // return count when it was kept
+};
+constexpr size_t KEEP_BLOCK = 128u << 20, KEEP_TOTAL = 512u << 20;
+constexpr uint64_t KEEP_RETURNS = 512;
+std::mutex g_kept_mu;
+std::vector<KeptBlock> g_kept; // oldest first
+size_t g_kept_bytes = 0;
+uint64_t g_returns = 0;
+thread_local int t_device_idle = 0;
+
+// takes block k out of the list (the caller holds the mutex)
+KeptBlock take_kept(size_t k)
+{
+    const KeptBlock b = g_kept[k];
+    g_kept.erase(g_kept.begin() + (ptrdiff_t)k);
+    g_kept_bytes -= b.bytes;
+    return b;
+}
+
+} // namespace
+
+rg::DeviceIdle::DeviceIdle() { t_device_idle++; }
+rg::DeviceIdle::~DeviceIdle() { t_device_idle--; }
+
+cudaError_t rg::device_take(void** p, size_t& bytes, int& dev)
+{
+    dev = 0;
+    cudaGetDevice(&dev);
+    {
+        std::lock_guard<std::mutex> lock(g_kept_mu);
+        size_t best = g_kept.size();
+        for (size_t k = 0; k < g_kept.size(); k++) // the smallest that fits, at most twice as large
+            if (g_kept[k].dev == dev && g_kept[k].bytes >= bytes && g_kept[k].bytes <= 2 * bytes + 4096 &&
+                (best == g_kept.size() || g_kept[k].bytes < g_kept[best].bytes))
+                best = k;
+        if (best < g_kept.size()) {
+            const KeptBlock b = take_kept(best);
+            *p = b.p;
+            bytes = b.bytes;
+            return cudaSuccess;
+        }
+    }
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) { // give back what is kept, and once more
+        cudaGetLastError();
+        std::vector<KeptBlock> all;
+        {
+            std::lock_guard<std::mutex> lock(g_kept_mu);
+            all.swap(g_kept);
+            g_kept_bytes = 0;
+        }
+        for (const KeptBlock& b : all) cudaFree(b.p);
+        if (!all.empty()) e = cudaMalloc(p, bytes);
+    }
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+void rg::device_give_back(void* p, size_t bytes, int dev)
+{
+    int cur = -1;
+    if (bytes > KEEP_BLOCK || cudaGetDevice(&cur) != cudaSuccess || cur != dev ||
+        (t_device_idle == 0 && cudaDeviceSynchronize() != cudaSuccess)) {
+        cudaFree(p);
+        return;
+    }
+    std::vector<KeptBlock> out;
+    {
+        std::lock_guard<std::mutex> lock(g_kept_mu);
+        g_returns++;
+        g_kept.push_back({p, bytes, dev, g_returns});
+        g_kept_bytes += bytes;
+        while (!g_kept.empty() && (g_kept_bytes > KEEP_TOTAL || g_kept[0].at + KEEP_RETURNS < g_returns))
+            out.push_back(take_kept(0));
+    }
+    for (const KeptBlock& b : out) cudaFree(b.p);
+}
+
 // grow-only device allocation (contents are not preserved)
 rg_status rg::ensure(DevBuf& b, size_t bytes, const char* what)
 {
     if (bytes == 0) bytes = 16;
     if (b.p && b.bytes >= bytes) return RG_OK;
     b.release();
-    cudaError_t e = cudaMalloc(&b.p, bytes);
+    b.bytes = bytes;
+    cudaError_t e = device_take(&b.p, b.bytes, b.dev);
     if (e != cudaSuccess) {
-        cudaGetLastError();
         b.p = nullptr;
+        b.bytes = 0;
         return fail(RG_ERR_OOM, std::string("cudaMalloc failed for ") + what + " (" + std::to_string(bytes) + " bytes): " +
                                     cudaGetErrorString(e));
     }
-    b.bytes = bytes;
     return RG_OK;
 }
 
@@ -724,23 +809,20 @@ rg_status rg_scene_create(const rg_scene_desc* desc, void* stream, rg_scene** ou
     RG_STEP(ensure(s->sticky, sizeof(Sticky), "sticky"));
     if (cudaMemsetAsync(s->sticky.p, 0, sizeof(Sticky), st) != cudaSuccess) RG_STEP(fail(RG_ERR_CUDA, "memset"));
     if (cudaMemsetAsync(flag.p, 0, 16, st) != cudaSuccess) RG_STEP(fail(RG_ERR_CUDA, "memset"));
-    launch_check_finite(dm, n * 3, flag.as<unsigned>(), st);
-    launch_check_finite(ds, n * 3, flag.as<unsigned>(), st);
-    launch_check_finite(dq, n * 4, flag.as<unsigned>(), st);
-    launch_check_finite(dop, n, flag.as<unsigned>(), st);
-    launch_check_finite(dsh, n * 48, flag.as<unsigned>(), st);
-    // opacities on the host: range check and log o (FP64 log, rounded to FP32)
-    std::vector<float> o((size_t)n), lo((size_t)n);
-    if (n && cudaMemcpyAsync(o.data(), dop, (size_t)n * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        RG_STEP(fail(RG_ERR_CUDA, "copy opacities"));
+    launch_check_attributes(dm, ds, dq, dop, dsh, n, flag.as<unsigned>(), st);
+    // the compact storage needs the opacities on the host: log o (FP64 log, rounded to FP32)
+    std::vector<float> lo;
+    if (s->storage & RG_STORE_COMPACT) {
+        lo.resize((size_t)n);
+        if (n && cudaMemcpyAsync(lo.data(), dop, (size_t)n * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            RG_STEP(fail(RG_ERR_CUDA, "copy opacities"));
+    }
     unsigned hflag = 0;
     if (cudaMemcpyAsync(&hflag, flag.p, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess) RG_STEP(fail(RG_ERR_CUDA, "copy flag"));
     if (cudaStreamSynchronize(st) != cudaSuccess) RG_STEP(fail(RG_ERR_CUDA, std::string("scene upload: ") + cudaGetErrorString(cudaGetLastError())));
-    if (hflag) RG_STEP(fail(RG_ERR_INVALID_ARG, "scene attributes contain non-finite values"));
-    for (int64_t i = 0; i < n; i++) {
-        if (!(o[i] >= 0.0f && o[i] <= 1.0f)) RG_STEP(fail(RG_ERR_INVALID_ARG, "opacity outside [0, 1]"));
-        lo[i] = (float)std::log((double)o[i]);
-    }
+    if (hflag & 1u) RG_STEP(fail(RG_ERR_INVALID_ARG, "scene attributes contain non-finite values"));
+    if (hflag & 2u) RG_STEP(fail(RG_ERR_INVALID_ARG, "opacity outside [0, 1]"));
+    for (float& o : lo) o = (float)std::log((double)o);
     if (s->storage & RG_STORE_COMPACT) {
         RG_STEP(ensure(logo, (size_t)n * 4, "log o"));
         RG_STEP(ensure(maxbits, 12 * 4, "sh max"));
@@ -765,7 +847,10 @@ rg_status rg_scene_create(const rg_scene_desc* desc, void* stream, rg_scene** ou
     }
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
         RG_STEP(fail(RG_ERR_CUDA, "scene conversion failed"));
-    cleanup();
+    {
+        DeviceIdle idle; // the staging buffers were only used on st
+        cleanup();
+    }
 #undef RG_STEP
     *out = s;
     return RG_OK;
@@ -774,9 +859,14 @@ rg_status rg_scene_create(const rg_scene_desc* desc, void* stream, rg_scene** ou
 rg_status rg_scene_destroy(rg_scene* scene)
 {
     if (!scene) return RG_OK;
-    cudaDeviceSynchronize();
-    drop_plans_of(scene);
-    destroy_scene(scene);
+    if (cudaDeviceSynchronize() == cudaSuccess) {
+        DeviceIdle idle;
+        drop_plans_of(scene);
+        destroy_scene(scene);
+    } else {
+        drop_plans_of(scene);
+        destroy_scene(scene);
+    }
     return RG_OK;
 }
 

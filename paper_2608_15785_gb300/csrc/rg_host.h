@@ -27,12 +27,30 @@ rg_status fail(rg_status s, const std::string& msg);
         if (s_ != RG_OK) return s_;  \
     } while (0)
 
+// Device memory of at least `bytes` on the current device (bytes: what it got), from the blocks that
+// released buffers left or from cudaMalloc; and its return. A program that makes and drops a scene per
+// step (the autograd wrapper) would otherwise spend most of the step in cudaMalloc and cudaFree.
+// Blocks above 128 MiB are not kept, at most 512 MiB are, those that 512 later returns did not take up
+// again go back to CUDA, and all of them do when an allocation fails. A returned block is idle: the device
+// is synchronised first (as cudaFree does), unless the caller has done so (DeviceIdle).
+cudaError_t device_take(void** p, size_t& bytes, int& dev);
+void device_give_back(void* p, size_t bytes, int dev);
+
+// While one lives, this thread's releases need not synchronise: no work of theirs is in flight.
+struct DeviceIdle {
+    DeviceIdle();
+    ~DeviceIdle();
+    DeviceIdle(const DeviceIdle&) = delete;
+    DeviceIdle& operator=(const DeviceIdle&) = delete;
+};
+
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
+    int dev = 0;
     void release()
     {
-        if (p) cudaFree(p);
+        if (p) device_give_back(p, bytes, dev);
         p = nullptr;
         bytes = 0;
     }

@@ -827,7 +827,9 @@ int device_sm_count();
 void set_last_error(const char* msg);
 
 // Scene creation kernels
-void launch_check_finite(const float* p, long long count, unsigned* flag, cudaStream_t s);
+// ORs into *flag: 1 if an attribute is not finite, 2 if an opacity lies outside [0, 1]
+void launch_check_attributes(const float* means, const float* scales, const float* quats, const float* opac,
+                             const float* sh, long long n, unsigned* flag, cudaStream_t s);
 void launch_sh_absmax(const float* sh, long long n, unsigned* maxbits /*[12]*/, cudaStream_t s);
 void launch_compact(const float* means, const float* scales, const float* quats, const float* logo,
                     const float* sh, long long n, const float* band_scale /*host [12]*/, int per_gauss,
