@@ -108,7 +108,7 @@ extern "C" rg_status rg_sort_pairs_noalloc(uint32_t* keys, uint32_t* vals, int64
     a.keys[1] = base + OFF_KEYS;
     a.vals[0] = vals;
     a.vals[1] = reinterpret_cast<unsigned*>(base + OFF_VALS);
-    a.cap = NA_MAX;
+    a.cap = n;
     a.key_bytes = 4;
     a.passes = key_bits / 8;
     // arbitrary keys hold many distinct digits per warp: every pass ranks with the peer masks

@@ -125,3 +125,26 @@ def test_exact_runs_leave_out_only_pairs_below_the_threshold(n, scale, thin, wh,
         img = gs.render(cam, mode="exact", tile=tile)
     assert torch.equal(img, full)
     gs.check()
+
+
+@pytest.mark.parametrize("n", [1, 31, 1_024, 1_025, 24_577, 311_296, 311_297])
+def test_depth_orders(n):
+    """Around the sizes where the depth keys' grid changes (one block, 304 blocks of 1,024): many equal
+    depth codes (ties by index), culled Gaussians; RoofGS entries equal those of the full 32-bit key
+    sort, which orders no Gaussians beforehand, exact ones the oracle's."""
+    sc = _scene(n, 1.5 if n < 100_000 else 0.2, seed=n)
+    sc.means[: n // 3, 2] = np.float32(0.25)  # equal depths at the camera below
+    sc.means[n // 2:: 7, 2] = np.float32(-9.0)  # behind it
+    if n > 10:
+        sc.opacities[5:: 11] = np.float32(1e-3)
+    cam = synth.look_at_camera((0.0, 0.0, -3.0), 200, 120, zfar=4.5)
+    gs = binding.Scene(sc)
+    gs.render(cam, stats=True)
+    a = _entries(gs)
+    gs.render(cam, stats=True, flags=binding.RG_FLAG_SORT_FULL_KEY)
+    for x, y in zip(a, _entries(gs)):
+        assert np.array_equal(x, y)
+    gs.render(cam, mode="exact", stats=True)
+    k, v, _, _ = oracle.keys(sc, cam, oracle.EXACT)
+    assert np.array_equal(gs.inspect(binding.RG_INSPECT_KEYS).view(np.uint64), k)
+    assert np.array_equal(gs.inspect(binding.RG_INSPECT_VALUES), v)
