@@ -150,6 +150,36 @@ __device__ __forceinline__ void blend_one_fast(float P, float nr, float ng, floa
     T = Tn;
 }
 
+// The same blend without branches, for frames of few tiles, where the latency of each warp's own chain
+// of records bounds the rasterizer and not the issue slots: with selects instead of the skip and stop
+// branches the records' exponents overlap the blends before them. Bit-identical to the two above.
+template <int NH>
+__device__ __forceinline__ void blend_pairs_straight(const float (&P)[2 * NH], float2 nr, float2 ng, float2 nb,
+                                                     float2 (&T)[NH], float2 (&cr)[NH], float2 (&cg)[NH],
+                                                     float2 (&cb)[NH], float (&thr)[2 * NH])
+{
+    const float inf = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int h = 0; h < NH; h++) {
+        const float2 w = __ffma2_rn(make_float2(P[2 * h], P[2 * h + 1]), make_float2(1.44269502f, 1.44269502f),
+                                    make_float2(126.954323f, 126.954323f));
+        const float ea = __uint_as_float(__float_as_uint(w.x) << 6); // -exp^(P)
+        const float eb = __uint_as_float(__float_as_uint(w.y) << 6);
+        const float2 na = make_float2(P[2 * h] >= thr[2 * h] ? fmaxf(-0.99f, ea) : 0.0f,
+                                      P[2 * h + 1] >= thr[2 * h + 1] ? fmaxf(-0.99f, eb) : 0.0f);
+        const float2 Tn = __ffma2_rn(T[h], na, T[h]);
+        float2 nw = __fmul2_rn(na, T[h]); // -alpha T
+        const bool sx = Tn.x < 1e-4f, sy = Tn.y < 1e-4f; // adds nothing, T kept, finished
+        nw = make_float2(sx ? 0.0f : nw.x, sy ? 0.0f : nw.y);
+        thr[2 * h] = sx ? inf : thr[2 * h];
+        thr[2 * h + 1] = sy ? inf : thr[2 * h + 1];
+        T[h] = make_float2(sx ? T[h].x : Tn.x, sy ? T[h].y : Tn.y);
+        cr[h] = __ffma2_rn(nr, nw, cr[h]);
+        cg[h] = __ffma2_rn(ng, nw, cg[h]);
+        cb[h] = __ffma2_rn(nb, nw, cb[h]);
+    }
+}
+
 // sums the per-thread work counters of a counting launch into the frame counters
 __device__ __forceinline__ void flush_counts(Counters* c, unsigned n_eval, unsigned n_blend)
 {
@@ -189,7 +219,7 @@ __device__ __forceinline__ unsigned warp_lower_bound(const K* __restrict__ keys,
 }
 
 // One tile of the RoofGS rasterizer (a block of 256 / PPT threads).
-template <bool FAST, int PPT, bool COUNT>
+template <bool FAST, int PPT, bool COUNT, bool STRAIGHT = false>
 __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
 {
     constexpr int NT = 256 / PPT; // threads per tile of 256 pixels (16 x 16, 32 x 8 or 8 x 32)
@@ -246,6 +276,21 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
     } else {
         range = a.ranges[tile];
     }
+    // the record of entry j, and whether it is fetched while the batch before it is blended (eight
+    // registers; two pixels per thread: 256 tiles 22.4 -> 20.4 us, 1080p 126 -> 123 us; four pixels, 4K:
+    // 391 -> 396 us, not done)
+    constexpr int UNROLL = PPT == 4 ? 2 : (STRAIGHT ? 8 : 4);
+    constexpr bool AHEAD = PPT == 2 && !COUNT;
+    float4 q0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), q1 = q0;
+    auto fetch = [&](unsigned j) {
+        if (j < range.y) {
+            unsigned id = a.vals[j];
+            if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
+            q0 = __ldg(&a.rec[2 * id]);
+            q1 = __ldg(&a.rec[2 * id + 1]);
+        }
+    };
+    if (AHEAD) fetch(range.x + t);
     for (unsigned start = range.x; start < range.y; start += NT) {
         bool all_done = true;
 #pragma unroll
@@ -253,11 +298,8 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
             all_done = all_done && ((PAIRS || ONE) ? thr[i] == __int_as_float(0x7f800000) : done[i]);
         if (__syncthreads_count(!all_done) == 0) break;
         const unsigned j = start + t;
+        if (!AHEAD) fetch(j);
         if (j < range.y) {
-            unsigned id = a.vals[j];
-            if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
-            const float4 q0 = __ldg(&a.rec[2 * id]);
-            const float4 q1 = __ldg(&a.rec[2 * id + 1]);
             const float u = q0.x - (float)x0, v = q0.y - (float)y0;
             const float ca = q0.z, cbq = q0.w, cc = q1.x, logo = q1.y;
             // Eq. (15): folded coefficients
@@ -280,9 +322,10 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
             }
         }
         __syncthreads();
+        if (AHEAD) fetch(j + NT);
         const int cnt = min((unsigned)NT, range.y - start);
         if (!__all_sync(0xffffffffu, all_done)) {
-#pragma unroll(PPT == 4 ? 2 : 4) // records per iteration, 4K raster: 4 pixels 0.564 -> 0.558 ms (2), 2 pixels 0.549 -> 0.540 ms and 1 pixel 1.059 -> 0.900 ms (4)
+#pragma unroll(UNROLL) // records per iteration, 4K raster: 4 pixels 0.564 -> 0.558 ms (2), 2 pixels 0.549 -> 0.540 ms and 1 pixel 1.059 -> 0.900 ms (4)
             for (int k = 0; k < cnt; k++) {
                 const float4 c0 = s_c0[k];
                 const float4 c1 = s_c1[k];
@@ -312,7 +355,10 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
                         P[i] = P[i - 1] + d;
                     }
                 }
-                if constexpr (PAIRS) {
+                if constexpr (PAIRS && STRAIGHT) {
+                    blend_pairs_straight<NH>(P, make_float2(cn.x, cn.y), make_float2(cn.z, cn.w), make_float2(c1.z, c1.w),
+                                             T2, R2, G2, B2, thr);
+                } else if constexpr (PAIRS) {
                     blend_pairs_fast<NH>(P, make_float2(cn.x, cn.y), make_float2(cn.z, cn.w), make_float2(c1.z, c1.w),
                                          T2, R2, G2, B2, thr);
                 } else if constexpr (ONE) {
@@ -344,11 +390,11 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
     }
 }
 
-template <bool FAST, int PPT, bool COUNT>
+template <bool FAST, int PPT, bool COUNT, bool STRAIGHT = false>
 __global__ void __launch_bounds__(256 / PPT) k_raster_roofgs(RasterArgs a)
 {
     grid_dependency_wait();
-    raster_tile<FAST, PPT, COUNT>(a, (int)ordered_tile(a.order, blockIdx.x));
+    raster_tile<FAST, PPT, COUNT, STRAIGHT>(a, (int)ordered_tile(a.order, blockIdx.x));
 }
 
 // Every view of a batch in one persistent launch: each block takes (view, tile) items
@@ -400,7 +446,13 @@ template <bool COUNT>
 static void raster_roofgs_variant(const RasterArgs& a, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)(a.tiles_x * a.tiles_y);
-    if (a.fast_exp) {
+    // two pixels per thread and at most 20 tiles per SM: the blend without branches. 256 tiles, 10 k Gaussians
+    // 32.5 -> 20.2 us; 256 to 2,451 tiles, 30 k / 400 k Gaussians 20-35 % / 0-10 % less; 3,600 tiles and more fill
+    // the issue slots, and branches win (82 against 98 us, 1080p 124 against 150), as with four pixels per thread
+    // at any size once pixels finish early (256 tiles, 400 k: 1,043 against 1,120)
+    if (a.fast_exp && !COUNT && a.ppt == 2 && tiles <= 20u * (unsigned)device_sm_count()) {
+        launch_dependent(k_raster_roofgs<true, 2, false, true>, dim3(tiles), dim3(128), 0, s, a);
+    } else if (a.fast_exp) {
         if (a.ppt == 1) launch_dependent(k_raster_roofgs<true, 1, COUNT>, dim3(tiles), dim3(256), 0, s, a);
         else if (a.ppt == 4) launch_dependent(k_raster_roofgs<true, 4, COUNT>, dim3(tiles), dim3(64), 0, s, a);
         else launch_dependent(k_raster_roofgs<true, 2, COUNT>, dim3(tiles), dim3(128), 0, s, a);
@@ -522,17 +574,29 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
 #pragma unroll
     for (int i = 0; i < PPT; i++) lim[i] = px < W && py + i < H ? -INF : INF;
     const uint2 range = a.ranges[tile];
+    // the record of entry j, and whether it is fetched while the batch before it is blended (few tiles:
+    // 672 tiles 49.8 -> 47.0 us; four pixels per thread at 4K 676 -> 701 us, not done)
+    constexpr bool AHEAD = PPT == 2;
+    float4 m = make_float4(0.0f, 0.0f, 0.0f, 0.0f), q = m, c = m;
+    auto fetch = [&](unsigned j) {
+        if (j < range.y) {
+            unsigned id = a.vals[j];
+            if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
+            const float4* const rec = a.erec + 3 * (size_t)id;
+            m = __ldg(rec);
+            q = __ldg(rec + 1);
+            c = __ldg(rec + 2);
+        }
+    };
+    if (AHEAD) fetch(range.x + t);
     for (unsigned start = range.x; start < range.y; start += NT) {
         bool all_done = true;
 #pragma unroll
         for (int i = 0; i < PPT; i++) all_done = all_done && lim[i] == INF;
         if (__syncthreads_count(!all_done) == 0) break;
         const unsigned j = start + t;
+        if (!AHEAD) fetch(j);
         if (j < range.y) {
-            unsigned id = a.vals[j];
-            if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
-            const float4* const rec = a.erec + 3 * (size_t)id;
-            const float4 m = __ldg(rec), q = __ldg(rec + 1), c = __ldg(rec + 2);
             const float mz = m.z - (float)y0;
             s_a[t] = make_float4(m.x - (float)x0, exact_skip_below(q.w), q.w, 0.0f);
             s_b[t] = make_float4(-mz, -mz, -m.w, -m.w);
@@ -542,6 +606,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
             s_bb[t] = make_float2(c.z, c.z);
         }
         __syncthreads();
+        if (AHEAD) fetch(j + NT);
         const int cnt = min((unsigned)NT, range.y - start);
         if (__all_sync(0xffffffffu, all_done)) continue;
 #pragma unroll 2
