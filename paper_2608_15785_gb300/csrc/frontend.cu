@@ -638,25 +638,26 @@ void launch_frontend_runs(const FrontendArgs& a, const RunArgs& r, cudaStream_t 
 // ---------------------------------------------------------------------------
 constexpr int EX_THREADS = 256;
 
-// The raster record of Gaussian i, binned as b: the exponent of Eq. (10) with the quadratic form
+// The raster record of a Gaussian binned as b: the exponent of Eq. (10) with the quadratic form
 // completed in dx, -1/2 ((Sigma'_yy / det) (dx - c dy)^2 + dy^2 / Sigma'_yy), c = Sigma'_xy / Sigma'_yy
-// (no cancellation for thin Gaussians), the mean as double-floats (b's FP32 u, v only bin the
-// Gaussian), and the degree-3 SH colour from FP32 coefficients.
-__device__ __forceinline__ void exact_record(const ExactArgs& a, long long i, const Binned& b, float mx, float my,
-                                             float mz, float4& mean, float4& quad, float4& rgb)
+// (no cancellation for thin Gaussians), and the mean as double-floats (b's FP32 u, v only bin the
+// Gaussian).
+__device__ __forceinline__ void exact_record(const ExactArgs& a, float opacity, const Binned& b, float mx, float my,
+                                             float mz, float4& mean, float4& quad)
 {
-    quad = make_float4(-0.5f * __fdiv_rn(b.sc, b.det), __fdiv_rn(b.sb, b.sc), __fdiv_rn(-0.5f, b.sc), a.opac[i]);
+    quad = make_float4(-0.5f * __fdiv_rn(b.sc, b.det), __fdiv_rn(b.sb, b.sc), __fdiv_rn(-0.5f, b.sc), opacity);
     mean = project_mean_df(a.cam, mx, my, mz);
-    float dx, dy, dz;
-    view_dir(a.cam, mx, my, mz, dx, dy, dz);
-    float Y[16];
-    sh_basis(dx, dy, dz, Y);
-    const int nk = (a.sh_degree + 1) * (a.sh_degree + 1);
-    const float4* shp = reinterpret_cast<const float4*>(a.sh + 48 * i);
-    float c[3] = {0.5f, 0.5f, 0.5f};
+}
+
+// Adds the terms of words 4 V0 .. 4 V1 - 1 of a Gaussian's degree-3 SH coefficients (FP32) to its colour
+// c; word4(v) gives words 4 v .. 4 v + 3.
+template <int V0, int V1, class F>
+__device__ __forceinline__ void exact_colour(const float (&Y)[16], int sh_degree, float (&c)[3], F word4)
+{
+    const int nk = (sh_degree + 1) * (sh_degree + 1);
 #pragma unroll
-    for (int v4 = 0; v4 < 12; v4++) {
-        const float4 f = shp[v4];
+    for (int v4 = V0; v4 < V1; v4++) {
+        const float4 f = word4(v4);
         const float e[4] = {f.x, f.y, f.z, f.w};
 #pragma unroll
         for (int u = 0; u < 4; u++) {
@@ -665,7 +666,6 @@ __device__ __forceinline__ void exact_record(const ExactArgs& a, long long i, co
             if (k < nk) c[ch] = fmaf(Y[k], e[u], c[ch]);
         }
     }
-    rgb = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), 0.0f);
 }
 
 // Front end in index order: the frames whose tile grid is too large for runs.
@@ -691,7 +691,13 @@ __global__ void __launch_bounds__(EX_THREADS) k_exact_preprocess(ExactArgs a)
     a.depth[i] = pz;
     a.rect[i] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
     a.touched[i] = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
-    exact_record(a, i, b, mx, my, mz, a.rec[3 * i], a.rec[3 * i + 1], a.rec[3 * i + 2]);
+    exact_record(a, a.opac[i], b, mx, my, mz, a.rec[3 * i], a.rec[3 * i + 1]);
+    float dx, dy, dz, Y[16], c[3] = {0.5f, 0.5f, 0.5f};
+    view_dir(a.cam, mx, my, mz, dx, dy, dz);
+    sh_basis(dx, dy, dz, Y);
+    const float4* const shp = reinterpret_cast<const float4*>(a.sh + 48 * i);
+    exact_colour<0, 12>(Y, a.sh_degree, c, [&](int v) { return shp[v]; });
+    a.rec[3 * i + 2] = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), 0.0f);
 }
 
 __global__ void __launch_bounds__(DK_THREADS) k_exact_depth_keys(ExactArgs a, unsigned* keys, unsigned* vals, Counters* ctr,
@@ -772,46 +778,88 @@ __device__ __forceinline__ bool exact_row_range(const ExactRow& g, int ty, const
 // The front end of an exact frame of runs: one slot (Gaussian in depth order) per thread. Its record
 // goes to its slot; the frame's entries are counted by the rectangles (plain 3DGS's entries), while the
 // runs leave out the tiles where the Gaussian stays below 1/255 (about two thirds of the entries at
-// 4K), which the rasterizer would skip pixel by pixel. Bound by its depth-ordered gathers (236 B per
-// Gaussian; 405 us at 4K with 3 M, where the index-ordered preprocessing took 265). It pays for them many
-// times: with the entries in depth order no 64-bit key is written or sorted, and the whole exact frame
-// goes from 13.3 to 2.1 ms (4K, 3 M), 1.40 to 0.50 ms (1080p, 500 k).
+// 4K), which the rasterizer would skip pixel by pixel. Bound by its depth-ordered gathers (240 B per
+// Gaussian), which fill the L1 pipe (0.78 of its wavefronts) before HBM: 418 us at 4K with 3 M Gaussians with
+// every attribute array gathered by itself, 374 with the geometry in one 48-byte row (three or five
+// blocks per SM: 434 / 374), 321 with the SH rows fetched asynchronously as below as well (three / five: 351 /
+// 407). It replaced an index-ordered preprocessing of 265 us and pays for that many times: with
+// the entries in depth order no 64-bit key is written or sorted, and the whole exact frame went from 13.3 to
+// 2.1 ms (4K, 3 M), 1.40 to 0.50 ms (1080p, 500 k) by it.
 __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunArgs r, int keep_all)
 {
-    __shared__ ExactRow s_row[FE_THREADS];
+    // the warps' SH rows, half a row at a time; then the slots' row tests
+    constexpr int SH_HALF = 24, SH_PITCH = 28; // words (the pitch: 16-byte reads without bank conflicts)
+    __shared__ __align__(16) float s_sh[FE_WARPS][32 * SH_PITCH];
+    ExactRow* const s_row = reinterpret_cast<ExactRow*>(s_sh);
     __shared__ unsigned long long s_sum[FE_WARPS];
-    static_assert(sizeof(s_row) >= FE_WARPS * RUN_CACHE * 4, "the runs are staged over the rows");
+    static_assert(sizeof(s_sh) >= FE_THREADS * sizeof(ExactRow) && sizeof(s_sh) >= FE_WARPS * RUN_CACHE * 4,
+                  "the row tests, then the staged runs, lie over the SH rows");
     grid_dependency_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long slot = (long long)blockIdx.x * FE_THREADS + tid;
     bool front = false, vis = false;
     int rows_l = 0;
     unsigned tiles = 0;
-    if (slot < a.n) {
-        const long long i = (long long)a.order[slot]; // below n
-        const float mx = a.means[3 * i], my = a.means[3 * i + 1], mz = a.means[3 * i + 2];
-        const float pz = view_z(a.cam, mx, my, mz);
-        front = pz > a.cam.zn && pz <= a.cam.zf;
-        if (front) {
-            const float4 q = *reinterpret_cast<const float4*>(&a.quats[4 * i]);
-            Binned b;
-            vis = project_bin(a.cam, mx, my, mz, pz, q.x, q.y, q.z, q.w, a.scales[3 * i], a.scales[3 * i + 1],
-                              a.scales[3 * i + 2], false, 0.0f, b);
-            if (vis) {
-                float4 mean, quad, rgb;
-                exact_record(a, i, b, mx, my, mz, mean, quad, rgb);
-                a.rec[3 * slot] = mean;
-                a.rec[3 * slot + 1] = quad;
-                a.rec[3 * slot + 2] = rgb;
-                a.rect[slot] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
-                tiles = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
-                bool any;
-                s_row[tid] = exact_row(b, mean, quad, any);
-                if (any || keep_all) rows_l = b.ty1 - b.ty0 + 1;
+    const unsigned i = slot < a.n ? a.order[slot] : 0u; // below n
+    // The colour's SH rows (192 bytes each, in depth order anywhere in memory) come asynchronously, half a
+    // row at a time, six lanes to a row; each thread reads its own from shared memory. A thread loading its
+    // own row touched 32 lines with every instruction, which filled the L1 pipe.
+    auto fetch = [&](unsigned rows, int half) {
+#pragma unroll
+        for (int it = 0; it < 6; it++) {
+            const int q = it * 32 + lane, g = q / 6, part = q % 6;
+            const unsigned j = __shfl_sync(0xffffffffu, i, g);
+            if ((rows >> g) & 1u) {
+                const unsigned dst = (unsigned)__cvta_generic_to_shared(&s_sh[warp][g * SH_PITCH + 4 * part]);
+                const float* src = a.sh + 48 * (size_t)j + SH_HALF * half + 4 * part;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
             }
         }
-        a.touched[i] = tiles;
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    auto arrived = [&]() {
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncwarp();
+    };
+    const float4 m = slot < a.n ? __ldg(&a.geo[3 * (size_t)i]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float pz = view_z(a.cam, m.x, m.y, m.z);
+    front = slot < a.n && pz > a.cam.zn && pz <= a.cam.zf;
+    fetch(__ballot_sync(0xffffffffu, front), 0);
+    Binned b;
+    if (front) {
+        const float4 q = __ldg(&a.geo[3 * (size_t)i + 1]), s = __ldg(&a.geo[3 * (size_t)i + 2]);
+        vis = project_bin(a.cam, m.x, m.y, m.z, pz, q.x, q.y, q.z, q.w, s.x, s.y, s.z, false, 0.0f, b);
     }
+    const unsigned seen = __ballot_sync(0xffffffffu, vis);
+    const float4* const own = reinterpret_cast<const float4*>(&s_sh[warp][lane * SH_PITCH]);
+    float Y[16], c[3] = {0.5f, 0.5f, 0.5f};
+    float dx, dy, dz;
+    view_dir(a.cam, m.x, m.y, m.z, dx, dy, dz);
+    sh_basis(dx, dy, dz, Y);
+    arrived();
+    if (vis) exact_colour<0, 6>(Y, a.sh_degree, c, [&](int v) { return own[v]; });
+    __syncwarp();
+    fetch(seen, 1);
+    ExactRow row;
+    bool any = false;
+    if (vis) {
+        float4 mean, quad;
+        exact_record(a, m.w, b, m.x, m.y, m.z, mean, quad);
+        a.rec[3 * slot] = mean;
+        a.rec[3 * slot + 1] = quad;
+        a.rect[slot] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
+        tiles = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
+        row = exact_row(b, mean, quad, any);
+        if (any || keep_all) rows_l = b.ty1 - b.ty0 + 1;
+    }
+    if (slot < a.n) a.touched[i] = tiles;
+    arrived();
+    if (vis) {
+        exact_colour<6, 12>(Y, a.sh_degree, c, [&](int v) { return own[v - 6]; });
+        a.rec[3 * slot + 2] = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), 0.0f);
+    }
+    __syncthreads(); // the row tests lie over the SH rows of other warps
+    if (rows_l) s_row[tid] = row;
     emit_runs(r, blockIdx.x, rows_l, reinterpret_cast<unsigned*>(s_row), [&](int t, int k, int& ty, int& txa, int& txb) {
         const ExactRow& G = s_row[t];
         ty = G.ty0 + k;
@@ -1078,6 +1126,23 @@ void launch_check_attributes(const float* means, const float* scales, const floa
     long long blocks = (48 * n + 255) / 256;
     if (blocks > 16ll * device_sm_count()) blocks = 16ll * device_sm_count();
     k_check_attributes<<<(unsigned)blocks, 256, 0, s>>>(means, scales, quats, opac, sh, n, flag);
+}
+
+__global__ void k_pack_geometry(const float* means, const float* scales, const float* quats, const float* opac,
+                                long long n, float4* geo)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    geo[3 * i] = make_float4(means[3 * i], means[3 * i + 1], means[3 * i + 2], opac[i]);
+    geo[3 * i + 1] = make_float4(quats[4 * i], quats[4 * i + 1], quats[4 * i + 2], quats[4 * i + 3]);
+    geo[3 * i + 2] = make_float4(scales[3 * i], scales[3 * i + 1], scales[3 * i + 2], 0.0f);
+}
+
+void launch_pack_geometry(const float* means, const float* scales, const float* quats, const float* opac, long long n,
+                          float4* geo, cudaStream_t s)
+{
+    if (n <= 0) return;
+    k_pack_geometry<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(means, scales, quats, opac, n, geo);
 }
 
 // max |SH| per (degree, channel): float bits of non-negative values order like integers

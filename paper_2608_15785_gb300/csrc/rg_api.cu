@@ -571,6 +571,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         a.quats = s->quats.as<float>();
         a.opac = s->opac.as<float>();
         a.sh = s->sh.as<float>();
+        a.geo = s->geo.as<float4>();
         a.sh_degree = s->sh_degree;
         a.n = n;
         a.cam = F.cam;
@@ -740,7 +741,7 @@ rg_status upload(DevBuf& dst, const float* src, size_t count, int on_device, cud
 
 void destroy_scene(rg_scene* s)
 {
-    DevBuf* bufs[] = {&s->means, &s->scales, &s->quats, &s->opac, &s->sh, &s->geoA, &s->geoB, &s->shq, &s->sticky};
+    DevBuf* bufs[] = {&s->means, &s->scales, &s->quats, &s->opac, &s->sh, &s->geoA, &s->geoB, &s->shq, &s->sticky, &s->geo};
     for (DevBuf* b : bufs) b->release();
     s->ws.release();
     delete s;
@@ -810,6 +811,10 @@ rg_status rg_scene_create(const rg_scene_desc* desc, void* stream, rg_scene** ou
     if (cudaMemsetAsync(s->sticky.p, 0, sizeof(Sticky), st) != cudaSuccess) RG_STEP(fail(RG_ERR_CUDA, "memset"));
     if (cudaMemsetAsync(flag.p, 0, 16, st) != cudaSuccess) RG_STEP(fail(RG_ERR_CUDA, "memset"));
     launch_check_attributes(dm, ds, dq, dop, dsh, n, flag.as<unsigned>(), st);
+    if (keep32) {
+        RG_STEP(ensure(s->geo, (size_t)n * 48, "geometry"));
+        launch_pack_geometry(dm, ds, dq, dop, n, s->geo.as<float4>(), st);
+    }
     // the compact storage needs the opacities on the host: log o (FP64 log, rounded to FP32)
     std::vector<float> lo;
     if (s->storage & RG_STORE_COMPACT) {
@@ -1021,6 +1026,14 @@ rg_status rg_scene_load(const char* path, void* stream, rg_scene** out)
         }
     }
     std::fclose(f);
+    if (e == RG_OK && (s->storage & RG_STORE_FP32)) {
+        e = ensure(s->geo, (size_t)s->n * 48, "geometry");
+        if (e == RG_OK) {
+            launch_pack_geometry(s->means.as<float>(), s->scales.as<float>(), s->quats.as<float>(), s->opac.as<float>(),
+                                 s->n, s->geo.as<float4>(), st);
+            if (cudaStreamSynchronize(st) != cudaSuccess) e = fail(RG_ERR_CUDA, "scene conversion failed");
+        }
+    }
     if (e != RG_OK) {
         cudaStreamSynchronize(st);
         destroy_scene(s);

@@ -127,6 +127,7 @@ struct rg_scene {
     int sh_scale_mode = 0;
     // exact-mode attributes (FP32)
     rg::DevBuf means, scales, quats, opac, sh;
+    rg::DevBuf geo; // their geometry again, 48 contiguous bytes per Gaussian (launch_pack_geometry)
     // compact attributes (RoofGS mode)
     rg::DevBuf geoA, geoB, shq;
     float band_scale[12] = {0};

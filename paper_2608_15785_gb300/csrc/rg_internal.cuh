@@ -655,6 +655,7 @@ struct ExactArgs {
     long long n;
     CamDev cam;
     Layout lay;
+    const float4* geo;     // [N][3] (mean, opacity), quaternion, (scales, -): what a frame gathers in depth order
     const unsigned* order; // [N] Gaussian of each slot (depth order) in a frame of tile-row runs, else null
     // per slot (index without an order):
     float4* rec;           // [N][3] projected mean as double-floats (u.hi, u.lo, v.hi, v.lo);
@@ -830,6 +831,9 @@ void set_last_error(const char* msg);
 // ORs into *flag: 1 if an attribute is not finite, 2 if an opacity lies outside [0, 1]
 void launch_check_attributes(const float* means, const float* scales, const float* quats, const float* opac,
                              const float* sh, long long n, unsigned* flag, cudaStream_t s);
+// geo [n][3] = (mean, opacity), quaternion, (scales, 0)
+void launch_pack_geometry(const float* means, const float* scales, const float* quats, const float* opac, long long n,
+                          float4* geo, cudaStream_t s);
 void launch_sh_absmax(const float* sh, long long n, unsigned* maxbits /*[12]*/, cudaStream_t s);
 void launch_compact(const float* means, const float* scales, const float* quats, const float* logo,
                     const float* sh, long long n, const float* band_scale /*host [12]*/, int per_gauss,
