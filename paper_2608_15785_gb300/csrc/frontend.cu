@@ -580,14 +580,11 @@ __device__ __forceinline__ unsigned emit_runs(const RunArgs& r, const unsigned v
     return __reduce_or_sync(0xffffffffu, vis);
 }
 
-// resident blocks per SM: 6 (40 registers, no spills); the fused kernel's 8 (32 registers) spill.
-// The tile rows found by the counting walk are kept for the placing one (8 KB; 217 -> 201 us at 4K
-// against walking twice)
-#ifndef RG_FER_MIN_BLOCKS
-#define RG_FER_MIN_BLOCKS 6
-#endif
-
-__global__ void __launch_bounds__(FE_THREADS, RG_FER_MIN_BLOCKS) k_frontend_runs(FrontendArgs a, RunArgs r)
+// Resident blocks per SM: 5 (48 registers). What shared memory leaves of the L1 holds the depth-ordered
+// gathers, so more blocks cost more than they hide, above all with the per-row words of 8K: 4 / 5 / 6
+// blocks 213 / 196 / 207 us at 4K, 105 / 101 / 130 us at 8K, 37 / 33 / 33 us at 1080p. The tile rows found
+// by the counting walk are kept for the placing one (8 KB; 217 -> 201 us at 4K against walking twice).
+__global__ void __launch_bounds__(FE_THREADS, 5) k_frontend_runs(FrontendArgs a, RunArgs r)
 {
     __shared__ RowTestS s_rt[FE_THREADS];
     static_assert(sizeof(s_rt) >= FE_WARPS * RUN_CACHE * 4, "the runs are staged over the row tests");

@@ -273,7 +273,8 @@ __device__ __forceinline__ void collect_chunk(const RunArgs& a, const RunRow& r,
 }
 
 // Grid (blocks per row, rows): block x of a row takes its chunks x, x + gridDim.x, ...
-__global__ void __launch_bounds__(RUN_THREADS) k_run_collect(RunArgs a)
+// (six blocks per SM: latency-bound; four, five, eight: 4K 98, 99, 103 us with k_run_rows, six 92)
+__global__ void __launch_bounds__(RUN_THREADS, 6) k_run_collect(RunArgs a)
 {
     __shared__ CollectSmem S;
     grid_dependency_wait();
@@ -638,9 +639,10 @@ void launch_runs(const RunArgs& a, cudaStream_t s, cudaEvent_t ev_after_collect)
         launch_dependent(k_run_expand<true>, grid, block, sizeof(ExpandSmem), s, a);
         return;
     }
-    // at most the chunks a row can have, and about 8 waves of blocks over all rows
+    // at most the chunks a row can have, and about 4 waves of blocks over all rows (2 / 8 waves: 1080p 53 / 57 us
+    // of collection and expansion, 4K 407 / 375; 4: 53 and 379)
     const unsigned most = a.blocks * (unsigned)RUN_SLOTS / CHUNK_STEP + a.blocks / CHUNK_BLOCKS + 1;
-    const unsigned want = (unsigned)(8 * 5 * device_sm_count() / a.rows + 1);
+    const unsigned want = (unsigned)(4 * 5 * device_sm_count() / a.rows + 1);
     const dim3 grid(most < want ? most : want, (unsigned)a.rows);
     launch_dependent(k_run_rows, dim3((unsigned)a.rows), dim3(1024), 0, s, a);
     launch_dependent(k_run_collect, grid, block, 0, s, a);
