@@ -69,7 +69,7 @@ __device__ __forceinline__ void blend(float P, float r, float g, float b, float&
 
 // A thread's pixels blended in pairs with packed FP32x2 arithmetic (FFMA2 / FMUL2: one
 // instruction for both pixels of a pair). Per pixel the operations and roundings of
-// blend<true, false>, written with -alpha (the shift-add of Eq. (24) without its + 2^31
+// blend<FAST, false>, written with -alpha (the shift-add of Eq. (24) without its + 2^31
 // is -exp^(P): that addition only sets the sign bit) and with the negated colours nr, ng,
 // nb: T + T (-alpha) = T (1 - alpha) and c + (-r)(-alpha T) = c + r (alpha T) round to the
 // same values. A pixel's state is its skip threshold thr: -ln 255 while it blends, +inf
@@ -79,8 +79,8 @@ __device__ __forceinline__ void blend(float P, float r, float g, float b, float&
 // (4K raster 0.558 -> 0.476 ms against selects on every pair and a finished flag beside
 // the threshold test; 0.476 -> 0.453 ms with the branches taken once for all of the
 // thread's pairs instead of once per pair).
-template <int NH>
-__device__ __forceinline__ void blend_pairs_fast(const float (&P)[2 * NH], float2 nr, float2 ng, float2 nb,
+template <bool FAST, int NH>
+__device__ __forceinline__ void blend_pairs(const float (&P)[2 * NH], float2 nr, float2 ng, float2 nb,
                                                  float2 (&T)[NH], float2 (&cr)[NH], float2 (&cg)[NH],
                                                  float2 (&cb)[NH], float (&thr)[2 * NH])
 {
@@ -96,10 +96,16 @@ __device__ __forceinline__ void blend_pairs_fast(const float (&P)[2 * NH], float
     bool stop = false;
 #pragma unroll
     for (int h = 0; h < NH; h++) {
-        const float2 w = __ffma2_rn(make_float2(P[2 * h], P[2 * h + 1]), make_float2(1.44269502f, 1.44269502f),
-                                    make_float2(126.954323f, 126.954323f));
-        const float ea = __uint_as_float(__float_as_uint(w.x) << 6); // -exp^(P)
-        const float eb = __uint_as_float(__float_as_uint(w.y) << 6);
+        float ea, eb; // -exp^(P), or -expf(P)
+        if constexpr (FAST) {
+            const float2 w = __ffma2_rn(make_float2(P[2 * h], P[2 * h + 1]), make_float2(1.44269502f, 1.44269502f),
+                                        make_float2(126.954323f, 126.954323f));
+            ea = __uint_as_float(__float_as_uint(w.x) << 6);
+            eb = __uint_as_float(__float_as_uint(w.y) << 6);
+        } else {
+            ea = -expf(P[2 * h]);
+            eb = -expf(P[2 * h + 1]);
+        }
         const float2 na = make_float2(u[2 * h] ? fmaxf(-0.99f, ea) : 0.0f, u[2 * h + 1] ? fmaxf(-0.99f, eb) : 0.0f);
         Tn[h] = __ffma2_rn(T[h], na, T[h]);
         nw[h] = __fmul2_rn(na, T[h]); // -alpha T
@@ -130,13 +136,16 @@ __device__ __forceinline__ void blend_pairs_fast(const float (&P)[2 * NH], float
 }
 
 // The same blend for a thread with one pixel: the skip threshold as its state, the stop
-// below 1e-4 a branch around the common path (bit-identical to blend<true, false>).
-__device__ __forceinline__ void blend_one_fast(float P, float nr, float ng, float nb, float& T, float& cr, float& cg,
+// below 1e-4 a branch around the common path (bit-identical to blend<FAST, false>).
+template <bool FAST>
+__device__ __forceinline__ void blend_one(float P, float nr, float ng, float nb, float& T, float& cr, float& cg,
                                                float& cb, float& thr)
 {
     if (!(P >= thr)) return;
-    const float w = fmaf(P, 1.44269502f, 126.954323f);
-    const float na = fmaxf(-0.99f, __uint_as_float(__float_as_uint(w) << 6)); // -alpha
+    float e; // -exp^(P), or -expf(P)
+    if constexpr (FAST) e = __uint_as_float(__float_as_uint(fmaf(P, 1.44269502f, 126.954323f)) << 6);
+    else e = -expf(P);
+    const float na = fmaxf(-0.99f, e); // -alpha
     float Tn = fmaf(T, na, T);
     float nw = na * T; // -alpha T
     if (Tn < 1e-4f) { // once in the pixel's life: adds nothing, T kept, finished
@@ -240,8 +249,8 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
     bool done[PPT];
     // the packed pair blend keeps a pixel's state as its skip threshold instead: -ln 255 while it
     // blends, +inf once finished (one compare per pixel and Gaussian instead of two tests)
-    constexpr bool PAIRS = FAST && !COUNT && PPT >= 2;
-    constexpr bool ONE = FAST && !COUNT && PPT == 1;
+    constexpr bool PAIRS = !COUNT && PPT >= 2;
+    constexpr bool ONE = !COUNT && PPT == 1;
     float thr[PPT];
     // transmittance and colour of pixel i in component i & 1 of pair i / 2
     float2 T2[NH], R2[NH], G2[NH], B2[NH];
@@ -359,10 +368,10 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
                     blend_pairs_straight<NH>(P, make_float2(cn.x, cn.y), make_float2(cn.z, cn.w), make_float2(c1.z, c1.w),
                                              T2, R2, G2, B2, thr);
                 } else if constexpr (PAIRS) {
-                    blend_pairs_fast<NH>(P, make_float2(cn.x, cn.y), make_float2(cn.z, cn.w), make_float2(c1.z, c1.w),
+                    blend_pairs<FAST, NH>(P, make_float2(cn.x, cn.y), make_float2(cn.z, cn.w), make_float2(c1.z, c1.w),
                                          T2, R2, G2, B2, thr);
                 } else if constexpr (ONE) {
-                    blend_one_fast(P[0], nr, ng, nb, T2[0].x, R2[0].x, G2[0].x, B2[0].x, thr[0]);
+                    blend_one<FAST>(P[0], nr, ng, nb, T2[0].x, R2[0].x, G2[0].x, B2[0].x, thr[0]);
                 } else {
 #pragma unroll
                     for (int i = 0; i < PPT; i++) {

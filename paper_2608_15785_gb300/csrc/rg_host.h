@@ -70,6 +70,7 @@ constexpr size_t CTRL_BYTES = sizeof(Counters) + 8 * 256 * sizeof(unsigned);
 constexpr size_t FE_HIST_BYTES = (size_t)FE_HIST_COPIES * 8 * 256 * sizeof(unsigned);
 constexpr size_t RUN_TOT_AT = (2 * CTRL_BYTES + FE_HIST_BYTES + 15) / 16 * 16; // then RunArgs::tot
 constexpr size_t CTRL_ALLOC = RUN_TOT_AT + (size_t)RUN_MAX_GRID * 8;
+static_assert(CTRL_ALLOC % 16 == 0, "cleared 16 bytes at a time");
 
 // Frame workspace: everything one frame in flight needs besides the scene.
 // rg_render uses the scene's own workspace; a batch lane or a server slot owns one.
