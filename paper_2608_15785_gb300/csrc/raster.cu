@@ -227,8 +227,14 @@ __device__ __forceinline__ unsigned warp_lower_bound(const K* __restrict__ keys,
     return lo + (unsigned)__popc(__ballot_sync(0xffffffffu, less));
 }
 
+// Limited frames (RunArgs::limit) have the first RUN_LIMIT entries of every tile in vals. A tile that is read
+// further before its pixels are finished is left to a second launch (REST), before which its other entries are
+// written: its pixels' T stand in the place of its first entries (negative: finished), their colours in the image.
+// (With the further entries fetched by the tile's own block the code around the loop cost every tile 3 to 5 %.)
+enum { WHOLE = 0, LIMITED = 1, REST = 2 };
+
 // One tile of the RoofGS rasterizer (a block of 256 / PPT threads).
-template <bool FAST, int PPT, bool COUNT, bool STRAIGHT = false>
+template <bool FAST, int PPT, bool COUNT, bool STRAIGHT = false, int MODE = WHOLE>
 __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
 {
     constexpr int NT = 256 / PPT; // threads per tile of 256 pixels (16 x 16, 32 x 8 or 8 x 32)
@@ -269,7 +275,7 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
     const float xx = x * x, xy = x * y, yy = y * y, y2p1 = 2.0f * y + 1.0f;
     unsigned n_eval = 0, n_blend = 0;
     uint2 range;
-    if (a.skeys || a.skeys16) { // warps 0 and 1 search the first entries of tiles `tile` and `tile + 1`
+    if (MODE == WHOLE && (a.skeys || a.skeys16)) { // warps 0 and 1 search the first entries of tiles `tile` and `tile + 1`
         __shared__ unsigned s_bound[2];
         const int warp = t >> 5;
         if (warp < 2) {
@@ -289,26 +295,51 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
     // registers; two pixels per thread: 256 tiles 22.4 -> 20.4 us, 1080p 126 -> 123 us; four pixels, 4K:
     // 391 -> 396 us, not done)
     constexpr int UNROLL = PPT == 4 ? 2 : (STRAIGHT ? 8 : 4);
-    constexpr bool AHEAD = PPT == 2 && !COUNT;
+    constexpr bool AHEAD = PPT == 2 && !COUNT && MODE != REST;
     float4 q0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), q1 = q0;
+    unsigned first = range.x, end = range.y; // entries blended next
+    if (MODE != WHOLE) {
+        const unsigned limit = a.row_limit[ty];
+        if (range.y - range.x > limit) end = range.x + limit;
+    }
     auto fetch = [&](unsigned j) {
-        if (j < range.y) {
+        if (j < end) {
             unsigned id = a.vals[j];
             if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
             q0 = __ldg(&a.rec[2 * id]);
             q1 = __ldg(&a.rec[2 * id + 1]);
         }
     };
-    if (AHEAD) fetch(range.x + t);
-    for (unsigned start = range.x; start < range.y; start += NT) {
-        bool all_done = true;
+    auto finished = [&](bool& all_done) { // every pixel of the thread, of the block
+        all_done = true;
 #pragma unroll
         for (int i = 0; i < PPT; i++)
             all_done = all_done && ((PAIRS || ONE) ? thr[i] == __int_as_float(0x7f800000) : done[i]);
-        if (__syncthreads_count(!all_done) == 0) break;
+        return __syncthreads_count(!all_done) == 0;
+    };
+    bool all_done = false;
+    if constexpr (MODE == REST) { // the pixels as the first kernel left them
+        first = end;
+        end = range.y;
+#pragma unroll
+        for (int i = 0; i < PPT; i++) {
+            const float Ti = __uint_as_float(a.vals[range.x + (unsigned)(i * NT + t)]);
+            thr[i] = Ti < 0.0f ? __int_as_float(0x7f800000) : -LN255F;
+            ((i & 1) ? T2[i >> 1].y : T2[i >> 1].x) = fabsf(Ti);
+            if (px < W && py + i < H) {
+                const size_t plane = (size_t)W * H, o = (size_t)(py + i) * W + px;
+                ((i & 1) ? R2[i >> 1].y : R2[i >> 1].x) = a.out[o];
+                ((i & 1) ? G2[i >> 1].y : G2[i >> 1].x) = a.out[plane + o];
+                ((i & 1) ? B2[i >> 1].y : B2[i >> 1].x) = a.out[2 * plane + o];
+            }
+        }
+    }
+    if (AHEAD) fetch(first + t);
+    for (unsigned start = first; start < end; start += NT) {
+        if (finished(all_done)) break;
         const unsigned j = start + t;
         if (!AHEAD) fetch(j);
-        if (j < range.y) {
+        if (j < end) {
             const float u = q0.x - (float)x0, v = q0.y - (float)y0;
             const float ca = q0.z, cbq = q0.w, cc = q1.x, logo = q1.y;
             // Eq. (15): folded coefficients
@@ -332,7 +363,7 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
         }
         __syncthreads();
         if (AHEAD) fetch(j + NT);
-        const int cnt = min((unsigned)NT, range.y - start);
+        const int cnt = min((unsigned)NT, end - start);
         if (!__all_sync(0xffffffffu, all_done)) {
 #pragma unroll(UNROLL) // records per iteration, 4K raster: 4 pixels 0.564 -> 0.558 ms (2), 2 pixels 0.549 -> 0.540 ms and 1 pixel 1.059 -> 0.900 ms (4)
             for (int k = 0; k < cnt; k++) {
@@ -385,6 +416,21 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
             }
         }
     }
+    const bool rest = MODE == LIMITED && end < range.y && !finished(all_done);
+    if constexpr (MODE == LIMITED) {
+        if (rest) {
+            if (t == 0) {
+                a.rest_list[atomicAdd(a.rest_count, 1u)] = (unsigned)tile;
+                a.rest_flag[tile] = 1u;
+            }
+#pragma unroll
+            for (int i = 0; i < PPT; i++) {
+                const float Ti = (i & 1) ? T2[i >> 1].y : T2[i >> 1].x;
+                a.vals_out[range.x + (unsigned)(i * NT + t)] =
+                    __float_as_uint(thr[i] == __int_as_float(0x7f800000) ? -Ti : Ti);
+            }
+        }
+    }
     if (COUNT) flush_counts(a.count, n_eval, n_blend);
     const size_t plane = (size_t)W * H;
 #pragma unroll
@@ -392,19 +438,35 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
         if (px < W && py + i < H) {
             const size_t o = (size_t)(py + i) * W + px;
             const float Ti = (i & 1) ? T2[i >> 1].y : T2[i >> 1].x;
-            a.out[o] = ((i & 1) ? R2[i >> 1].y : R2[i >> 1].x) + Ti * a.cam.bg[0];
-            a.out[plane + o] = ((i & 1) ? G2[i >> 1].y : G2[i >> 1].x) + Ti * a.cam.bg[1];
-            a.out[2 * plane + o] = ((i & 1) ? B2[i >> 1].y : B2[i >> 1].x) + Ti * a.cam.bg[2];
+            const float r = (i & 1) ? R2[i >> 1].y : R2[i >> 1].x, g = (i & 1) ? G2[i >> 1].y : G2[i >> 1].x,
+                        b = (i & 1) ? B2[i >> 1].y : B2[i >> 1].x;
+            a.out[o] = rest ? r : r + Ti * a.cam.bg[0];
+            a.out[plane + o] = rest ? g : g + Ti * a.cam.bg[1];
+            a.out[2 * plane + o] = rest ? b : b + Ti * a.cam.bg[2];
         }
     }
 }
 
-template <bool FAST, int PPT, bool COUNT, bool STRAIGHT = false>
+template <bool FAST, int PPT, bool COUNT, bool STRAIGHT = false, int MODE = WHOLE>
 __global__ void __launch_bounds__(256 / PPT) k_raster_roofgs(RasterArgs a)
 {
     grid_dependency_wait();
-    raster_tile<FAST, PPT, COUNT, STRAIGHT>(a, (int)ordered_tile(a.order, blockIdx.x));
+    raster_tile<FAST, PPT, COUNT, STRAIGHT, MODE>(a, (int)ordered_tile(a.order, blockIdx.x));
 }
+
+// the tiles that a LIMITED launch left unfinished
+template <bool FAST, int PPT>
+__global__ void __launch_bounds__(256 / PPT) k_raster_roofgs_rest(RasterArgs a)
+{
+    grid_dependency_wait();
+    const unsigned n = *a.rest_count;
+    for (unsigned b = blockIdx.x; b < n; b += gridDim.x) {
+        raster_tile<FAST, PPT, false, false, REST>(a, (int)a.rest_list[b]);
+        __syncthreads(); // the staged records are written again
+    }
+}
+// blocks of such a launch (its list is in about the order of the first one, the longest tiles first)
+static unsigned rest_blocks(int ppt) { return (unsigned)(4 * ppt * device_sm_count()); }
 
 // Every view of a batch in one persistent launch: each block takes (view, tile) items
 // from one work counter (views in order, tiles in order) until all are done, and
@@ -452,9 +514,28 @@ void launch_raster_views(const RasterViews& m, int fast_exp, int ppt, cudaStream
 }
 
 template <bool COUNT>
-static void raster_roofgs_variant(const RasterArgs& a, cudaStream_t s)
+static void raster_roofgs_variant(const RasterArgs& a, const RunArgs* runs, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)(a.tiles_x * a.tiles_y);
+    if constexpr (!COUNT) {
+        if (a.limit != RUN_ALL) {
+            auto launch = [&](auto kernel, auto rest, unsigned ppt) {
+                launch_dependent(kernel, dim3(tiles), dim3(256 / ppt), 0, s, a);
+                launch_runs_rest(*runs, s);
+                launch_dependent(rest, dim3(rest_blocks((int)ppt)), dim3(256 / ppt), 0, s, a);
+            };
+            if (a.fast_exp) {
+                if (a.ppt == 1) launch(k_raster_roofgs<true, 1, false, false, LIMITED>, k_raster_roofgs_rest<true, 1>, 1);
+                else if (a.ppt == 4) launch(k_raster_roofgs<true, 4, false, false, LIMITED>, k_raster_roofgs_rest<true, 4>, 4);
+                else launch(k_raster_roofgs<true, 2, false, false, LIMITED>, k_raster_roofgs_rest<true, 2>, 2);
+            } else {
+                if (a.ppt == 1) launch(k_raster_roofgs<false, 1, false, false, LIMITED>, k_raster_roofgs_rest<false, 1>, 1);
+                else if (a.ppt == 4) launch(k_raster_roofgs<false, 4, false, false, LIMITED>, k_raster_roofgs_rest<false, 4>, 4);
+                else launch(k_raster_roofgs<false, 2, false, false, LIMITED>, k_raster_roofgs_rest<false, 2>, 2);
+            }
+            return;
+        }
+    }
     // two pixels per thread and at most 20 tiles per SM: the blend without branches. 256 tiles, 10 k Gaussians
     // 32.5 -> 20.2 us; 256 to 2,451 tiles, 30 k / 400 k Gaussians 20-35 % / 0-10 % less; 3,600 tiles and more fill
     // the issue slots, and branches win (82 against 98 us, 1080p 124 against 150), as with four pixels per thread
@@ -472,10 +553,10 @@ static void raster_roofgs_variant(const RasterArgs& a, cudaStream_t s)
     }
 }
 
-void launch_raster_roofgs(const RasterArgs& a, cudaStream_t s)
+void launch_raster_roofgs(const RasterArgs& a, const RunArgs* runs, cudaStream_t s)
 {
-    if (a.count) raster_roofgs_variant<true>(a, s);
-    else raster_roofgs_variant<false>(a, s);
+    if (a.count) raster_roofgs_variant<true>(a, runs, s);
+    else raster_roofgs_variant<false>(a, runs, s);
 }
 
 // Plain 3DGS rasterizer: expf, the exponent of Eq. (10) in the completed-square form of
@@ -553,8 +634,8 @@ __global__ void __launch_bounds__(E_THREADS) k_raster_exact_count(RasterArgs a)
 // cycle at 1080p, the last wave of heavy tiles aside): 4K, 3 M Gaussians 950 -> 730 us against one
 // pixel per thread with expf on every pair, 1080p, 500 k 300 -> 240 us.
 // Records are staged with the operands of the packed instructions doubled.
-template <int PPT>
-__global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
+template <int PPT, int MODE>
+__device__ __forceinline__ void exact_tile(const RasterArgs& a, const int tile)
 {
     constexpr int NT = 256 / PPT, NH = PPT / 2;
     __shared__ float4 s_a[NT]; // u - x0, skip threshold, opacity
@@ -563,8 +644,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
     __shared__ float4 s_d[NT]; // quad.x twice, quad.z twice
     __shared__ float4 s_rg[NT]; // r, r, g, g
     __shared__ float2 s_bb[NT]; // b, b
-    grid_dependency_wait();
-    const int tile = (int)ordered_tile(a.order, blockIdx.x), t = threadIdx.x;
+    const int t = threadIdx.x;
     const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
     const int x0 = tx * a.cam.tw, y0 = ty * a.cam.th;
     const int lxi = t & (a.cam.tw - 1), lyi = (t >> a.cam.tw_log2) * PPT;
@@ -585,10 +665,15 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
     const uint2 range = a.ranges[tile];
     // the record of entry j, and whether it is fetched while the batch before it is blended (few tiles:
     // 672 tiles 49.8 -> 47.0 us; four pixels per thread at 4K 676 -> 701 us, not done)
-    constexpr bool AHEAD = PPT == 2;
+    constexpr bool AHEAD = PPT == 2 && MODE != REST;
     float4 m = make_float4(0.0f, 0.0f, 0.0f, 0.0f), q = m, c = m;
+    unsigned first = range.x, end = range.y; // entries blended next
+    if (MODE != WHOLE) {
+        const unsigned limit = a.row_limit[ty];
+        if (range.y - range.x > limit) end = range.x + limit;
+    }
     auto fetch = [&](unsigned j) {
-        if (j < range.y) {
+        if (j < end) {
             unsigned id = a.vals[j];
             if (id >= (unsigned long long)a.n) id = 0; // only after a failed (timed-out) sort
             const float4* const rec = a.erec + 3 * (size_t)id;
@@ -597,15 +682,35 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
             c = __ldg(rec + 2);
         }
     };
-    if (AHEAD) fetch(range.x + t);
-    for (unsigned start = range.x; start < range.y; start += NT) {
-        bool all_done = true;
+    auto finished = [&](bool& all_done) { // every pixel of the thread, of the block
+        all_done = true;
 #pragma unroll
         for (int i = 0; i < PPT; i++) all_done = all_done && lim[i] == INF;
-        if (__syncthreads_count(!all_done) == 0) break;
+        return __syncthreads_count(!all_done) == 0;
+    };
+    bool all_done = false;
+    if constexpr (MODE == REST) { // the pixels as the first kernel left them
+        first = end;
+        end = range.y;
+#pragma unroll
+        for (int i = 0; i < PPT; i++) {
+            const float Ti = __uint_as_float(a.vals[range.x + (unsigned)(i * NT + t)]);
+            lim[i] = Ti < 0.0f ? INF : -INF;
+            (i & 1 ? T[i / 2].y : T[i / 2].x) = fabsf(Ti);
+            if (px < W && py + i < H) {
+                const size_t plane = (size_t)W * H, o = (size_t)(py + i) * W + px;
+                (i & 1 ? R[i / 2].y : R[i / 2].x) = a.out[o];
+                (i & 1 ? G[i / 2].y : G[i / 2].x) = a.out[plane + o];
+                (i & 1 ? B[i / 2].y : B[i / 2].x) = a.out[2 * plane + o];
+            }
+        }
+    }
+    if (AHEAD) fetch(first + t);
+    for (unsigned start = first; start < end; start += NT) {
+        if (finished(all_done)) break;
         const unsigned j = start + t;
         if (!AHEAD) fetch(j);
-        if (j < range.y) {
+        if (j < end) {
             const float mz = m.z - (float)y0;
             s_a[t] = make_float4(m.x - (float)x0, exact_skip_below(q.w), q.w, 0.0f);
             s_b[t] = make_float4(-mz, -mz, -m.w, -m.w);
@@ -616,7 +721,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
         }
         __syncthreads();
         if (AHEAD) fetch(j + NT);
-        const int cnt = min((unsigned)NT, range.y - start);
+        const int cnt = min((unsigned)NT, end - start);
         if (__all_sync(0xffffffffu, all_done)) continue;
 #pragma unroll 2
         for (int k = 0; k < cnt; k++) {
@@ -682,16 +787,47 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
             }
         }
     }
+    const bool rest = MODE == LIMITED && end < range.y && !finished(all_done);
+    if constexpr (MODE == LIMITED) {
+        if (rest) {
+            if (t == 0) {
+                a.rest_list[atomicAdd(a.rest_count, 1u)] = (unsigned)tile;
+                a.rest_flag[tile] = 1u;
+            }
+#pragma unroll
+            for (int i = 0; i < PPT; i++) {
+                const float Ti = i & 1 ? T[i / 2].y : T[i / 2].x;
+                a.vals_out[range.x + (unsigned)(i * NT + t)] = __float_as_uint(lim[i] == INF ? -Ti : Ti);
+            }
+        }
+    }
     const size_t plane = (size_t)W * H;
 #pragma unroll
     for (int i = 0; i < PPT; i++) {
         if (px < W && py + i < H) {
             const size_t o = (size_t)(py + i) * W + px;
             const float Ti = i & 1 ? T[i / 2].y : T[i / 2].x;
-            a.out[o] = fmaf(Ti, a.cam.bg[0], i & 1 ? R[i / 2].y : R[i / 2].x);
-            a.out[plane + o] = fmaf(Ti, a.cam.bg[1], i & 1 ? G[i / 2].y : G[i / 2].x);
-            a.out[2 * plane + o] = fmaf(Ti, a.cam.bg[2], i & 1 ? B[i / 2].y : B[i / 2].x);
+            const float r = i & 1 ? R[i / 2].y : R[i / 2].x, g = i & 1 ? G[i / 2].y : G[i / 2].x,
+                        b = i & 1 ? B[i / 2].y : B[i / 2].x;
+            a.out[o] = rest ? r : fmaf(Ti, a.cam.bg[0], r);
+            a.out[plane + o] = rest ? g : fmaf(Ti, a.cam.bg[1], g);
+            a.out[2 * plane + o] = rest ? b : fmaf(Ti, a.cam.bg[2], b);
         }
+    }
+}
+
+template <int PPT, int MODE>
+__global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
+{
+    grid_dependency_wait();
+    if constexpr (MODE == REST) {
+        const unsigned n = *a.rest_count;
+        for (unsigned b = blockIdx.x; b < n; b += gridDim.x) {
+            exact_tile<PPT, MODE>(a, (int)a.rest_list[b]);
+            __syncthreads(); // the staged records are written again
+        }
+    } else {
+        exact_tile<PPT, MODE>(a, (int)ordered_tile(a.order, blockIdx.x));
     }
 }
 
@@ -699,12 +835,19 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_exact(RasterArgs a)
 // are resident); below that a tile's own chain of pairs bounds the frame, and four warps per tile get
 // through it faster than two. Per pass, two / four pixels per thread: 672 tiles (499x333) 106 / 113 us,
 // 8,160 (1080p) 477 / 445 us, 32,400 (4K) 1988 / 1876 us.
-void launch_raster_exact(const RasterArgs& a, cudaStream_t s)
+void launch_raster_exact(const RasterArgs& a, const RunArgs* runs, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)(a.tiles_x * a.tiles_y);
     if (a.count) launch_dependent(k_raster_exact_count, dim3(tiles), dim3(E_THREADS), 0, s, a);
-    else if (tiles <= 16u * (unsigned)device_sm_count()) launch_dependent(k_raster_exact<2>, dim3(tiles), dim3(128), 0, s, a);
-    else launch_dependent(k_raster_exact<4>, dim3(tiles), dim3(64), 0, s, a);
+    else if (a.limit != RUN_ALL) { // only with many tiles
+        launch_dependent(k_raster_exact<4, LIMITED>, dim3(tiles), dim3(64), 0, s, a);
+        launch_runs_rest(*runs, s);
+        launch_dependent(k_raster_exact<4, REST>, dim3(rest_blocks(4)), dim3(64), 0, s, a);
+    } else if (tiles <= 16u * (unsigned)device_sm_count()) {
+        launch_dependent(k_raster_exact<2, WHOLE>, dim3(tiles), dim3(128), 0, s, a);
+    } else {
+        launch_dependent(k_raster_exact<4, WHOLE>, dim3(tiles), dim3(64), 0, s, a);
+    }
 }
 
 void launch_fast_exp_eval(const float* P, float* out, long long n, cudaStream_t s)

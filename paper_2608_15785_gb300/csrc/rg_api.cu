@@ -231,6 +231,13 @@ static TileOrder tile_order(const Workspace& w, int tiles)
     return o;
 }
 
+// Large frames write the first RUN_LIMIT entries of every tile and the others only for tiles whose pixels need them
+// (few: of 4K's 1,723 entries per tile, 3 M Gaussians, some 100 are read before the pixels are finished; 465 and 73 at
+// 8K, 1 M). Per frame, all entries / limited: 4K 3 M 1064 / 963 us (exact 1496 / 1396), 8K 1 M 1646 / 1567, 4K 1 M
+// 605 / 579, 4K 700 k 517 / 502, 4K 500 k 447 / 445, 2560 x 1440 2 M 548 / 513 and 500 k 290 / 284; two launches more
+// outweigh it below: 4K 100 k 260 / 265, 1080p 500 k 228 / 228 (exact 339 / 355).
+static constexpr int LIMIT_TILES = 12288, LIMIT_GAUSSIANS = 500000;
+
 // Arguments of runs.cu for a frame on workspace w: the runs live in the key buffers (list in
 // keys[0], the blocks' runs in keys[1]), the rest in runbuf. Returns the bytes of runbuf the frame
 // needs; the pointers are valid if runbuf has them.
@@ -246,6 +253,7 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     a.list = w.keys[0].as<uint2>();
     a.runs = w.keys[1].as<unsigned>();
     a.vals = w.vals[0].as<unsigned>();
+    a.limit = RUN_ALL;
     a.ranges = w.ranges.as<uint2>();
     a.ctr = w.ctrl.as<Counters>();
     a.order = tile_order(w, a.rows * a.cols);
@@ -264,6 +272,7 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
         a.tot = reinterpret_cast<unsigned long long*>(w.ctrl.as<unsigned char>() + RUN_TOT_AT);
     a.chunk = reinterpret_cast<RunChunk*>(part((size_t)a.chunk_cap * sizeof(RunChunk)));
     a.row = reinterpret_cast<RunRow*>(part((size_t)a.rows * sizeof(RunRow)));
+    a.row_limit = reinterpret_cast<unsigned*>(part((size_t)a.rows * 4));
     a.col = reinterpret_cast<unsigned*>(part((size_t)a.chunk_cap * run_pitch(a.cols) * 4));
     return at;
 }
@@ -298,7 +307,7 @@ rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameL
         for (int k = 0; k < 2; k++) RG_TRY(ensure(w.sort_status[k], (size_t)max_tiles * 256 * 4, "sort status"));
         w.cap = cap;
     }
-    RG_TRY(ensure(w.ranges, (size_t)F.tiles * (sizeof(uint2) + 8 * 4), "ranges and tile order"));
+    RG_TRY(ensure(w.ranges, (size_t)F.tiles * (sizeof(uint2) + (8 + 2) * 4), "ranges and tile order"));
     RG_TRY(ensure(w.ctrl, CTRL_ALLOC, "counters"));
     const int64_t fe_blocks = (n + frontend_block_threads() - 1) / frontend_block_threads();
     RG_TRY(ensure(w.lb_status, (size_t)(std::max<int64_t>(fe_blocks, (n + 2047) / 2048) + 1) * 8, "look-back status"));
@@ -502,6 +511,7 @@ void roofgs_raster_args(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_
     r.ranges = w.ranges.as<uint2>();
     r.vals = w.vals[fin].as<unsigned>();
     r.n = s->n;
+    r.limit = RUN_ALL;
     r.tiles_x = F.lay.tiles_x;
     r.tiles_y = F.lay.tiles_y;
     r.cam = F.cam;
@@ -518,6 +528,18 @@ void roofgs_raster_args(rg_scene* s, Workspace& w, const FrameLayout& F, uint32_
     r.ctr = w.ctrl.as<Counters>();
     r.fast_exp = (flags & RG_FLAG_EXACT_EXP) ? 0 : 1;
     r.ppt = (flags & RG_FLAG_SINGLE_PIXEL) ? 1 : ((flags & RG_FLAG_QUAD_PIXEL) ? 4 : 2);
+}
+
+// A frame of runs: the order of its tiles, and where their entries past the limit are found.
+static void raster_runs(const RunArgs& a, RasterArgs& r)
+{
+    r.order = a.order;
+    r.limit = a.limit;
+    r.row_limit = a.row_limit;
+    r.vals_out = a.vals;
+    r.rest_list = reinterpret_cast<unsigned*>(a.ranges + a.rows * a.cols) + 9 * a.rows * a.cols;
+    r.rest_count = &a.ctr->n_rest;
+    r.rest_flag = a.rest_flag;
 }
 
 // One frame on `st`; the caller has checked arguments and the workspace.
@@ -543,6 +565,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     w.last_key16 = false;
     w.last_tilesort = false;
     w.last_runs = false;
+    w.last_limited.limit = RUN_ALL;
     // a kernel launched like the others: a memset costs a full stream-ordered boundary on both sides (256 x 256
     // frames 61.8 -> 58.3 us); not in a graph, where a memset node overlaps other views' work
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -685,7 +708,13 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     if (ev && !runs && (sa.passes <= 0 || tile_sort)) RG_CK(cudaEventRecord(E[3], st));
     if (runs) {
         NvtxScope r_("rg sort");
+        if (!ra.tot && out && !count && F.tiles > LIMIT_TILES && n > LIMIT_GAUSSIANS) {
+            ra.limit = RUN_LIMIT;
+            ra.rec = mode == RG_MODE_EXACT ? w.erec.as<float4>() : w.rec.as<float4>();
+            ra.rest_flag = reinterpret_cast<unsigned*>(ra.ranges + F.tiles) + 8 * F.tiles;
+        }
         launch_runs(ra, st, ev ? E[3] : nullptr);
+        if (ra.limit != RUN_ALL) w.last_limited = ra;
     } else if (tile_sort) {
         NvtxScope r_("rg sort");
         launch_tile_counting_sort(tsa, st);
@@ -723,6 +752,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     r.ranges = w.ranges.as<uint2>();
     r.vals = w.vals[fin].as<unsigned>();
     r.n = n;
+    r.limit = RUN_ALL;
     r.tiles_x = F.lay.tiles_x;
     r.tiles_y = F.lay.tiles_y;
     r.cam = F.cam;
@@ -730,15 +760,15 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     r.count = count ? ctr : nullptr;
     if (mode == RG_MODE_EXACT) {
         r.erec = w.erec.as<float4>();
-        if (runs) r.order = ra.order;
+        if (runs) raster_runs(ra, r);
         NvtxScope r_("rg raster");
-        launch_raster_exact(r, st);
+        launch_raster_exact(r, &ra, st);
     } else {
         roofgs_raster_args(s, w, F, flags, out, r);
         r.count = count ? ctr : nullptr;
-        if (runs) r.order = ra.order;
+        if (runs) raster_runs(ra, r);
         NvtxScope r_("rg raster");
-        launch_raster_roofgs(r, st);
+        launch_raster_roofgs(r, &ra, st);
     }
     if (ev) RG_CK(cudaEventRecord(E[6], st));
     RG_CK(cudaGetLastError());
@@ -1235,6 +1265,15 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
         if (s->ws.last_runs && what != RG_INSPECT_RANGES) {
             std::vector<uint32_t> order(ng);
             val.resize(ne);
+            RunArgs& z = s->ws.last_limited;
+            if (ne && z.cap && z.limit != RUN_ALL) { // the frame left values out
+                if (z.list != s->ws.keys[0].p || z.vals != s->ws.vals[0].p || (void*)z.cnt != s->ws.runbuf.p ||
+                    (void*)z.ranges != s->ws.ranges.p || z.cap != s->ws.cap)
+                    return fail(RG_ERR_INVALID_ARG, "the workspace was resized after the frame");
+                launch_runs_all(z, 0);
+                RG_CK(cudaDeviceSynchronize());
+                z.limit = RUN_ALL;
+            }
             if (ne) RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
             if (ng) RG_CK(cudaMemcpy(order.data(), g.vals[s->ws.last_gfin], ng * 4, cudaMemcpyDeviceToHost));
             for (uint32_t& v : val) v = v < ng ? order[v] : 0u;

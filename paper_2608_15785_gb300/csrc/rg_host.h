@@ -95,6 +95,7 @@ struct Workspace {
     int last_tiles_x = 0;
     bool last_key16 = false; // entries carried 16-bit tile ids (the 32-bit keys are rebuilt on inspection)
     bool last_tilesort = false; // the entries were grouped by the per-tile counting sort (keys rebuilt from ranges)
+    RunArgs last_limited = {}; // runs of the last frame if its values were not all written; else limit = RUN_ALL or 0
     bool last_runs = false;  // the entries were written from tile-row runs: values are slots of the depth order
                              // in tile-id order, in vals[0]
     int last_bd = 0;         // b_d of the last RoofGS frame

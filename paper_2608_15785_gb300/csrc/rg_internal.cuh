@@ -76,7 +76,7 @@ struct Counters {
     unsigned n_front;
     unsigned n_row_runs;         // tile-row runs given a place in the rows' lists (runs.cu)
     unsigned n_chunks;           // chunks of runs
-    unsigned pad;
+    unsigned n_rest;             // tiles that a limited frame's rasterizer left to its second kernel
     alignas(16) unsigned tiles[8]; // tiles of each size class (TileOrder)
     unsigned long long n_runs;   // tile-row runs the front end's blocks asked room for
     unsigned long long n_pairs;  // rasterizer work counters (counting launches only)
@@ -536,6 +536,9 @@ __host__ __device__ __forceinline__ unsigned run_pack(unsigned slot, unsigned ta
 __host__ __device__ __forceinline__ unsigned run_slot(unsigned v) { return v & 255u; }
 __host__ __device__ __forceinline__ unsigned run_first(unsigned v) { return (v >> 8) & 0xfffu; }
 __host__ __device__ __forceinline__ unsigned run_last(unsigned v) { return v >> 20; }
+// RunArgs::limit: every entry is written; a large frame that is rasterized only writes the first ones of every tile
+constexpr unsigned RUN_ALL = 0xffffffffu, RUN_LIMIT = 512;
+static_assert(RUN_LIMIT >= 256, "an unfinished tile's pixels take the place of its first entries");
 // words per chunk of the column counts
 __host__ __device__ __forceinline__ int run_pitch(int cols) { return (cols + 31) / 32 * 32; }
 
@@ -609,6 +612,12 @@ struct RunArgs {
     RunRow* row;       // [rows]
     unsigned* col;     // [chunk_cap][run_pitch(cols)] entries per column, then their first slot in vals
     unsigned* vals;    // [cap] slots, by tile id, by slot
+    unsigned limit;    // RUN_ALL, or a limited frame: a tile's entries before this one are written first, the others if
+                       // the tile is flagged; row by row as row_limit says
+    unsigned* row_limit; // [rows] limit or RUN_ALL
+    const float4* rec; // the front end's records (FrontendArgs::rec, ExactArgs::rec)
+    unsigned* rest_flag; // [rows * cols] nonzero: the rasterizer needs more of the tile's entries (cleared with the ranges)
+    int rest;          // 1: the second launch
     uint2* ranges;     // [rows * cols] [start, end) of every tile, [0, 0) if empty
     TileOrder order;   // filled too if order.list is set
     Counters* ctr;
@@ -617,6 +626,9 @@ struct RunArgs {
 unsigned run_chunk_cap(unsigned run_cap, int rows, unsigned blocks);
 // groups the runs the front end left in a.runs by tile: fills vals and ranges
 void launch_runs(const RunArgs& a, cudaStream_t s, cudaEvent_t ev_after_collect);
+// after launch_runs with a limit: writes the other entries of the tiles flagged since (nothing without one); of every tile
+void launch_runs_rest(const RunArgs& a, cudaStream_t s);
+void launch_runs_all(const RunArgs& a, cudaStream_t s);
 // the front end of a frame of runs: projection, culling, colour, record per slot, runs per block
 void launch_frontend_runs(const FrontendArgs& a, const RunArgs& r, cudaStream_t s);
 
@@ -751,9 +763,17 @@ struct RasterArgs {
     int fast_exp;
     int ppt;              // pixels per thread: 1, 2 (Eq. (20)) or 4
     const float4* erec;   // exact (ExactArgs::rec)
+    // a frame of runs whose vals were not all written (RunArgs::limit); otherwise limit = RUN_ALL
+    unsigned limit;
+    const unsigned* row_limit;
+    unsigned* vals_out;   // vals
+    unsigned* rest_list;  // [tiles] tiles left unfinished, *rest_count of them
+    unsigned* rest_count;
+    unsigned* rest_flag;  // [tiles] RunArgs::rest_flag
     Counters* count;      // non-null: count evaluated / blended pairs (separate kernel variant)
 };
-void launch_raster_roofgs(const RasterArgs& a, cudaStream_t s);
+// runs: of a limited frame (RasterArgs::limit), else unused
+void launch_raster_roofgs(const RasterArgs& a, const RunArgs* runs, cudaStream_t s);
 
 struct RasterViews {
     RasterArgs views[MAX_BATCH_VIEWS];          // RoofGS tile-search arguments of each view
@@ -764,7 +784,7 @@ struct RasterViews {
 static_assert(sizeof(RasterViews) <= 32000, "the views' rasterizer arguments must fit the kernel parameters");
 // one persistent launch over the (view, tile) items of every view
 void launch_raster_views(const RasterViews& m, int fast_exp, int ppt, cudaStream_t s);
-void launch_raster_exact(const RasterArgs& a, cudaStream_t s);
+void launch_raster_exact(const RasterArgs& a, const RunArgs* runs, cudaStream_t s);
 void launch_fast_exp_eval(const float* P, float* out, long long n, cudaStream_t s);
 
 // Per-tile counting sort of 16-bit-tile-id entries (tilesort.cu): stable, one scatter.

@@ -353,6 +353,12 @@ __global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
                   !a.box_total && s_all > (unsigned long long)a.cap, 0, s_before & RUN_TOT_ENTRIES, S);
 }
 
+
+// A row of a limited frame is limited from this mean opacity of its entries. Per pass, limited / not, opacities drawn
+// around 0.5 (trained scenes) and scaled: 4K, 1 M Gaussians x 1 579 / 605 us, x 0.5 743 / 764, x 0.35 852 / 855, x 0.1
+// 1243 / 1123; 2560 x 1440, 2 M x 1 513 / 548, x 0.5 660 / 661, x 0.35 752 / 728 (exact mode alike)
+constexpr float LIMIT_OPACITY = 0.3f;
+
 // One block per tile row: OFF_SEGS segments of the row's chunks x OFF_COLS columns at a time.
 constexpr int OFF_SEGS = 4, OFF_COLS = 256;
 
@@ -392,6 +398,26 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
             }
         }
     }
+    // A limited frame pays where pixels are finished early, under opaque Gaussians: the mean opacity of the row's
+    // entries, from 256 runs spread over its list, decides
+    if (a.limit != RUN_ALL && warp == OFF_SEGS * OFF_COLS / 32 - 2) {
+        float sum = 0.0f, len = 0.0f;
+#pragma unroll
+        for (unsigned k = 0; k < 8; k++) {
+            if (r.runs == 0) break;
+            const uint2 q = __ldg(&a.list[r.base + (unsigned)((unsigned long long)r.runs * (32u * k + lane) / 256u)]);
+            const float o = a.box_total ? __ldg(&a.rec[3 * (size_t)q.x + 1].w) : __expf(__ldg(&a.rec[2 * (size_t)q.x + 1].y));
+            const float n = (float)((q.y >> 16) + 1u - (q.y & 0xffffu)); // (0 for a dropped run)
+            sum += o * n;
+            len += n;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            len += __shfl_xor_sync(0xffffffffu, len, o);
+        }
+        if (lane == 0) a.row_limit[row] = sum >= LIMIT_OPACITY * len ? a.limit : RUN_ALL;
+    }
     unsigned run = 0; // entries of the row's earlier columns
     for (int g = 0; g < a.cols; g += OFF_COLS) {
         const int col = g + (int)c;
@@ -424,6 +450,7 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
                 const unsigned b = first < a.cap ? first : (unsigned)a.cap;
                 const unsigned e = first + total < a.cap ? first + total : (unsigned)a.cap;
                 a.ranges[(size_t)row * a.cols + col] = e > b ? make_uint2(b, e) : make_uint2(0u, 0u);
+                if (a.rest_flag) a.rest_flag[(size_t)row * a.cols + col] = 0u;
             }
             if (a.order.list) add_tile(a.order, a.ctr->tiles, col < a.cols, row * (unsigned)a.cols + (unsigned)col, total);
         }
@@ -453,7 +480,9 @@ struct ExpandSmem {
     unsigned first[RUN_MAX_GRID]; // first slot in vals of the chunk's entries of each column
     unsigned w[RUN_WARPS];
     unsigned start;
+    unsigned need[3][2]; // bit b: columns 8 b .. 8 b + 7 have an entry to be written; of three chunks in turn
 };
+static_assert(RUN_MAX_GRID <= 64 * 8 && COLS % 8 == 0, "a bit for every eight columns, a window of whole bits");
 static_assert(sizeof(ExpandSmem) <= 48 * 1024, "no opt-in to more shared memory");
 
 // k_run_offsets for the chunk of one block of a small frame: the first slot of each of its columns
@@ -520,13 +549,18 @@ __device__ __forceinline__ void put_first(unsigned& m, unsigned* vals, unsigned&
     d++;
 }
 
-// Grid as the collect kernel's.
+constexpr unsigned NONE = 0xffffffffu;
+
+// Grid as the collect kernel's. In a limited frame (RunArgs::limit) a chunk's columns of which no entry is to be written
+// are left out, with their masks where eight of them lie together at the edge of a window: 4K, 3 M Gaussians (83 % of the
+// entries lie past their tile's first 512) 286 -> 175 us, 8K, 1 M 321 -> 232 us.
 template <bool SMALL>
 __global__ void __launch_bounds__(RUN_THREADS, 5) k_run_expand(RunArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ExpandSmem& S = *reinterpret_cast<ExpandSmem*>(smem_raw);
     grid_dependency_wait();
+    if (!SMALL && a.rest && a.ctr->n_rest == 0u) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned row = blockIdx.y;
     const RunRow r = a.row[row];
@@ -535,14 +569,41 @@ __global__ void __launch_bounds__(RUN_THREADS, 5) k_run_expand(RunArgs a)
     const int pitch = run_pitch(a.cols);
     const unsigned cap = (unsigned)a.cap;
     const bool over = a.ctr->n_entries_total > (unsigned long long)a.cap;
-    // groups of an even number of columns
-    const int groups = (a.cols + COLS - 1) / COLS, group = ((a.cols + groups - 1) / groups + 1) & ~1;
+    const unsigned limit = a.limit == RUN_ALL ? RUN_ALL : a.row_limit[row];
+    int turn = 0;
+    if (!SMALL) {
+        if (tid < 6) S.need[tid / 2][tid & 1] = 0u;
+        __syncthreads();
+    }
     for (unsigned c = blockIdx.x; c < r.nchunks; c += gridDim.x) {
         RunChunk k;
         unsigned bend, rend;
         chunk_bounds(a, r, c, k, bend, rend);
         const unsigned n = rend - k.run; // at most CHUNK_RUNS
         if (n == 0) continue;
+        unsigned long long need = ~0ull >> (64 - (a.cols + 7) / 8);
+        if (!SMALL) { // NONE: no entry of the chunk is to be written, being past the tile's first `limit` ones (or, at rest, not)
+            for (int j0 = 0; j0 < a.cols; j0 += RUN_THREADS) {
+                const int j = j0 + tid;
+                bool write = false;
+                if (j < a.cols) {
+                    const unsigned f = __ldg(&a.col[(size_t)(r.chunk + c) * pitch + j]);
+                    const uint2 tile = __ldg(&a.ranges[(size_t)row * a.cols + j]);
+                    write = f < tile.y && (a.rest ? f - tile.x >= limit && a.rest_flag[row * a.cols + j] : f - tile.x < limit);
+                    S.first[j] = write ? f : NONE;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, write);
+                if (lane == 0 && m)
+                    atomicOr(&S.need[turn][j0 / RUN_THREADS], ((m & 0xffu ? 1u : 0u) | (m & 0xff00u ? 2u : 0u) |
+                             (m & 0xff0000u ? 4u : 0u) | (m & 0xff000000u ? 8u : 0u)) << (4 * warp));
+            }
+            __syncthreads();
+            need = S.need[turn][0] | ((unsigned long long)S.need[turn][1] << 32);
+            // the words of the turn after the next: read by nobody since the barrier, and zero before the next one
+            turn = turn == 2 ? 0 : turn + 1;
+            if (tid < 2) S.need[turn == 2 ? 0 : turn + 1][tid] = 0u;
+        }
+        if (!need) continue;
         const uint2* const list = a.list + r.base + k.run;
         unsigned ends[CHUNK_RUNS / RUN_THREADS]; // the thread's runs: first and last column
 #pragma unroll
@@ -552,10 +613,11 @@ __global__ void __launch_bounds__(RUN_THREADS, 5) k_run_expand(RunArgs a)
             if (j < n) S.id[j] = q.x;
             ends[u] = q.y;
         }
-        if (!SMALL)
-            for (int j = tid; j < a.cols; j += RUN_THREADS) S.first[j] = __ldg(&a.col[(size_t)(r.chunk + c) * pitch + j]);
-        for (int g = 0; g < a.cols; g += group) {
-            const int cols = a.cols - g < group ? a.cols - g : group;
+        while (need) { // a window of columns
+            const int g = 8 * (__ffsll((long long)need) - 1);
+            const unsigned long long in = (need >> (g / 8)) & ((1ull << (COLS / 8)) - 1ull);
+            const int width = 8 * (64 - __clzll((long long)in)), cols = a.cols - g < width ? a.cols - g : width;
+            need &= ~(in << (g / 8));
             for (int j = tid; j < cols * PITCH / 2; j += RUN_THREADS)
                 reinterpret_cast<uint2*>(&S.mask[0][0])[j] = make_uint2(0u, 0u);
             __syncthreads();
@@ -590,10 +652,14 @@ __global__ void __launch_bounds__(RUN_THREADS, 5) k_run_expand(RunArgs a)
             // a warp takes two columns at a time (one scan of 16-bit counts, two chains of stores)
             for (int q = 2 * warp; q < cols; q += 2 * RUN_WARPS) {
                 const bool two = q + 1 < cols;
+                const bool use0 = SMALL || S.first[g + q] != NONE, use1 = SMALL || (two && S.first[g + q + 1] != NONE);
+                if (!use0 && !use1) continue;
                 const uint2 b = *reinterpret_cast<const uint2*>(&S.seg[q / SEG_COLS][2 * lane]);
                 const uint2 m0 = *reinterpret_cast<const uint2*>(&S.mask[q][2 * lane]);
                 const uint2 m1 = two ? *reinterpret_cast<const uint2*>(&S.mask[q + 1][2 * lane]) : b;
                 unsigned lo0 = m0.x ^ b.x, hi0 = m0.y ^ b.y, lo1 = m1.x ^ b.x, hi1 = m1.y ^ b.y;
+                if (!use0) lo0 = hi0 = 0u; // nothing is written
+                if (!use1) lo1 = hi1 = 0u;
                 const unsigned n0 = (unsigned)__popc(lo0), n1 = (unsigned)__popc(lo1);
                 const unsigned cnt = (n0 + (unsigned)__popc(hi0)) + ((n1 + (unsigned)__popc(hi1)) << 16);
                 const unsigned excl = run_warp_scan(cnt) - cnt;
@@ -628,6 +694,29 @@ __global__ void __launch_bounds__(RUN_THREADS, 5) k_run_expand(RunArgs a)
     }
 }
 
+// at most the chunks a row can have, and about 4 waves of blocks over all rows (2 / 8 waves: 1080p 53 / 57 us
+// of collection and expansion, 4K 407 / 375; 4: 53 and 379)
+static dim3 run_grid(const RunArgs& a, int waves = 4)
+{
+    const unsigned most = a.blocks * (unsigned)RUN_SLOTS / CHUNK_STEP + a.blocks / CHUNK_BLOCKS + 1;
+    const unsigned want = (unsigned)(waves * 5 * device_sm_count() / a.rows + 1);
+    return dim3(most < want ? most : want, (unsigned)a.rows);
+}
+
+void launch_runs_rest(const RunArgs& limited, cudaStream_t s)
+{
+    RunArgs a = limited;
+    a.rest = 1;
+    launch_dependent(k_run_expand<false>, run_grid(a, 1), dim3(RUN_THREADS), sizeof(ExpandSmem), s, a);
+}
+
+void launch_runs_all(const RunArgs& limited, cudaStream_t s)
+{
+    RunArgs a = limited;
+    a.limit = RUN_ALL;
+    launch_dependent(k_run_expand<false>, run_grid(a), dim3(RUN_THREADS), sizeof(ExpandSmem), s, a);
+}
+
 void launch_runs(const RunArgs& a, cudaStream_t s, cudaEvent_t ev_after_collect)
 {
     if (a.blocks == 0) return;
@@ -639,11 +728,7 @@ void launch_runs(const RunArgs& a, cudaStream_t s, cudaEvent_t ev_after_collect)
         launch_dependent(k_run_expand<true>, grid, block, sizeof(ExpandSmem), s, a);
         return;
     }
-    // at most the chunks a row can have, and about 4 waves of blocks over all rows (2 / 8 waves: 1080p 53 / 57 us
-    // of collection and expansion, 4K 407 / 375; 4: 53 and 379)
-    const unsigned most = a.blocks * (unsigned)RUN_SLOTS / CHUNK_STEP + a.blocks / CHUNK_BLOCKS + 1;
-    const unsigned want = (unsigned)(4 * 5 * device_sm_count() / a.rows + 1);
-    const dim3 grid(most < want ? most : want, (unsigned)a.rows);
+    const dim3 grid = run_grid(a);
     launch_dependent(k_run_rows, dim3((unsigned)a.rows), dim3(1024), 0, s, a);
     launch_dependent(k_run_collect, grid, block, 0, s, a);
     if (ev_after_collect) cudaEventRecord(ev_after_collect, s);

@@ -148,3 +148,43 @@ def test_depth_orders(n):
     k, v, _, _ = oracle.keys(sc, cam, oracle.EXACT)
     assert np.array_equal(gs.inspect(binding.RG_INSPECT_KEYS).view(np.uint64), k)
     assert np.array_equal(gs.inspect(binding.RG_INSPECT_VALUES), v)
+
+
+# 12,288 tiles and 500,000 Gaussians, the largest frames whose entries are all written, and above them limited ones (the
+# first 512 entries of every tile; the last one is too faint for it). Specks: tiles with more than 1,024 entries whose
+# pixels are not all finished after 512
+LIMIT_CASES = [(500_001, (2048, 1536), (16, 16), 0.4), (500_000, (2048, 1537), (16, 16), 0.4),
+               (500_001, (2048, 1537), (16, 16), 0.4), (500_001, (1999, 1777), (32, 8), 0.4),
+               (500_001, (1777, 1999), (8, 32), 0.4), (500_001, (2048, 1537), (16, 16), 0.01)]
+
+
+@pytest.mark.parametrize("n,wh,tile,opacity", LIMIT_CASES)
+def test_limited_frames_render_every_entry(n, wh, tile, opacity):
+    """Tiles read past the entries written for them are resumed by a second launch: the images equal, bit by bit,
+    those of the ordered front end and of the counting launch, and so do the entries that an inspection sees."""
+    sc = _scene(n, 0.15, seed=5)
+    rng = np.random.default_rng(2)
+    sc.opacities = (opacity * rng.uniform(0.9, 1.1, n)).astype(np.float32)
+    sc.means[n // 4:] *= np.float32(0.25)  # most of them in the middle
+    cam = synth.tiny_camera(*wh, bg=(0.2, 0.1, 0.3))
+    gs = binding.Scene(sc)
+    for mode in ("roofgs", "exact"):
+        gs.render(cam, mode=mode, tile=tile, stats=True)  # sizes the workspace
+    for flags in (0, binding.RG_FLAG_QUAD_PIXEL, binding.RG_FLAG_SINGLE_PIXEL | binding.RG_FLAG_EXACT_EXP,
+                  binding.RG_FLAG_QUAD_PIXEL | binding.RG_FLAG_EXACT_EXP):
+        a = gs.render(cam, flags=flags, tile=tile)
+        ea = _entries(gs)
+        assert torch.equal(a, gs.render(cam, flags=flags, tile=tile))  # nothing of the inspection is left
+        b = gs.render(cam, flags=flags | binding.RG_FLAG_ORDERED_FRONT_END, tile=tile)
+        eb = _entries(gs)
+        for x, y in zip(ea, eb):
+            assert np.array_equal(x, y)
+        assert torch.equal(a, b)
+    r = ea[2].view(np.uint32).reshape(-1, 2).astype(np.int64)
+    assert (r[:, 1] - r[:, 0]).max() > 1_024
+    a = gs.render(cam, mode="exact", tile=tile)
+    b, _ = gs.render(cam, mode="exact", tile=tile, stats=True)
+    b = b.clone()
+    assert torch.equal(a, gs.render(cam, mode="exact", tile=tile))
+    assert torch.equal(a, b)
+    gs.check()
