@@ -43,11 +43,10 @@ REASONS = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_powe
 # clock. Warp instructions per evaluated (Gaussian, pixel) pair of the timed kernel
 # (k_raster_roofgs<fast exp, 4 pixels per thread>: pixel pairs blended with packed FP32x2
 # FMAs, skip thresholds, one skip and one stop branch per thread and Gaussian, two records
-# per loop iteration), from ncu on the 1M-Gaussian 4K case: sm__inst_issued.sum 388.1 M for
-# 615.1 M evaluated pairs (per pair: FMA pipe 0.302, ALU pipe 0.188, LSU 0.033, XU 0.001,
-# the rest branches and uniform datapath). The pair count of the timed frames comes from the
-# counting variant of the same kernel.
-RASTER_WARP_INST_PER_PAIR = 388.1 / 615.1
+# per loop iteration), from ncu on a 1M-Gaussian 4K frame: smsp__inst_executed.sum 334.3 M for
+# 534.0 M evaluated pairs. The pair count of the timed frames comes from the counting variant
+# of the same kernel.
+RASTER_WARP_INST_PER_PAIR = 334.3 / 534.0
 # Source-level FP32/ALU-pipe instruction counts of the rasterizers' inner loops (per
 # evaluated exponent, per pair inside the alpha >= 1/255 range), kept as a second,
 # model-based view: RoofGS 4 + 1 range test, blend 11; exact 10, blend 20.
@@ -83,7 +82,7 @@ def parse():
                    help="skip the per-pose median frame times (100 frames per pose in RoofGS mode)")
     p.add_argument("--ordered-front-end", action="store_true",
                    help="RoofGS: the fused front end with the ordered allocation and two tile-bit passes "
-                        "instead of the row-bucketed front end")
+                        "instead of tile-row runs")
     return p.parse_args()
 
 
@@ -157,9 +156,40 @@ class ClockSampler:
 # ---------------------------------------------------------------------------
 # algorithmic work per stage (bytes for the HBM-bound stages, ops for raster)
 # ---------------------------------------------------------------------------
+def runs_frame(st, ordered):
+    """Whether a frame's entries came from tile-row runs (no sort of the entries): the default up to
+    512 x 512 tiles."""
+    return not ordered and st["tiles_x"] <= 512 and st["tiles_y"] <= 512
+
+
+def run_launches(st, ordered, mode="roofgs"):
+    """Kernels of a frame of runs: clear, depth keys, depth passes, front end, grouping (rows, collect,
+    offsets, expand; collect and expand up to 32,768 Gaussians), rasterizer, and in a limited frame (more
+    than 500,000 Gaussians and 12,288 tiles) the two launches for unfinished tiles. Otherwise None."""
+    if not runs_frame(st, ordered):
+        return None
+    n, tiles = st["n_gaussians"], st["tiles_x"] * st["tiles_y"]
+    depth = 1 + (4 if mode == "exact" else (int(st["b_d"]) + 7) // 8)
+    return 1 + depth + 1 + (2 if n <= 32768 else 4) + 1 + (2 if n > 500000 and tiles > 12288 else 0)
+
+
+def run_work(st):
+    """Bytes that the stages of a RoofGS frame of runs cannot do without. Depth order: 16 B mean + log o
+    read, 8 B (code, index) written per Gaussian, 16 B per depth pass. Front end: 4 B order + 16 B mean +
+    log o per Gaussian, 16 B geometry if in front, 48 B INT8 SH + 32 B record if visible. Expansion: a 4 B
+    value per entry, at most 512 a tile where the frame is limited (the runs themselves, a fifth of the
+    entries, are not counted)."""
+    N, nf, nv, nd = st["n_gaussians"], st["n_front"], st["n_visible"], st["n_entries"]
+    tiles = st["tiles_x"] * st["tiles_y"]
+    gpasses = (st["b_d"] + 7) // 8
+    limited = N > 500000 and tiles > 12288
+    return {"depth": 24 * N + 16 * gpasses * N, "front": 20 * N + 16 * nf + 80 * nv,
+            "expand": 4 * (min(nd, 512 * tiles) if limited else nd)}
+
+
 def row_buckets(st, ordered):
-    """Whether a RoofGS frame with an image ran the row-bucketed front end: the default with the
-    depth pre-sort, 16-bit tile ids and at most 256 x 256 tiles."""
+    """Whether a grid has at most 256 x 256 tiles and 16 tile bits: one pass over the tile column is what
+    rg_stats reports for its frames."""
     return not ordered and st["b_t"] <= 16 and st["tiles_x"] <= 256 and st["tiles_y"] <= 256
 
 
@@ -434,13 +464,13 @@ def run_ours(a, rank, world, local_rank):
             cfg["exact_per_pose"] = ex["per_pose"]
     line["config"] = cfg
     line["roofline"], line["stages"] = rooflines(r, a, props, clocks)
-    # per frame: depth keys (which also clear the depth sort's look-back status), depth-sort
-    # passes, the front end (row-bucketed: count, row scan, scatter; else the fused kernel),
-    # entry histogram + tile-bit passes, rasterizer (which finds the tile ranges itself)
+    # per frame: run_launches; without runs: clear, depth keys (which also clear the depth sort's
+    # look-back status), depth-sort passes, the fused front end, entry histogram + tile-bit passes,
+    # rasterizer (which finds the tile ranges itself)
     gp = (int(r["stats"]["b_d"]) + 7) // 8
-    fe = 3 if row_buckets(r["stats"], a.ordered_front_end) else 1
-    cfg["front_end"] = "row-bucketed (count, row scan, scatter)" if fe == 3 else "fused, ordered allocation"
-    line["gpu_launches"] = r["steps"] * (1 + gp + fe + 1 + int(r["stats"]["sort_passes"]) + 1)
+    launches = run_launches(r["stats"], a.ordered_front_end)
+    cfg["front_end"] = "tile-row runs" if launches else "fused, ordered allocation"
+    line["gpu_launches"] = r["steps"] * (launches or (2 + gp + 1 + 1 + int(r["stats"]["sort_passes"]) + 1))
     line["e2e"] = {"value": round(job_fps(e2e_steps, world, e2e_ms), 2), "unit": UNIT,
                    "h2d_bytes_per_step": 100,  # the rg_camera struct, passed by value per call
                    "d2h_bytes_per_step": 3 * a.width * a.height * 4,
@@ -529,8 +559,8 @@ def run_batch(a, sc3, gs3, dev):
 
 def run_tile_sort(a, gs, cams, dev, rflags):
     """The ways of grouping the entries by tile, on this workload and on the 1080p one (500k
-    Gaussians, pose 0): frame rate and stage times of the row-bucketed front end with its one
-    column pass (the default), the fused front end with two tile-bit radix passes
+    Gaussians, pose 0): frame rate and stage times of the tile-row runs (the default), the fused
+    front end with two tile-bit radix passes
     (RG_FLAG_ORDERED_FRONT_END) and the fused front end with the per-tile counting sort
     (RG_FLAG_TILE_COUNTING_SORT)."""
     import torch
@@ -545,7 +575,7 @@ def run_tile_sort(a, gs, cams, dev, rflags):
         img = torch.empty((3, cs[0].height, cs[0].width), device=dev)
         row = {}
         rf = rflags & ~binding.RG_FLAG_ORDERED_FRONT_END
-        for name, fl in (("row_buckets", 0), ("ordered_radix", binding.RG_FLAG_ORDERED_FRONT_END),
+        for name, fl in (("runs", 0), ("ordered_radix", binding.RG_FLAG_ORDERED_FRONT_END),
                          ("counting", binding.RG_FLAG_TILE_COUNTING_SORT)):
             for c in cs:
                 scene.render(c, mode="roofgs", flags=rf | fl, out=img, stats=True)
@@ -567,7 +597,7 @@ def run_tile_sort(a, gs, cams, dev, rflags):
                          "front_end_ms": round(per[1], 4)}
         row["counting_sort_speedup_vs_radix"] = round(row["ordered_radix"]["sort_ms"] /
                                                       max(row["counting"]["sort_ms"], 1e-9), 3)
-        row["row_buckets_frame_speedup"] = round(row["row_buckets"]["fps"] / max(row["ordered_radix"]["fps"], 1e-9), 3)
+        row["runs_frame_speedup"] = round(row["runs"]["fps"] / max(row["ordered_radix"]["fps"], 1e-9), 3)
         out[label] = row
         scene.check()
     g2.close()
@@ -758,8 +788,10 @@ def rooflines(r, a, props, clocks):
     hbm, src = measured_peaks()
     W, H = a.width, a.height
     st = r["stats"]
-    rows = row_buckets(st, a.ordered_front_end)
-    work = stage_work("roofgs", st, W, H, rows)
+    runs = runs_frame(st, a.ordered_front_end)
+    work = stage_work("roofgs", st, W, H)
+    if runs:
+        work.update(run_work(st))
     sms = props.multi_processor_count
     mhz = (clocks or {}).get("sm_mhz") or 2070.0
     issue_peak = sms * 4 * mhz * 1e6 / 1e9  # warp instructions per second (G/s): 4 schedulers per SM
@@ -774,8 +806,10 @@ def rooflines(r, a, props, clocks):
     stages = {
         "depth_order": hbm_stage(work["depth"], ms["depth_order"]),
         "front_end": hbm_stage(work["front"], ms["front_end"]),
-        "sort_hist": hbm_stage(work["hist"], ms["sort_hist"]),
-        "sort_pass": hbm_stage(work["sort_pass"], ms["sort_passes"] / passes),
+        "sort_hist": None if runs else hbm_stage(work["hist"], ms["sort_hist"]),
+        "sort_pass": None if runs else hbm_stage(work["sort_pass"], ms["sort_passes"] / passes),
+        # rows and collection of the runs lie between the front end and the expansion: issue- and latency-bound
+        "run_expand": hbm_stage(work["expand"], ms["sort_passes"]) if runs else None,
         "ranges": hbm_stage(work["ranges"], ms["ranges"]) if work["ranges"] else None,
         "raster": {"bound": "alu", "achieved": RASTER_WARP_INST_PER_PAIR * st["n_pairs"] / (ms["raster"] * 1e-3) / 1e9,
                    "peak": issue_peak, "unit": "G warp instructions/s", "ms": ms["raster"],
@@ -784,10 +818,12 @@ def rooflines(r, a, props, clocks):
                                        "peak": round(alu_peak, 1), "unit": "Gop/s",
                                        "frac": round(work["raster_ops"] / (ms["raster"] * 1e-3) / 1e9 / alu_peak, 4)}},
     }
-    stages["sort_pass"]["launches_per_frame"] = work["passes"]
     stages["depth_order"]["kernels"] = 1 + (st["b_d"] + 7) // 8
-    stages["front_end"]["kernels"] = 3 if rows else 1
     stages = {k: v for k, v in stages.items() if v is not None}
+    if runs:
+        stages["run_expand"]["kernels"] = 2 if st["n_gaussians"] > 32768 else 1
+    else:
+        stages["sort_pass"]["launches_per_frame"] = work["passes"]
     for v in stages.values():
         v["frac"] = round(v["achieved"] / v["peak"], 4)
         v["achieved"] = round(v["achieved"], 1)
@@ -802,8 +838,8 @@ def rooflines(r, a, props, clocks):
         traffic = round(SORT_PASS_TRAFFIC_PER_ENTRY * st["n_entries"])
     names = {"sort_pass": "k_onesweep<uint16 tile id> (one tile-bit pass)",
              "raster": "k_raster_roofgs<fast exp, %d pixels per thread>" % a.ppt,
-             "front_end": "k_frontend_count + k_row_scan + k_frontend_scatter" if rows else "k_frontend_fused",
-             "depth_order": "k_depth_keys + per-Gaussian sort",
+             "front_end": "k_frontend_runs" if runs else "k_frontend_fused",
+             "run_expand": "k_run_offsets + k_run_expand", "depth_order": "k_depth_keys + per-Gaussian sort",
              "sort_hist": "k_sort_hist<uint32>", "ranges": "k_ranges<uint32>"}
     roof = {"kernel": names[dom], "bound": d["bound"], "achieved": d["achieved"], "peak": d["peak"],
             "unit": d["unit"], "frac": d["frac"], "traffic": traffic,

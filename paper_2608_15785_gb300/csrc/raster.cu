@@ -416,7 +416,7 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
             }
         }
     }
-    const bool rest = MODE == LIMITED && end < range.y && !finished(all_done);
+    const bool rest = MODE == LIMITED && end < a.ranges[tile].y && !finished(all_done); // (loaded again: no register meanwhile)
     if constexpr (MODE == LIMITED) {
         if (rest) {
             if (t == 0) {
@@ -426,7 +426,7 @@ __device__ __forceinline__ void raster_tile(const RasterArgs& a, const int tile)
 #pragma unroll
             for (int i = 0; i < PPT; i++) {
                 const float Ti = (i & 1) ? T2[i >> 1].y : T2[i >> 1].x;
-                a.vals_out[range.x + (unsigned)(i * NT + t)] =
+                a.vals_out[a.ranges[tile].x + (unsigned)(i * NT + t)] =
                     __float_as_uint(thr[i] == __int_as_float(0x7f800000) ? -Ti : Ti);
             }
         }
@@ -787,7 +787,7 @@ __device__ __forceinline__ void exact_tile(const RasterArgs& a, const int tile)
             }
         }
     }
-    const bool rest = MODE == LIMITED && end < range.y && !finished(all_done);
+    const bool rest = MODE == LIMITED && end < a.ranges[tile].y && !finished(all_done); // (loaded again: no register meanwhile)
     if constexpr (MODE == LIMITED) {
         if (rest) {
             if (t == 0) {
@@ -797,7 +797,7 @@ __device__ __forceinline__ void exact_tile(const RasterArgs& a, const int tile)
 #pragma unroll
             for (int i = 0; i < PPT; i++) {
                 const float Ti = i & 1 ? T[i / 2].y : T[i / 2].x;
-                a.vals_out[range.x + (unsigned)(i * NT + t)] = __float_as_uint(lim[i] == INF ? -Ti : Ti);
+                a.vals_out[a.ranges[tile].x + (unsigned)(i * NT + t)] = __float_as_uint(lim[i] == INF ? -Ti : Ti);
             }
         }
     }
