@@ -931,6 +931,14 @@ rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries)
     const int64_t max_tiles = (cap + sort_tile_items() - 1) / sort_tile_items();
     for (int k = 0; k < 2; k++) RG_TRY(ensure(scene->ws.sort_status[k], (size_t)max_tiles * 256 * 4, "sort status"));
     scene->ws.cap = cap;
+    if (scene->ws.last_tiles_x > 0) { // the last frame's grid can be captured next, without an allocation
+        Layout L;
+        memset(&L, 0, sizeof(L));
+        L.tiles_x = scene->ws.last_tiles_x;
+        L.tiles_y = scene->ws.last_tiles / scene->ws.last_tiles_x;
+        RunArgs ra;
+        if (runs_possible(L, scene->n)) RG_TRY(ensure(scene->ws.runbuf, run_views(scene->ws, scene->n, L, ra), "tile-row runs"));
+    }
     return RG_OK;
 }
 

@@ -84,3 +84,22 @@ def test_invalid_attributes_are_refused(storage, field, at, value, text):
     with pytest.raises(binding.RgError, match=text) as e:
         binding.Scene(sc, storage=storage)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("n,mode", [(5_000, "roofgs"), (40_000, "roofgs"), (40_000, "exact")])
+def test_a_reserved_workspace_can_be_captured(n, mode):
+    """After a frame and a larger reserve the same view is captured into a graph without an allocation."""
+    cam = synth.tiny_camera(320, 240)
+    gs = binding.Scene(synth.tiny_scene(n, seed=4))
+    want = gs.render(cam, mode=mode).clone()
+    gs.reserve(6_000_000)
+    out = torch.empty_like(want)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        gs.render(cam, mode=mode, out=out)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    gs.check()
