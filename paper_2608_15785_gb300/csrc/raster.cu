@@ -6,9 +6,9 @@
 // pairs with alpha < 1/255 are skipped, the loop stops (without adding) once
 // the transmittance would fall below 1e-4, C += c alpha T, out = C + T bg.
 //
-// RoofGS mode (Sec. IV-B): the block first finds its tile's [start, end) in
-// the sorted keys (warp-cooperative search). While a batch of records is
-// staged in shared memory, each Gaussian's coefficients are folded (Eqs.
+// RoofGS mode (Sec. IV-B): the tile's [start, end) comes with the entries of a frame of
+// runs (runs.cu); with sorted entries the block finds it in the sorted keys (warp-cooperative
+// search). While a batch of records is staged in shared memory, each Gaussian's coefficients are folded (Eqs.
 // (13)-(15)) -- -1/2 and log o absorbed, C1..C6 -- in TILE-LOCAL coordinates
 // (pixel and mean shifted by the tile origin, so the FP32 terms stay small at
 // 4K); every thread owns PPT vertically adjacent pixels (x, y) ... (x,
