@@ -536,7 +536,9 @@ __host__ __device__ __forceinline__ unsigned run_pack(unsigned slot, unsigned ta
 __host__ __device__ __forceinline__ unsigned run_slot(unsigned v) { return v & 255u; }
 __host__ __device__ __forceinline__ unsigned run_first(unsigned v) { return (v >> 8) & 0xfffu; }
 __host__ __device__ __forceinline__ unsigned run_last(unsigned v) { return v >> 20; }
-// RunArgs::limit: every entry is written; a large frame that is rasterized only writes the first ones of every tile
+// RunArgs::limit: every entry is written; a large frame that is rasterized only writes the first ones of every tile.
+// 512: at 4K with 3 M Gaussians the expansion takes 197 us with 1,024, 189 with 768, 180 with 512, 167 with 256, and
+// next to no tile is read past 512, in either mode (with 256 the exact frames' tiles often are)
 constexpr unsigned RUN_ALL = 0xffffffffu, RUN_LIMIT = 512;
 static_assert(RUN_LIMIT >= 256, "an unfinished tile's pixels take the place of its first entries");
 // words per chunk of the column counts

@@ -180,6 +180,16 @@ def test_limited_frames_render_every_entry(n, wh, tile, opacity):
         for x, y in zip(ea, eb):
             assert np.array_equal(x, y)
         assert torch.equal(a, b)
+    out = torch.empty_like(a)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        gs.render(cam, flags=flags, tile=tile, out=out)
+    for _ in range(2):
+        out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(a, out)
     r = ea[2].view(np.uint32).reshape(-1, 2).astype(np.int64)
     assert (r[:, 1] - r[:, 0]).max() > 1_024
     a = gs.render(cam, mode="exact", tile=tile)
