@@ -484,7 +484,9 @@ __device__ __forceinline__ unsigned emit_runs(const RunArgs& r, const unsigned v
 {
     extern __shared__ __align__(16) unsigned char run_smem[];
     RunRowSmem* const R = reinterpret_cast<RunRowSmem*>(run_smem);
-    __shared__ unsigned s_cache[FE_WARPS][RUN_CACHE]; // owner | ty << 5 | first << 14 | last << 23; ~0: no tiles
+    __shared__ unsigned s_cache[FE_WARPS][RUN_CACHE]; // owner | ty << 5 | first << 14 | last << 23
+    constexpr unsigned NO_TILES = 1u << 14; // first 1, last 0: no run has it (every one of the 32 bits is used: a run of
+                                            // lane 31 in the last tile of a 512 x 512 grid is ~0)
     __shared__ unsigned s_w[FE_WARPS];
     __shared__ unsigned s_base;
     static_assert(RUN_MAX_GRID <= 512, "nine bits for a tile row or column");
@@ -504,13 +506,13 @@ __device__ __forceinline__ unsigned emit_runs(const RunArgs& r, const unsigned v
         int ty, txa, txb;
         if (k < wrows && range(warp * 32 + owner, (int)rl, ty, txa, txb))
             return (unsigned)owner | ((unsigned)ty << 5) | ((unsigned)txa << 14) | ((unsigned)txb << 23);
-        return 0xffffffffu;
+        return NO_TILES;
     };
     unsigned vis = 0;
     for (unsigned r0 = 0; r0 < wrows; r0 += 32) {
         const unsigned v = tiles_of(r0 + (unsigned)lane);
         if (r0 + 32 <= RUN_CACHE) s_cache[warp][r0 + lane] = v;
-        if (v != 0xffffffffu) {
+        if (v != NO_TILES) {
             const unsigned owner = v & 31u, ty = (v >> 5) & 511u;
             atomicOr(&R[ty].mask[warp], 1u << owner);
             atomicAdd(&R[ty].ents, (v >> 23) - ((v >> 14) & 511u) + 1u);
@@ -564,7 +566,7 @@ __device__ __forceinline__ unsigned emit_runs(const RunArgs& r, const unsigned v
     if (ok) {
         for (unsigned r0 = 0; r0 < wrows; r0 += 32) {
             const unsigned v = r0 + 32 <= RUN_CACHE ? s_cache[warp][r0 + lane] : tiles_of(r0 + (unsigned)lane);
-            if (v == 0xffffffffu) continue;
+            if (v == NO_TILES) continue;
             const unsigned owner = v & 31u;
             const RunRowSmem& q = R[(v >> 5) & 511u];
             const unsigned pos = q.first + q.before[warp] + (unsigned)__popc(q.mask[warp] & ((1u << owner) - 1u));

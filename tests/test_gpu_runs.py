@@ -198,3 +198,47 @@ def test_limited_frames_render_every_entry(n, wh, tile, opacity):
     assert torch.equal(a, gs.render(cam, mode="exact", tile=tile))
     assert torch.equal(a, b)
     gs.check()
+
+
+def _specks(cam, tile, n, seed=0):
+    """Gaussians about a pixel wide: three of four in the bottom-right tile, the others anywhere in the image."""
+    rng = np.random.default_rng(seed)
+    lo = np.array([cam.width - tile[0] + 2, cam.height - tile[1] + 2])
+    px = rng.uniform(lo, [cam.width - 1, cam.height - 1], size=(n, 2))
+    px[::4] = rng.uniform(0, [cam.width - 1, cam.height - 1], size=px[::4].shape)
+    z = rng.uniform(2.0, 4.0, n)
+    sc = synth.tiny_scene(n, seed=seed)
+    sc.means = np.stack([(px[:, 0] - cam.cx) / cam.fx * z, (px[:, 1] - cam.cy) / cam.fy * z, z], 1).astype(np.float32)
+    sc.scales = (rng.uniform(0.2, 0.6, (n, 3)) * (z / cam.fx)[:, None]).astype(np.float32)
+    return sc
+
+
+@pytest.mark.parametrize("wh,tile", [((8192, 8192), (16, 16)), ((16384, 4096), (32, 8)), ((4096, 16384), (8, 32))])
+def test_the_largest_grid_keeps_its_last_tile(wh, tile):
+    """512 x 512 tiles: runs of every lane in the last column of the last row. RoofGS against the ordered front end;
+    exact against a view one tile column wider, whose entries are sorted by 64-bit keys (the same Gaussians in the same
+    order, so the same pixels)."""
+    f = float(wh[0] // 2)
+    eye = np.eye(3, dtype=np.float32).reshape(9)
+
+    def camera(w):
+        return synth.Camera(eye, np.zeros(3, np.float32), f, f, (wh[0] - 1) / 2.0, (wh[1] - 1) / 2.0, w, wh[1], 0.5, 8.0,
+                            np.array([0.2, 0.1, 0.3], np.float32))
+
+    cam = camera(wh[0])
+    gs = binding.Scene(_specks(cam, tile, 3_000))
+    a, sa = gs.render(cam, stats=True, tile=tile)
+    ea = _entries(gs)
+    b, sb = gs.render(cam, flags=binding.RG_FLAG_ORDERED_FRONT_END, stats=True, tile=tile)
+    eb = _entries(gs)
+    last = ea[2].view(np.uint32).reshape(-1, 2)[-1]
+    assert int(last[1]) - int(last[0]) > 1_000
+    assert torch.equal(a, b)
+    for k in ("n_entries", "n_visible", "n_front", "n_pairs", "n_blends"):
+        assert sa[k] == sb[k], k
+    for x, y in zip(ea, eb):
+        assert np.array_equal(x, y)
+    a = gs.render(cam, mode="exact", tile=tile)
+    b = gs.render(camera(wh[0] + tile[0]), mode="exact", tile=tile)
+    assert torch.equal(a, b[:, :, :wh[0]])
+    gs.check()
