@@ -83,17 +83,21 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
     const float lx = (float)lxi;
     const uint2 range = a.ranges[tile];
     if (th == 0) s_last = -1;
-    auto stage = [&](unsigned j, bool colour) {
+    // the record of entry j; blended: the block's last blended entry (colours are staged too), -1 in the replay
+    auto stage = [&](unsigned j, int blended) {
         unsigned id = a.vals[j];
         if (id >= (unsigned long long)a.n) id = 0;
         const float4* const rec = a.erec + 3 * (size_t)id;
         const float4 m = __ldg(rec), q = __ldg(rec + 1);
-        const float mz = m.z - (float)y0;
         unsigned g = 0;
-        if (colour) {
-            s_rgb[th] = __ldg(rec + 2);
+        if (blended >= 0) {
+            const float4 c = __ldg(rec + 2);
+            s_rgb[th] = c;
             g = a.order ? a.order[id] : id;
+            if (c.w != 0.0f && (int)j <= blended) // its exponent is undefined: of its gradients only the colour's is a number
+                for (int k = 0; k < 6; k++) atomicAdd(a.gbuf + (size_t)g * GBUF + k, __int_as_float(0x7fffffff));
         }
+        const float mz = m.z - (float)y0;
         s_a[th] = make_float4(m.x - (float)x0, exact_skip_below(q.w), q.w, __uint_as_float(g));
         s_b[th] = make_float4(-mz, -mz, -m.w, -m.w);
         s_c[th] = make_float4(-q.y, -q.y, -m.y, -m.y);
@@ -120,7 +124,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
 #pragma unroll
         for (int i = 0; i < PPT; i++) all_done = all_done && lim[i] == INF;
         if (__syncthreads_count(!all_done) == 0) break;
-        if (start + th < range.y) stage(start + th, false);
+        if (start + th < range.y) stage(start + th, -1);
         __syncthreads();
         const int cnt = min((unsigned)NT, range.y - start);
         if (__all_sync(0xffffffffu, all_done)) continue;
@@ -183,7 +187,7 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
     const unsigned first_batch = range.x + (((unsigned)block_last - range.x) / NT) * NT;
     for (long long start = first_batch; start >= (long long)range.x; start -= NT) {
         __syncthreads();
-        if ((unsigned)start + th < range.y) stage((unsigned)start + th, true);
+        if ((unsigned)start + th < range.y) stage((unsigned)start + th, block_last);
         __syncthreads();
         const int cnt = (int)min((long long)NT, (long long)top + 1 - start); // the warp's last pair
         for (int k = cnt - 1; k >= 0; k--) {

@@ -640,12 +640,17 @@ constexpr int EX_THREADS = 256;
 // The raster record of a Gaussian binned as b: the exponent of Eq. (10) with the quadratic form
 // completed in dx, -1/2 ((Sigma'_yy / det) (dx - c dy)^2 + dy^2 / Sigma'_yy), c = Sigma'_xy / Sigma'_yy
 // (no cancellation for thin Gaussians), and the mean as double-floats (b's FP32 u, v only bin the
-// Gaussian).
-__device__ __forceinline__ void exact_record(const ExactArgs& a, float opacity, const Binned& b, float mx, float my,
+// Gaussian). Where the exponent is undefined, one of 0 and an alpha of 0.99 are written (the rasterizers compare exponents
+// before they evaluate alpha): returns whether it is.
+__device__ __forceinline__ bool exact_record(const ExactArgs& a, float opacity, const Binned& b, float mx, float my,
                                              float mz, float4& mean, float4& quad)
 {
     quad = make_float4(-0.5f * __fdiv_rn(b.sc, b.det), __fdiv_rn(b.sb, b.sc), __fdiv_rn(-0.5f, b.sc), opacity);
     mean = project_mean_df(a.cam, mx, my, mz);
+    if (!exact_undefined(mean)) return false;
+    mean = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    quad = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
+    return true;
 }
 
 // Adds the terms of words 4 V0 .. 4 V1 - 1 of a Gaussian's degree-3 SH coefficients (FP32) to its colour
@@ -690,13 +695,13 @@ __global__ void __launch_bounds__(EX_THREADS) k_exact_preprocess(ExactArgs a)
     a.depth[i] = pz;
     a.rect[i] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
     a.touched[i] = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
-    exact_record(a, a.opac[i], b, mx, my, mz, a.rec[3 * i], a.rec[3 * i + 1]);
+    const bool undefined = exact_record(a, a.opac[i], b, mx, my, mz, a.rec[3 * i], a.rec[3 * i + 1]);
     float dx, dy, dz, Y[16], c[3] = {0.5f, 0.5f, 0.5f};
     view_dir(a.cam, mx, my, mz, dx, dy, dz);
     sh_basis(dx, dy, dz, Y);
     const float4* const shp = reinterpret_cast<const float4*>(a.sh + 48 * i);
     exact_colour<0, 12>(Y, a.sh_degree, c, [&](int v) { return shp[v]; });
-    a.rec[3 * i + 2] = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), 0.0f);
+    a.rec[3 * i + 2] = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), undefined ? 1.0f : 0.0f);
 }
 
 __global__ void __launch_bounds__(DK_THREADS) k_exact_depth_keys(ExactArgs a, unsigned* keys, unsigned* vals, Counters* ctr,
@@ -738,14 +743,19 @@ struct ExactRow {
     int tx0, tx1, ty0;
 };
 
-__device__ __forceinline__ ExactRow exact_row(const Binned& b, const float4& mean, const float4& quad, bool& any)
+__device__ __forceinline__ ExactRow exact_row(const Binned& b, const float4& mean, const float4& quad, bool undefined,
+                                              bool& any)
 {
     ExactRow r;
     const float ext = sqrtf(12.0f * fmaxf(b.sa, b.sc)); // at least sqrt(2 level Sigma'_xx), level <= ln 255
     r.level = LN255F + logf(quad.w) + 0.01f + 1e-5f * ext;
-    any = r.level > 0.0f;
     r.u = mean.x;
     r.v = mean.z;
+    if (undefined) { // blends in every tile of the rectangle: NaN keeps them all
+        r.u = r.v = __int_as_float(0x7fffffff);
+        r.level = __int_as_float(0x7f800000);
+    }
+    any = r.level > 0.0f;
     r.kx = -1.0f / quad.x;
     r.sz = -quad.z;
     r.c = quad.y;
@@ -840,22 +850,22 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
     __syncwarp();
     fetch(seen, 1);
     ExactRow row;
-    bool any = false;
+    bool any = false, undefined = false;
     if (vis) {
         float4 mean, quad;
-        exact_record(a, m.w, b, m.x, m.y, m.z, mean, quad);
+        undefined = exact_record(a, m.w, b, m.x, m.y, m.z, mean, quad);
         a.rec[3 * slot] = mean;
         a.rec[3 * slot + 1] = quad;
         a.rect[slot] = make_int4(b.tx0, b.ty0, b.tx1, b.ty1);
         tiles = (unsigned)((b.tx1 - b.tx0 + 1) * (b.ty1 - b.ty0 + 1));
-        row = exact_row(b, mean, quad, any);
+        row = exact_row(b, mean, quad, undefined, any);
         if (any || keep_all) rows_l = b.ty1 - b.ty0 + 1;
     }
     if (slot < a.n) a.touched[i] = tiles;
     arrived();
     if (vis) {
         exact_colour<6, 12>(Y, a.sh_degree, c, [&](int v) { return own[v - 6]; });
-        a.rec[3 * slot + 2] = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), 0.0f);
+        a.rec[3 * slot + 2] = make_float4(clamp01(c[0]), clamp01(c[1]), clamp01(c[2]), undefined ? 1.0f : 0.0f);
     }
     __syncthreads(); // the row tests lie over the SH rows of other warps
     if (rows_l) s_row[tid] = row;

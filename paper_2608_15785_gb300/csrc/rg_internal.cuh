@@ -480,6 +480,11 @@ __device__ __forceinline__ float exact_power(const float4& m, const float4& quad
     return __fmaf_rn(__fmul_rn(quad.x, t), t, __fmul_rn(__fmul_rn(quad.z, dy), dy));
 }
 
+// Whether the exponent is not a number, at every pixel: z cancels to nothing in the double-float projection (coordinates of
+// 1e7 and more) and does not in FP32, which culls and bins the Gaussian, so u or v is NaN or infinite and its low part NaN.
+// Such a pair blends with alpha = min(0.99, NaN) = 0.99 (the minimum drops a NaN) all over its rectangle.
+__device__ __forceinline__ bool exact_undefined(const float4& m) { return isnan(m.y + m.w); }
+
 // The exponent below which a pair of opacity o is surely skipped: o exp(p) < 1/255 for every p below
 // it, whatever expf and the product round to (both within 1e-6; the margin is 1e-4). +inf for o = 0.
 __device__ __forceinline__ float exact_skip_below(float o) { return -(LN255F + logf(o)) - 1e-4f; }
@@ -673,7 +678,8 @@ struct ExactArgs {
     const unsigned* order; // [N] Gaussian of each slot (depth order) in a frame of tile-row runs, else null
     // per slot (index without an order):
     float4* rec;           // [N][3] projected mean as double-floats (u.hi, u.lo, v.hi, v.lo);
-                           // (-Sigma'_yy / (2 det), Sigma'_xy / Sigma'_yy, -1 / (2 Sigma'_yy), opacity); rgb
+                           // (-Sigma'_yy / (2 det), Sigma'_xy / Sigma'_yy, -1 / (2 Sigma'_yy), opacity); rgb, and 0, or
+                           // 1 where the exponent was undefined: one of exponent 0 and alpha 0.99 takes its place
     int4* rect;            // [N] tx0, ty0, tx1, ty1
     // per Gaussian:
     unsigned* touched;     // [N] tiles of the rectangle, 0 if culled

@@ -181,3 +181,50 @@ def test_backward_matches_fp64_oracle_gradient_everywhere():
             float(np.percentile(rel[np.abs(b) > 1e-3 * scale], 99))))
         bad = err > 2e-4 * np.abs(b) + 2e-5 * scale
         assert not bad.any(), (f, int(bad.sum()), np.argwhere(bad)[:5].tolist())
+
+
+def _cancelling_camera(width, height):
+    """z of the mean (2^24 + 2, 1, 3) is 2 in FP32 and 0 exactly, so its projected mean is no number."""
+    R = np.array([0, 1, 0, 0, 0, 1, 1, 1, 1], np.float32)
+    t = np.array([-1.0, -3.0, -(2.0 ** 24 + 6.0)], np.float32)
+    return synth.Camera(R, t, 100.0, 100.0, (width - 1) / 2.0, (height - 1) / 2.0, width, height, 0.5, 100.0)
+
+
+def _undefined_scene(opacity):
+    """That Gaussian, its rectangle about 30 pixels wide, in front of an ordinary one as wide."""
+    sc = synth.tiny_scene(2, seed=1)
+    sc.means = np.array([[2 ** 24 + 2, 1, 3], [2 ** 24 + 40, 1, 3]], np.float32)
+    sc.scales = np.array([[0.1] * 3, [2.0] * 3], np.float32)
+    sc.opacities = np.array([opacity, 0.7], np.float32)
+    return sc
+
+
+# two and four pixels per thread
+@pytest.mark.parametrize("wh", [(160, 120), (1024, 1040)])
+@pytest.mark.parametrize("opacity", [0.0, 0.5, 1.0])
+def test_a_gaussian_without_an_exponent(wh, opacity):
+    """alpha = min(0.99, o expf(NaN)) = 0.99: the timed image equals the counting launch's, which has the Gaussian all over
+    its rectangle, and the gradients are of that image: what lies behind gets 1 - 0.99 of its own (to rounding: 1e-4), the
+    Gaussian itself a number for its colour alone."""
+    cam = _cancelling_camera(*wh)
+    sc = _undefined_scene(opacity)
+    gs = binding.Scene(sc, storage=binding.RG_STORE_FP32)
+    img = gs.render(cam, mode="exact").clone()
+    full, st = gs.render(cam, mode="exact", stats=True)
+    assert st["n_visible"] == 2
+    behind = binding.Scene(sc.subset([1]), storage=binding.RG_STORE_FP32)
+    alone = behind.render(cam, mode="exact")
+    inside = (full != alone).any(0)
+    assert int(inside.sum()) >= 256
+    assert torch.equal(img, full)
+    w = torch.randn((3, wh[1], wh[0]), generator=torch.Generator().manual_seed(5)).cuda() * inside
+    g, ref = gs.backward(cam, w), behind.backward(cam, w)
+    left = float(np.float32(1) - np.float32(0.99))
+    for f in ref:
+        b = ref[f][0] * left
+        if f != "quats":  # (zero for equal scales: rounding alone)
+            assert torch.allclose(g[f][1], b, rtol=1e-4, atol=1e-4 * float(b.abs().max())), f
+        if f == "sh":
+            assert bool(torch.isfinite(g[f][0]).all()) and bool((g[f][0] != 0).any())
+        else:
+            assert bool(torch.isnan(g[f][0]).all()), f
