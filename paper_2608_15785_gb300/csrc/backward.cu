@@ -65,16 +65,16 @@ __device__ __forceinline__ float2 power_pair(float dx, float2 ly, const float4& 
 // time). With one pixel per thread a warp summed nine values over its lanes in 45 shuffles and nine
 // atomics for each of its eight warps and every pair, reached or not: 1250 us at 1080p with 500 k Gaussians,
 // now 760 us (two warps per tile, 14 shuffles, one atomic instruction of nine lanes).
-template <int PPT>
-__global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
+// SINGLY: pixel by pixel, for a large or non-finite dL/dimage (k_backward_begin).
+template <int PPT, bool SINGLY>
+__device__ __forceinline__ void backward_tile(const BackwardArgs& a, const int tile)
 {
     constexpr int NT = 256 / PPT, NH = PPT / 2;
     __shared__ float4 s_a[NT]; // u - x0, skip threshold, opacity, Gaussian
     __shared__ float4 s_b[NT], s_c[NT], s_d[NT]; // as power_pair() takes them
     __shared__ float4 s_rgb[NT];
     __shared__ int s_last;
-    grid_dependency_wait();
-    const int tile = (int)ordered_tile(a.tile_order, blockIdx.x), th = threadIdx.x, lane = th & 31;
+    const int th = threadIdx.x, lane = th & 31;
     const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
     const int x0 = tx * a.cam.tw, y0 = ty * a.cam.th;
     const int lxi = th & (a.cam.tw - 1), lyi = (th >> a.cam.tw_log2) * PPT;
@@ -184,6 +184,12 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
     if (block_last < 0) return;
 
     // 2) back to front over the same pairs
+    float2 R[NH][3]; // SINGLY: the colour behind the pair
+    if constexpr (SINGLY)
+#pragma unroll
+        for (int h = 0; h < NH; h++)
+#pragma unroll
+            for (int c = 0; c < 3; c++) R[h][c] = make_float2(a.cam.bg[c] * T[h].x, a.cam.bg[c] * T[h].y);
     const unsigned first_batch = range.x + (((unsigned)block_last - range.x) / NT) * NT;
     for (long long start = first_batch; start >= (long long)range.x; start -= NT) {
         __syncthreads();
@@ -207,7 +213,34 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
             float v[9];
 #pragma unroll
             for (int g = 0; g < 9; g++) v[g] = 0.0f;
-            if (any) {
+            if constexpr (SINGLY) {
+                const float4 c = s_rgb[k];
+                const float rgb[3] = {c.x, c.y, c.z};
+#pragma unroll
+                for (int i = 0; i < PPT; i++) {
+                    auto of = [&](float2& x) -> float& { return i & 1 ? x.y : x.x; };
+                    const int h = i / 2;
+                    const float e = expf(of(P[h])), oe = va.z * e, alpha = fminf(0.99f, oe);
+                    if (!u[i] || alpha < 1.0f / 255.0f) continue;
+                    const float inv = __frcp_rn(1.0f - alpha);
+                    const float Ti = of(T[h]) *= inv, w = alpha * Ti;
+                    float dal = 0.0f;
+#pragma unroll
+                    for (int g = 0; g < 3; g++) {
+                        dal += of(G[h][g]) * (rgb[g] * Ti - of(R[h][g]) * inv);
+                        of(R[h][g]) += rgb[g] * w;
+                        v[6 + g] += of(G[h][g]) * w;
+                    }
+                    if (oe > 0.99f) continue; // clamped
+                    const float dp = dal * alpha, ti = of(t[h]), dyi = of(dy[h]);
+                    v[0] += dp * ti;
+                    v[1] += dp * dyi;
+                    v[2] += dp * ti * ti;
+                    v[3] += dp * ti * dyi;
+                    v[4] += dp * dyi * dyi;
+                    v[5] += dal * e;
+                }
+            } else if (any) {
                 const float4 c = s_rgb[k];
 #pragma unroll
                 for (int h = 0; h < NH; h++) {
@@ -252,6 +285,43 @@ __global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
             else if (lane == 1) atomicAdd(out + 8, ninth);
         }
     }
+}
+
+template <int PPT>
+__global__ void __launch_bounds__(256 / PPT) k_raster_backward(BackwardArgs a)
+{
+    grid_dependency_wait();
+    if (*a.singly) return;
+    backward_tile<PPT, false>(a, (int)ordered_tile(a.tile_order, blockIdx.x));
+}
+
+// Its work in a frame of such a dL/dimage. (A choice within one kernel takes 92 registers instead of 72: 1080p 987 -> 1,028 us.)
+__global__ void __launch_bounds__(128) k_raster_backward_singly(BackwardArgs a)
+{
+    grid_dependency_wait();
+    if (!*a.singly) return;
+    const unsigned tiles = (unsigned)(a.tiles_x * a.tiles_y);
+    for (unsigned b = blockIdx.x; b < tiles; b += gridDim.x) {
+        backward_tile<2, true>(a, (int)ordered_tile(a.tile_order, b));
+        __syncthreads(); // the staged records are written again
+    }
+}
+
+// Clears the sums, and sees whether the pairs' sums will do: they take the pixel that skips a Gaussian with weight 0, which is
+// nothing only while every factor is finite. |G| and |G . bg| up to about 1e30 are enough (colours lie in [0, 1], the weights
+// add up to at most 1, 1 / (1 - alpha) is at most 100).
+__global__ void __launch_bounds__(256) k_backward_begin(BackwardArgs a, float limit)
+{
+    grid_dependency_wait();
+    const long long stride = (long long)gridDim.x * 256, i0 = (long long)blockIdx.x * 256 + threadIdx.x;
+    float4* const sums = reinterpret_cast<float4*>(a.gbuf);
+#pragma unroll 4
+    for (long long i = i0; i < a.n * (GBUF / 4); i += stride) sums[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const long long values = 3ll * a.cam.W * a.cam.H;
+    bool large = false;
+#pragma unroll 4
+    for (long long i = i0; i < values; i += stride) large |= !(fabsf(a.dL_dimg[i]) <= limit);
+    if (large) *a.singly = 1u;
 }
 
 // gradient of the real SH basis (polynomial form; the tangential projection of the
@@ -469,10 +539,16 @@ __global__ void __launch_bounds__(PB_THREADS) k_preprocess_backward(BackwardArgs
 void launch_raster_backward(const BackwardArgs& a, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)(a.tiles_x * a.tiles_y);
+    float bg = 1.0f;
+    for (int c = 0; c < 3; c++) bg = fmaxf(bg, fabsf(a.cam.bg[c]));
+    const long long work = a.n * (GBUF / 4) + 3ll * a.cam.W * a.cam.H, blocks = (work + 1023) / 1024, all = 8ll * device_sm_count();
+    launch_dependent(k_backward_begin, dim3((unsigned)(blocks < all ? blocks : all)), dim3(256), 0, s, a, 1e30f / bg);
     // the forward's rule (launch_raster_exact): a small image's tiles (475 at 400x304) want more warps per tile (two / four
     // pixels per thread: autograd step 1.94 / 2.00 ms), 1080p fewer sums over warps (1.04 / 1.01 ms)
     if (tiles <= 16u * (unsigned)device_sm_count()) launch_dependent(k_raster_backward<2>, dim3(tiles), dim3(128), 0, s, a);
     else launch_dependent(k_raster_backward<4>, dim3(tiles), dim3(64), 0, s, a);
+    const unsigned most = 8u * (unsigned)device_sm_count();
+    launch_dependent(k_raster_backward_singly, dim3(tiles < most ? tiles : most), dim3(128), 0, s, a);
 }
 
 void launch_preprocess_backward(const BackwardArgs& a, cudaStream_t s)

@@ -1429,7 +1429,6 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
         RG_TRY(ensure_workspace(s->ws, s->n, RG_MODE_EXACT, F, s->ws.cap));
     }
     RG_TRY(ensure(s->ws.gbuf, (size_t)(s->n > 0 ? s->n : 1) * GBUF * 4, "gradient buffer"));
-    RG_CK(cudaMemsetAsync(s->ws.gbuf.p, 0, (size_t)(s->n > 0 ? s->n : 1) * GBUF * 4, st));
     BackwardArgs b;
     memset(&b, 0, sizeof(b));
     const int fin = s->ws.last_passes & 1;
@@ -1450,6 +1449,7 @@ rg_status rg_backward(rg_scene* s, const rg_camera* cam, const rg_render_opts* o
     b.sh_degree = s->sh_degree;
     b.dL_dimg = dL_dimg;
     b.gbuf = s->ws.gbuf.as<float>();
+    b.singly = &s->ws.ctrl.as<Counters>()->singly;
     b.dmeans = grads->means;
     b.dscales = grads->scales;
     b.dquats = grads->quats;

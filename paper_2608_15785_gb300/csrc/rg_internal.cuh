@@ -77,6 +77,7 @@ struct Counters {
     unsigned n_row_runs;         // tile-row runs given a place in the rows' lists (runs.cu)
     unsigned n_chunks;           // chunks of runs
     unsigned n_rest;             // tiles that a limited frame's rasterizer left to its second kernel
+    unsigned singly;             // BackwardArgs::singly
     alignas(16) unsigned tiles[8]; // tiles of each size class (TileOrder)
     unsigned long long n_runs;   // tile-row runs the front end's blocks asked room for
     unsigned long long n_pairs;  // rasterizer work counters (counting launches only)
@@ -839,6 +840,7 @@ struct BackwardArgs {
     // dy^2 (backward.cu), d(opacity), d(rgb)
     const float* dL_dimg;
     float* gbuf;
+    unsigned* singly; // 0; set where dL/dimage is large or not finite
     // outputs
     float* dmeans;
     float* dscales;
@@ -846,6 +848,7 @@ struct BackwardArgs {
     float* dopac;
     float* dsh;
 };
+// clears gbuf before
 void launch_raster_backward(const BackwardArgs& a, cudaStream_t s);
 void launch_preprocess_backward(const BackwardArgs& a, cudaStream_t s);
 

@@ -228,3 +228,40 @@ def test_a_gaussian_without_an_exponent(wh, opacity):
             assert bool(torch.isfinite(g[f][0]).all()) and bool((g[f][0] != 0).any())
         else:
             assert bool(torch.isnan(g[f][0]).all()), f
+
+
+# two and four pixels per thread; a pixel of each half of a pair
+@pytest.mark.parametrize("wh", [(256, 192), (1024, 1040)])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan, 3e38])
+def test_a_non_finite_gradient_stays_with_its_pixel(wh, value):
+    """A Gaussian that the pixel does not blend (alpha < 1/255 there by a wide margin, or culled) has the gradients that a
+    zero in the pixel's place gives it, to rounding (the sums use atomics); the first one that it surely blends has no number."""
+    rng = np.random.default_rng(3)
+    sc = synth.tiny_scene(600, seed=8)
+    sc.scales = (sc.scales * 2.0).astype(np.float32)
+    cam = synth.tiny_camera(*wh, bg=(0.1, 0.3, 0.2))
+    # specks about the two pixels, many of which reach only the neighbours that share a thread
+    sc.means[:200] = np.append(rng.uniform(-5, 10, (200, 2)) / cam.fx * 3.0, rng.uniform(-0.01, 0.01, (200, 1)), 1)
+    sc.scales[:200] = np.float32(1.0 / cam.fx)
+    sc.opacities[:200] = 0.1
+    gs = binding.Scene(sc, storage=binding.RG_STORE_FP32)
+    w = torch.from_numpy(rng.normal(size=(3, wh[1], wh[0])).astype(np.float32)).cuda()
+    far = np.zeros(sc.n, bool)
+    for x, y in ((wh[0] // 2, wh[1] // 2), (wh[0] // 2 + 5, wh[1] // 2 + 1)):
+        d2, z = np.empty(sc.n), np.empty(sc.n)
+        for i in range(sc.n):
+            p = oracle.project64(sc.means[i], sc.quats[i], sc.scales[i], cam)
+            d = np.array([p["u"] - x, p["v"] - y])
+            d2[i], z[i] = d @ np.linalg.solve(p["cov2d"], d), p["z"]
+        power = np.log(np.maximum(sc.opacities, 1e-30)) - 0.5 * d2
+        far = power < np.log(0.5 / 255.0)
+        front = int(np.argmin(np.where((power > np.log(0.05)) & (sc.opacities < 0.98), z, np.inf)))
+        zero, bad = w.clone(), w.clone()
+        zero[1, y, x] = 0.0
+        bad[1, y, x] = float(value)
+        ref, g = gs.backward(cam, zero), gs.backward(cam, bad)
+        keep = torch.from_numpy(far).cuda()
+        assert 100 < int(keep.sum()) < sc.n
+        for f in FIELDS:
+            assert torch.allclose(g[f][keep], ref[f][keep], rtol=1e-4, atol=1e-5 * float(ref[f].abs().max())), f
+        assert np.isfinite(value) or not bool(torch.isfinite(g["opacities"][front]))
