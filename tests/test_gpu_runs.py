@@ -242,3 +242,39 @@ def test_the_largest_grid_keeps_its_last_tile(wh, tile):
     b = gs.render(camera(wh[0] + tile[0]), mode="exact", tile=tile)
     assert torch.equal(a, b[:, :, :wh[0]])
     gs.check()
+
+
+def _ms(gs, cam, out):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for _ in range(5):
+        a.record()
+        for _ in range(10):
+            gs.render(cam, out=out)
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("part", [0.07, 0.5, 0.9])
+def test_a_large_frame_beyond_the_capacity(part):
+    """Rows of many chunks: the kept entries are the first ones in (tile row, depth code, index, tile column) order of the
+    complete frame's, and the frame takes no longer than the complete one (0.5 to 0.95 of it; the bound leaves room for
+    noise on a busy machine)."""
+    sc = synth.clustered_scene(400_000, 1)
+    cam = synth.orbit_camera(0, 1920, 1080, radius=2.5)
+    full, small = binding.Scene(sc), binding.Scene(sc)
+    _, st = full.render(cam, stats=True)
+    k, v, _ = _entries(full)
+    k = k.view(np.uint32).astype(np.uint64)
+    room = int(k.size * part)
+    small.reserve(room)
+    out = small.render(cam)
+    gk, gv, _ = _entries(small)
+    b_d = np.uint64(st["b_d"])
+    tx, ty = (k >> b_d) % np.uint64(st["tiles_x"]), (k >> b_d) // np.uint64(st["tiles_x"])
+    kept = np.lexsort((tx, v, k & ((np.uint64(1) << b_d) - np.uint64(1)), ty))[:room]
+    expect = kept[np.lexsort((v[kept], k[kept]))]
+    assert np.array_equal(gk.view(np.uint32), k[expect].astype(np.uint32)) and np.array_equal(gv, v[expect])
+    assert _ms(small, cam, out) <= 1.15 * _ms(full, cam, out)
