@@ -218,7 +218,9 @@ rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries);
  * (dual-pixel), 1 or 4 pixels per thread (Sec. IV).
  * The number of entries stays on the device: with stats == NULL the call does
  * not synchronise; if the entries exceed the workspace the image is
- * incomplete and the overflow is recorded (see rg_scene_check). With stats
+ * incomplete (exact: the entries that fit are the first ones Gaussian by Gaussian in
+ * index order, row by row of each rectangle; RoofGS: those first by tile row, depth,
+ * index and tile column) and the overflow is recorded (see rg_scene_check). With stats
  * != NULL the call synchronises, grows the workspace and renders again if
  * needed, and fills *stats.
  * Errors: RG_ERR_INVALID_ARG (NULL, width/height <= 0, zfar <= znear, a mode

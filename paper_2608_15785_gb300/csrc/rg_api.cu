@@ -254,6 +254,7 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     a.runs = w.keys[1].as<unsigned>();
     a.vals = w.vals[0].as<unsigned>();
     a.limit = RUN_ALL;
+    a.kept = reinterpret_cast<unsigned*>(w.ctrl.as<unsigned char>() + RUN_KEPT_AT);
     a.ranges = w.ranges.as<uint2>();
     a.ctr = w.ctrl.as<Counters>();
     a.order = tile_order(w, a.rows * a.cols);
@@ -268,8 +269,8 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     a.cnt = reinterpret_cast<unsigned*>(part(per_row));
     a.seg = reinterpret_cast<unsigned*>(part(per_row));
     a.pre = reinterpret_cast<unsigned*>(part(per_row));
-    if (a.blocks <= RUN_SMALL_BLOCKS)
-        a.tot = reinterpret_cast<unsigned long long*>(w.ctrl.as<unsigned char>() + RUN_TOT_AT);
+    a.parts = reinterpret_cast<unsigned long long*>(w.ctrl.as<unsigned char>() + RUN_TOT_AT); // (tot's place)
+    if (a.blocks <= RUN_SMALL_BLOCKS) a.tot = a.parts;
     a.chunk = reinterpret_cast<RunChunk*>(part((size_t)a.chunk_cap * sizeof(RunChunk)));
     a.row = reinterpret_cast<RunRow*>(part((size_t)a.rows * sizeof(RunRow)));
     a.row_limit = reinterpret_cast<unsigned*>(part((size_t)a.rows * 4));
@@ -637,6 +638,10 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
             SortArgs ga;
             depth_sort_args(w, n, 4, sticky, ga);
             a.order = ga.vals[0]; // four passes
+            ra.n = n;
+            ra.gauss = a.order;
+            ra.rect = a.rect;
+            ra.touched = a.touched;
             w.last_gfin = 0;
             w.last_runs = true;
             w.last_passes = 0;

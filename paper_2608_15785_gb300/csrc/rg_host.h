@@ -68,8 +68,9 @@ constexpr size_t CTRL_BYTES = sizeof(Counters) + 8 * 256 * sizeof(unsigned);
 // frame counters, the per-Gaussian depth sort's, then the producers' digit-count copies
 // ([copy][2][256] from the fused front end, [copy][8][256] from the exact duplicate)
 constexpr size_t FE_HIST_BYTES = (size_t)FE_HIST_COPIES * 8 * 256 * sizeof(unsigned);
-constexpr size_t RUN_TOT_AT = (2 * CTRL_BYTES + FE_HIST_BYTES + 15) / 16 * 16; // then RunArgs::tot
-constexpr size_t CTRL_ALLOC = RUN_TOT_AT + (size_t)RUN_MAX_GRID * 8;
+constexpr size_t RUN_TOT_AT = (2 * CTRL_BYTES + FE_HIST_BYTES + 15) / 16 * 16; // then RunArgs::tot or parts
+constexpr size_t RUN_KEPT_AT = RUN_TOT_AT + (size_t)RUN_MAX_GRID * 8; // RunArgs::kept
+constexpr size_t CTRL_ALLOC = RUN_KEPT_AT + (size_t)RUN_MAX_GRID * 4;
 static_assert(CTRL_ALLOC % 16 == 0, "cleared 16 bytes at a time");
 
 // Frame workspace: everything one frame in flight needs besides the scene.

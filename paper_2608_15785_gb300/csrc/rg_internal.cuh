@@ -78,6 +78,9 @@ struct Counters {
     unsigned n_chunks;           // chunks of runs
     unsigned n_rest;             // tiles that a limited frame's rasterizer left to its second kernel
     unsigned singly;             // BackwardArgs::singly
+    unsigned cut, cut_tiles;     // an exact frame beyond its capacity: the Gaussian (in index order) with which the tiles of the
+                                 // rectangles pass it, and how many of its tiles fit
+    unsigned cut_ctr;            // blocks that added up their part of the tiles
     alignas(16) unsigned tiles[8]; // tiles of each size class (TileOrder)
     unsigned long long n_runs;   // tile-row runs the front end's blocks asked room for
     unsigned long long n_pairs;  // rasterizer work counters (counting launches only)
@@ -609,6 +612,13 @@ struct RunArgs {
     int box_total;     // 1: the front end counted the frame's entries (n_entries_total; exact mode, whose
                        // lists leave out entries below 1/255 on the whole tile); 0: the runs' entries
     long long cap;     // entries the workspace holds
+    unsigned* kept;    // [rows] entries of a frame beyond its capacity that it keeps (zeroed for every frame)
+    // box_total, for such a frame (ExactArgs):
+    long long n;
+    const unsigned* gauss; // order
+    const int4* rect;
+    const unsigned* touched;
+    unsigned long long* parts; // [rows] tiles of a part of the Gaussians (k_run_rows)
     unsigned* cnt;     // [rows][blocks] entries | runs << RUN_CNT_SHIFT
     unsigned* pre;     // [rows][blocks] runs of the row in the blocks before
     unsigned long long* tot; // [rows] entries | runs << RUN_TOT_SHIFT, zeroed for every frame; null in a frame that

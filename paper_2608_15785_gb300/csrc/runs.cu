@@ -91,6 +91,87 @@ __device__ __forceinline__ unsigned chunk_of(unsigned run, unsigned block)
     return run / CHUNK_STEP + block / CHUNK_BLOCKS;
 }
 
+// An exact frame beyond its capacity keeps the tiles of the rectangles Gaussian by Gaussian in index order, row by row, as
+// the entries that fit are the first ones plain 3DGS duplicates: the Gaussian with which they pass `cap`, and how many of its
+// tiles fit. It is one of the `len` from lo on, `before` tiles lie before those. Every thread of the block calls it; s_w: one
+// word per warp. A part of the Gaussians per warp, then the part that passes the capacity again, down to a warp's lanes.
+template <int WARPS>
+__device__ __noinline__ uint2 find_cut(const unsigned* touched, unsigned lo, unsigned len, unsigned long long before,
+                                       unsigned long long cap, unsigned long long* s_w)
+{
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    while (len > 32) {
+        const unsigned part = (len + WARPS - 1) / WARPS, end = lo + len;
+        const unsigned w0 = lo + warp * part, w1 = w0 + part < end ? w0 + part : end;
+        unsigned long long sum = 0;
+#pragma unroll 8
+        for (unsigned i = w0 + lane; i < w1; i += 32) sum += touched[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) s_w[warp] = sum;
+        __syncthreads();
+        unsigned k = 0;
+        while (k + 1 < WARPS && before + s_w[k] <= cap) before += s_w[k++];
+        __syncthreads();
+        lo += k * part;
+        len = lo < end ? (part < end - lo ? part : end - lo) : 0u;
+    }
+    const unsigned t = lane < len ? touched[lo + lane] : 0u;
+    const unsigned long long upto = before + run_warp_scan((unsigned long long)t);
+    const int first = __ffs((int)__ballot_sync(0xffffffffu, upto > cap)) - 1; // there is one
+    const unsigned fits = (unsigned)(cap - (upto - t));
+    return make_uint2(lo + (unsigned)(first < 0 ? 0 : first), __shfl_sync(0xffffffffu, fits, first < 0 ? 0 : first));
+}
+
+// find_cut over the blocks of k_run_rows: each adds up a part of the Gaussians, the last one to finish looks into the part that
+// passes the capacity. (One block for all of 3 M Gaussians took 0.4 ms.)
+template <int WARPS>
+__device__ __noinline__ void cut_by_rows(const RunArgs& a, unsigned long long* s_w)
+{
+    __shared__ bool s_last;
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, n = (unsigned)a.n, rows = (unsigned)a.rows;
+    const unsigned long long cap = (unsigned long long)a.cap;
+    const unsigned part = (n + rows - 1u) / rows, lo = blockIdx.x * part;
+    unsigned long long sum = 0;
+#pragma unroll 8
+    for (unsigned i = threadIdx.x; i < part; i += 32 * WARPS)
+        if (lo + i < n) sum += a.touched[lo + i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) s_w[warp] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sum = 0;
+        for (int q = 0; q < WARPS; q++) sum += s_w[q];
+        st_volatile_u64(&a.parts[blockIdx.x], sum);
+        __threadfence();
+        s_last = atomicAdd(&a.ctr->cut_ctr, 1u) == rows - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    unsigned k = 0; // the part that passes the capacity
+    unsigned long long before = 0;
+    for (; k < rows; k += 32) {
+        const unsigned long long t = k + lane < rows ? ld_volatile_u64(&a.parts[k + lane]) : 0ull;
+        const unsigned long long upto = before + run_warp_scan(t);
+        const unsigned over = __ballot_sync(0xffffffffu, upto > cap);
+        if (over) {
+            const int first = __ffs((int)over) - 1;
+            before = __shfl_sync(0xffffffffu, upto - t, first);
+            k += (unsigned)first;
+            break;
+        }
+        before = __shfl_sync(0xffffffffu, upto, 31);
+    }
+    const unsigned from = k * part; // (there is one: k < rows and from < n)
+    const uint2 cut = find_cut<WARPS>(a.touched, from, from < n ? (part < n - from ? part : n - from) : 0u, before, cap, s_w);
+    if (threadIdx.x == 0) {
+        a.ctr->cut = cut.x;
+        a.ctr->cut_tiles = cut.y;
+    }
+}
+
 // One block of 1024 threads per tile row: a scan of the blocks' counts, and the row's chunks.
 __global__ void __launch_bounds__(1024) k_run_rows(RunArgs a)
 {
@@ -100,6 +181,7 @@ __global__ void __launch_bounds__(1024) k_run_rows(RunArgs a)
     __shared__ unsigned s_chunk;
     grid_dependency_wait();
     const unsigned row = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    if (a.box_total && a.ctr->n_entries_total > (unsigned long long)a.cap) cut_by_rows<WARPS>(a, s_e);
     const unsigned* const cnt = a.cnt + (size_t)row * a.blocks;
     const unsigned per = (a.blocks + 32u * WARPS - 1u) / (32u * WARPS), b0 = tid * per;
     const unsigned b1 = b0 + per < a.blocks ? b0 + per : a.blocks;
@@ -182,11 +264,12 @@ struct alignas(16) CollectSmem {
 // The runs of chunk `chunk` of a tile row: front-end blocks [block, bend), runs [run, run + n) of the
 // row. A thread takes eight consecutive runs; all its loads are in flight together. Which block a run
 // lies in follows from a maximum scan over the blocks' first runs. clip: the frame has more entries
-// than the workspace holds and keeps those whose place in (tile row, slot, column) order lies below
-// the capacity; `entry` entries of the frame lie before the chunk then.
+// than the workspace holds. It keeps those whose place in (tile row, slot, column) order lies below the
+// capacity; `entry` entries of the frame lie before the chunk then. An exact frame keeps the tiles that come first in
+// index order: cut.x, cut.y of find_cut.
 __device__ __forceinline__ void collect_chunk(const RunArgs& a, const RunRow& r, unsigned row, unsigned chunk,
                                               unsigned block, unsigned bend, unsigned run, unsigned n, bool clip,
-                                              unsigned long long entry, CollectSmem& S)
+                                              unsigned long long entry, uint2 cut, CollectSmem& S)
 {
     constexpr int PER = CHUNK_RUNS / RUN_THREADS;
     const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -235,8 +318,8 @@ __device__ __forceinline__ void collect_chunk(const RunArgs& a, const RunRow& r,
         const unsigned j = j0 + (unsigned)u;
         v[u] = j < n ? a.runs[S.from[own[u] - 1] + j] : 0u;
     }
-    unsigned room = 0; // clip: entries that still fit before the thread's first run (0: none)
-    if (clip) { // (a walk over the runs before each run instead of this scan: frames of half the room 1,407 us at 4K, 275 at 1080p)
+    unsigned room = 0, kept = 0; // clip: entries that still fit before the thread's first run; entries of its runs
+    if (clip && !a.box_total) { // (a walk over the runs before each run instead of this scan: frames of half the room 1,407 us at 4K, 275 at 1080p)
         int sum = 0, all;
 #pragma unroll
         for (int u = 0; u < PER; u++)
@@ -253,17 +336,33 @@ __device__ __forceinline__ void collect_chunk(const RunArgs& a, const RunRow& r,
         if (j >= n) break;
         unsigned ta = run_first(v[u]), tb = run_last(v[u]);
         const unsigned b = block + own[u] - 1;
-        if (clip) {
-            const unsigned width = tb - ta + 1u, kept = width < room ? width : room;
-            tb = ta + kept - 1u;
-            if (kept == 0u) { // an empty run
+        if (clip && a.box_total) {
+            const unsigned g = a.gauss[b * RUN_SLOTS + run_slot(v[u])];
+            if (g >= cut.x) {
+                int left = 0; // of the rectangle's tiles in the row, those kept
+                if (g == cut.x) {
+                    const int4 q = a.rect[b * RUN_SLOTS + run_slot(v[u])];
+                    left = (int)cut.y - ((int)row - q.y) * (q.z - q.x + 1) + q.x;
+                }
+                if (left <= (int)ta) { // an empty run
+                    ta = 1;
+                    tb = 0;
+                } else if ((int)tb >= left) {
+                    tb = (unsigned)left - 1u;
+                }
+            }
+        } else if (clip) {
+            const unsigned width = tb - ta + 1u, fits = width < room ? width : room;
+            tb = ta + fits - 1u;
+            if (fits == 0u) { // an empty run
                 ta = 1;
                 tb = 0;
             }
-            room -= kept;
+            room -= fits;
         }
         list[j] = make_uint2(b * RUN_SLOTS + run_slot(v[u]), ta | (tb << 16));
         if (ta <= tb) {
+            kept += tb - ta + 1u;
             atomicAdd(&S.d[ta], 1);
             atomicSub(&S.d[tb + 1], 1);
         }
@@ -278,6 +377,11 @@ __device__ __forceinline__ void collect_chunk(const RunArgs& a, const RunRow& r,
         if (col < a.cols) a.col[(size_t)chunk * pitch + col] = (unsigned)(carry + x);
         carry += all;
     }
+    if (clip) {
+        int all;
+        run_block_scan<RUN_WARPS>((int)kept, S.w, all);
+        if (tid == 0 && all) atomicAdd(&a.kept[row], (unsigned)all);
+    }
 }
 
 // Grid (blocks per row, rows): block x of a row takes its chunks x, x + gridDim.x, ...
@@ -289,16 +393,17 @@ __global__ void __launch_bounds__(RUN_THREADS, 6) k_run_collect(RunArgs a)
     const unsigned row = blockIdx.y;
     const RunRow r = a.row[row];
     if (blockIdx.x >= r.nchunks) return;
-    const bool clip = !a.box_total && a.ctr->n_entries_total > (unsigned long long)a.cap;
+    const bool clip = a.ctr->n_entries_total > (unsigned long long)a.cap;
+    const uint2 cut = make_uint2(a.ctr->cut, a.ctr->cut_tiles);
     unsigned long long start = 0;
-    if (clip)
+    if (clip && !a.box_total)
         for (unsigned q = 0; q < row; q++) start += a.row[q].entries;
     for (unsigned c = blockIdx.x; c < r.nchunks; c += gridDim.x) {
         RunChunk k;
         unsigned bend, rend;
         chunk_bounds(a, r, c, k, bend, rend);
         if (rend > k.run)
-            collect_chunk(a, r, row, r.chunk + c, k.block, bend, k.run, rend - k.run, clip, start + k.entry, S);
+            collect_chunk(a, r, row, r.chunk + c, k.block, bend, k.run, rend - k.run, clip, start + k.entry, cut, S);
         else // no run: no entries in any column
             for (int j = (int)threadIdx.x; j < a.cols; j += RUN_THREADS)
                 a.col[(size_t)(r.chunk + c) * run_pitch(a.cols) + j] = 0u;
@@ -357,14 +462,18 @@ __global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
     }
     if (blockIdx.x >= r.nchunks) return;
     if (tid == s_first) a.chunk[r.chunk + blockIdx.x] = RunChunk{tid, p, 0ull};
-    const bool clip = !a.box_total && s_all > (unsigned long long)a.cap;
+    const bool clip = (a.box_total ? a.ctr->n_entries_total : s_all) > (unsigned long long)a.cap;
     unsigned long long entry = s_before & RUN_TOT_ENTRIES;
-    if (clip) { // and the row's entries before the chunk
+    uint2 cut = make_uint2(0u, 0u);
+    if (clip && a.box_total) {
+        __shared__ unsigned long long s_cut[RUN_WARPS];
+        cut = find_cut<RUN_WARPS>(a.touched, 0u, (unsigned)a.n, 0ull, (unsigned long long)a.cap, s_cut);
+    } else if (clip) { // and the row's entries before the chunk
         unsigned all;
         run_block_scan<RUN_WARPS>(tid < s_first ? a.cnt[(size_t)row * a.blocks + tid] & RUN_CNT_ENTRIES : 0u, s_w, all);
         entry += all;
     }
-    collect_chunk(a, r, row, r.chunk + blockIdx.x, s_first, s_end, s_run, s_rend - s_run, clip, entry, S);
+    collect_chunk(a, r, row, r.chunk + blockIdx.x, s_first, s_end, s_run, s_rend - s_run, clip, entry, cut, S);
 }
 
 
@@ -372,6 +481,22 @@ __global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
 // around 0.5 (trained scenes) and scaled: 4K, 1 M Gaussians x 1 579 / 605 us, x 0.5 743 / 764, x 0.35 852 / 855, x 0.1
 // 1243 / 1123; 2560 x 1440, 2 M x 1 513 / 548, x 0.5 660 / 661, x 0.35 752 / 728 (exact mode alike)
 constexpr float LIMIT_OPACITY = 0.3f;
+
+// A frame beyond its capacity: the entries kept in the rows before `row`, and in all (called by one warp).
+__device__ __forceinline__ void kept_before(const RunArgs& a, unsigned row, unsigned long long& before, unsigned long long& all)
+{
+    before = all = 0;
+    for (unsigned q = threadIdx.x & 31u; (int)q < a.rows; q += 32) {
+        const unsigned e = a.kept[q];
+        before += q < row ? e : 0u;
+        all += e;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+    }
+}
 
 // One block per tile row: OFF_SEGS segments of the row's chunks x OFF_COLS columns at a time.
 constexpr int OFF_SEGS = 4, OFF_COLS = 256;
@@ -402,10 +527,11 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
             before += __shfl_xor_sync(0xffffffffu, before, o);
             all += __shfl_xor_sync(0xffffffffu, all, o);
         }
-        if (lane == 0) s_start = (unsigned)(before < cap ? before : cap);
+        const unsigned long long total = a.box_total ? a.ctr->n_entries_total : all;
+        if (total > cap) kept_before(a, row, before, all);
+        if (lane == 0) s_start = (unsigned)before;
         if (lane == 0 && row == 0) {
-            const unsigned long long total = a.box_total ? a.ctr->n_entries_total : all;
-            a.ctr->n_entries = (unsigned)(total < cap ? total : cap);
+            a.ctr->n_entries = (unsigned)(total <= cap ? total : (a.box_total ? cap : all));
             if (total > cap) {
                 atomicOr(&a.ctr->overflow, 1u);
                 atomicOr(&a.sticky->overflow, 1u);
@@ -506,18 +632,22 @@ __device__ __forceinline__ void small_offsets(const RunArgs& a, const RunRow& r,
     const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const unsigned long long cap = (unsigned long long)a.cap;
     if (warp == RUN_WARPS - 1) {
-        unsigned long long before = 0;
-        for (unsigned q = lane; q < row; q += 32) before += a.tot[q] & RUN_TOT_ENTRIES;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-        if (lane == 0) S.start = (unsigned)(before < cap ? before : cap);
-    }
-    if (blockIdx.x == 0 && row == 0 && tid == 0) {
         const unsigned long long total = a.ctr->n_entries_total;
-        a.ctr->n_entries = (unsigned)(total < cap ? total : cap);
+        unsigned long long before = 0, all = 0;
         if (total > cap) {
-            atomicOr(&a.ctr->overflow, 1u);
-            atomicOr(&a.sticky->overflow, 1u);
+            kept_before(a, row, before, all);
+        } else {
+            for (unsigned q = lane; q < row; q += 32) before += a.tot[q] & RUN_TOT_ENTRIES;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        }
+        if (lane == 0) S.start = (unsigned)before;
+        if (lane == 0 && blockIdx.x == 0 && row == 0) {
+            a.ctr->n_entries = (unsigned)(total <= cap ? total : (a.box_total ? cap : all));
+            if (total > cap) {
+                atomicOr(&a.ctr->overflow, 1u);
+                atomicOr(&a.sticky->overflow, 1u);
+            }
         }
     }
     const int pitch = run_pitch(a.cols);

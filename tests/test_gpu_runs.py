@@ -278,3 +278,37 @@ def test_a_large_frame_beyond_the_capacity(part):
     expect = kept[np.lexsort((v[kept], k[kept]))]
     assert np.array_equal(gk.view(np.uint32), k[expect].astype(np.uint32)) and np.array_equal(gv, v[expect])
     assert _ms(small, cam, out) <= 1.15 * _ms(full, cam, out)
+
+
+# a small frame, a larger one, a limited one
+@pytest.mark.parametrize("n,wh,scale", [(3_000, (200, 150), 2.0), (40_000, (320, 200), 1.0), (520_000, (2064, 1552), 0.5)])
+def test_exact_frames_beyond_the_capacity(n, wh, scale):
+    """The entries that an exact frame keeps, and blends, are the first ones Gaussian by Gaussian in index order, row by row
+    of its rectangle: the image equals that of the scene cut off there, with the last Gaussian in its first tiles only."""
+    sc = _scene(n, scale, seed=6)
+    cam = synth.tiny_camera(*wh, bg=(0.2, 0.1, 0.3))
+    bins = oracle.keys(sc, cam, oracle.EXACT)[3]
+    rows, cols = bins[:, 4] - bins[:, 2] + 1, bins[:, 3] - bins[:, 1] + 1
+    k = int(np.flatnonzero((np.arange(n) > n // 2) & (bins[:, 0] > 0) & (rows > 1) & (cols > 1))[0])
+    sc.opacities[k] = 0.9
+    fits = int(cols[k]) + 1  # its first row, and a tile of the second
+    room = int(bins[:k, 6].sum()) + fits
+    assert room < int(bins[:, 6].sum())
+    small = binding.Scene(sc, storage=binding.RG_STORE_FP32)
+    small.reserve(room)
+    img = small.render(cam, mode="exact")
+    want = []
+    for m in (k, k + 1):
+        gs = binding.Scene(sc.subset(np.arange(m)), storage=binding.RG_STORE_FP32)
+        gs.render(cam, mode="exact", stats=True)
+        want.append(gs.render(cam, mode="exact").clone())
+        gs.close()
+    ref = want[0]
+    for t in range(fits):
+        x, y = 16 * (int(bins[k, 1]) + t % int(cols[k])), 16 * (int(bins[k, 2]) + t // int(cols[k]))
+        ref[:, y:y + 16, x:x + 16] = want[1][:, y:y + 16, x:x + 16]
+    assert torch.equal(img, ref)
+    assert small.inspect(binding.RG_INSPECT_VALUES).size == room
+    with pytest.raises(binding.RgError) as e:
+        small.check()
+    assert e.value.status == 4
