@@ -253,7 +253,9 @@ rg_status rg_stage_times(rg_scene* scene, float* ms7, int32_t* frames);
                                     that sort at most 16 tile bits keep 16-bit tile ids: the 32-bit keys
                                     (tile << b_d | q_d) are rebuilt on the host from the tile ranges or
                                     ids, the values and the per-Gaussian depth codes, so every frame
-                                    reports the order of the 32-bit key */
+                                    reports the order of the 32-bit key; exact frames without stats
+                                    leave tiles below 1/255 out of their lists, and they are added
+                                    here (RG_ERR_CUDA if the lists do not lie among the result) */
 #define RG_INSPECT_VALUES 2      /* sorted values: uint32 Gaussian indices (in the same order) */
 #define RG_INSPECT_RANGES 3      /* uint32 [tiles][2] = [start, end) per tile (of the same order) */
 #define RG_INSPECT_SH_CODES 4    /* int8 [n][16][3] compact SH codes */

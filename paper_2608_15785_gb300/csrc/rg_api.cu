@@ -643,6 +643,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
             ra.rect = a.rect;
             ra.touched = a.touched;
             w.last_gfin = 0;
+            w.last_all_tiles = count;
             w.last_runs = true;
             w.last_passes = 0;
             {
@@ -719,6 +720,8 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
             ra.rest_flag = reinterpret_cast<unsigned*>(ra.ranges + F.tiles) + 8 * F.tiles;
         }
         launch_runs(ra, st, ev ? E[3] : nullptr);
+        w.last_lists[0] = ra.vals;
+        w.last_lists[1] = ra.ranges;
         if (ra.limit != RUN_ALL) w.last_limited = ra;
     } else if (tile_sort) {
         NvtxScope r_("rg sort");
@@ -1198,52 +1201,105 @@ rg_status rg_stage_times(rg_scene* s, float* ms7, int32_t* frames)
     return RG_OK;
 }
 
-// The entries of an exact frame of runs as plain 3DGS has them: every tile of every rectangle (the device
-// lists leave out tiles below 1/255), in the order of the 64-bit key tile << 32 | float depth, ties by
-// index; those that the capacity keeps are the first ones Gaussian by Gaussian, tiles ascending.
+// Writes the values that a limited frame left out (over the state of its unfinished tiles).
+static rg_status write_all_values(Workspace& w)
+{
+    RunArgs& z = w.last_limited;
+    if (!z.cap || z.limit == RUN_ALL) return RG_OK;
+    if (z.list != w.keys[0].p || z.vals != w.vals[0].p || (void*)z.cnt != w.runbuf.p || (void*)z.ranges != w.ranges.p ||
+        z.cap != w.cap)
+        return fail(RG_ERR_INVALID_ARG, "the workspace was resized after the frame");
+    launch_runs_all(z, 0);
+    RG_CK(cudaDeviceSynchronize());
+    z.limit = RUN_ALL;
+    return RG_OK;
+}
+
+// The entries of an exact frame of runs as plain 3DGS has them: every tile of every rectangle, in the order of the 64-bit
+// key tile << 32 | float depth, ties by index; those that the capacity keeps are the first ones Gaussian by Gaussian, row by
+// row. A counting frame's lists on the device are these; the others leave out tiles below 1/255: what was left out is added
+// from the rectangles, and what the device has must lie among the result in the same order.
 static rg_status exact_runs_entries(rg_scene* s, const Counters& c, int32_t what, std::vector<unsigned char>& out)
 {
-    const Workspace& w = s->ws;
+    Workspace& w = s->ws;
     const size_t n = (size_t)s->n, tiles = (size_t)w.last_tiles, tx = (size_t)w.last_tiles_x, ne = c.n_entries;
-    std::vector<uint32_t> order(n), depth(n), touched(n), kept(n, 0u);
-    std::vector<int4> rect(n);
+    const bool lists = w.last_lists[0] == w.vals[0].p && w.last_lists[1] == w.ranges.p; // not resized since
+    std::vector<uint32_t> order(n), depth(n);
     const DepthSortViews g = depth_sort_views(w, s->n);
     RG_CK(cudaMemcpy(order.data(), g.vals[w.last_gfin], n * 4, cudaMemcpyDeviceToHost));
     RG_CK(cudaMemcpy(depth.data(), g.keys[w.last_gfin], n * 4, cudaMemcpyDeviceToHost));
-    RG_CK(cudaMemcpy(touched.data(), w.touched.p, n * 4, cudaMemcpyDeviceToHost));
-    RG_CK(cudaMemcpy(rect.data(), w.rect.p, n * 16, cudaMemcpyDeviceToHost));
-    for (size_t k = 0; k < n; k++)
-        kept[k] = touched[k];
-    for (size_t i = 0, left = ne; i < n; i++) {
-        kept[i] = (uint32_t)std::min<size_t>(kept[i], left);
-        left -= kept[i];
+    std::vector<uint2> have(lists ? tiles : 0); // the device's lists (slots)
+    std::vector<uint32_t> slots;
+    if (lists) {
+        if (what != RG_INSPECT_RANGES || !w.last_all_tiles) RG_TRY(write_all_values(w));
+        RG_CK(cudaMemcpy(have.data(), w.ranges.p, tiles * 8, cudaMemcpyDeviceToHost));
+        uint32_t end = 0;
+        for (const uint2& r : have) end = std::max(end, r.y);
+        if ((int64_t)end > w.cap) return fail(RG_ERR_CUDA, "the device's ranges are not the frame's");
+        slots.resize(end);
+        if (end) RG_CK(cudaMemcpy(slots.data(), w.vals[0].p, (size_t)end * 4, cudaMemcpyDeviceToHost));
+        for (uint32_t k : slots)
+            if (k >= n || order[k] >= n) return fail(RG_ERR_CUDA, "the device's entries are not the frame's");
     }
-    auto each = [&](auto&& f) { // f(slot, Gaussian, tile) in depth order, tiles ascending
-        for (size_t k = 0; k < n; k++) {
-            if (order[k] >= n) continue;
-            uint32_t left = kept[order[k]];
-            const int4 r = rect[k];
-            for (int y = r.y; left && y <= r.w; y++)
-                for (int x = r.x; left && x <= r.z; x++, left--) f(k, order[k], (size_t)y * tx + (size_t)x);
+    std::vector<uint2> range(tiles);
+    std::vector<uint32_t> list; // slots by tile
+    if (lists && w.last_all_tiles) {
+        range.swap(have);
+        list.swap(slots);
+        if (list.size() != ne) return fail(RG_ERR_CUDA, "the device's entries are not the frame's");
+    } else {
+        std::vector<uint32_t> touched(n), kept(n);
+        std::vector<int4> rect(n);
+        RG_CK(cudaMemcpy(touched.data(), w.touched.p, n * 4, cudaMemcpyDeviceToHost));
+        RG_CK(cudaMemcpy(rect.data(), w.rect.p, n * 16, cudaMemcpyDeviceToHost));
+        size_t left = ne;
+        for (size_t i = 0; i < n; i++) {
+            kept[i] = (uint32_t)std::min<size_t>(touched[i], left);
+            left -= kept[i];
         }
-    };
-    std::vector<uint32_t> first(tiles + 1, 0u);
-    each([&](size_t, uint32_t, size_t t) { first[t + 1]++; });
-    for (size_t t = 0; t < tiles; t++) first[t + 1] += first[t];
+        for (size_t k = 0; k < n; k++) { // (the rectangle of a slot without tiles is not written)
+            const int4 r = rect[k];
+            if (order[k] >= n || (kept[order[k]] &&
+                                  (r.x < 0 || r.y < 0 || r.z >= (int)tx || r.w >= (int)(tiles / tx))))
+                return fail(RG_ERR_CUDA, "the device's rectangles are not the frame's");
+        }
+        auto each = [&](auto&& f) { // f(slot, tile) in depth order, tiles ascending
+            for (size_t k = 0; k < n; k++) {
+                uint32_t more = kept[order[k]];
+                const int4 r = rect[k];
+                for (int y = r.y; more && y <= r.w; y++)
+                    for (int x = r.x; more && x <= r.z; x++, more--) f(k, (size_t)y * tx + (size_t)x);
+            }
+        };
+        std::vector<uint32_t> first(tiles + 1, 0u);
+        each([&](size_t, size_t t) { first[t + 1]++; });
+        for (size_t t = 0; t < tiles; t++) {
+            first[t + 1] += first[t];
+            range[t] = first[t + 1] > first[t] ? make_uint2(first[t], first[t + 1]) : make_uint2(0u, 0u);
+        }
+        if (first[tiles] != ne) return fail(RG_ERR_CUDA, "the device's rectangles are not the frame's");
+        list.resize(ne);
+        each([&](size_t k, size_t t) { list[first[t]++] = (uint32_t)k; });
+        for (size_t t = 0; t < have.size(); t++) {
+            uint32_t j = range[t].x;
+            for (uint32_t k = have[t].x; k < have[t].y; k++, j++) {
+                while (j < range[t].y && list[j] != slots[k]) j++;
+                if (j >= range[t].y) return fail(RG_ERR_CUDA, "the device's entries are not the frame's");
+            }
+        }
+    }
     if (what == RG_INSPECT_RANGES) {
-        std::vector<uint2> rr(tiles);
-        for (size_t t = 0; t < tiles; t++)
-            rr[t] = first[t + 1] > first[t] ? make_uint2(first[t], first[t + 1]) : make_uint2(0u, 0u);
         out.resize(tiles * 8);
-        memcpy(out.data(), rr.data(), out.size());
+        memcpy(out.data(), range.data(), out.size());
         return RG_OK;
     }
     const size_t item = what == RG_INSPECT_KEYS ? 8 : 4;
     out.resize(ne * item);
-    each([&](size_t k, uint32_t i, size_t t) {
-        const uint64_t key = ((uint64_t)t << 32) | depth[k];
-        memcpy(&out[(size_t)first[t]++ * item], what == RG_INSPECT_KEYS ? (const void*)&key : (const void*)&i, item);
-    });
+    for (size_t t = 0; t < tiles; t++)
+        for (uint32_t j = range[t].x; j < range[t].y; j++) {
+            const uint64_t key = ((uint64_t)t << 32) | depth[list[j]];
+            memcpy(&out[(size_t)j * item], what == RG_INSPECT_KEYS ? (const void*)&key : (const void*)&order[list[j]], item);
+        }
     return RG_OK;
 }
 
@@ -1278,15 +1334,7 @@ rg_status rg_inspect(rg_scene* s, int32_t what, void* host_dst, int64_t cap_byte
         if (s->ws.last_runs && what != RG_INSPECT_RANGES) {
             std::vector<uint32_t> order(ng);
             val.resize(ne);
-            RunArgs& z = s->ws.last_limited;
-            if (ne && z.cap && z.limit != RUN_ALL) { // the frame left values out
-                if (z.list != s->ws.keys[0].p || z.vals != s->ws.vals[0].p || (void*)z.cnt != s->ws.runbuf.p ||
-                    (void*)z.ranges != s->ws.ranges.p || z.cap != s->ws.cap)
-                    return fail(RG_ERR_INVALID_ARG, "the workspace was resized after the frame");
-                launch_runs_all(z, 0);
-                RG_CK(cudaDeviceSynchronize());
-                z.limit = RUN_ALL;
-            }
+            if (ne) RG_TRY(write_all_values(s->ws));
             if (ne) RG_CK(cudaMemcpy(val.data(), s->ws.vals[fin].p, ne * 4, cudaMemcpyDeviceToHost));
             if (ng) RG_CK(cudaMemcpy(order.data(), g.vals[s->ws.last_gfin], ng * 4, cudaMemcpyDeviceToHost));
             for (uint32_t& v : val) v = v < ng ? order[v] : 0u;

@@ -99,6 +99,8 @@ struct Workspace {
     RunArgs last_limited = {}; // runs of the last frame if its values were not all written; else limit = RUN_ALL or 0
     bool last_runs = false;  // the entries were written from tile-row runs: values are slots of the depth order
                              // in tile-id order, in vals[0]
+    bool last_all_tiles = false; // an exact frame of runs whose lists hold every tile of the rectangles (a counting frame)
+    const void* last_lists[2] = {nullptr, nullptr}; // vals[0], ranges of a frame of runs
     int last_bd = 0;         // b_d of the last RoofGS frame
     int last_gfin = 0;       // buffer of the per-Gaussian depth sort's result
     // stage events

@@ -312,3 +312,32 @@ def test_exact_frames_beyond_the_capacity(n, wh, scale):
     with pytest.raises(binding.RgError) as e:
         small.check()
     assert e.value.status == 4
+
+
+@pytest.mark.parametrize("stats", [True, False])
+@pytest.mark.parametrize("n", [20_000, 40_000])
+def test_inspection_reads_the_device_lists(n, stats):
+    """What rg_inspect reports of an exact frame is the counting frame's lists, and for the others is held against the lists
+    that the device blends: once a replayed graph has put another frame's in their place, it reports those or refuses."""
+    sc = _scene(n)
+    cam = synth.tiny_camera(320, 200)
+    gs = binding.Scene(sc)
+    out = gs.render(cam)
+    gs.render(cam, mode="exact", stats=True)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        gs.render(cam, out=out)
+    gs.render(cam, mode="exact", stats=stats)
+    k, v, r, _ = oracle.keys(sc, cam, oracle.EXACT)
+    gk, gv, gr = _entries(gs)
+    assert np.array_equal(gk.view(np.uint64), k) and np.array_equal(gv, v)
+    assert np.array_equal(gr.view(np.uint32).reshape(-1, 2), r)
+    g.replay()
+    if stats:
+        assert not np.array_equal(gs.inspect(binding.RG_INSPECT_VALUES), v)
+    else:
+        with pytest.raises(binding.RgError):
+            gs.inspect(binding.RG_INSPECT_VALUES)
+    gs.render(cam, mode="exact", stats=stats)
+    assert np.array_equal(_entries(gs)[1], v)
