@@ -1201,17 +1201,17 @@ rg_status rg_stage_times(rg_scene* s, float* ms7, int32_t* frames)
     return RG_OK;
 }
 
-// Writes the values that a limited frame left out (over the state of its unfinished tiles).
-static rg_status write_all_values(Workspace& w)
+// Writes the values that a limited frame left out (over the state of its unfinished tiles). For every inspection: a replayed
+// graph leaves them out again.
+static rg_status write_all_values(const Workspace& w)
 {
-    RunArgs& z = w.last_limited;
+    const RunArgs& z = w.last_limited;
     if (!z.cap || z.limit == RUN_ALL) return RG_OK;
     if (z.list != w.keys[0].p || z.vals != w.vals[0].p || (void*)z.cnt != w.runbuf.p || (void*)z.ranges != w.ranges.p ||
         z.cap != w.cap)
         return fail(RG_ERR_INVALID_ARG, "the workspace was resized after the frame");
     launch_runs_all(z, 0);
     RG_CK(cudaDeviceSynchronize());
-    z.limit = RUN_ALL;
     return RG_OK;
 }
 
@@ -1221,7 +1221,7 @@ static rg_status write_all_values(Workspace& w)
 // from the rectangles, and what the device has must lie among the result in the same order.
 static rg_status exact_runs_entries(rg_scene* s, const Counters& c, int32_t what, std::vector<unsigned char>& out)
 {
-    Workspace& w = s->ws;
+    const Workspace& w = s->ws;
     const size_t n = (size_t)s->n, tiles = (size_t)w.last_tiles, tx = (size_t)w.last_tiles_x, ne = c.n_entries;
     const bool lists = w.last_lists[0] == w.vals[0].p && w.last_lists[1] == w.ranges.p; // not resized since
     std::vector<uint32_t> order(n), depth(n);

@@ -341,3 +341,25 @@ def test_inspection_reads_the_device_lists(n, stats):
             gs.inspect(binding.RG_INSPECT_VALUES)
     gs.render(cam, mode="exact", stats=stats)
     assert np.array_equal(_entries(gs)[1], v)
+
+
+@pytest.mark.parametrize("mode", ["roofgs", "exact"])
+def test_a_replayed_limited_frame_is_inspected_again(mode):
+    """A replay leaves values out again, and the state of unfinished tiles in their place: every inspection completes them."""
+    n, cam = 500_001, synth.tiny_camera(2048, 1537)
+    sc = _scene(n, 0.15, seed=5)
+    sc.opacities = np.full(n, 0.4, np.float32)
+    sc.means[n // 4:] *= np.float32(0.25)
+    gs = binding.Scene(sc)
+    out, _ = gs.render(cam, mode=mode, stats=True)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        gs.render(cam, mode=mode, out=out)
+    frames = []
+    for _ in range(3):
+        g.replay()
+        frames.append(_entries(gs))
+    for f in frames[1:]:
+        for x, y in zip(frames[0], f):
+            assert np.array_equal(x, y)
