@@ -238,9 +238,20 @@ static TileOrder tile_order(const Workspace& w, int tiles)
 // outweigh it below: 4K 100 k 260 / 265, 1080p 500 k 228 / 228 (exact 339 / 355).
 static constexpr int LIMIT_TILES = 12288, LIMIT_GAUSSIANS = 500000;
 
+// Bytes of runbuf for any tile grid of at most `tiles` tiles, so that a frame of another shape needs no allocation (in a
+// capture, on a server's slot) where its tiles fit: at most RUN_MAX_GRID rows; rows x run_pitch(cols) <= tiles + 31 rows.
+static size_t run_bytes(int64_t n, int64_t cap, int64_t tiles)
+{
+    const size_t side = (size_t)std::min<int64_t>(RUN_MAX_GRID, tiles), blocks = (size_t)((n + RUN_SLOTS - 1) / RUN_SLOTS);
+    const unsigned run_cap = (unsigned)key_items(n, cap);
+    const size_t none = run_chunk_cap(run_cap, 0, (unsigned)blocks), a_row = run_chunk_cap(run_cap, 1, (unsigned)blocks) - none;
+    const size_t words = 3 * side * blocks + side + none * run_pitch((int)side) + a_row * ((size_t)tiles + 31 * side);
+    return words * 4 + (none + a_row * side) * sizeof(RunChunk) + side * sizeof(RunRow) + 8 * 256;
+}
+
 // Arguments of runs.cu for a frame on workspace w: the runs live in the key buffers (list in
 // keys[0], the blocks' runs in keys[1]), the rest in runbuf. Returns the bytes of runbuf the frame
-// needs; the pointers are valid if runbuf has them.
+// needs (at most run_bytes); the pointers are valid if runbuf has them.
 size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
 {
     memset(&a, 0, sizeof(a));
@@ -324,10 +335,8 @@ rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameL
         RG_TRY(ensure(w.tsort, tilesort_matrix_bytes_max() + (size_t)tilesort_max_tiles() * 4, "tile counting sort"));
     }
     RG_TRY(ensure(w.gsort, depth_sort_views(w, n).bytes, "depth sort"));
-    if (runs_possible(F.lay, n)) {
-        RunArgs ra;
-        RG_TRY(ensure(w.runbuf, run_views(w, n, F.lay, ra), "tile-row runs"));
-    }
+    w.max_tiles = std::max(w.max_tiles, F.tiles);
+    RG_TRY(ensure(w.runbuf, run_bytes(n, w.cap, w.max_tiles), "tile-row runs"));
     return RG_OK;
 }
 
@@ -939,14 +948,9 @@ rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries)
     const int64_t max_tiles = (cap + sort_tile_items() - 1) / sort_tile_items();
     for (int k = 0; k < 2; k++) RG_TRY(ensure(scene->ws.sort_status[k], (size_t)max_tiles * 256 * 4, "sort status"));
     scene->ws.cap = cap;
-    if (scene->ws.last_tiles_x > 0) { // the last frame's grid can be captured next, without an allocation
-        Layout L;
-        memset(&L, 0, sizeof(L));
-        L.tiles_x = scene->ws.last_tiles_x;
-        L.tiles_y = scene->ws.last_tiles / scene->ws.last_tiles_x;
-        RunArgs ra;
-        if (runs_possible(L, scene->n)) RG_TRY(ensure(scene->ws.runbuf, run_views(scene->ws, scene->n, L, ra), "tile-row runs"));
-    }
+    // frames of the grids rendered so far can be captured next, without an allocation
+    if (scene->ws.max_tiles > 0)
+        RG_TRY(ensure(scene->ws.runbuf, run_bytes(std::max<int64_t>(scene->n, 1), cap, scene->ws.max_tiles), "tile-row runs"));
     return RG_OK;
 }
 

@@ -77,6 +77,7 @@ static_assert(CTRL_ALLOC % 16 == 0, "cleared 16 bytes at a time");
 // rg_render uses the scene's own workspace; a batch lane or a server slot owns one.
 struct Workspace {
     int64_t cap = 0;
+    int max_tiles = 0; // tiles of the largest grid it was sized for
     DevBuf keys[2], vals[2];
     DevBuf ranges;
     DevBuf ctrl; // Counters followed by hist[8][256] (twice: frame, depth sort)
@@ -119,6 +120,7 @@ struct Workspace {
                 for (int k = 0; k < EV_PER_FRAME; k++) cudaEventDestroy(ev[f][k]);
         ev_init = false;
         cap = 0;
+        max_tiles = 0;
     }
 };
 

@@ -103,3 +103,33 @@ def test_a_reserved_workspace_can_be_captured(n, mode):
     torch.cuda.synchronize()
     assert torch.equal(out, want)
     gs.check()
+
+
+@pytest.mark.parametrize("mode", ["roofgs", "exact"])
+@pytest.mark.parametrize("n", [5_000, 40_000])
+def test_any_grid_within_the_largest_can_be_captured(n, mode):
+    """A view whose tiles are no more than an earlier one's is captured without an allocation, whatever its shape, and so is
+    every earlier view after a reserve."""
+    wide, tall, small = synth.tiny_camera(960, 64), synth.tiny_camera(64, 960), synth.tiny_camera(160, 120)
+    sc = synth.tiny_scene(n, seed=4)
+    other = binding.Scene(sc)
+    want = [other.render(c, mode=mode).clone() for c in (wide, tall, small)]
+    gs = binding.Scene(sc)
+    gs.render(wide, mode=mode)
+
+    def captured(cam):
+        out = torch.empty((3, cam.height, cam.width), device="cuda")
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            gs.render(cam, mode=mode, out=out)
+        g.replay()
+        torch.cuda.synchronize()
+        return out
+
+    assert torch.equal(captured(tall), want[1])
+    gs.render(small, mode=mode)
+    gs.reserve(6_000_000)
+    for cam, w in zip((wide, tall, small), want):
+        assert torch.equal(captured(cam), w)
+    gs.check()
