@@ -178,8 +178,15 @@ typedef struct {
  */
 rg_status rg_scene_create(const rg_scene_desc* desc, void* stream, rg_scene** out);
 
-/* Free every device buffer of the scene (synchronises the device). NULL is a no-op. */
+/*
+ * Release every device buffer of the scene (synchronises the device). NULL is a no-op. The library keeps released
+ * buffers of at most 128 MiB each, 512 MiB in all, for its next allocations (programs that make and drop a scene per
+ * step); those that 512 later releases did not take up go back to CUDA, and all do when an allocation of the library
+ * fails or at rg_trim.
+ */
 rg_status rg_scene_destroy(rg_scene* scene);
+/* Give the kept buffers of every device back to CUDA, for a program whose other allocations need the room. */
+rg_status rg_trim(void);
 
 /*
  * Scene files (checkpoint / resume of a resident scene; the paper has no counterpart):

@@ -48,7 +48,7 @@ EXPORTS = ["rg_scene_create", "rg_scene_destroy", "rg_scene_reserve", "rg_render
            "rg_stage_times", "rg_inspect", "rg_eval_fast_exp", "rg_render_batch", "rg_backward", "rg_submit",
            "rg_poll", "rg_last_error", "rg_version", "rg_sort_pairs_noalloc", "rg_batch_plan_info",
            "rg_server_create", "rg_server_destroy", "rg_server_stats", "rg_server_reset_stats", "rg_scene_save",
-           "rg_scene_load"]
+           "rg_scene_load", "rg_trim"]
 
 
 class RgError(RuntimeError):
@@ -116,6 +116,7 @@ def lib():
         P = C.c_void_p
         L.rg_scene_create.argtypes = [C.POINTER(RgSceneDesc), P, C.POINTER(P)]
         L.rg_scene_destroy.argtypes = [P]
+        L.rg_trim.argtypes = []
         L.rg_scene_reserve.argtypes = [P, C.c_int64]
         L.rg_render.argtypes = [P, C.POINTER(RgCamera), C.POINTER(RgOpts), P, C.POINTER(RgStats), P]
         L.rg_scene_check.argtypes = [P, P]
@@ -366,6 +367,11 @@ def eval_fast_exp(P, stream=None):
     out = torch.empty_like(P)
     check(lib().rg_eval_fast_exp(C.c_void_p(P.data_ptr()), C.c_void_p(out.data_ptr()), P.numel(), _stream_ptr(stream)))
     return out
+
+
+def trim():
+    """Give the device memory that the library keeps from dropped scenes back to CUDA (rg_trim)."""
+    check(lib().rg_trim())
 
 
 def version() -> int:

@@ -58,6 +58,18 @@ KeptBlock take_kept(size_t k)
 rg::DeviceIdle::DeviceIdle() { t_device_idle++; }
 rg::DeviceIdle::~DeviceIdle() { t_device_idle--; }
 
+bool rg::device_trim()
+{
+    std::vector<KeptBlock> all;
+    {
+        std::lock_guard<std::mutex> lock(g_kept_mu);
+        all.swap(g_kept);
+        g_kept_bytes = 0;
+    }
+    for (const KeptBlock& b : all) cudaFree(b.p);
+    return !all.empty();
+}
+
 cudaError_t rg::device_take(void** p, size_t& bytes, int& dev)
 {
     dev = 0;
@@ -79,14 +91,7 @@ cudaError_t rg::device_take(void** p, size_t& bytes, int& dev)
     cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation) { // give back what is kept, and once more
         cudaGetLastError();
-        std::vector<KeptBlock> all;
-        {
-            std::lock_guard<std::mutex> lock(g_kept_mu);
-            all.swap(g_kept);
-            g_kept_bytes = 0;
-        }
-        for (const KeptBlock& b : all) cudaFree(b.p);
-        if (!all.empty()) e = cudaMalloc(p, bytes);
+        if (device_trim()) e = cudaMalloc(p, bytes);
     }
     if (e != cudaSuccess) cudaGetLastError();
     return e;
@@ -932,6 +937,12 @@ rg_status rg_scene_destroy(rg_scene* scene)
         drop_plans_of(scene);
         destroy_scene(scene);
     }
+    return RG_OK;
+}
+
+rg_status rg_trim(void)
+{
+    device_trim();
     return RG_OK;
 }
 

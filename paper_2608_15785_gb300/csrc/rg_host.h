@@ -35,6 +35,8 @@ rg_status fail(rg_status s, const std::string& msg);
 // is synchronised first (as cudaFree does), unless the caller has done so (DeviceIdle).
 cudaError_t device_take(void** p, size_t& bytes, int& dev);
 void device_give_back(void* p, size_t bytes, int dev);
+// gives every kept block back to CUDA (those of other devices too); false if there was none
+bool device_trim();
 
 // While one lives, this thread's releases need not synchronise: no work of theirs is in flight.
 struct DeviceIdle {

@@ -133,3 +133,19 @@ def test_any_grid_within_the_largest_can_be_captured(n, mode):
     for cam, w in zip((wide, tall, small), want):
         assert torch.equal(captured(cam), w)
     gs.check()
+
+
+def test_trim_gives_the_kept_memory_back():
+    """A dropped scene's buffers stay with the library until rg_trim; then other allocators have them, and a new scene is
+    made as before."""
+    cam = synth.tiny_camera(160, 120)
+    sc = synth.tiny_scene(200_000, seed=3)  # 40 MB of SH coefficients
+    gs = binding.Scene(sc)
+    want = gs.render(cam).clone()
+    torch.cuda.synchronize()
+    gs.close()
+    kept = torch.cuda.mem_get_info()[0]
+    binding.trim()
+    assert torch.cuda.mem_get_info()[0] - kept >= 30 << 20
+    binding.trim()  # nothing left
+    assert torch.equal(binding.Scene(sc).render(cam), want)
