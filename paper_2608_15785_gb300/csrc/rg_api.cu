@@ -294,10 +294,9 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     return at;
 }
 
-DepthSortViews depth_sort_views(const Workspace& w, int64_t n)
+static DepthSortViews depth_sort_at(unsigned char* p, int64_t n)
 {
     DepthSortViews v;
-    unsigned char* const p = w.gsort.as<unsigned char>();
     size_t at = 0;
     auto part = [&](size_t words) {
         unsigned* q = reinterpret_cast<unsigned*>(p + at);
@@ -313,35 +312,60 @@ DepthSortViews depth_sort_views(const Workspace& w, int64_t n)
     return v;
 }
 
-rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameLayout& F, int64_t cap)
+DepthSortViews depth_sort_views(const Workspace& w, int64_t n) { return depth_sort_at(w.gsort.as<unsigned char>(), n); }
+
+WorkspaceBytes workspace_bytes(int64_t n_gauss, int mode, int64_t tiles, int64_t cap)
 {
     const int64_t n = n_gauss > 0 ? n_gauss : 1;
-    if (cap > MAX_CAP) return fail(RG_ERR_CAPACITY, "entry capacity above 2^30 - 1");
-    for (int k = 0; k < 2; k++) RG_TRY(ensure(w.keys[k], (size_t)key_items(n, std::max(cap, w.cap)) * 8, "keys"));
-    if (cap > w.cap || !w.vals[0].p) {
-        for (int k = 0; k < 2; k++) RG_TRY(ensure(w.vals[k], (size_t)cap * 4, "values"));
-        const int64_t max_tiles = (cap + sort_tile_items() - 1) / sort_tile_items();
-        for (int k = 0; k < 2; k++) RG_TRY(ensure(w.sort_status[k], (size_t)max_tiles * 256 * 4, "sort status"));
-        w.cap = cap;
-    }
-    RG_TRY(ensure(w.ranges, (size_t)F.tiles * (sizeof(uint2) + (8 + 2) * 4), "ranges and tile order"));
-    RG_TRY(ensure(w.ctrl, CTRL_ALLOC, "counters"));
+    WorkspaceBytes b;
+    b.keys = (size_t)key_items(n, cap) * 8;
+    b.vals = (size_t)cap * 4;
+    b.sort_status = (size_t)((cap + sort_tile_items() - 1) / sort_tile_items()) * 256 * 4;
+    b.ranges = (size_t)tiles * (sizeof(uint2) + (8 + 2) * 4);
+    b.ctrl = CTRL_ALLOC;
     const int64_t fe_blocks = (n + frontend_block_threads() - 1) / frontend_block_threads();
-    RG_TRY(ensure(w.lb_status, (size_t)(std::max<int64_t>(fe_blocks, (n + 2047) / 2048) + 1) * 8, "look-back status"));
+    b.lb_status = (size_t)(std::max<int64_t>(fe_blocks, (n + 2047) / 2048) + 1) * 8;
     if (mode == RG_MODE_EXACT) {
-        RG_TRY(ensure(w.erec, (size_t)n * 48, "records"));
-        RG_TRY(ensure(w.rect, (size_t)n * 16, "rect"));
-        RG_TRY(ensure(w.touched, (size_t)n * 4, "touched"));
+        b.erec = (size_t)n * 48;
+        b.rect = (size_t)n * 16;
+        b.touched = (size_t)n * 4;
     } else {
-        RG_TRY(ensure(w.rec, (size_t)n * 32, "records"));
+        b.rec = (size_t)n * 32;
         // the per-tile counting sort's count matrix (chunks x tiles, at most SMs x one block's shared
         // memory for any tile count) and tile totals: sized for any frame, so a workspace shared by
         // views of several resolutions never runs short
-        RG_TRY(ensure(w.tsort, tilesort_matrix_bytes_max() + (size_t)tilesort_max_tiles() * 4, "tile counting sort"));
+        b.tsort = tilesort_matrix_bytes_max() + (size_t)tilesort_max_tiles() * 4;
     }
-    RG_TRY(ensure(w.gsort, depth_sort_views(w, n).bytes, "depth sort"));
+    b.gsort = depth_sort_at(nullptr, n).bytes;
+    b.runs = run_bytes(n, cap, tiles);
+    return b;
+}
+
+rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameLayout& F, int64_t cap)
+{
+    if (cap > MAX_CAP) return fail(RG_ERR_CAPACITY, "entry capacity above 2^30 - 1");
+    const bool grow = cap > w.cap || !w.vals[0].p;
+    const WorkspaceBytes b = workspace_bytes(n_gauss, mode, std::max(w.max_tiles, F.tiles), std::max(cap, w.cap));
+    for (int k = 0; k < 2; k++) RG_TRY(ensure(w.keys[k], b.keys, "keys"));
+    if (grow) {
+        for (int k = 0; k < 2; k++) RG_TRY(ensure(w.vals[k], b.vals, "values"));
+        for (int k = 0; k < 2; k++) RG_TRY(ensure(w.sort_status[k], b.sort_status, "sort status"));
+        w.cap = cap;
+    }
+    RG_TRY(ensure(w.ranges, b.ranges, "ranges and tile order"));
+    RG_TRY(ensure(w.ctrl, b.ctrl, "counters"));
+    RG_TRY(ensure(w.lb_status, b.lb_status, "look-back status"));
+    if (mode == RG_MODE_EXACT) {
+        RG_TRY(ensure(w.erec, b.erec, "records"));
+        RG_TRY(ensure(w.rect, b.rect, "rect"));
+        RG_TRY(ensure(w.touched, b.touched, "touched"));
+    } else {
+        RG_TRY(ensure(w.rec, b.rec, "records"));
+        RG_TRY(ensure(w.tsort, b.tsort, "tile counting sort"));
+    }
+    RG_TRY(ensure(w.gsort, b.gsort, "depth sort"));
+    RG_TRY(ensure(w.runbuf, b.runs, "tile-row runs"));
     w.max_tiles = std::max(w.max_tiles, F.tiles);
-    RG_TRY(ensure(w.runbuf, run_bytes(n, w.cap, w.max_tiles), "tile-row runs"));
     return RG_OK;
 }
 

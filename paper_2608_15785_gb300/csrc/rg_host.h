@@ -170,6 +170,16 @@ rg_status tile_shape(const rg_render_opts* o, int& tw, int& th);
 rg_status make_layout(const rg_camera* c, FrameLayout& f, int tw = TILE, int th = TILE);
 // grows a workspace for a frame of n_gauss Gaussians, F's tile grid and `cap` entries
 rg_status ensure_workspace(Workspace& w, int64_t n_gauss, int mode, const FrameLayout& F, int64_t cap);
+// bytes of each of a workspace's buffers for n_gauss Gaussians, any grid of at most `tiles` tiles and `cap` entries
+struct WorkspaceBytes {
+    size_t keys = 0, vals = 0, sort_status = 0; // of each of two
+    size_t ranges = 0, ctrl = 0, lb_status = 0, erec = 0, rect = 0, touched = 0, rec = 0, tsort = 0, gsort = 0, runs = 0;
+    size_t total() const
+    {
+        return 2 * (keys + vals + sort_status) + ranges + ctrl + lb_status + erec + rect + touched + rec + tsort + gsort + runs;
+    }
+};
+WorkspaceBytes workspace_bytes(int64_t n_gauss, int mode, int64_t tiles, int64_t cap);
 // creates the stage events of a workspace on first use
 void init_events(Workspace& w);
 // enqueues one frame on `st` (arguments and workspace already checked); out == nullptr stops

@@ -196,6 +196,7 @@ rg_status rg_server_create(rg_scene* const* scenes, int32_t n_scenes, const rg_s
     sv->max_w = cfg->max_width;
     sv->max_h = cfg->max_height;
     sv->budget = cfg->memory_budget > 0 ? cfg->memory_budget : (8ll << 30);
+    device_trim(); // (a kept block may be up to twice as large as what it is taken for)
     // calibrate one slot: the largest scene at the largest resolution, pose of the first camera
     int big = 0;
     for (int k = 1; k < n_scenes; k++)
@@ -227,16 +228,16 @@ rg_status rg_server_create(rg_scene* const* scenes, int32_t n_scenes, const rg_s
         RG_CK(cudaMemsetAsync(scenes[big]->sticky.p, 0, sizeof(Sticky), probe->stream));
     }
     const int64_t cap = std::min<int64_t>(MAX_CAP, std::max<int64_t>(1 << 20, entries + entries / 2 + 1024));
-    const int64_t ngauss = scenes[big]->n;
     FrameLayout largest; // the tile grid of the largest request
     largest.lay.tiles_x = (sv->max_w + TILE - 1) / TILE;
     largest.lay.tiles_y = (sv->max_h + TILE - 1) / TILE;
     const int64_t tiles = (int64_t)largest.lay.tiles_x * largest.lay.tiles_y;
     largest.tiles = (int)tiles;
-    // bytes of one slot: 2 x (keys 8 B + values 4 B) per entry, sort status, per-Gaussian arrays (RoofGS:
-    // records, depth order), ranges, image
-    sv->slot_bytes = cap * 24 + (cap / 4096 + 1) * 2048 + ngauss * (sv->mode == RG_MODE_EXACT ? 92 : 112) +
-                     tiles * 8 + (int64_t)out_bytes;
+    // bytes of one slot: the workspace that serves every scene (that of the largest one, whose buffers are all at least as
+    // large but the runs' beside a scene of at most 32,768 Gaussians), and the image
+    WorkspaceBytes slot = workspace_bytes(scenes[big]->n, sv->mode, tiles, cap);
+    for (int j = 0; j < n_scenes; j++) slot.runs = std::max(slot.runs, workspace_bytes(scenes[j]->n, sv->mode, tiles, cap).runs);
+    sv->slot_bytes = (int64_t)(slot.total() + out_bytes);
     int nslots = cfg->max_slots > 0 ? cfg->max_slots : 8;
     nslots = (int)std::max<int64_t>(1, std::min<int64_t>(nslots, sv->budget / std::max<int64_t>(sv->slot_bytes, 1)));
     for (int k = 0; k < nslots; k++) {

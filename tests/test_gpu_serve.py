@@ -115,3 +115,28 @@ def test_result_delivered_into_pinned_host_memory(scenes):
     torch.cuda.synchronize()
     assert torch.equal(host, ref.cpu())
     srv.close()
+
+
+@pytest.mark.parametrize("mode", ["roofgs", "exact"])
+def test_the_memory_budget_holds(mode):
+    """A slot takes the bytes that admission books for it (to 2 MiB for each of its buffers, what CUDA rounds up to), also
+    with far more Gaussians than entries, and the budget limits the slots."""
+    scene = binding.Scene(synth.tiny_scene(2_000_000, seed=1),
+                          storage=binding.RG_STORE_FP32 if mode == "exact" else binding.RG_STORE_COMPACT)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    binding.trim()
+    before = free()
+    srv = binding.Server([scene], 640, 360, mode=mode, max_slots=3)
+    st, used = srv.stats(), before - free()
+    assert st["slots"] == 3
+    assert used <= 3 * (st["slot_bytes"] + 18 * (2 << 20))
+    srv.close()
+    srv = binding.Server([scene], 640, 360, mode=mode, max_slots=8, memory_budget=int(2.5 * st["slot_bytes"]))
+    assert srv.stats()["slots"] == 2
+    srv.close()
