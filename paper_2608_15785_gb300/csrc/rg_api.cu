@@ -754,6 +754,8 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
         NvtxScope r_("rg sort");
         if (!ra.tot && out && !count && F.tiles > LIMIT_TILES && n > LIMIT_GAUSSIANS) {
             ra.limit = RUN_LIMIT;
+            ra.tw = F.cam.tw;
+            ra.th = F.cam.th;
             ra.rec = mode == RG_MODE_EXACT ? w.erec.as<float4>() : w.rec.as<float4>();
             ra.rest_flag = reinterpret_cast<unsigned*>(ra.ranges + F.tiles) + 8 * F.tiles;
         }

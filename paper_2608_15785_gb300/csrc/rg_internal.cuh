@@ -634,6 +634,7 @@ struct RunArgs {
                        // the tile is flagged; row by row as row_limit says
     unsigned* row_limit; // [rows] limit or RUN_ALL
     const float4* rec; // the front end's records (FrontendArgs::rec, ExactArgs::rec)
+    int tw, th;        // tile shape
     unsigned* rest_flag; // [rows * cols] nonzero: the rasterizer needs more of the tile's entries (cleared with the ranges)
     int rest;          // 1: the second launch
     uint2* ranges;     // [rows * cols] [start, end) of every tile, [0, 0) if empty

@@ -477,10 +477,14 @@ __global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
 }
 
 
-// A row of a limited frame is limited from this mean opacity of its entries. Per pass, limited / not, opacities drawn
-// around 0.5 (trained scenes) and scaled: 4K, 1 M Gaussians x 1 579 / 605 us, x 0.5 743 / 764, x 0.35 852 / 855, x 0.1
-// 1243 / 1123; 2560 x 1440, 2 M x 1 513 / 548, x 0.5 660 / 661, x 0.35 752 / 728 (exact mode alike)
-constexpr float LIMIT_OPACITY = 0.3f;
+// A row of a limited frame is limited where RUN_LIMIT of its entries bring this optical depth to a pixel on average (a pixel
+// is finished at ln 1e4 = 9.2, a tile when its last pixel is). Opacity alone does not tell: small Gaussians cover little of a
+// tile. Us per RoofGS frame, all entries / limited everywhere / from a depth of 12 / of 24, at 4K: opacities around 0.5 (trained scenes),
+// 3 M 1291 / 1046 / 1046 / 1047, all of them x 0.5 1468 / 1263 / 1263 / 1468, x 0.35 1599 / 1530 / 1615 / 1596, x 0.1 2238 / 2558 / 2239 /
+// 2238; specks of opacity 0.5 in the middle 6 % of the image, 2 px: 6 M 1148 / 1438 / 1151 / 1147, 3 M 686 / 840 / 686 / 685, 4 px, 3 M
+// 714 / 648 / 650 / 714; of opacity 0.9, 2 px, 6 M 1074 / 1097 / 1096 / 1073. 8: x 0.2 1997 against 1847. (Exact mode alike.) A rule
+// with the depth's variance beside its mean (z of 2 and 3) chose no better.
+constexpr float LIMIT_DEPTH = 12.0f;
 
 // A frame beyond its capacity: the entries kept in the rows before `row`, and in all (called by one warp).
 __device__ __forceinline__ void kept_before(const RunArgs& a, unsigned row, unsigned long long& before, unsigned long long& all)
@@ -498,6 +502,17 @@ __device__ __forceinline__ void kept_before(const RunArgs& a, unsigned row, unsi
     }
 }
 
+// What an entry of a Gaussian of opacity o and Sigma' = (sa, sb, sc) adds to the optical depth of its tile's pixels on average:
+// the integral of -ln(1 - o exp(-d^T Sigma'^-1 d / 2)) is 2 pi sqrt(det Sigma') Li2(o), spread over the tiles of the box of
+// alpha >= 1/255. (Li2(o) = o + o^2 / 4 + o^3 / 9 + ...: to 2 % by the cubic below.)
+__device__ __forceinline__ float entry_depth(float o, float sa, float sc, float det, float tw, float th)
+{
+    const float t = 2.0f * (__logf(fmaxf(o, 1e-6f)) + LN255F);
+    const float tiles = (__fdividef(2.0f * __fsqrt_rn(t * sa), tw) + 1.0f) * (__fdividef(2.0f * __fsqrt_rn(t * sc), th) + 1.0f);
+    const float x = __fdividef(6.2831853f * __fsqrt_rn(det) * o * (1.0f + o * (0.2f + 0.4f * o * o)), tiles * 256.0f);
+    return x >= 0.0f && x < 1e30f ? x : 0.0f; // (0 for what is no number)
+}
+
 // One block per tile row: OFF_SEGS segments of the row's chunks x OFF_COLS columns at a time.
 constexpr int OFF_SEGS = 4, OFF_COLS = 256;
 
@@ -507,6 +522,7 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
     __shared__ unsigned s_first[OFF_COLS];
     __shared__ unsigned s_w[OFF_COLS / 32];
     __shared__ unsigned s_start;
+    __shared__ float2 s_depth[OFF_COLS / 32];
     grid_dependency_wait();
     const unsigned row = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const unsigned long long cap = (unsigned long long)a.cap;
@@ -538,25 +554,35 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
             }
         }
     }
-    // A limited frame pays where pixels are finished early, under opaque Gaussians: the mean opacity of the row's
-    // entries, from 256 runs spread over its list, decides
-    if (a.limit != RUN_ALL && warp == OFF_SEGS * OFF_COLS / 32 - 2) {
+    // A limited frame pays where pixels are finished early: the optical depth of the row's entries, from 256 runs spread over
+    // its list, decides (one run per lane of eight warps: one warp for all of them took 10 us)
+    if (a.limit != RUN_ALL && sg == OFF_SEGS / 2) {
         float sum = 0.0f, len = 0.0f;
-#pragma unroll
-        for (unsigned k = 0; k < 8; k++) {
-            if (r.runs == 0) break;
-            const uint2 q = __ldg(&a.list[r.base + (unsigned)((unsigned long long)r.runs * (32u * k + lane) / 256u)]);
-            const float o = a.box_total ? __ldg(&a.rec[3 * (size_t)q.x + 1].w) : __expf(__ldg(&a.rec[2 * (size_t)q.x + 1].y));
-            const float n = (float)((q.y >> 16) + 1u - (q.y & 0xffffu)); // (0 for a dropped run)
-            sum += o * n;
-            len += n;
+        if (r.runs) {
+            const uint2 q = __ldg(&a.list[r.base + (unsigned)((unsigned long long)r.runs * c / OFF_COLS)]);
+            float o, sa, sc, det;
+            if (a.box_total) {
+                const float4 e = __ldg(&a.rec[3 * (size_t)q.x + 1]); // -Sigma'_yy / (2 det), Sigma'_xy / Sigma'_yy, -1 / (2 Sigma'_yy)
+                o = e.w;
+                sc = __fdividef(-0.5f, e.z);
+                det = __fdividef(-0.5f * sc, e.x);
+                sa = __fdividef(det, sc) + e.y * e.y * sc;
+            } else {
+                const float4 e = __ldg(&a.rec[2 * (size_t)q.x]), f = __ldg(&a.rec[2 * (size_t)q.x + 1]); // conic (a, b, c)
+                o = __expf(f.y);
+                det = __fdividef(1.0f, fmaf(e.z, f.x, -0.25f * e.w * e.w));
+                sa = f.x * det;
+                sc = e.z * det;
+            }
+            len = (float)((q.y >> 16) + 1u - (q.y & 0xffffu)); // (0 for a dropped run)
+            sum = entry_depth(o, sa, sc, det, (float)a.tw, (float)a.th) * len;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            len += __shfl_xor_sync(0xffffffffu, len, o);
+        for (int d = 16; d > 0; d >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, d);
+            len += __shfl_xor_sync(0xffffffffu, len, d);
         }
-        if (lane == 0) a.row_limit[row] = sum >= LIMIT_OPACITY * len ? a.limit : RUN_ALL;
+        if (lane == 0) s_depth[c / 32] = make_float2(sum, len);
     }
     unsigned run = 0; // entries of the row's earlier columns
     for (int g = 0; g < a.cols; g += OFF_COLS) {
@@ -607,6 +633,15 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
         }
         run += row_all;
         __syncthreads();
+    }
+    if (tid == 0 && a.limit != RUN_ALL) {
+        float sum = 0.0f, len = 0.0f;
+#pragma unroll
+        for (int q = 0; q < OFF_COLS / 32; q++) {
+            sum += s_depth[q].x;
+            len += s_depth[q].y;
+        }
+        a.row_limit[row] = sum * (float)RUN_LIMIT >= LIMIT_DEPTH * len ? a.limit : RUN_ALL;
     }
 }
 

@@ -363,3 +363,84 @@ def test_a_replayed_limited_frame_is_inspected_again(mode):
     for f in frames[1:]:
         for x, y in zip(frames[0], f):
             assert np.array_equal(x, y)
+
+
+def _frame_us(gs, cam, out):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for _ in range(4):
+        a.record()
+        for _ in range(10):
+            gs.render(cam, out=out, flags=binding.RG_FLAG_QUAD_PIXEL)
+        b.record()
+        b.synchronize()
+        best = min(best, 100.0 * a.elapsed_time(b))
+    return best
+
+
+def test_limited_frames_of_specks_are_not_slower():
+    """Specks of opacity 0.5, two pixels wide, in the middle of a 4K frame: most of their tiles need more than the first 512
+    entries, and a frame just above the largest whose entries are all written (500,000 Gaussians) may not pay for a second
+    pass over nearly all of them: that cost a quarter; 15 % are allowed for noise and the two launches."""
+    rng = np.random.default_rng(0)
+    w, h, n = 3840, 2160, 500_002
+    cam = synth.Camera(np.eye(3, dtype=np.float32).reshape(9), np.zeros(3, np.float32), w / 2.0, w / 2.0, (w - 1) / 2.0,
+                       (h - 1) / 2.0, w, h, 0.5, 50.0)
+    sc = synth.tiny_scene(n, seed=0)
+    z = rng.uniform(2, 20, n)
+    px = np.array([w, h]) / 2 + rng.normal(size=(n, 2)) * 0.02 * np.array([w, h])
+    sc.means = np.append((px - [cam.cx, cam.cy]) / cam.fx * z[:, None], z[:, None], 1).astype(np.float32)
+    sc.scales = (rng.uniform(1.5, 2.5, (n, 3)) * (z / cam.fx)[:, None]).astype(np.float32)
+    sc.opacities = np.full(n, 0.5, np.float32)
+    limited, full = binding.Scene(sc), binding.Scene(sc.subset(np.arange(500_000)))
+    out, _ = limited.render(cam, stats=True)
+    full.render(cam, stats=True)
+    assert _frame_us(limited, cam, out) <= 1.15 * _frame_us(full, cam, torch.empty_like(out))
+
+
+@pytest.mark.parametrize("wh,tile", [((2048, 1552), (16, 16)), ((1999, 1777), (32, 8)), ((1777, 1999), (8, 32))])
+def test_limited_frames_resume_unfinished_tiles(wh, tile):
+    """Rows that are limited, their left part being opaque soon, with tiles on the right whose pixels are still unfinished after
+    every one of their entries: image and entries as the ordered front end's and the counting launch's."""
+    rng = np.random.default_rng(4)
+    w, h, n = wh[0], wh[1], 600_000
+    cam = synth.Camera(np.eye(3, dtype=np.float32).reshape(9), np.zeros(3, np.float32), w / 2.0, w / 2.0, (w - 1) / 2.0,
+                       (h - 1) / 2.0, w, h, 0.5, 50.0, np.array([0.2, 0.9, 0.4], np.float32))
+    left = np.arange(n) % 3 > 0
+    x = np.where(left, rng.uniform(0.05, 0.4, n), rng.uniform(0.55, 0.75, n)) * w
+    y = rng.uniform(0.45, 0.55, n) * h
+    z, size = rng.uniform(2, 20, n), np.where(left, 5.0, 0.4)  # pixels
+    sc = synth.tiny_scene(n, seed=2)
+    sc.means = np.stack([(x - cam.cx) / cam.fx * z, (y - cam.cy) / cam.fy * z, z], 1).astype(np.float32)
+    sc.scales = np.repeat((size * z / cam.fx)[:, None], 3, 1).astype(np.float32)
+    sc.opacities = np.where(left, 0.9, 0.012).astype(np.float32)
+    # the optical depth that 512 entries bring, as the rule estimates it, in the rows between 0.46 and 0.54 of the height: far
+    # above its 12
+    s2, o = size ** 2 + 0.3, sc.opacities.astype(np.float64)
+    box = 2 * np.sqrt(2 * np.log(255 * o) * s2)
+    tiles = (box / tile[0] + 1) * (box / tile[1] + 1)
+    depth = 2 * np.pi * s2 * sum(o ** k / k ** 2 for k in range(1, 60)) / 256
+    for r in np.linspace(0.46, 0.54, 9):
+        row = np.abs(y - r * h) < 16
+        assert 512 * depth[row].sum() / tiles[row].sum() > 20
+    gs = binding.Scene(sc)
+    for flags in (0, binding.RG_FLAG_QUAD_PIXEL, binding.RG_FLAG_SINGLE_PIXEL | binding.RG_FLAG_EXACT_EXP):
+        gs.render(cam, flags=flags, tile=tile, stats=True)
+        a = gs.render(cam, flags=flags, tile=tile)
+        ea = _entries(gs)
+        b = gs.render(cam, flags=flags | binding.RG_FLAG_ORDERED_FRONT_END, tile=tile)
+        for p, q in zip(ea, _entries(gs)):
+            assert np.array_equal(p, q)
+        assert torch.equal(a, b)
+    b, st = gs.render(cam, mode="exact", tile=tile, stats=True)
+    r = gs.inspect(binding.RG_INSPECT_RANGES).reshape(-1, 2).astype(np.int64)
+    per_tile = (r[:, 1] - r[:, 0]).reshape(st["tiles_y"], st["tiles_x"])
+    a = gs.render(cam, mode="exact", tile=tile).clone()
+    assert torch.equal(a, b)
+    # unfinished: the background shows through
+    cam.bg = np.zeros(3, np.float32)
+    through = (a - gs.render(cam, mode="exact", tile=tile))[1].cpu().numpy() / 0.9
+    ty, tx = int(0.5 * h) // tile[1], int(0.65 * w) // tile[0]
+    assert per_tile[ty, tx] > 512
+    assert through[ty * tile[1]:(ty + 1) * tile[1], tx * tile[0]:(tx + 1) * tile[0]].max() > 1e-2
+    gs.check()
