@@ -35,7 +35,10 @@ constexpr int RUN_WARPS = RUN_THREADS / 32;
 constexpr int CHUNK_RUNS = 2048;                // runs of a chunk at most: 64 per lane of a warp
 constexpr int CHUNK_STEP = CHUNK_RUNS - RUN_SLOTS; // a chunk ends with the block that reaches this many
 constexpr int CHUNK_BLOCKS = 1024;              // blocks of a chunk at most (sparse tile rows)
-constexpr int COLS = 120;                       // tile columns expanded at a time (five blocks per SM)
+// tile columns expanded at a time: the most that five blocks per SM leave room for (45 KB each). k_run_offsets and k_run_expand with
+// 112 / 120 / 128: 2048 x 1152 37.8 / 37.7 / 35.6 us, 2560 x 1440 46.9 / 47.6 / 46.5, 5120 x 2880 144.4 / 146.3 / 143.5, 4K 71.3 / 69.4 / 68.8,
+// 1366 x 768 (86 columns) 25.9 / 25.9 / 25.8; 64 to 88 with five or six blocks took 1 to 3 % more at 4K
+constexpr int COLS = 128;
 constexpr int PITCH = CHUNK_RUNS / 32 + 2;      // words per column: 64 masks, padded (8-byte loads, no bank conflicts)
 
 // chunks a tile row of a small frame has at most: its row r has chunks r * small_chunks(blocks) and up

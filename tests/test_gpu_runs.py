@@ -444,3 +444,18 @@ def test_limited_frames_resume_unfinished_tiles(wh, tile):
     assert per_tile[ty, tx] > 512
     assert through[ty * tile[1]:(ty + 1) * tile[1], tx * tile[0]:(tx + 1) * tile[0]].max() > 1e-2
     gs.check()
+
+
+@pytest.mark.parametrize("cols", [127, 128, 129, 136, 137, 256, 257])
+def test_windows_of_columns(cols):
+    """Grids about a window of the expansion (128 tile columns) and two, a small frame and a larger one: entries and image as the
+    ordered front end's."""
+    cam = synth.tiny_camera(16 * cols - 3, 90, bg=(0.2, 0.1, 0.3))
+    for n in (6_000, 36_000):
+        gs = binding.Scene(_scene(n, 2.0, seed=cols))
+        gs.render(cam, stats=True)
+        a = gs.render(cam)
+        ea = _entries(gs)
+        assert torch.equal(a, gs.render(cam, flags=binding.RG_FLAG_ORDERED_FRONT_END))
+        for x, y in zip(ea, _entries(gs)):
+            assert np.array_equal(x, y)
