@@ -572,6 +572,7 @@ __global__ void __launch_bounds__(E_THREADS) k_raster_exact_count(RasterArgs a)
     __shared__ float4 s_q[E_THREADS];
     __shared__ float4 s_rgb[E_THREADS];
     grid_dependency_wait();
+    if (a.count->n_entries_total > (unsigned long long)a.cap) return; // the caller grows the workspace and renders again
     const int tile = blockIdx.x;
     const int tx = tile % a.tiles_x, ty = tile / a.tiles_x;
     const int x0 = tx * a.cam.tw, y0 = ty * a.cam.th;

@@ -808,6 +808,7 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
     r.count = count ? ctr : nullptr;
     if (mode == RG_MODE_EXACT) {
         r.erec = w.erec.as<float4>();
+        r.cap = w.cap;
         if (runs) raster_runs(ra, r);
         NvtxScope r_("rg raster");
         launch_raster_exact(r, &ra, st);

@@ -791,6 +791,7 @@ struct RasterArgs {
     unsigned* rest_count;
     unsigned* rest_flag;  // [tiles] RunArgs::rest_flag
     Counters* count;      // non-null: count evaluated / blended pairs (separate kernel variant)
+    long long cap;        // entries the workspace holds (exact counting launches)
 };
 // runs: of a limited frame (RasterArgs::limit), else unused
 void launch_raster_roofgs(const RasterArgs& a, const RunArgs* runs, cudaStream_t s);
