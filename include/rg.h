@@ -145,6 +145,8 @@ typedef struct {
  * is invalid, kernels finish with in-bounds writes only, and the next rg_scene_check (or this
  * call, given stats) returns RG_ERR_TIMEOUT. The scene renders normally afterwards. */
 #define RG_FLAG_TEST_STALL_SORT (1u << 10)
+/* the same for the sort of the Gaussians by depth (rg_render; frames that have one) */
+#define RG_FLAG_TEST_STALL_DEPTH (1u << 15)
 
 typedef struct {
     int32_t mode;   /* RG_MODE_EXACT or RG_MODE_ROOFGS */

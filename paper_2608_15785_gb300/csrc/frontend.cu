@@ -582,6 +582,12 @@ __device__ __forceinline__ unsigned emit_runs(const RunArgs& r, const unsigned v
     return __reduce_or_sync(0xffffffffu, vis);
 }
 
+// the depth sort's error bits, which are the frame's too (one thread of the grid reads them)
+__device__ __forceinline__ unsigned depth_error(const RunArgs& r)
+{
+    return blockIdx.x == 0 && threadIdx.x == 0 ? r.depth_ctr->error : 0u;
+}
+
 // Resident blocks per SM: 5 (48 registers). What shared memory leaves of the L1 holds the depth-ordered
 // gathers, so more blocks cost more than they hide, above all with the per-row words of 8K: 4 / 5 / 6
 // blocks 213 / 196 / 207 us at 4K, 105 / 101 / 130 us at 8K, 37 / 33 / 33 us at 1080p. The tile rows found
@@ -594,6 +600,7 @@ __global__ void __launch_bounds__(FE_THREADS, 5) k_frontend_runs(FrontendArgs a,
     const int tid = threadIdx.x;
     const long long slot = (long long)blockIdx.x * FE_THREADS + tid;
     const long long i = slot < a.n ? (long long)a.order[slot] : a.n;
+    const unsigned error = depth_error(r); // (loaded early, used late)
     RowTest rt;
     unsigned qd;
     const bool front = roofgs_project(a, i, slot, rt, qd);
@@ -609,6 +616,7 @@ __global__ void __launch_bounds__(FE_THREADS, 5) k_frontend_runs(FrontendArgs a,
     if (tid == 0) {
         if (nvis) atomicAdd(&a.ctr->n_visible, (unsigned)nvis);
         if (nfront) atomicAdd(&a.ctr->n_front, (unsigned)nfront);
+        if (error) atomicOr(&a.ctr->error, error);
     }
 }
 
@@ -809,7 +817,10 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
     bool front = false, vis = false;
     int rows_l = 0;
     unsigned tiles = 0;
-    const unsigned i = slot < a.n ? a.order[slot] : 0u; // below n
+    const unsigned error = depth_error(r); // (loaded early, used late)
+    const unsigned ordered = slot < a.n ? a.order[slot] : 0xffffffffu;
+    const bool here = ordered < (unsigned long long)a.n; // (a slot that a timed-out depth sort left out holds anything)
+    const unsigned i = here ? ordered : 0u;
     // The colour's SH rows (192 bytes each, in depth order anywhere in memory) come asynchronously, half a
     // row at a time, six lanes to a row; each thread reads its own from shared memory. A thread loading its
     // own row touched 32 lines with every instruction, which filled the L1 pipe.
@@ -830,9 +841,9 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         __syncwarp();
     };
-    const float4 m = slot < a.n ? __ldg(&a.geo[3 * (size_t)i]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const float4 m = here ? __ldg(&a.geo[3 * (size_t)i]) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float pz = view_z(a.cam, m.x, m.y, m.z);
-    front = slot < a.n && pz > a.cam.zn && pz <= a.cam.zf;
+    front = here && pz > a.cam.zn && pz <= a.cam.zf;
     fetch(__ballot_sync(0xffffffffu, front), 0);
     Binned b;
     if (front) {
@@ -861,7 +872,7 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
         row = exact_row(b, mean, quad, undefined, any);
         if (any || keep_all) rows_l = b.ty1 - b.ty0 + 1;
     }
-    if (slot < a.n) a.touched[i] = tiles;
+    if (here) a.touched[i] = tiles;
     arrived();
     if (vis) {
         exact_colour<6, 12>(Y, a.sh_degree, c, [&](int v) { return own[v - 6]; });
@@ -888,6 +899,7 @@ __global__ void __launch_bounds__(FE_THREADS, 4) k_exact_runs(ExactArgs a, RunAr
     if (tid == 0) {
         if (nvis) atomicAdd(&a.ctr->n_visible, (unsigned)nvis);
         if (nfront) atomicAdd(&a.ctr->n_front, (unsigned)nfront);
+        if (error) atomicOr(&a.ctr->error, error);
         sum = 0;
         for (int q = 0; q < FE_WARPS; q++) sum += s_sum[q];
         if (sum) atomicAdd(&a.ctr->n_entries_total, sum);

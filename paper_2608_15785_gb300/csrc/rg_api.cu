@@ -208,7 +208,7 @@ __global__ void k_clear(uint4* p, unsigned n)
     if (i < n) p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// one device word set from the stream (test hook of RG_FLAG_TEST_STALL_SORT)
+// one device word set from the stream (test hooks RG_FLAG_TEST_STALL_SORT, RG_FLAG_TEST_STALL_DEPTH)
 __global__ void k_set_word(unsigned* p, unsigned v) { *p = v; }
 
 // entries (8 B each) the key buffers are sized for: the capacity, and the runs of an ordinary frame
@@ -273,6 +273,7 @@ size_t run_views(const Workspace& w, int64_t n, const Layout& L, RunArgs& a)
     a.kept = reinterpret_cast<unsigned*>(w.ctrl.as<unsigned char>() + RUN_KEPT_AT);
     a.ranges = w.ranges.as<uint2>();
     a.ctr = w.ctrl.as<Counters>();
+    a.depth_ctr = reinterpret_cast<const Counters*>(w.ctrl.as<unsigned char>() + CTRL_BYTES);
     a.order = tile_order(w, a.rows * a.cols);
     unsigned char* const p = w.runbuf.as<unsigned char>();
     size_t at = 0;
@@ -614,6 +615,11 @@ rg_status render_once(rg_scene* s, Workspace& w, const FrameLayout& F, int mode,
                      (unsigned)(CTRL_ALLOC / 16));
     if (flags & RG_FLAG_TEST_STALL_SORT) { // tile 0 of the first entry-sort pass is never claimed
         k_set_word<<<1, 1, 0, st>>>(&ctr->sort_tile_ctr[0], 1u);
+        RG_CK(cudaGetLastError());
+    }
+    if (flags & RG_FLAG_TEST_STALL_DEPTH) { // the depth sort's
+        k_set_word<<<1, 1, 0, st>>>(
+            &reinterpret_cast<Counters*>(w.ctrl.as<unsigned char>() + CTRL_BYTES)->sort_tile_ctr[0], 1u);
         RG_CK(cudaGetLastError());
     }
     // (the stall hook needs an entry sort to stall: its frames take the radix passes)

@@ -640,6 +640,7 @@ struct RunArgs {
     uint2* ranges;     // [rows * cols] [start, end) of every tile, [0, 0) if empty
     TileOrder order;   // filled too if order.list is set
     Counters* ctr;
+    const Counters* depth_ctr; // the depth sort's
     Sticky* sticky;
 };
 unsigned run_chunk_cap(unsigned run_cap, int rows, unsigned blocks);

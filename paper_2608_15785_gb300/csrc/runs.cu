@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(OFF_SEGS* OFF_COLS) k_run_offsets(RunArgs a)
         }
         const unsigned long long total = a.box_total ? a.ctr->n_entries_total : all;
         if (total > cap) kept_before(a, row, before, all);
-        if (lane == 0) s_start = (unsigned)before;
+        if (lane == 0) s_start = (unsigned)(before < cap ? before : cap);
         if (lane == 0 && row == 0) {
             a.ctr->n_entries = (unsigned)(total <= cap ? total : (a.box_total ? cap : all));
             if (total > cap) {
@@ -679,7 +679,7 @@ __device__ __forceinline__ void small_offsets(const RunArgs& a, const RunRow& r,
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
         }
-        if (lane == 0) S.start = (unsigned)before;
+        if (lane == 0) S.start = (unsigned)(before < cap ? before : cap);
         if (lane == 0 && blockIdx.x == 0 && row == 0) {
             a.ctr->n_entries = (unsigned)(total <= cap ? total : (a.box_total ? cap : all));
             if (total > cap) {

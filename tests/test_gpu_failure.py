@@ -85,3 +85,25 @@ def test_server_request_reports_the_timeout():
                 torch.cuda.synchronize()
                 assert torch.equal(out, ref)
         srv.close()
+
+
+@pytest.mark.parametrize("mode", ["roofgs", "exact"])
+@pytest.mark.parametrize("n", [20_000, 60_000])
+def test_stalled_depth_order_times_out_and_reports(mode, n):
+    """The order of the Gaussians runs out its bounded wait: slots that it left out are no Gaussians, the call given stats and
+    the next check report the timeout, and the scene renders as before afterwards."""
+    cam = synth.tiny_camera(256, 256)
+    gs = binding.Scene(synth.tiny_scene(n, seed=0))
+    ref = gs.render(cam, mode=mode).clone()
+    gs.check()
+    gs.render(cam, mode=mode, flags=binding.RG_FLAG_TEST_STALL_DEPTH)
+    with pytest.raises(binding.RgError) as e:
+        gs.check()
+    assert e.value.status == RG_ERR_TIMEOUT
+    with pytest.raises(binding.RgError) as e:
+        gs.render(cam, mode=mode, flags=binding.RG_FLAG_TEST_STALL_DEPTH, stats=True)
+    assert e.value.status == RG_ERR_TIMEOUT
+    with pytest.raises(binding.RgError):
+        gs.check()
+    assert torch.equal(gs.render(cam, mode=mode), ref)
+    gs.check()
