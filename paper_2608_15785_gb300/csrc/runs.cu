@@ -176,7 +176,7 @@ __device__ __noinline__ void cut_by_rows(const RunArgs& a, unsigned long long* s
 }
 
 // One block of 1024 threads per tile row: a scan of the blocks' counts, and the row's chunks.
-__global__ void __launch_bounds__(1024) k_run_rows(RunArgs a)
+__global__ void __launch_bounds__(1024, 2) k_run_rows(RunArgs a)
 {
     constexpr int WARPS = 32;
     __shared__ unsigned s_r[WARPS];
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(1024) k_run_rows(RunArgs a)
     __shared__ unsigned s_chunk;
     grid_dependency_wait();
     const unsigned row = blockIdx.x, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    if (a.box_total && a.ctr->n_entries_total > (unsigned long long)a.cap) cut_by_rows<WARPS>(a, s_e);
+    const unsigned long long boxes = a.box_total ? a.ctr->n_entries_total : 0ull; // (loaded early, used late)
     const unsigned* const cnt = a.cnt + (size_t)row * a.blocks;
     const unsigned per = (a.blocks + 32u * WARPS - 1u) / (32u * WARPS), b0 = tid * per;
     const unsigned b1 = b0 + per < a.blocks ? b0 + per : a.blocks;
@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(1024) k_run_rows(RunArgs a)
         s_chunk = chunk;
     }
     __syncthreads();
+    if (boxes > (unsigned long long)a.cap) cut_by_rows<WARPS>(a, s_e);
     if (!rtot || b0 >= b1) return;
     p = rend - p;
     e = ebefore + ex - e;
@@ -394,10 +395,11 @@ __global__ void __launch_bounds__(RUN_THREADS, 6) k_run_collect(RunArgs a)
     __shared__ CollectSmem S;
     grid_dependency_wait();
     const unsigned row = blockIdx.y;
+    const unsigned long long total = a.ctr->n_entries_total;
+    const uint2 cut = make_uint2(a.ctr->cut, a.ctr->cut_tiles);
     const RunRow r = a.row[row];
     if (blockIdx.x >= r.nchunks) return;
-    const bool clip = a.ctr->n_entries_total > (unsigned long long)a.cap;
-    const uint2 cut = make_uint2(a.ctr->cut, a.ctr->cut_tiles);
+    const bool clip = total > (unsigned long long)a.cap;
     unsigned long long start = 0;
     if (clip && !a.box_total)
         for (unsigned q = 0; q < row; q++) start += a.row[q].entries;
@@ -424,6 +426,7 @@ __global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
     static_assert(RUN_SMALL_BLOCKS <= RUN_THREADS, "one thread per front-end block");
     grid_dependency_wait();
     const unsigned row = blockIdx.y, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const unsigned long long boxes = a.box_total ? a.ctr->n_entries_total : 0ull;
     if (warp == RUN_WARPS - 1) { // totals of the earlier rows, and of the frame
         unsigned long long before = 0, all = 0;
         for (unsigned q = lane; (int)q < a.rows; q += 32) {
@@ -465,7 +468,7 @@ __global__ void __launch_bounds__(RUN_THREADS) k_run_collect_small(RunArgs a)
     }
     if (blockIdx.x >= r.nchunks) return;
     if (tid == s_first) a.chunk[r.chunk + blockIdx.x] = RunChunk{tid, p, 0ull};
-    const bool clip = (a.box_total ? a.ctr->n_entries_total : s_all) > (unsigned long long)a.cap;
+    const bool clip = (a.box_total ? boxes : s_all) > (unsigned long long)a.cap;
     unsigned long long entry = s_before & RUN_TOT_ENTRIES;
     uint2 cut = make_uint2(0u, 0u);
     if (clip && a.box_total) {
@@ -672,13 +675,10 @@ __device__ __forceinline__ void small_offsets(const RunArgs& a, const RunRow& r,
     if (warp == RUN_WARPS - 1) {
         const unsigned long long total = a.ctr->n_entries_total;
         unsigned long long before = 0, all = 0;
-        if (total > cap) {
-            kept_before(a, row, before, all);
-        } else {
-            for (unsigned q = lane; q < row; q += 32) before += a.tot[q] & RUN_TOT_ENTRIES;
+        for (unsigned q = lane; q < row; q += 32) before += a.tot[q] & RUN_TOT_ENTRIES;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-        }
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        if (total > cap) kept_before(a, row, before, all);
         if (lane == 0) S.start = (unsigned)(before < cap ? before : cap);
         if (lane == 0 && blockIdx.x == 0 && row == 0) {
             a.ctr->n_entries = (unsigned)(total <= cap ? total : (a.box_total ? cap : all));
