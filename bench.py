@@ -43,10 +43,10 @@ REASONS = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_powe
 # clock. Warp instructions per evaluated (Gaussian, pixel) pair of the timed kernel
 # (k_raster_roofgs<fast exp, 4 pixels per thread>: pixel pairs blended with packed FP32x2
 # FMAs, skip thresholds, one skip and one stop branch per thread and Gaussian, two records
-# per loop iteration), from ncu on a 1M-Gaussian 4K frame: smsp__inst_executed.sum 334.3 M for
+# per loop iteration), from ncu on a 1M-Gaussian 4K frame: smsp__inst_executed.sum 335.3 M for
 # 534.0 M evaluated pairs. The pair count of the timed frames comes from the counting variant
 # of the same kernel.
-RASTER_WARP_INST_PER_PAIR = 334.3 / 534.0
+RASTER_WARP_INST_PER_PAIR = 335.3 / 534.0
 # Source-level FP32/ALU-pipe instruction counts of the rasterizers' inner loops (per
 # evaluated exponent, per pair inside the alpha >= 1/255 range), kept as a second,
 # model-based view: RoofGS 4 + 1 range test, blend 11; exact 10, blend 20.

@@ -3,7 +3,8 @@
  *
  * Forward render of 3D Gaussian Splatting in two modes:
  *   RG_MODE_EXACT   the plain 3DGS path: FP32 attributes (236 bytes per
- *                   Gaussian, paper Sec. III-A, Eq. (3)), entries in the order
+ *                   Gaussian, paper Sec. III-A, Eq. (3); a resident scene keeps their
+ *                   geometry a second time, 48 bytes), entries in the order
  *                   of 64-bit tile|float-depth keys (Sec. IV-A.2), IEEE expf in
  *                   the rasterizer (Eqs. (7), (10)-(12));
  *   RG_MODE_ROOFGS  the paper's method: compact attributes (FP32 mean, FP16
@@ -202,7 +203,9 @@ rg_status rg_trim(void);
 rg_status rg_scene_save(rg_scene* scene, const char* path);
 rg_status rg_scene_load(const char* path, void* stream, rg_scene** out);
 
-/* Grow the frame workspace to hold at least n_entries (tile, Gaussian) entries. Synchronous. */
+/* Grow the frame workspace to hold at least n_entries (tile, Gaussian) entries (24 bytes each; two buffers of 8 bytes
+ * an entry are sized for at least 4 entries per Gaussian). Synchronous. Frames of grids with no more tiles than an
+ * earlier one's can be captured into a graph afterwards. */
 rg_status rg_scene_reserve(rg_scene* scene, int64_t n_entries);
 
 /*

@@ -24,7 +24,8 @@
 // column at a time, 405 us at 4K with 3 M Gaussians; five blocks and two columns at a time 281 us).
 // Kernel times (ncu) of the front end and the grouping, with every entry written, against the scatter by
 // tile row with one radix pass it replaced: 4K, 3 M Gaussians 792 -> 591 us (front end 201, rows 14,
-// collect 85, offsets 11, expand 281; limited frames: expand 175, see k_run_expand); 8K, 1 M, against the fused front end with three radix passes 1295 -> 541 us; 1080p,
+// collect 85, offsets 11, expand 281, in windows of 120 columns; limited frames: expand 175, see k_run_expand); 8K, 1 M, against the fused front end with
+// three radix passes 1295 -> 541 us; 1080p,
 // 500 k 93 -> 89 us; 256 x 256, 10 k 35 -> 26 us.
 #include "rg_internal.cuh"
 
